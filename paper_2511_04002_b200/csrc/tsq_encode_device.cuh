@@ -1,0 +1,681 @@
+// Device code shared by the encode kernels: AIQ parameters of a level, the vector passes over a 32-element group,
+// the placement look-back and the blob's header and per-token fields.  Included by one .cu file per kernel.
+#ifndef TSQ_ENCODE_DEVICE_CUH_
+#define TSQ_ENCODE_DEVICE_CUH_
+
+#include "tsq_device.cuh"
+#include "tsq_internal.h"
+
+namespace tsq {
+namespace {
+
+constexpr float kRoundMagic = 8388608.0f;  // 2^23: adding it to 0 <= y < 2^23 rounds y to an integer, ties to even
+constexpr uint32_t kLookbackPollLimit = 1u << 20;  // polls of one descriptor (200 ns to 1 us apart): about a second
+constexpr uint32_t kHandshakeFactor = 4u;          // handshakes inside a CTA poll faster: four times as many polls
+
+// AIQ parameters of one candidate level for one row (Eq. "Proposed").
+struct __align__(16) Level {
+  float s;    // scale
+  float r;    // fl(1 / s)
+  int zp;     // zero-point rint(m_min / s)
+  int qmax;   // 2^(b-1) - 1
+};
+
+// *plain: the fast steps apply to the level: FMA quotient safe, zero-point 0, no code needs the clamp (see the file header).
+__device__ __forceinline__ Level make_level(float mmin, float mmax, int b, bool* plain) {
+  Level c;
+  c.qmax = (1 << (b - 1)) - 1;
+  const float range = __fsub_rn(mmax, mmin);
+  c.s = range > 0.0f ? __fdiv_rn(range, static_cast<float>(c.qmax)) : (mmax > 0.0f ? mmax : 1.0f);
+  c.zp = mmin > 0.0f ? __float2int_rn(__fdiv_rn(mmin, c.s)) : 0;  // 0 / s = 0: the usual row needs no division here
+  c.r = __frcp_rn(c.s);
+  // Plain: no intermediate of the FMA quotient can leave the normal range, the zero-point is 0 (so no code is
+  // negative) and the largest magnitude's code needs no clamp (codes grow with the magnitude).  With a minimum
+  // of 0 the scale is fl(max / Qmax) and max / scale rounds to Qmax: no division needed to know.
+  *plain = (c.s >= 0x1p-60f) && (c.s <= 0x1p60f) && c.zp == 0 &&
+           (mmin == 0.0f || __float2int_rn(__fdiv_rn(mmax, c.s)) <= c.qmax);
+  return c;
+}
+
+// The signed-values variant (Eq. "Proposed" on the signed inliers): Q_max = 2^b - 1, the zero-point may be
+// negative, a constant row takes its own magnitude as the scale.  *plain: the fast steps apply: the FMA quotient is
+// safe and no code needs a clamp (codes grow with the value, the smallest is 0 by construction, so the largest
+// value's code decides); the zero-point is then subtracted byte-wise, modulo 256.
+__device__ __forceinline__ Level make_level_signed(float vmin, float vmax, int b, bool* plain) {
+  Level c;
+  c.qmax = (1 << b) - 1;
+  // two finite values of opposite sign can lie further apart than binary32 holds: the largest finite value then
+  const float range = fminf(__fsub_rn(vmax, vmin), 3.40282346638528859811704183484516925e+38f);
+  const float a = fabsf(vmax);
+  c.s = range > 0.0f ? __fdiv_rn(range, static_cast<float>(c.qmax)) : (a > 0.0f ? a : 1.0f);
+  c.zp = __float2int_rn(__fdiv_rn(vmin, c.s));
+  c.r = __frcp_rn(c.s);
+  *plain = (c.s >= 0x1p-60f) && (c.s <= 0x1p60f) && (__float2int_rn(__fdiv_rn(vmax, c.s)) - c.zp <= c.qmax);
+  return c;
+}
+
+// 16-bit patterns of signed values <-> 16-bit keys that order like the values (-0 just below +0).
+__device__ __forceinline__ uint32_t order_keys2(uint32_t v2) {
+  return v2 ^ 0x80008000u ^ (((v2 >> 15) & 0x10001u) * 0x7fffu);
+}
+__device__ __forceinline__ uint32_t pattern_of_key(uint32_t key) { return (key & 0x8000u) ? key ^ 0x8000u : key ^ 0xffffu; }
+
+// Codes of the two elements of a 16-bit pair, as two 16-bit integers, by the division instruction: for rows
+// that are not plain.  SV = false: codes of the magnitudes (sign bits ignored); SV = true: of the signed values.
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ uint32_t codes2_divide(uint32_t x, const Level& c) {
+  using E = Elem<BF16>;
+  const float lo = SV ? E::lo_f32(x) : fabsf(E::lo_f32(x)), hi = SV ? E::hi_f32(x) : fabsf(E::hi_f32(x));
+  const int klo = __vimin_s32_relu(__float2int_rn(__fdiv_rn(lo, c.s)) - c.zp, c.qmax);
+  const int khi = __vimin_s32_relu(__float2int_rn(__fdiv_rn(hi, c.s)) - c.zp, c.qmax);
+  return static_cast<uint32_t>(klo) | (static_cast<uint32_t>(khi) << 16);
+}
+
+// ---- plain rows: two elements at a time with the packed binary32 instructions (each lane IEEE round-to-nearest-even) ----
+struct Level2 {
+  uint64_t r2, ns2;  // {r, r} and {-s, -s}
+  uint32_t zp4;      // signed-values variant: the zero-point modulo 256 in every byte
+};
+__device__ __forceinline__ Level2 make_level2(const Level& c) {
+  Level2 l;
+  l.r2 = pack2f(c.r, c.r);
+  l.ns2 = pack2f(-c.s, -c.s);
+  l.zp4 = (static_cast<uint32_t>(c.zp) & 0xffu) * 0x01010101u;
+  return l;
+}
+// Magnitudes of the two elements of a 16-bit pair as packed binary32.
+template <bool BF16>
+__device__ __forceinline__ uint64_t magnitudes2(uint32_t x) {
+  const uint32_t a = x & 0x7fff7fffu;
+  if (BF16) return pack2u(mad_u32(a, 65536u, 0u), a & 0xffff0000u);
+  const float2 f = __half22float2(Elem<false>::as2(a));
+  return pack2f(f.x, f.y);
+}
+// rint(fl(m / s)) + 2^23 in both lanes: q0 = fl(m r), the residual m - q0 s (one FMA, exact), q = fl(q0 + residual r),
+// then the addition that rounds to an integer.  The code is the low byte of the result's pattern.
+__device__ __forceinline__ uint64_t quotient2(uint64_t m2, const Level2& l, uint64_t magic2) {
+  const uint64_t q0 = mul2(m2, l.r2);
+  const uint64_t e = fma2(q0, l.ns2, m2);
+  const uint64_t q = fma2(e, l.r2, q0);
+  return add2(q, magic2);
+}
+// Low bytes of four patterns 2^23 + k (k < 256) as one word: bytes a.lo, b.lo, a.hi, b.hi.
+__device__ __forceinline__ uint32_t bytes4(uint64_t ta, uint64_t tb) {
+  uint32_t alo, ahi, blo, bhi;
+  unpack2u(ta, alo, ahi);
+  unpack2u(tb, blo, bhi);
+  return __byte_perm(mad_u32(blo, 256u, alo), mad_u32(bhi, 256u, ahi), 0x5410);
+}
+
+// 2^23 rounds a non-negative quotient to an integer; 2^23 + 2^22 does the same for |quotient| < 2^22 of either sign
+// and leaves the integer, modulo 2^22, in the low bits of the pattern (two's complement).
+constexpr float kRoundMagicSigned = 12582912.0f;
+// The signed values of the two elements of a 16-bit pair as packed binary32 (signed-values variant).
+template <bool BF16>
+__device__ __forceinline__ uint64_t values2(uint32_t x) {
+  if (BF16) return pack2u(mad_u32(x, 65536u, 0u), x & 0xffff0000u);
+  const float2 f = __half22float2(Elem<false>::as2(x));
+  return pack2f(f.x, f.y);
+}
+// Low bytes of four patterns as one word (bytes a.lo, b.lo, a.hi, b.hi) when the patterns' other bytes are not
+// zero (a negative rounded quotient): byte permutes only.
+__device__ __forceinline__ uint32_t bytes4_any(uint64_t ta, uint64_t tb) {
+  uint32_t alo, ahi, blo, bhi;
+  unpack2u(ta, alo, ahi);
+  unpack2u(tb, blo, bhi);
+  return __byte_perm(__byte_perm(alo, blo, 0x0040), __byte_perm(ahi, bhi, 0x0040), 0x5410);
+}
+// The codes of four elements (pairs xa, xb) at level l as bytes a.lo, b.lo, a.hi, b.hi.  SV: of the signed values,
+// zero-point subtracted modulo 256 (exact for a plain level: every code lies in [0, 255]).
+template <bool BF16, bool SV>
+__device__ __forceinline__ uint32_t codes4(uint32_t xa, uint32_t xb, const Level2& l) {
+  if (SV) {
+    const uint64_t magic2 = pack2f(kRoundMagicSigned, kRoundMagicSigned);
+    return __vsub4(bytes4_any(quotient2(values2<BF16>(xa), l, magic2), quotient2(values2<BF16>(xb), l, magic2)), l.zp4);
+  }
+  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+  return bytes4(quotient2(magnitudes2<BF16>(xa), l, magic2), quotient2(magnitudes2<BF16>(xb), l, magic2));
+}
+
+__device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.s16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t min_s16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("min.s16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// Pass A on one group held in x[16] (pair i of chunk j in x[4j + i]; chunks j >= nvalid lie past the
+// end of the row and hold zeros): outlier slots become +0, bit e of the result flags element e of
+// the group, mn2 / mx2 collect the inlier magnitudes.
+template <bool BF16>
+__device__ __forceinline__ uint32_t split_group(uint32_t (&x)[16], uint32_t nvalid, uint32_t thr2, uint32_t& mn2,
+                                                uint32_t& mx2) {
+  using E = Elem<BF16>;
+  uint32_t bitmap = 0u;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (static_cast<uint32_t>(j) >= nvalid) continue;
+    uint32_t acc = 0u;  // bit 2i / bit 17 + 2i flag the low / high element of pair i
+    uint32_t m2[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t a = x[4 * j + i] & 0x7fff7fffu;
+      const uint32_t mk = E::geu_mask(a, thr2);  // 0xffff in each half with |x| >= tau, NaN included
+      m2[i] = a & ~mk;
+      x[4 * j + i] &= ~mk;
+      acc |= mk & ((1u << (2 * i)) | (1u << (17 + 2 * i)));
+    }
+    // patterns of non-negative values order like the values: integer min / max
+    mx2 = __vimax3_u16x2(mx2, m2[0], m2[1]);
+    mx2 = __vimax3_u16x2(mx2, m2[2], m2[3]);
+    mn2 = __vimin3_u16x2(mn2, m2[0], m2[1]);
+    mn2 = __vimin3_u16x2(mn2, m2[2], m2[3]);
+    bitmap |= ((acc | (acc >> 16)) & 0xffu) << (8 * j);
+  }
+  return bitmap;
+}
+
+// Pass B on one group of a plain row: sum |(q0 >> sh) - q| over its 32 elements (Algorithm 1's distortion
+// numerator).  Four codes travel as the bytes of one word: the shift and mask take four at a time, and the
+// byte-wise sum-of-absolute-differences instruction adds the four differences.
+// SV (signed-values variant): 8-bit codes of the signed values; the chunks at and past `nvalid` lie beyond the end
+// of the row and do not count (their zeros would get the code of the value 0, which is not 0 there).
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ uint32_t distortion_group(const uint32_t (&x)[16], const Level2& top, const Level2& low, int sh,
+                                                     uint32_t nvalid = 4u) {
+  const uint32_t shmask = ((SV ? 0xffu : 0x7fu) >> sh) * 0x01010101u;
+  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+  uint32_t S = 0;
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) {
+    if (SV) {
+      if (static_cast<uint32_t>(i / 4) >= nvalid) continue;
+      S = __vsadu4((codes4<BF16, true>(x[i], x[i + 1], top) >> sh) & shmask, codes4<BF16, true>(x[i], x[i + 1], low)) + S;
+      continue;
+    }
+    const uint64_t ma = magnitudes2<BF16>(x[i]), mb = magnitudes2<BF16>(x[i + 1]);
+    const uint32_t ct4 = bytes4(quotient2(ma, top, magic2), quotient2(mb, top, magic2));
+    const uint32_t q4 = bytes4(quotient2(ma, low, magic2), quotient2(mb, low, magic2));
+    S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
+  }
+  return S;
+}
+
+// Pass B for the first lower candidate, keeping what pass C needs if that candidate fails: on return tb[4h + i]
+// holds the top-level bytes (code | sign << 7) of elements 16h + 2i, 16h + 8 + 2i, 16h + 2i + 1, 16h + 8 + 2i + 1 (pair i
+// of chunks 2h and 2h + 1, low elements first) and ql the candidate's own codes in the same grouping, no signs.
+// (Any grouping of four serves the sum; this one costs the byte assembly least, and two byte permutes per i
+// turn it into the input of the bit transpose.)
+// SV: bytes are the 8-bit codes of the signed values, no signs; bytes of chunks at and past `nvalid` are 0.
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ uint32_t distortion_first(const uint32_t (&x)[16], const Level2& top, const Level2& low, int sh,
+                                                     uint32_t (&tb)[8], uint32_t (&ql)[8], uint32_t nvalid = 4u) {
+  const uint32_t shmask = ((SV ? 0xffu : 0x7fu) >> sh) * 0x01010101u;
+  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+  uint32_t S = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    // bytes 0 and 2 of a word belong to chunk 2h, bytes 1 and 3 to chunk 2h + 1
+    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];  // pairs i of chunks 2h and 2h + 1
+      if (SV) {
+        const uint32_t ct4 = codes4<BF16, true>(xa, xb, top) & inside, q4 = codes4<BF16, true>(xa, xb, low) & inside;
+        S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
+        tb[4 * h + i] = ct4;
+        ql[4 * h + i] = q4;
+        continue;
+      }
+      const uint64_t ma = magnitudes2<BF16>(xa), mb = magnitudes2<BF16>(xb);
+      const uint32_t ct4 = bytes4(quotient2(ma, top, magic2), quotient2(mb, top, magic2));
+      const uint32_t q4 = bytes4(quotient2(ma, low, magic2), quotient2(mb, low, magic2));
+      S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
+      tb[4 * h + i] = ct4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);  // the sign bits sit in bytes 1 and 3 of a pair
+      ql[4 * h + i] = q4;
+    }
+  }
+  return S;
+}
+
+// Pass B for a further candidate: the top-level codes come from the bytes the first turn left.
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ uint32_t distortion_next(const uint32_t (&x)[16], const uint32_t (&tb)[8], const Level2& low, int sh,
+                                                    uint32_t (&ql)[8], uint32_t nvalid = 4u) {
+  // a byte of tb is code | sign << 7 (SV: an 8-bit code): shifted right by sh >= 1, the sign bit and the bits that
+  // come in from the next byte all land above the mask
+  const uint32_t shmask = ((SV ? 0xffu : 0x7fu) >> sh) * 0x01010101u;
+  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+  uint32_t S = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (SV) {
+        const uint32_t q4 = codes4<BF16, true>(x[8 * h + i], x[8 * h + 4 + i], low) & inside;
+        S = __vsadu4((tb[4 * h + i] >> sh) & shmask, q4) + S;
+        ql[4 * h + i] = q4;
+        continue;
+      }
+      const uint32_t q4 = bytes4(quotient2(magnitudes2<BF16>(x[8 * h + i]), low, magic2),
+                                 quotient2(magnitudes2<BF16>(x[8 * h + 4 + i]), low, magic2));
+      S = __vsadu4((tb[4 * h + i] >> sh) & shmask, q4) + S;
+      ql[4 * h + i] = q4;
+    }
+  }
+  return S;
+}
+
+// Bytes of one group as distortion_first leaves them -> bit-planes: on return r[k] = bit k of every byte,
+// k < 7 code bits, k = 7 signs.
+__device__ __forceinline__ void planes_of_bytes(const uint32_t (&tb)[8], uint32_t (&r)[8]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    r[2 * i] = __byte_perm(tb[i], tb[4 + i], 0x5410);      // byte c = element 8c + 2i
+    r[2 * i + 1] = __byte_perm(tb[i], tb[4 + i], 0x7632);  // byte c = element 8c + 2i + 1
+  }
+  transpose8x32_select(r);
+}
+
+// Pass C on one group of a row whose chosen level is plain: codes as bytes (code | sign << 7), transposed into
+// bit-planes: on return r[k] = bit k of every byte, k < 7 code bits, k = 7 signs.
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ void pack_group(const uint32_t (&x)[16], const Level2& lv, uint32_t (&r)[8], uint32_t nvalid = 4u) {
+  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+  uint32_t tb[8];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
+      if (SV) {
+        tb[4 * h + i] = codes4<BF16, true>(xa, xb, lv) & inside;
+        continue;
+      }
+      const uint32_t c4 = bytes4(quotient2(magnitudes2<BF16>(xa), lv, magic2), quotient2(magnitudes2<BF16>(xb), lv, magic2));
+      tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
+    }
+  }
+  planes_of_bytes(tb, r);
+}
+
+// The same steps with the division instruction, for one group held in registers (the one-CTA-per-row kernel).
+// (SV: the zeros past the end of a row would get non-zero codes under a negative zero-point, so only the
+// first `pairs` registers, the ones inside the row, count.)
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ uint32_t divide_distortion_regs(const uint32_t (&x)[16], const Level& top, const Level& low, int sh,
+                                                           uint32_t pairs = 16u) {
+  const uint32_t shmask = (0xffffu >> sh) * 0x10001u;
+  uint32_t S = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    if (SV && static_cast<uint32_t>(i) >= pairs) continue;
+    const uint32_t a = (codes2_divide<BF16, SV>(x[i], top) >> sh) & shmask;
+    const uint32_t q = codes2_divide<BF16, SV>(x[i], low);
+    const uint32_t d = max_s16x2(a, q) - min_s16x2(a, q);
+    S += (d & 0xffffu) + (d >> 16);
+  }
+  return S;
+}
+
+struct Planes8 {
+  uint32_t v[8];
+};
+template <bool BF16, bool SV = false>
+__device__ __forceinline__ void divide_pack_regs(const uint32_t (&x)[16], const Level& lv, uint32_t (&r)[8]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) r[k] = 0u;  // r[k] bit e = bit k of the byte (code | sign << 7; SV: the 8-bit code) of element e
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    // elements 2i (byte 0) and 2i + 1 (byte 2)
+    const uint32_t b2 = codes2_divide<BF16, SV>(x[i], lv) | (SV ? 0u : ((x[i] >> 8) & 0x00800080u));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r[k] |= (((b2 >> k) & 1u) << (2 * i)) | (((b2 >> (16 + k)) & 1u) << (2 * i + 1));
+  }
+}
+
+// The same two steps for rows that need the division instruction, written as loops over the parked
+// row's words (xw: the row as 32-bit words) so that they take little room in the instruction stream.
+__device__ __forceinline__ uint32_t park_index(uint32_t nt, uint32_t u, uint32_t j);
+// (SV: only the first `pairs` words, the ones inside the row, count: see divide_distortion_regs.)
+template <bool BF16, bool SV = false>
+__device__ __noinline__ uint32_t rolled_distortion(const uint32_t* xw, uint32_t nt, uint32_t u, Level top, Level low, int sh,
+                                                   uint32_t pairs = 16u) {
+  const uint32_t shmask = (0xffffu >> sh) * 0x10001u;
+  uint32_t S = 0;
+#pragma unroll 1
+  for (uint32_t i = 0; i < (SV ? pairs : 16u); ++i) {
+    const uint32_t x = xw[4u * park_index(nt, u, i >> 2) + (i & 3u)];
+    const uint32_t a = (codes2_divide<BF16, SV>(x, top) >> sh) & shmask;
+    const uint32_t q = codes2_divide<BF16, SV>(x, low);
+    const uint32_t d = max_s16x2(a, q) - min_s16x2(a, q);
+    S += (d & 0xffffu) + (d >> 16);
+  }
+  return S;
+}
+template <bool BF16, bool SV = false>
+__device__ __noinline__ Planes8 rolled_pack(const uint32_t* xw, uint32_t nt, uint32_t u, Level lv, uint32_t pairs = 16u) {
+  uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // r[k] bit e = bit k of the byte (code | sign << 7; SV: the 8-bit code) of element e
+#pragma unroll 1
+  for (uint32_t i = 0; i < (SV ? pairs : 16u); ++i) {
+    const uint32_t x = xw[4u * park_index(nt, u, i >> 2) + (i & 3u)];
+    // elements 2i (byte 0) and 2i + 1 (byte 2)
+    const uint32_t b2 = codes2_divide<BF16, SV>(x, lv) | (SV ? 0u : ((x >> 8) & 0x00800080u));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r[k] |= (((b2 >> k) & 1u) << (2u * i)) | (((b2 >> (16 + k)) & 1u) << (2u * i + 1u));
+  }
+  Planes8 out;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) out.v[k] = r[k];
+  return out;
+}
+
+// Shared-memory index (in 16-byte chunks) of chunk j of group u inside a parked row of nt groups: a group's
+// four chunks stay together, rotated so that the 16-byte accesses of neighbouring threads fall into
+// different banks.  (Keeping the chunks with the same j side by side instead measured 8 % slower while the
+// copies bypassed L1, and no faster than this since they do not.)
+__device__ __forceinline__ uint32_t park_index(uint32_t /*nt*/, uint32_t u, uint32_t j) { return 4u * u + ((j + (u >> 1)) & 3u); }
+
+// Number of 16-byte chunks of group u that lie inside the row (4, fewer in the last group, 0 beyond it).
+// Recomputed where it is needed: a value kept alive across the whole row loop costs a register there.
+__device__ __forceinline__ uint32_t group_chunks(const EncodeParams& p, uint32_t u) {
+  return 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
+}
+
+// Asynchronous copy of the 64 bytes of group u of row `tile` into parked row `slot` (chunks
+// j >= nvalid lie past the end of the row and are not copied).
+__device__ __forceinline__ void fetch_group(const EncodeParams& p, uint4* xpark, uint32_t tile, uint32_t slot, uint32_t u,
+                                            uint32_t nvalid) {
+  const uint4* xrow = reinterpret_cast<const uint4*>(p.x + static_cast<size_t>(tile) * p.hidden);
+  uint4* xp = xpark + slot * (p.park_stride / 16u);
+#pragma unroll
+  for (uint32_t j = 0; j < 4; ++j) {
+    if (j < nvalid) cp_async16(&xp[park_index(p.compute_threads, u, j)], &xrow[4u * u + j]);
+  }
+  cp_async_commit();
+}
+
+// The CSR entries (column << 16 | original pattern) of the elements of one group that `bm` flags, in
+// ascending column order, from the group's 64 bytes as they stand in the input (v[j] = chunk j): f(entry) is
+// called once per flagged element.  All 32 positions are visited under a predicate: no data-dependent loads.
+template <typename F>
+__device__ __forceinline__ void for_each_flagged(uint32_t bm, const uint4 (&v)[4], uint32_t col0, F&& f) {
+#pragma unroll
+  for (uint32_t j = 0; j < 4; ++j) {
+    const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) {
+      const uint32_t e = 8u * j + 2u * i;
+      if ((bm >> e) & 1u) f(((col0 + e) << 16) | (w[i] & 0xffffu));
+      if ((bm >> (e + 1u)) & 1u) f(((col0 + e + 1u) << 16) | (w[i] >> 16));
+    }
+  }
+}
+
+// The b* plane words of one group, in blob order (plane 0 = sign, plane 1 + k = code bit k), to dst.
+// SV: plane k = code bit k, no sign plane.
+template <bool SV = false>
+__device__ __forceinline__ void store_planes(uint32_t* dst, const uint32_t (&r)[8], int bstar, bool vec) {
+  if (SV) {
+    if (vec && bstar == 8) {
+      reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[0], r[1], r[2], r[3]);
+      reinterpret_cast<uint4*>(dst)[1] = make_uint4(r[4], r[5], r[6], r[7]);
+    } else if (vec && bstar == 4) {
+      reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[0], r[1], r[2], r[3]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (q < bstar) dst[q] = r[q];
+      }
+    }
+    return;
+  }
+  if (vec && bstar == 8) {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[7], r[0], r[1], r[2]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(r[3], r[4], r[5], r[6]);
+  } else if (vec && bstar == 4) {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[7], r[0], r[1], r[2]);
+  } else {
+    dst[0] = r[7];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      if (q < bstar - 1) dst[1 + q] = r[q];
+    }
+  }
+}
+
+// The row's min / max patterns, outlier total and per-warp outlier offsets from the per-warp partial
+// results, and the AIQ parameters of every candidate: run by one full warp, lane i takes candidate i.
+// Returns (in every lane) 1 when some level needs the division instruction.
+template <int NW>  // the most warps that contribute
+struct RowPartials {
+  uint32_t warp_min[NW], warp_max[NW], warp_cnt[NW];  // warp_cnt becomes an exclusive scan
+};
+template <bool BF16, int NW, bool SV = false>
+__device__ __forceinline__ uint32_t row_levels(const EncodeParams& p, RowPartials<NW>& part, uint32_t nwarps, uint32_t lane,
+                                               Level* lv_out, int* S_out, uint32_t* row_cnt) {
+  using E = Elem<BF16>;
+  const uint32_t pmin = __reduce_min_sync(kFull, lane < nwarps ? part.warp_min[lane] : 0xffffu);
+  const uint32_t pmax = __reduce_max_sync(kFull, lane < nwarps ? part.warp_max[lane] : 0u);
+  const uint32_t wc = lane < nwarps ? part.warp_cnt[lane] : 0u;
+  uint32_t incl = wc;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t n = __shfl_up_sync(kFull, incl, d);
+    if (lane >= static_cast<uint32_t>(d)) incl += n;
+  }
+  if (lane < nwarps) part.warp_cnt[lane] = incl - wc;
+  const uint32_t total = __shfl_sync(kFull, incl, 31);
+  // SV: the partial results are order keys of signed values
+  const int b = p.bits[min(lane, static_cast<uint32_t>(p.n_bits - 1))];
+  bool plain = false;
+  const Level lv = SV ? make_level_signed(E::pattern_f32(pattern_of_key(pmin)), E::pattern_f32(pattern_of_key(pmax)), b, &plain)
+                      : make_level(E::pattern_f32(pmin), E::pattern_f32(pmax), b, &plain);
+  if (lane < static_cast<uint32_t>(p.n_bits)) {
+    lv_out[lane] = lv;
+    S_out[lane] = 0;
+  }
+  if (lane == 0) *row_cnt = total;
+  return __all_sync(kFull, plain) ? 0u : 1u;
+}
+
+// The limit on device-side waits: the workspace's setting, else the built-in one.
+__device__ __forceinline__ uint32_t lookback_limit(const EncodeParams& p) {
+  const uint32_t set = *reinterpret_cast<volatile const uint32_t*>(&p.ws->poll_limit);
+  return set != 0u ? set : kLookbackPollLimit;
+}
+
+__device__ __forceinline__ unsigned long long pack_desc(uint32_t tag, uint32_t value) {
+  return (static_cast<unsigned long long>(tag) << 32) | value;
+}
+
+// Decoupled look-back over the tile descriptors.
+// Tile t owns two adjacent descriptors, desc[2t] for plane words and desc[2t + 1] for outliers, each
+// (generation * 4 + flag) << 32 | payload: an AGGREGATE payload is the tile's own size, a PREFIX
+// payload the inclusive prefix sum up to and including the tile.  Both are read in the same round
+// trip; a tile counts as published once both carry the same flag of the current generation.
+__device__ __forceinline__ void publish(const EncodeParams& p, uint32_t tag, uint32_t tile, uint32_t w, uint32_t o) {
+  st_relaxed_u64(p.desc + 2 * static_cast<size_t>(tile), pack_desc(tag, w));
+  st_relaxed_u64(p.desc + 2 * static_cast<size_t>(tile) + 1, pack_desc(tag, o));
+}
+
+__device__ __forceinline__ void publish_aggregate(const EncodeParams& p, uint32_t gen4, uint32_t tile, uint32_t agg_w,
+                                                  uint32_t agg_o) {
+  if (tile > 0) publish(p, gen4 | kFlagAggregate, tile, agg_w, agg_o);
+}
+
+// State of a tile from its two descriptors: 0 = not (consistently) published yet, else the common flag.
+__device__ __forceinline__ uint32_t tile_state(uint32_t gen4, unsigned long long vw, unsigned long long vo) {
+  const uint32_t tw = static_cast<uint32_t>(vw >> 32), to = static_cast<uint32_t>(vo >> 32);
+  const uint32_t fw = ((tw & ~3u) == gen4) ? (tw & 3u) : 0u, fo = ((to & ~3u) == gen4) ? (to & 3u) : 0u;
+  if (fw == kFlagAbort || fo == kFlagAbort) return kFlagAbort;
+  return fw == fo ? fw : 0u;
+}
+
+// Run by one full warp for its tile, after publish_aggregate: walk back to the nearest published
+// prefix, then publish this tile's own.
+// Returns TSQ_OK, TSQ_ERR_TIMEOUT (gave up) or -1 when a predecessor has aborted.
+// DEPTH = descriptor pairs each lane reads per step (32 * DEPTH tiles per round trip).  The one-CTA-per-row
+// kernel, whose rows all finish at about the same time, looks back 256 tiles at once; the pipelined
+// kernel, where the nearest finished prefix is rarely more than a few dozen tiles away and the look-back
+// runs in a lone warp that issues slowly, takes 32 (measured: 6 % faster at hidden 8192 and 20 % at
+// 1024 than with 256).
+template <int DEPTH>
+__device__ int resolve_prefix(const EncodeParams& p, uint32_t gen4, uint32_t tile, uint32_t agg_w, uint32_t agg_o,
+                              uint32_t lane, uint32_t* excl_w, uint32_t* excl_o, uint32_t poll_limit) {
+  uint32_t base_w = 0, base_o = 0;  // prefix found at the end of the walk
+  uint32_t part_w = 0, part_o = 0;  // this lane's share of the aggregates walked over
+  if (tile > 0) {
+    int pos = static_cast<int>(tile) - 1;  // nearest tile not yet accounted for
+    uint32_t polls = 0;
+    bool done = false;
+    while (!done) {
+      unsigned long long vw[DEPTH], vo[DEPTH];
+#pragma unroll
+      for (int k = 0; k < DEPTH; ++k) {
+        const int j = pos - (32 * k + static_cast<int>(lane));
+        // before tile 0: prefix 0
+        vw[k] = vo[k] = pack_desc(gen4 | kFlagPrefix, 0u);
+        if (j >= 0) ld_relaxed_u64x2(p.desc + 2 * static_cast<size_t>(j), vw[k], vo[k]);
+      }
+      int consumed = 32 * DEPTH;
+      bool stopped = false;
+      int verdict = TSQ_OK;
+#pragma unroll
+      for (int k = 0; k < DEPTH; ++k) {
+        if (stopped) continue;
+        // the usual window: 32 aggregates
+        const uint32_t agg_tag = gen4 | kFlagAggregate;
+        if (__all_sync(kFull, static_cast<uint32_t>(vw[k] >> 32) == agg_tag && static_cast<uint32_t>(vo[k] >> 32) == agg_tag)) {
+          part_w += static_cast<uint32_t>(vw[k]);
+          part_o += static_cast<uint32_t>(vo[k]);
+          continue;
+        }
+        const uint32_t state = tile_state(gen4, vw[k], vo[k]);
+        const uint32_t stop = __ballot_sync(kFull, state != kFlagAggregate);
+        const uint32_t first = stop ? static_cast<uint32_t>(__ffs(stop) - 1) : 32u;
+        if (lane < first) {
+          part_w += static_cast<uint32_t>(vw[k]);
+          part_o += static_cast<uint32_t>(vo[k]);
+        }
+        if (stop == 0u) continue;
+        stopped = true;
+        const uint32_t first_state = __shfl_sync(kFull, state, first);
+        if (first_state == kFlagAbort) {
+          verdict = -1;
+        } else if (first_state == kFlagPrefix) {
+          base_w = __shfl_sync(kFull, static_cast<uint32_t>(vw[k]), first);
+          base_o = __shfl_sync(kFull, static_cast<uint32_t>(vo[k]), first);
+          done = true;
+        } else {  // not published yet: keep what was walked over, poll again from there
+          consumed = 32 * k + static_cast<int>(first);
+        }
+      }
+      if (verdict != TSQ_OK) return verdict;
+      if (!done) {
+        pos -= consumed;
+        if (consumed == 0) {
+          // tile `pos` has published nothing yet: watch its two descriptors alone until it has
+          for (;;) {
+            uint32_t state = 0u;
+            if (lane == 0) {
+              unsigned long long w0, w1;
+              ld_relaxed_u64x2(p.desc + 2 * static_cast<size_t>(pos), w0, w1);
+              state = tile_state(gen4, w0, w1);
+            }
+            if (__shfl_sync(kFull, state, 0) != 0u) break;
+            if (++polls > poll_limit) return TSQ_ERR_TIMEOUT;
+            __nanosleep(polls < 32u ? 200u : 1000u);
+          }
+        }
+      }
+    }
+    base_w += __reduce_add_sync(kFull, part_w);
+    base_o += __reduce_add_sync(kFull, part_o);
+  }
+  if (lane == 0) publish(p, gen4 | kFlagPrefix, tile, base_w + agg_w, base_o + agg_o);
+  *excl_w = base_w;
+  *excl_o = base_o;
+  return TSQ_OK;
+}
+
+__device__ void write_header(const EncodeParams& p, unsigned long long total_words, unsigned long long total_outliers) {
+  BlobHeader* h = reinterpret_cast<BlobHeader*>(p.blob);
+  h->magic = kMagic;
+  h->version = kVersion;
+  h->dtype = p.dtype;
+  h->hidden = p.hidden;
+  h->tokens = p.tokens;
+  h->n_bits = static_cast<uint32_t>(p.n_bits);
+#pragma unroll
+  for (int i = 0; i < 7; ++i) h->bits[i] = (i < p.n_bits) ? static_cast<uint8_t>(p.bits[i]) : 0;
+  h->bits[7] = static_cast<uint8_t>(p.variant);  // at most seven candidates: the last entry carries the variant
+  h->tau = p.tau;
+  h->delta = p.delta;
+  h->total_words = total_words;
+  h->total_outliers = total_outliers;
+  h->outlier_capacity = static_cast<uint32_t>(p.lay.outlier_capacity);
+}
+
+// The CTA that finishes last publishes the totals and the status, and re-arms the workspace.
+__device__ void finish_call(const EncodeParams& p, uint32_t gen4) {
+  __threadfence();
+  const uint32_t prev = atomicAdd(&p.ws->done, 1u);
+  if (prev != gridDim.x - 1u) return;
+  __threadfence();
+  const uint32_t e = atomicExch(&p.ws->err, 0u);
+  // totals = the last tile's inclusive prefixes, if it got that far
+  unsigned long long tw = 0ull, to = 0ull;
+  if (p.tokens != 0u) {
+    const unsigned long long dw = ld_relaxed_u64(p.desc + 2 * static_cast<size_t>(p.tokens - 1u));
+    const unsigned long long dout = ld_relaxed_u64(p.desc + 2 * static_cast<size_t>(p.tokens - 1u) + 1);
+    if (tile_state(gen4, dw, dout) == kFlagPrefix) {
+      tw = static_cast<uint32_t>(dw);
+      to = static_cast<uint32_t>(dout);
+    }
+  }
+  write_header(p, tw, to);
+  reinterpret_cast<BlobHeader*>(p.blob)->status = e;
+  if (p.tokens == 0u) {  // no row writes the leading zeros of the two prefix-sum sections
+    reinterpret_cast<uint32_t*>(p.blob + p.lay.off_word_off)[0] = 0u;
+    reinterpret_cast<uint32_t*>(p.blob + p.lay.off_out_ptr)[0] = 0u;
+  }
+  if (e != 0u) atomicCAS(&p.ws->enc_status, 0u, e);
+  uint32_t g = (gen4 >> 2);
+  if (g >= kGenWrap) {
+    // generation counter about to wrap: wipe the descriptors so that old tags cannot alias
+    const uint32_t n = p.ws->desc_capacity;
+    for (uint32_t i = 0; i < 2u * n; ++i) p.desc[i] = 0ull;
+    g = 0u;
+  }
+  p.ws->ticket = 0u;
+  p.ws->done = 0u;
+  p.ws->gen = g;
+}
+
+// The per-token fields of the blob, written by one thread.
+__device__ __forceinline__ void write_token_fields(const EncodeParams& p, uint32_t tile, int bstar, float scale, int zp,
+                                                   uint32_t word_end, uint32_t out_end) {
+  reinterpret_cast<uint8_t*>(p.blob + p.lay.off_bits)[tile] = static_cast<uint8_t>(bstar);
+  reinterpret_cast<float*>(p.blob + p.lay.off_scale)[tile] = scale;
+  reinterpret_cast<int32_t*>(p.blob + p.lay.off_zp)[tile] = zp;
+  uint32_t* o_word_off = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_word_off);
+  uint32_t* o_out_ptr = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_out_ptr);
+  if (tile == 0) {
+    o_word_off[0] = 0;
+    o_out_ptr[0] = 0;
+  }
+  o_word_off[tile + 1] = word_end;
+  o_out_ptr[tile + 1] = out_end;
+}
+
+}  // namespace
+}  // namespace tsq
+
+#endif  // TSQ_ENCODE_DEVICE_CUH_
