@@ -134,10 +134,12 @@ __device__ __noinline__ void restore_units_signed_values(const DecodeParams& p, 
 }
 
 template <bool BF16>
-__global__ void __launch_bounds__(kMaxThreads) decode_kernel(const DecodeParams p) {
+__global__ void __launch_bounds__(kMaxThreads) decode_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ __align__(128) unsigned char smem_dyn[];  // one output row
   const uint32_t tid = threadIdx.x;
   const uint32_t t = blockIdx.x;
+  launch_dependents();
+  wait_for_prior_grids();
 
   // ---- header against the plan and the call ----
   const BlobHeader* h = reinterpret_cast<const BlobHeader*>(p.blob);
@@ -243,12 +245,7 @@ cudaError_t decode_kernel_attrs(bool bf16, int threads, size_t smem, int* blocks
 }
 
 cudaError_t launch_decode(const DecodeParams& p, int grid, int threads, size_t smem, cudaStream_t stream) {
-  if (p.dtype == TSQ_BF16) {
-    decode_kernel<true><<<grid, threads, smem, stream>>>(p);
-  } else {
-    decode_kernel<false><<<grid, threads, smem, stream>>>(p);
-  }
-  return cudaGetLastError();
+  return launch_overlapped(p.dtype == TSQ_BF16 ? decode_kernel<true> : decode_kernel<false>, grid, threads, smem, stream, p);
 }
 
 }  // namespace tsq

@@ -142,12 +142,14 @@ __device__ __forceinline__ bool wait_beyond(volatile uint32_t* counter, uint32_t
 // checks for short or missing groups is needed.
 // SV: the signed-values variant.
 template <bool BF16, bool FULL, int MAXT, int MINB, bool SV>
-__global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const EncodeParams p) {
+__global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   __shared__ PipeShared sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t nt = p.compute_threads, nwarps = nt >> 5;
+  launch_dependents();
+  wait_for_prior_grids();
   const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
   uint4* const xpark = reinterpret_cast<uint4*>(smem_dyn);
   uint32_t* const planes = reinterpret_cast<uint32_t*>(smem_dyn + 3u * p.park_stride);
@@ -697,29 +699,17 @@ cudaError_t encode_pipe_attrs(bool bf16, bool full, bool sv, int threads, size_t
 }
 
 template <bool SV>
-static void launch_pipe_variant(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream) {
+static cudaError_t launch_pipe_variant(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream) {
   const bool bf16 = p.dtype == TSQ_BF16;
   if (full) {
-    if (bf16) {
-      encode_pipe_kernel<true, true, kPipeMaxThreads, 2, SV><<<grid, threads, smem, stream>>>(p);
-    } else {
-      encode_pipe_kernel<false, true, kPipeMaxThreads, 2, SV><<<grid, threads, smem, stream>>>(p);
-    }
-  } else if (bf16) {
-    encode_pipe_kernel<true, false, kPipeMaxThreads, 2, SV><<<grid, threads, smem, stream>>>(p);
-  } else {
-    encode_pipe_kernel<false, false, kPipeMaxThreads, 2, SV><<<grid, threads, smem, stream>>>(p);
+    return launch_overlapped(bf16 ? encode_pipe_kernel<true, true, kPipeMaxThreads, 2, SV> : encode_pipe_kernel<false, true, kPipeMaxThreads, 2, SV>, grid, threads, smem, stream, p);
   }
+  return launch_overlapped(bf16 ? encode_pipe_kernel<true, false, kPipeMaxThreads, 2, SV> : encode_pipe_kernel<false, false, kPipeMaxThreads, 2, SV>, grid, threads, smem, stream, p);
 }
 
 cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream) {
   if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
-  if (p.variant != 0u) {
-    launch_pipe_variant<true>(p, full, grid, threads, smem, stream);
-  } else {
-    launch_pipe_variant<false>(p, full, grid, threads, smem, stream);
-  }
-  return cudaGetLastError();
+  return p.variant != 0u ? launch_pipe_variant<true>(p, full, grid, threads, smem, stream) : launch_pipe_variant<false>(p, full, grid, threads, smem, stream);
 }
 
 }  // namespace tsq

@@ -623,16 +623,24 @@ __device__ void write_header(const EncodeParams& p, unsigned long long total_wor
   h->outlier_capacity = static_cast<uint32_t>(p.lay.outlier_capacity);
 }
 
-// The CTA that finishes last publishes the totals and the status, and re-arms the workspace.
-__device__ void finish_call(const EncodeParams& p, uint32_t gen4) {
+// The CTA that finishes last publishes the totals and the status, and re-arms the workspace.  `direct`: the descriptors
+// are those of a call without look-back (encode_rows_kernel), which comes here only when the generation wraps.
+__device__ void finish_call(const EncodeParams& p, uint32_t gen4, bool direct = false) {
   __threadfence();
   const uint32_t prev = atomicAdd(&p.ws->done, 1u);
   if (prev != gridDim.x - 1u) return;
   __threadfence();
-  const uint32_t e = atomicExch(&p.ws->err, 0u);
+  uint32_t e = atomicExch(&p.ws->err, 0u);
   // totals = the last tile's inclusive prefixes, if it got that far
   unsigned long long tw = 0ull, to = 0ull;
-  if (p.tokens != 0u) {
+  if (direct) {
+    for (uint32_t i = 0; i < p.tokens; ++i) {
+      const uint32_t v = static_cast<uint32_t>(ld_relaxed_u64(p.desc + i));
+      tw += v >> 17;
+      to += v & 0x1ffffu;
+    }
+    if (e == 0u && to > p.lay.outlier_capacity) e = TSQ_ERR_OUTLIER_OVERFLOW;
+  } else if (p.tokens != 0u) {
     const unsigned long long dw = ld_relaxed_u64(p.desc + 2 * static_cast<size_t>(p.tokens - 1u));
     const unsigned long long dout = ld_relaxed_u64(p.desc + 2 * static_cast<size_t>(p.tokens - 1u) + 1);
     if (tile_state(gen4, dw, dout) == kFlagPrefix) {

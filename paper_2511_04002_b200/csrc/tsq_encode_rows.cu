@@ -17,24 +17,73 @@ struct RowShared {
   uint32_t row_cnt;    // outliers of the row
   uint32_t word_off, out_base;
   uint32_t status;     // TSQ_OK, or why the row is not written
+  uint32_t warp_w[32], warp_o[32], warp_status[32];  // direct_offsets: by warp
 };
+
+// Offsets of a row of a call whose rows are all being encoded at once: thread i polls the descriptors of rows i,
+// i + blockDim, ... until they carry the call's tag (payload: plane words << 17 | outliers, 15 and 17 bits for any row),
+// so the wait is one round trip past the last predecessor's store.  The sums are left by warp; the caller adds them up
+// behind its barrier.  (A walk back by one warp took 3600 of the 10100 cycles of a 64 x 4096 call: its first look found
+// nothing published, and every retry was another round trip.)
+__device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared& sh) {
+  const uint32_t limit = lookback_limit(p), tag = gen4 | kFlagAggregate;
+  uint32_t w = 0u, o = 0u, status = TSQ_OK;
+  for (uint32_t i = threadIdx.x; i < tile; i += blockDim.x) {
+    unsigned long long v = ld_relaxed_u64(p.desc + i);
+    for (uint32_t polls = 0; static_cast<uint32_t>(v >> 32) != tag; v = ld_relaxed_u64(p.desc + i)) {
+      if (++polls > limit) {
+        status = TSQ_ERR_TIMEOUT;
+        break;
+      }
+      if (polls > 32u) __nanosleep(1000u);
+    }
+    w += static_cast<uint32_t>(v) >> 17;
+    o += static_cast<uint32_t>(v) & 0x1ffffu;
+  }
+  w = __reduce_add_sync(kFull, w);
+  o = __reduce_add_sync(kFull, o);
+  status = __reduce_or_sync(kFull, status);
+  if ((threadIdx.x & 31u) == 0u) {
+    const uint32_t warp = threadIdx.x >> 5;
+    sh.warp_w[warp] = w;
+    sh.warp_o[warp] = o;
+    sh.warp_status[warp] = status;
+  }
+}
+
+// The last row's CTA ends such a call: it knows the totals, and every other CTA has read the generation (it has published
+// under it), so nothing has to wait for the others.  (A counter of finished CTAs and the atomics around it cost 1650 cycles.)
+__device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t gen4, uint32_t status, uint32_t total_w, uint32_t total_o) {
+  if (status == TSQ_OK && total_o > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
+  const bool ok = status != TSQ_ERR_TIMEOUT;
+  write_header(p, ok ? total_w : 0ull, ok ? total_o : 0ull);
+  reinterpret_cast<BlobHeader*>(p.blob)->status = status;
+  if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
+  p.ws->gen = gen4 >> 2;
+}
 
 // MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instance,
 // which may use four times the registers of the 1024-thread one).  SV: the signed-values variant.
-template <bool BF16, int UPT, int MAXT, bool SV>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(const EncodeParams p) {
+// DIRECT: calls of at most one row per SM.  Every CTA is resident, so row = CTA index needs no ticket, and a row's offsets
+// are read straight from the sizes of the rows before it (direct_offsets) instead of walked back to.
+template <bool BF16, int UPT, int MAXT, bool SV, bool DIRECT>
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
   __shared__ RowShared sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  launch_dependents();
+  wait_for_prior_grids();
   const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
 
-  if (tid == 0) {
-    // a call whose rows all get a CTA at once needs no ticket: every CTA is running, so row = CTA index is safe
-    sh.tile = p.direct_tiles != 0u ? blockIdx.x : atomicAdd(&p.ws->ticket, 1u);
-    sh.status = TSQ_OK;
+  uint32_t tile = blockIdx.x;
+  if (!DIRECT) {
+    if (tid == 0) {
+      sh.tile = atomicAdd(&p.ws->ticket, 1u);
+      sh.status = TSQ_OK;
+    }
+    __syncthreads();
+    tile = sh.tile;
   }
-  __syncthreads();
-  const uint32_t tile = sh.tile;
 
   if (tile < p.tokens) {
     // ---- the row, 64 bytes per group, straight into registers; thread t owns groups UPT * t + k ----
@@ -129,7 +178,13 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
     const uint32_t agg_w = static_cast<uint32_t>(bstar) * p.lay.wpp;
 
     // ---- this row's sizes are known: let the rows behind it see them, then pack ----
-    if (tid == 0) publish_aggregate(p, gen4, tile, agg_w, row_cnt);
+    if (tid == 0) {
+      if (DIRECT) {
+        st_relaxed_u64(p.desc + tile, pack_desc(gen4 | kFlagAggregate, agg_w << 17 | row_cnt));
+      } else {
+        publish_aggregate(p, gen4, tile, agg_w, row_cnt);
+      }
+    }
     uint32_t r[UPT][8];
 #pragma unroll
     for (int k = 0; k < UPT; ++k) {
@@ -146,7 +201,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
     }
 
     // ---- placement: exclusive prefix sums over the tokens before this one ----
-    if (warp == 0) {
+    if (DIRECT) {
+      direct_offsets(p, gen4, tile, sh);
+    } else if (warp == 0) {
       uint32_t word_off = 0, out_base = 0;
       const int st = resolve_prefix<8>(p, gen4, tile, agg_w, row_cnt, lane, &word_off, &out_base, lookback_limit(p));
       if (lane == 0) {
@@ -160,9 +217,18 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
       }
     }
     __syncthreads();
+    uint32_t word_off = sh.word_off, out_base = sh.out_base, status = sh.status;
+    if (DIRECT) {
+      word_off = out_base = status = 0u;
+      for (uint32_t w = 0; w < nwarps; ++w) {
+        word_off += sh.warp_w[w];
+        out_base += sh.warp_o[w];
+        status |= sh.warp_status[w];
+      }
+      if (tile == p.tokens - 1u && tid == blockDim.x - 1u && (gen4 >> 2) < kGenWrap) finish_direct(p, gen4, status, word_off + agg_w, out_base + row_cnt);
+    }
 
-    if (sh.status == TSQ_OK) {
-      const uint32_t word_off = sh.word_off, out_base = sh.out_base;
+    if (status == TSQ_OK) {
       // ---- plane words: group u owns words u * b* .. u * b* + b* - 1 ----
       uint32_t* wrow = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
 #pragma unroll
@@ -199,49 +265,36 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
               ++at;
             }
           }
-          if (overflow) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_OUTLIER_OVERFLOW));
+          if (overflow && !DIRECT) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_OUTLIER_OVERFLOW));
         }
       }
     }
   }
 
+  if (DIRECT && (gen4 >> 2) < kGenWrap) return;
   __syncthreads();
-  if (tid == 0) finish_call(p, gen4);
+  if (tid == 0) finish_call(p, gen4, DIRECT);
 }
 
 }  // namespace
 
-template <bool SV>
-static void launch_rows_variant(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
+template <bool SV, bool DIRECT>
+static cudaError_t launch_rows_variant(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
   const bool bf16 = p.dtype == TSQ_BF16;
   if (upt == 1 && threads <= 256) {
-    if (bf16) {
-      encode_rows_kernel<true, 1, 256, SV><<<grid, threads, 0, stream>>>(p);
-    } else {
-      encode_rows_kernel<false, 1, 256, SV><<<grid, threads, 0, stream>>>(p);
-    }
-  } else if (upt == 1) {
-    if (bf16) {
-      encode_rows_kernel<true, 1, 1024, SV><<<grid, threads, 0, stream>>>(p);
-    } else {
-      encode_rows_kernel<false, 1, 1024, SV><<<grid, threads, 0, stream>>>(p);
-    }
-  } else {
-    if (bf16) {
-      encode_rows_kernel<true, 2, 1024, SV><<<grid, threads, 0, stream>>>(p);
-    } else {
-      encode_rows_kernel<false, 2, 1024, SV><<<grid, threads, 0, stream>>>(p);
-    }
+    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 256, SV, DIRECT> : encode_rows_kernel<false, 1, 256, SV, DIRECT>, grid, threads, 0, stream, p);
   }
+  if (upt == 1) {
+    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 1024, SV, DIRECT> : encode_rows_kernel<false, 1, 1024, SV, DIRECT>, grid, threads, 0, stream, p);
+  }
+  return launch_overlapped(bf16 ? encode_rows_kernel<true, 2, 1024, SV, DIRECT> : encode_rows_kernel<false, 2, 1024, SV, DIRECT>, grid, threads, 0, stream, p);
 }
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
-  if (p.variant != 0u) {
-    launch_rows_variant<true>(p, grid, threads, upt, stream);
-  } else {
-    launch_rows_variant<false>(p, grid, threads, upt, stream);
+  if (p.direct_tiles != 0u) {
+    return p.variant != 0u ? launch_rows_variant<true, true>(p, grid, threads, upt, stream) : launch_rows_variant<false, true>(p, grid, threads, upt, stream);
   }
-  return cudaGetLastError();
+  return p.variant != 0u ? launch_rows_variant<true, false>(p, grid, threads, upt, stream) : launch_rows_variant<false, false>(p, grid, threads, upt, stream);
 }
 
 }  // namespace tsq

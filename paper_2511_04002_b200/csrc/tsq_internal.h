@@ -106,6 +106,24 @@ struct DecodeParams {
   unsigned long long blob_bytes;
 };
 
+// Launch with programmatic stream serialisation: the grid's CTAs may be set up while the stream's previous grid still runs
+// (where that is one of this library's kernels, which allow it from their start), and each begins with
+// wait_for_prior_grids().  Only the launch overlaps: a kernel reads and writes nothing before that wait.
+template <typename... Args>
+cudaError_t launch_overlapped(void (*kernel)(Args...), int grid, int threads, size_t smem, cudaStream_t stream, const Args&... args) {
+  cudaLaunchConfig_t config = {};
+  config.gridDim = dim3(static_cast<unsigned>(grid));
+  config.blockDim = dim3(static_cast<unsigned>(threads));
+  config.dynamicSmemBytes = smem;
+  config.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  config.attrs = attr;
+  config.numAttrs = 1;
+  return cudaLaunchKernelEx(&config, kernel, args...);
+}
+
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int groups_per_thread, cudaStream_t stream);
 cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream);
 cudaError_t encode_pipe_attrs(bool bf16, bool full, bool signed_values, int threads, size_t smem, int* blocks_per_sm);
