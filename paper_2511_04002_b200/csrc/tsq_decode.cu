@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kMaxThreads) decode_kernel(const __grid_consta
   extern __shared__ __align__(128) unsigned char smem_dyn[];  // one output row
   const uint32_t tid = threadIdx.x;
   const uint32_t t = blockIdx.x;
-  launch_dependents();
+  if (p.overlap_next != 0u) launch_dependents();
   wait_for_prior_grids();
 
   // ---- header against the plan and the call ----

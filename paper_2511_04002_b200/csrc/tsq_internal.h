@@ -103,6 +103,7 @@ struct DecodeParams {
   uint32_t tokens, hidden, units, chunks;
   uint32_t bmax, dtype;
   uint32_t variant;
+  uint32_t overlap_next;                     // 1: the stream's next grid may be set up while this one runs
   unsigned long long blob_bytes;
 };
 
