@@ -83,6 +83,12 @@ namespace {
 // keeps the compute warps busy while a slow predecessor (a row whose descent goes on) holds everybody up.
 constexpr int kMetaRing = kMaxRing + 2;  // row records: one row in pass A and one being packed on top of those
 
+// How the pipelined kernel decides the first lower candidate:
+constexpr int kKind84 = 0;      // 8 bits against 4: from the 8-bit codes' planes, the exact sum only when the open codes matter
+constexpr int kKindExact = 1;   // any other candidates: the exact distortion sum
+constexpr int kKindSigned = 2;  // signed-values variant, exact sum
+constexpr int kExactSlot = kMaxCand - 1;  // kKind84 (at most four candidates): the distortion slot of the exact first sum
+
 struct RowMeta {
   Level lv[kMaxCand];
   int S[kMaxCand];
@@ -91,6 +97,8 @@ struct RowMeta {
   uint32_t bstar, agg_w;
   float scale;
   int zp;
+  float lo, hi;    // smallest and largest magnitude
+  float one_fma;   // kKind84: the factor of the one-FMA codes (one_fma_factor), 0: the three-operation quotient
   uint32_t heavy;  // 1: the side buffer holds the row's outlier bitmaps (more outliers than a list holds)
 };
 
@@ -141,9 +149,11 @@ __device__ __forceinline__ bool wait_beyond(volatile uint32_t* counter, uint32_t
 // FULL: every compute thread owns a whole 32-element group (hidden is a multiple of 1024), so none of the
 // checks for short or missing groups is needed.
 // SV: the signed-values variant.
-template <bool BF16, bool FULL, int MAXT, int MINB, bool SV>
+// KIND: how the first lower candidate is decided (see the kKind constants).
+template <bool BF16, bool FULL, int MAXT, int MINB, int KIND>
 __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
+  constexpr bool SV = KIND == kKindSigned;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   __shared__ PipeShared sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -345,20 +355,50 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
               y[4 * j + 2] = c.z;
               y[4 * j + 3] = c.w;
             }
-            const int c0 = ci >= 0 ? ci : 0;
-            const Level low = m.lv[c0];
-            uint32_t S = distortion_first<BF16, SV>(y, make_level2(top), make_level2(low), bmax - p.bits[c0], tb, lb,
-                                                    (FULL || !SV) ? 4u : group_chunks(p, u));
-            if (ci >= 0) {
-              S = __reduce_add_sync(kFull, S);
-              if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
+            if (KIND == kKind84) {
+              if (m.one_fma != 0.0f) {
+                top_bytes_one_fma<BF16>(y, pack2f(m.one_fma, m.one_fma), tb);
+              } else {
+                top_bytes<BF16>(y, make_level2(top), tb);
+              }
+            } else {
+              const int c0 = ci >= 0 ? ci : 0;
+              const Level low = m.lv[c0];
+              uint32_t S = distortion_first<BF16, SV>(y, make_level2(top), make_level2(low), bmax - p.bits[c0], tb, lb,
+                                                      (FULL || !SV) ? 4u : group_chunks(p, u));
+              if (ci >= 0) {
+                S = __reduce_add_sync(kFull, S);
+                if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
+              }
             }
           }
           // pass C at the top level right away: the usual outcome, and work to do while the other warps
           // arrive at the barrier (a row that goes lower transposes once more, below)
           planes_of_bytes(tb, r);
           bool passed = false;
-          if (ci >= 0) {
+          if (KIND == kKind84) {
+            const uint32_t sum = __reduce_add_sync(kFull, distortion_8_to_4(r));
+            if (lane == 0 && sum != 0u) atomicAdd(&m.S[ci], static_cast<int>(sum));
+            compute_barrier(nt);
+            // usually the certain differences alone exceed the tolerance; when they do not, the exact sum is formed (its
+            // codes are needed anyway if the candidate passes)
+            if (static_cast<int>(static_cast<uint32_t>(m.S[ci]) & 0xffffu) <= p.s_max) {
+              uint32_t y[16];
+#pragma unroll
+              for (uint32_t j = 0; j < 4; ++j) {
+                const uint4 c = xp[park_index(nt, u, j)];
+                y[4 * j + 0] = c.x;
+                y[4 * j + 1] = c.y;
+                y[4 * j + 2] = c.z;
+                y[4 * j + 3] = c.w;
+              }
+              uint32_t S = distortion_next<BF16, false>(y, tb, make_level2(m.lv[ci]), bmax - p.bits[ci], lb);
+              S = __reduce_add_sync(kFull, S);
+              if (lane == 0 && S != 0u) atomicAdd(&m.S[kExactSlot], static_cast<int>(S));
+              compute_barrier(nt);
+              passed = m.S[kExactSlot] <= p.s_max;
+            }
+          } else if (ci >= 0) {
             compute_barrier(nt);
             passed = m.S[ci] <= p.s_max;
           }
@@ -503,8 +543,18 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
       if (!wait_beyond(&sh.a_ready, n, sh, true, 500u)) break;
       __threadfence_block();
       RowMeta& m = sh.meta[n % kMetaRing];
-      const uint32_t divide = row_levels<BF16, (kPipeMaxThreads - 64) / 32, SV>(p, m.part, nwarps, lane, m.lv, m.S, &m.row_cnt);
-      if (lane == 0) m.divide = divide;
+      const uint32_t divide = row_levels<BF16, (kPipeMaxThreads - 64) / 32, SV>(p, m.part, nwarps, lane, m.lv, m.S, &m.row_cnt, &m.lo, &m.hi);
+      __syncwarp();
+      float one = 0.0f;
+      if (KIND == kKind84) {
+        const Level top = m.lv[p.n_bits - 1];
+        if (divide == 0u) one = one_fma_factor<BF16>(m.lo, m.hi, top, lane);
+        if (lane == 0) m.S[kExactSlot] = 0;
+      }
+      if (lane == 0) {
+        m.divide = divide;
+        m.one_fma = one;
+      }
       __syncwarp();
       if (lane == 0) {
         __threadfence_block();
@@ -664,31 +714,34 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
 
 // The pipelined kernel is built for CTAs of up to kPipeMaxThreads threads (rows of up to 8192 elements)
 // and may use up to 102 registers per thread; longer rows take encode_rows_kernel.
-template <bool SV>
-static const void* pipe_kernel_of(bool bf16, bool full) {
-  if (full) {
-    return bf16 ? reinterpret_cast<const void*>(&encode_pipe_kernel<true, true, kPipeMaxThreads, 2, SV>)
-                : reinterpret_cast<const void*>(&encode_pipe_kernel<false, true, kPipeMaxThreads, 2, SV>);
-  }
-  return bf16 ? reinterpret_cast<const void*>(&encode_pipe_kernel<true, false, kPipeMaxThreads, 2, SV>)
-              : reinterpret_cast<const void*>(&encode_pipe_kernel<false, false, kPipeMaxThreads, 2, SV>);
+using PipeKernel = void (*)(EncodeParams);
+template <int KIND>
+static PipeKernel pipe_kernel_of(bool bf16, bool full) {
+  if (full) return bf16 ? encode_pipe_kernel<true, true, kPipeMaxThreads, 2, KIND> : encode_pipe_kernel<false, true, kPipeMaxThreads, 2, KIND>;
+  return bf16 ? encode_pipe_kernel<true, false, kPipeMaxThreads, 2, KIND> : encode_pipe_kernel<false, false, kPipeMaxThreads, 2, KIND>;
 }
-static const void* pipe_kernel(bool bf16, bool full, bool sv) { return sv ? pipe_kernel_of<true>(bf16, full) : pipe_kernel_of<false>(bf16, full); }
+static PipeKernel pipe_kernel(const EncodeParams& p, bool full, int* index) {
+  const bool bf16 = p.dtype == TSQ_BF16;
+  const int kind = p.variant != 0u ? kKindSigned : p.n_bits >= 2 && p.bits[p.n_bits - 1] == 8 && p.bits[p.n_bits - 2] == 4 ? kKind84 : kKindExact;
+  *index = kind * 4 + (bf16 ? 2 : 0) + (full ? 1 : 0);
+  return kind == kKindSigned ? pipe_kernel_of<kKindSigned>(bf16, full) : kind == kKind84 ? pipe_kernel_of<kKind84>(bf16, full) : pipe_kernel_of<kKindExact>(bf16, full);
+}
 
-cudaError_t encode_pipe_attrs(bool bf16, bool full, bool sv, int threads, size_t smem, int* blocks_per_sm) {
+cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, int threads, size_t smem, int* blocks_per_sm) {
   if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
-  const void* fn = pipe_kernel(bf16, full, sv);
+  int index = 0;
+  const void* fn = reinterpret_cast<const void*>(pipe_kernel(p, full, &index));
   // the attribute belongs to the kernel on the current device, not to a plan: it only ever grows, so
   // that every plan can launch
   static std::mutex mu;
-  static size_t granted[kMaxDevices][2][2][2] = {};
+  static size_t granted[kMaxDevices][12] = {};
   {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
-    size_t& have = granted[dev][bf16 ? 1 : 0][full ? 1 : 0][sv ? 1 : 0];
+    size_t& have = granted[dev][index];
     if (smem > have) {
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
       if (e != cudaSuccess) return e;
@@ -698,18 +751,10 @@ cudaError_t encode_pipe_attrs(bool bf16, bool full, bool sv, int threads, size_t
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
-template <bool SV>
-static cudaError_t launch_pipe_variant(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream) {
-  const bool bf16 = p.dtype == TSQ_BF16;
-  if (full) {
-    return launch_overlapped(bf16 ? encode_pipe_kernel<true, true, kPipeMaxThreads, 2, SV> : encode_pipe_kernel<false, true, kPipeMaxThreads, 2, SV>, grid, threads, smem, stream, p);
-  }
-  return launch_overlapped(bf16 ? encode_pipe_kernel<true, false, kPipeMaxThreads, 2, SV> : encode_pipe_kernel<false, false, kPipeMaxThreads, 2, SV>, grid, threads, smem, stream, p);
-}
-
 cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream) {
   if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
-  return p.variant != 0u ? launch_pipe_variant<true>(p, full, grid, threads, smem, stream) : launch_pipe_variant<false>(p, full, grid, threads, smem, stream);
+  int index = 0;
+  return launch_overlapped(pipe_kernel(p, full, &index), grid, threads, smem, stream, p);
 }
 
 }  // namespace tsq

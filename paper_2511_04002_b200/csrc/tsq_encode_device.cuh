@@ -282,6 +282,79 @@ __device__ __forceinline__ void planes_of_bytes(const uint32_t (&tb)[8], uint32_
   transpose8x32_select(r);
 }
 
+// ---- 8-bit top level: codes by one FMA, and the distortion from the codes' bit-planes ----------------------------
+
+// Top-level codes of a group as bytes (grouping and signs as in distortion_first) when one FMA per element gets them right
+// (see one_fma_factor): r2 = {r, r}.  On the signed value, rounded as 128 + q: the distance of the low byte from 128 is the
+// code, which saves the absolute values.
+template <bool BF16>
+__device__ __forceinline__ void top_bytes_one_fma(const uint32_t (&x)[16], uint64_t r2, uint32_t (&tb)[8]) {
+  const uint64_t magic2 = pack2f(kRoundMagicSigned + 128.0f, kRoundMagicSigned + 128.0f);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
+      const uint32_t c4 = __vabsdiffu4(bytes4(fma2(values2<BF16>(xa), r2, magic2), fma2(values2<BF16>(xb), r2, magic2)), 0x80808080u);
+      tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
+    }
+  }
+}
+// The same with the three-operation quotient.
+template <bool BF16>
+__device__ __forceinline__ void top_bytes(const uint32_t (&x)[16], const Level2& top, uint32_t (&tb)[8]) {
+  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
+      const uint32_t c4 = bytes4(quotient2(magnitudes2<BF16>(xa), top, magic2), quotient2(magnitudes2<BF16>(xb), top, magic2));
+      tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
+    }
+  }
+}
+
+// A factor r for which fma(m, r, 2^23) rounds to the 8-bit level's code rint(fl(m / s)) of every 16-bit magnitude m of the
+// row, or 0 when none is known; run by one full warp.  The two can only disagree where m / s lies within about 2^-22
+// (relative) of a boundary k + 1/2, and a 16-bit m that close to one is rare:
+//   - lo = 0 (the usual row, s = fl(hi / 127)): m / hi is a ratio of two integers below 2^11, so that m / s is either at least
+//     2^-19 away from every boundary or, in exact arithmetic, on one.  254 m = (2k + 1) hi then, which only m = hi / 2 solves
+//     (k = 63) unless 127 divides hi's significand.  So 1 / s is moved by 2^-21 to the side that fl((hi / 2) / s) rounds to,
+//     and rows with such a significand (1 in 127) are left out.
+//   - else the 16-bit magnitude next to each of the 127 boundaries is tried, four per lane.
+template <bool BF16>
+__device__ __forceinline__ float one_fma_factor(float lo, float hi, const Level& top, uint32_t lane) {
+  if (lo == 0.0f) {
+    const uint32_t f = __float_as_uint(hi), m = (f & 0x7fffffu) | 0x800000u;  // 127 divides it iff it divides the significand
+    if (m % 127u == 0u || f < 0x00800000u) return 0.0f;
+    const float half = 0.5f * hi, q0 = __fmul_rn(half, top.r), q = __fmaf_rn(__fmaf_rn(q0, -top.s, half), top.r, q0);
+    return __fmul_rn(top.r, q >= 63.5f ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
+  }
+  bool same = true;
+#pragma unroll
+  for (uint32_t i = 0; i < 4; ++i) {
+    const float b = __fmul_rn(static_cast<float>(lane + 32u * i) + 0.5f, top.s);
+    const float m = Elem<BF16>::lo_f32(Elem<BF16>::pack_rn(b, 0.0f));
+    const float q0 = __fmul_rn(m, top.r), q = __fmaf_rn(__fmaf_rn(q0, -top.s, m), top.r, q0);
+    same = same && __fadd_rn(q, kRoundMagic) == __fmaf_rn(m, top.r, kRoundMagic);
+  }
+  return __all_sync(kFull, same) ? top.r : 0.0f;
+}
+
+// Distortion of a group between the 8-bit level (7 code bits) and the 4-bit level, from the 8-bit codes' bit-planes alone
+// (r[k] = bit k of the codes).  Both levels round the same magnitude m, q = rint(m 127 / R) and low = rint(m 7 / R) up to
+// binary32 rounding, so |(q >> 4) - low| is 0 or 1 and is fixed by q except for the codes whose rounding interval contains
+// one of the low level's boundaries (k + 1/2) 127 / 7 = 9.07, 27.2, 45.4, 63.5, 81.6, 99.8, 117.9.  With q folded to
+// q' = min(q, 127 - q), j = q' >> 4 and n = q' & 15: the difference is 1 for n > 9 + 2j, 0 for n < 9 + 2j, open for
+// n = 9 + 2j.  Returns the number of certain differences, and of open codes in the upper half of the word.
+__device__ __forceinline__ uint32_t distortion_8_to_4(const uint32_t (&r)[8]) {
+  const uint32_t f = r[6], j1 = r[5] ^ f, j0 = r[4] ^ f, n3 = r[3] ^ f, n2 = r[2] ^ f, n1 = r[1] ^ f, n0 = r[0] ^ f;
+  const uint32_t one = n3 & ((~j1 & (n2 | (~j0 & n1))) | (j1 & ~j0 & n2 & n1));
+  const uint32_t open = n3 & n0 & ~(n2 ^ j1) & ~(n1 ^ j0);
+  return mad_u32(static_cast<uint32_t>(__popc(open)), 65536u, static_cast<uint32_t>(__popc(one)));
+}
+
 // Pass C on one group of a row whose chosen level is plain: codes as bytes (code | sign << 7), transposed into
 // bit-planes: on return r[k] = bit k of every byte, k < 7 code bits, k = 7 signs.
 template <bool BF16, bool SV = false>
@@ -459,7 +532,8 @@ struct RowPartials {
 };
 template <bool BF16, int NW, bool SV = false>
 __device__ __forceinline__ uint32_t row_levels(const EncodeParams& p, RowPartials<NW>& part, uint32_t nwarps, uint32_t lane,
-                                               Level* lv_out, int* S_out, uint32_t* row_cnt) {
+                                               Level* lv_out, int* S_out, uint32_t* row_cnt, float* lo_out = nullptr,
+                                               float* hi_out = nullptr) {
   using E = Elem<BF16>;
   const uint32_t pmin = __reduce_min_sync(kFull, lane < nwarps ? part.warp_min[lane] : 0xffffu);
   const uint32_t pmax = __reduce_max_sync(kFull, lane < nwarps ? part.warp_max[lane] : 0u);
@@ -481,7 +555,13 @@ __device__ __forceinline__ uint32_t row_levels(const EncodeParams& p, RowPartial
     lv_out[lane] = lv;
     S_out[lane] = 0;
   }
-  if (lane == 0) *row_cnt = total;
+  if (lane == 0) {
+    *row_cnt = total;
+    if (lo_out) {  // magnitudes (not meant for SV)
+      *lo_out = E::pattern_f32(pmin);
+      *hi_out = E::pattern_f32(pmax);
+    }
+  }
   return __all_sync(kFull, plain) ? 0u : 1u;
 }
 

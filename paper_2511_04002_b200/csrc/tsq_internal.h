@@ -127,7 +127,7 @@ cudaError_t launch_overlapped(void (*kernel)(Args...), int grid, int threads, si
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int groups_per_thread, cudaStream_t stream);
 cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream);
-cudaError_t encode_pipe_attrs(bool bf16, bool full, bool signed_values, int threads, size_t smem, int* blocks_per_sm);
+cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, int threads, size_t smem, int* blocks_per_sm);
 cudaError_t launch_decode(const DecodeParams& p, int grid, int threads, size_t smem, cudaStream_t stream);
 cudaError_t decode_kernel_attrs(bool bf16, int threads, size_t smem, int* blocks_per_sm);
 size_t decode_smem_bytes(uint32_t row_bytes);
