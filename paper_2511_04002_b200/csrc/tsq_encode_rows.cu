@@ -59,13 +59,15 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
   write_header(p, ok ? total_w : 0ull, ok ? total_o : 0ull);
   reinterpret_cast<BlobHeader*>(p.blob)->status = status;
   if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
+  p.ws->ticket = 0u;  // every CTA has taken its own
   p.ws->gen = gen4 >> 2;
 }
 
 // MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instance,
 // which may use four times the registers of the 1024-thread one).  SV: the signed-values variant.
-// DIRECT: calls of at most one row per SM.  Every CTA is resident, so row = CTA index needs no ticket, and a row's offsets
-// are read straight from the sizes of the rows before it (direct_offsets) instead of walked back to.
+// DIRECT: calls of at most two rows per SM: a row's offsets are read straight from the sizes of the rows before it
+// (direct_offsets) instead of walked back to.  With at most one row per SM every CTA is resident, so row = CTA index needs
+// no ticket.
 template <bool BF16, int UPT, int MAXT, bool SV, bool DIRECT>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
   const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
 
   uint32_t tile = blockIdx.x;
-  if (!DIRECT) {
+  if (!DIRECT || p.direct_tiles == 2u) {
     if (tid == 0) {
       sh.tile = atomicAdd(&p.ws->ticket, 1u);
       sh.status = TSQ_OK;
