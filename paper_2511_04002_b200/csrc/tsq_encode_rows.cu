@@ -65,7 +65,7 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
 
 // MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instance,
 // which may use four times the registers of the 1024-thread one).  SV: the signed-values variant.
-// DIRECT: calls of at most two rows per SM: a row's offsets are read straight from the sizes of the rows before it
+// DIRECT: calls of a few rows per SM: a row's offsets are read straight from the sizes of the rows before it
 // (direct_offsets) instead of walked back to.  With at most one row per SM every CTA is resident, so row = CTA index needs
 // no ticket.
 template <bool BF16, int UPT, int MAXT, bool SV, bool DIRECT>
