@@ -1,6 +1,7 @@
 // Host side of the tsq C ABI: plan creation, buffer sizing, argument checks, launches.
 
 #include <atomic>
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -84,6 +85,86 @@ __global__ void workspace_wait_limit_kernel(WsControl* ws, uint32_t polls) { ws-
 }  // namespace
 }  // namespace tsq
 
+namespace tsq {
+namespace {
+
+// What a host-buffer call needs to overlap its copies with the kernels: two copy streams, events and a few pinned words.
+// A plan keeps up to kMaxHostPipes of them between calls (one per call in flight) and destroys them with itself.
+constexpr int kMaxHostPipes = 4;
+constexpr int kPipeSlots = 8;  // parts in flight
+struct HostPipe {
+  cudaStream_t in = nullptr, out = nullptr;
+  cudaEvent_t begin = nullptr, landed[kPipeSlots] = {}, ready[kPipeSlots] = {};
+  unsigned long long* totals = nullptr;  // [kPipeSlots][4], pinned
+  bool create() {
+    bool ok = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&begin, cudaEventDisableTiming) == cudaSuccess &&
+              cudaHostAlloc(reinterpret_cast<void**>(&totals), kPipeSlots * 4 * sizeof(unsigned long long), cudaHostAllocPortable) == cudaSuccess;
+    for (int i = 0; ok && i < kPipeSlots; ++i) {
+      ok = cudaEventCreateWithFlags(&landed[i], cudaEventDisableTiming) == cudaSuccess && cudaEventCreateWithFlags(&ready[i], cudaEventDisableTiming) == cudaSuccess;
+    }
+    return ok;
+  }
+  void destroy() {
+    if (in) cudaStreamDestroy(in);
+    if (out) cudaStreamDestroy(out);
+    if (begin) cudaEventDestroy(begin);
+    for (int i = 0; i < kPipeSlots; ++i) {
+      if (landed[i]) cudaEventDestroy(landed[i]);
+      if (ready[i]) cudaEventDestroy(ready[i]);
+    }
+    if (totals) cudaFreeHost(totals);
+    cudaGetLastError();
+  }
+};
+struct HostPipes {
+  std::mutex mutex;
+  HostPipe* idle[kMaxHostPipes] = {};
+  HostPipe* take() {
+    {
+      std::lock_guard<std::mutex> lock(mutex);
+      for (HostPipe*& p : idle) {
+        if (p) {
+          HostPipe* got = p;
+          p = nullptr;
+          return got;
+        }
+      }
+    }
+    HostPipe* p = new (std::nothrow) HostPipe();
+    if (p && !p->create()) {
+      p->destroy();
+      delete p;
+      p = nullptr;
+    }
+    return p;
+  }
+  void give_back(HostPipe* p) {
+    {
+      std::lock_guard<std::mutex> lock(mutex);
+      for (HostPipe*& slot : idle) {
+        if (!slot) {
+          slot = p;
+          return;
+        }
+      }
+    }
+    p->destroy();
+    delete p;
+  }
+  ~HostPipes() {
+    for (HostPipe* p : idle) {
+      if (p) {
+        p->destroy();
+        delete p;
+      }
+    }
+  }
+};
+
+}  // namespace
+}  // namespace tsq
+
 struct tsq_plan {
   int device;
   tsq_dtype_t dtype;
@@ -107,6 +188,7 @@ struct tsq_plan {
   int sms;
   size_t dec_smem;
   size_t workspace_bytes;
+  mutable tsq::HostPipes host_pipes;
 };
 
 using namespace tsq;
@@ -318,10 +400,7 @@ static tsq_status_t check_encode_args(const tsq_plan_t* plan, const void* x_dev,
   return TSQ_OK;
 }
 
-tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, size_t blob_bytes,
-                        void* ws_dev, size_t ws_bytes, void* cuda_stream) {
-  const tsq_status_t args_ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
-  if (args_ok != TSQ_OK) return args_ok;
+static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, void* ws_dev) {
   const BlobLayout L = layout_for(plan, static_cast<unsigned long long>(tokens));
 
   EncodeParams p;
@@ -344,13 +423,24 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
   p.variant = plan->variant;
   p.tau = plan->tau;
   p.delta = plan->delta;
+  p.write_header = 1u;
+  p.header_tokens = p.tokens;
+  return p;
+}
 
+// Rows up to which a call goes through the one-CTA-per-row kernel with direct offsets.  It has no pipeline to fill, and up to
+// six rows per SM that is worth more than overlapping the stages of a row (4096 fp16: 300 rows 9.1 us against 14.5, 900 rows
+// 15.3 against 18.9, 1300 rows 20.1 against 21.7, 2048 rows 29.7 against 26.6).  Each row reads the sizes of all rows before
+// it, so the work of that grows with the square.
+static int64_t direct_rows(const tsq_plan_t* plan) { return 6 * static_cast<int64_t>(plan->sms); }
+
+tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, size_t blob_bytes,
+                        void* ws_dev, size_t ws_bytes, void* cuda_stream) {
+  const tsq_status_t args_ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
+  if (args_ok != TSQ_OK) return args_ok;
+  EncodeParams p = encode_params(plan, x_dev, tokens, blob_dev, ws_dev);
   cudaError_t e;
-  // The one-CTA-per-row kernel with direct offsets has no pipeline to fill, and up to this many rows that is worth more than
-  // overlapping the stages of a row (4096 fp16: 300 rows 9.1 us against 14.5, 900 rows 15.3 against 18.9, 1300 rows 20.1 against
-  // 21.7, 2048 rows 29.7 against 26.6).  Each row reads the sizes of all rows before it, so the work of that grows with the square.
-  const int64_t direct_rows = 6 * static_cast<int64_t>(plan->sms);
-  if (plan->pipe_ctas_per_sm > 0 && tokens > direct_rows) {
+  if (plan->pipe_ctas_per_sm > 0 && tokens > direct_rows(plan)) {
     // many rows: persistent CTAs that overlap the stages of consecutive rows
     p.compute_threads = plan->pipe_compute;
     p.park_stride = plan->pipe_park;
@@ -366,23 +456,15 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
     const int grid = tokens > 0 ? static_cast<int>(tokens) : 1;
     // up to one CTA per SM is resident whatever the CTA's size: such a call needs no tickets
     const int64_t sms = plan->sms;
-    p.direct_tiles = tokens < 1 || tokens > direct_rows ? 0u : tokens <= sms ? 1u : 2u;
+    p.direct_tiles = tokens < 1 || tokens > direct_rows(plan) ? 0u : tokens <= sms ? 1u : 2u;
     e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, static_cast<cudaStream_t>(cuda_stream));
   }
   g_launches.fetch_add(1);
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
 }
 
-tsq_status_t tsq_decode(const tsq_plan_t* plan, const void* blob_dev, size_t blob_bytes, int64_t tokens, void* y_dev,
-                        void* ws_dev, size_t ws_bytes, void* cuda_stream) {
-  if (!plan || !blob_dev || !ws_dev || tokens < 0 || static_cast<unsigned long long>(tokens) > plan->max_tokens)
-    return TSQ_ERR_INVALID_ARG;
-  if (tokens > 0 && !y_dev) return TSQ_ERR_INVALID_ARG;
-  if (!aligned16(y_dev) || !aligned16(blob_dev) || !aligned16(ws_dev)) return TSQ_ERR_INVALID_ARG;
+static DecodeParams decode_params(const tsq_plan_t* plan, const void* blob_dev, size_t blob_bytes, int64_t tokens, void* y_dev, void* ws_dev) {
   const BlobLayout L = layout_for(plan, static_cast<unsigned long long>(tokens));
-  if (blob_bytes < L.total || ws_bytes < plan->workspace_bytes) return TSQ_ERR_BUFFER_TOO_SMALL;
-  if (tokens == 0) return TSQ_OK;
-
   DecodeParams p;
   std::memset(&p, 0, sizeof p);
   p.blob = static_cast<const unsigned char*>(blob_dev);
@@ -397,6 +479,12 @@ tsq_status_t tsq_decode(const tsq_plan_t* plan, const void* blob_dev, size_t blo
   p.dtype = static_cast<uint32_t>(plan->dtype);
   p.variant = plan->variant;
   p.blob_bytes = blob_bytes;
+  p.header_tokens = p.tokens;
+  return p;
+}
+
+static tsq_status_t launch_decode_part(const tsq_plan_t* plan, DecodeParams& p, void* cuda_stream) {
+  const int64_t tokens = p.tokens;
   // A call that fills the device once lets the next grid in early (0.6 us per call at 64 rows).  A longer one does not: an
   // encode that follows it would be set up unevenly over the SMs that become free first, which costs its persistent CTAs
   // more than the launch (32768 x 4096 encode + decode: 312 us with, 295 us without).
@@ -408,6 +496,19 @@ tsq_status_t tsq_decode(const tsq_plan_t* plan, const void* blob_dev, size_t blo
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
 }
 
+tsq_status_t tsq_decode(const tsq_plan_t* plan, const void* blob_dev, size_t blob_bytes, int64_t tokens, void* y_dev,
+                        void* ws_dev, size_t ws_bytes, void* cuda_stream) {
+  if (!plan || !blob_dev || !ws_dev || tokens < 0 || static_cast<unsigned long long>(tokens) > plan->max_tokens)
+    return TSQ_ERR_INVALID_ARG;
+  if (tokens > 0 && !y_dev) return TSQ_ERR_INVALID_ARG;
+  if (!aligned16(y_dev) || !aligned16(blob_dev) || !aligned16(ws_dev)) return TSQ_ERR_INVALID_ARG;
+  const BlobLayout L = layout_for(plan, static_cast<unsigned long long>(tokens));
+  if (blob_bytes < L.total || ws_bytes < plan->workspace_bytes) return TSQ_ERR_BUFFER_TOO_SMALL;
+  if (tokens == 0) return TSQ_OK;
+
+  DecodeParams p = decode_params(plan, blob_dev, blob_bytes, tokens, y_dev, ws_dev);
+  return launch_decode_part(plan, p, cuda_stream);
+}
 tsq_status_t tsq_encode_noalloc(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev,
                                 size_t blob_bytes, void* cuda_stream) {
   if (!plan) return TSQ_ERR_INVALID_ARG;
@@ -471,6 +572,136 @@ tsq_status_t tsq_workspace_status(const void* ws_dev, uint32_t* encode_status, u
   return TSQ_OK;
 }
 
+// Host-buffer calls of more than a few megabytes go in parts of consecutive rows, so that the link is busy in both directions
+// while the kernels run: a part is copied in, encoded (or decoded) and copied out, each on its own stream.  The copies are what
+// such a call costs (2048 x 4096 fp16: 16.8 MB one way and 8.5 MB the other at about 55 GB/s, against 30 us of kernels).  Rows
+// of a part: an eighth of the call, at least 1 MB and at most what direct calls take.
+static int64_t part_rows(const tsq_plan_t* plan, int64_t tokens) {
+  int device = -1;
+  if (cudaGetDevice(&device) != cudaSuccess || device != plan->device) return tokens;  // the copy streams belong to the plan's device
+  const int64_t row = static_cast<int64_t>(plan->row_bytes), least = ((1 << 20) + row - 1) / row;
+  const int64_t rows = std::min(std::max((tokens + 7) / 8, least), direct_rows(plan));
+  return rows * row < (1 << 20) || tokens * row < (4 << 20) ? tokens : rows;
+}
+
+// The per-token sections of a part that starts at row t0.
+static BlobLayout part_layout(BlobLayout lay, int64_t t0) {
+  const unsigned long long t = static_cast<unsigned long long>(t0);
+  lay.off_bits += t;
+  lay.off_scale += 4 * t;
+  lay.off_zp += 4 * t;
+  lay.off_word_off += 4 * t;
+  lay.off_out_ptr += 4 * t;
+  return lay;
+}
+
+static tsq_status_t encode_host_parts(const tsq_plan_t* plan, HostPipe& pipe, const void* x_host, int64_t tokens, int64_t part, unsigned char* bh,
+                                      uint64_t* payload_bytes, void* x_dev, void* blob_dev, void* ws_dev, cudaStream_t st) {
+  const BlobLayout L = layout_for(plan, static_cast<unsigned long long>(tokens));
+  const int64_t parts = (tokens + part - 1) / part;
+  const unsigned char* bd = static_cast<const unsigned char*>(blob_dev);
+  const size_t row = plan->row_bytes;
+  cudaError_t e = cudaEventRecord(pipe.begin, st);  // what the caller has queued may still use the buffers
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe.in, pipe.begin, 0);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe.out, pipe.begin, 0);
+  unsigned long long words = 0, outliers = 0;
+  uint32_t status = TSQ_OK;
+  int64_t queued = 0;
+  for (int64_t c = 0; e == cudaSuccess && c < parts; ++c) {
+    for (; e == cudaSuccess && queued < parts && queued < c + kPipeSlots / 2; ++queued) {
+      const int64_t t0 = queued * part, n = std::min(part, tokens - t0);
+      const int slot = static_cast<int>(queued % kPipeSlots);
+      unsigned char* xd = static_cast<unsigned char*>(x_dev) + static_cast<size_t>(t0) * row;
+      e = cudaMemcpyAsync(xd, static_cast<const unsigned char*>(x_host) + static_cast<size_t>(t0) * row, static_cast<size_t>(n) * row, cudaMemcpyHostToDevice, pipe.in);
+      if (e == cudaSuccess) e = cudaEventRecord(pipe.landed[slot], pipe.in);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(st, pipe.landed[slot], 0);
+      if (e != cudaSuccess) break;
+      EncodeParams p = encode_params(plan, xd, tokens, blob_dev, ws_dev);
+      p.lay = part_layout(L, t0);
+      p.tokens = static_cast<uint32_t>(n);
+      p.direct_tiles = n <= plan->sms ? 1u : 2u;
+      p.chained = t0 > 0 ? 1u : 0u;
+      p.write_header = queued == parts - 1 ? 1u : 0u;
+      p.totals = pipe.totals + 4 * slot;
+      e = launch_encode_rows(p, static_cast<int>(n), plan->enc_threads, plan->enc_upt, st);
+      g_launches.fetch_add(1);
+      if (e == cudaSuccess) e = cudaEventRecord(pipe.ready[slot], st);
+    }
+    if (e == cudaSuccess) e = cudaEventSynchronize(pipe.ready[c % kPipeSlots]);
+    if (e != cudaSuccess) break;
+    const unsigned long long* t = pipe.totals + 4 * (c % kPipeSlots);
+    if (t[2] != TSQ_OK) status = static_cast<uint32_t>(t[2]);
+    const unsigned long long w1 = t[0], o1 = std::min(t[1], L.outlier_capacity);
+    if (w1 < words || w1 > L.words_capacity || o1 < outliers) break;  // a part that failed: its status says so
+    if (w1 > words) e = cudaMemcpyAsync(bh + L.off_words + 4 * words, bd + L.off_words + 4 * words, 4 * (w1 - words), cudaMemcpyDeviceToHost, pipe.out);
+    if (e == cudaSuccess && o1 > outliers) e = cudaMemcpyAsync(bh + L.off_outl + 4 * outliers, bd + L.off_outl + 4 * outliers, 4 * (o1 - outliers), cudaMemcpyDeviceToHost, pipe.out);
+    words = w1;
+    outliers = o1;
+  }
+  // the header and the per-token fields, once the last part is through
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(bh, bd, static_cast<size_t>(L.off_words), cudaMemcpyDeviceToHost, pipe.out);
+  const cudaError_t done[3] = {cudaStreamSynchronize(pipe.in), cudaStreamSynchronize(st), cudaStreamSynchronize(pipe.out)};
+  if (e != cudaSuccess || done[0] != cudaSuccess || done[1] != cudaSuccess || done[2] != cudaSuccess) return TSQ_ERR_CUDA;
+  BlobHeader h;
+  std::memcpy(&h, bh, sizeof h);
+  if (h.magic != kMagic) return TSQ_ERR_CORRUPT_BLOB;
+  if (payload_bytes) *payload_bytes = payload_of(h.tokens, h.total_words, std::min<unsigned long long>(h.total_outliers, L.outlier_capacity));
+  return static_cast<tsq_status_t>(h.status != TSQ_OK ? h.status : status);
+}
+
+// Whether the offsets at the parts' boundaries can be used to copy a blob in parts.
+static bool parts_in_order(const BlobLayout& L, const unsigned char* bh, int64_t tokens, int64_t part, unsigned long long words, unsigned long long outliers) {
+  uint32_t w = 0, o = 0;
+  for (int64_t t = 0;; t = std::min(t + part, tokens)) {
+    uint32_t w1, o1;
+    std::memcpy(&w1, bh + L.off_word_off + 4 * t, 4);
+    std::memcpy(&o1, bh + L.off_out_ptr + 4 * t, 4);
+    if (w1 < w || o1 < o || w1 > words || o1 > outliers || (t == 0 && (w1 != 0 || o1 != 0))) return false;
+    w = w1;
+    o = o1;
+    if (t == tokens) return w == words && o == outliers;
+  }
+}
+
+static tsq_status_t decode_host_parts(const tsq_plan_t* plan, HostPipe& pipe, const unsigned char* bh, size_t blob_bytes, int64_t tokens, int64_t part,
+                                      void* y_host, void* blob_dev, void* y_dev, void* ws_dev, cudaStream_t st) {
+  const BlobLayout L = layout_for(plan, static_cast<unsigned long long>(tokens));
+  unsigned char* bd = static_cast<unsigned char*>(blob_dev);
+  const size_t row = plan->row_bytes;
+  const auto at = [&](unsigned long long section, int64_t t) {
+    uint32_t v;
+    std::memcpy(&v, bh + section + 4 * t, 4);
+    return static_cast<size_t>(v);
+  };
+  cudaError_t e = cudaEventRecord(pipe.begin, st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe.in, pipe.begin, 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(bd, bh, static_cast<size_t>(L.off_words), cudaMemcpyHostToDevice, pipe.in);
+  int slot = 0;
+  for (int64_t t0 = 0; e == cudaSuccess && t0 < tokens; t0 += part, slot = (slot + 1) % kPipeSlots) {
+    const int64_t n = std::min(part, tokens - t0);
+    const size_t w0 = at(L.off_word_off, t0), w1 = at(L.off_word_off, t0 + n), o0 = at(L.off_out_ptr, t0), o1 = at(L.off_out_ptr, t0 + n);
+    if (w1 > w0) e = cudaMemcpyAsync(bd + L.off_words + 4 * w0, bh + L.off_words + 4 * w0, 4 * (w1 - w0), cudaMemcpyHostToDevice, pipe.in);
+    if (e == cudaSuccess && o1 > o0) e = cudaMemcpyAsync(bd + L.off_outl + 4 * o0, bh + L.off_outl + 4 * o0, 4 * (o1 - o0), cudaMemcpyHostToDevice, pipe.in);
+    if (e == cudaSuccess) e = cudaEventRecord(pipe.landed[slot], pipe.in);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, pipe.landed[slot], 0);
+    if (e != cudaSuccess) break;
+    unsigned char* yd = static_cast<unsigned char*>(y_dev) + static_cast<size_t>(t0) * row;
+    DecodeParams p = decode_params(plan, blob_dev, blob_bytes, tokens, yd, ws_dev);
+    p.lay = part_layout(L, t0);
+    p.tokens = static_cast<uint32_t>(n);
+    if (launch_decode_part(plan, p, st) != TSQ_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess) e = cudaEventRecord(pipe.ready[slot], st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe.out, pipe.ready[slot], 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(static_cast<unsigned char*>(y_host) + static_cast<size_t>(t0) * row, yd, static_cast<size_t>(n) * row, cudaMemcpyDeviceToHost, pipe.out);
+  }
+  uint32_t dec = 0;
+  const tsq_status_t ws = tsq_workspace_status(ws_dev, nullptr, &dec, st);
+  const cudaError_t done[2] = {cudaStreamSynchronize(pipe.in), cudaStreamSynchronize(pipe.out)};
+  if (e != cudaSuccess || done[0] != cudaSuccess || done[1] != cudaSuccess) return TSQ_ERR_CUDA;
+  return ws != TSQ_OK ? ws : static_cast<tsq_status_t>(dec);
+}
+
 tsq_status_t tsq_encode_host(const tsq_plan_t* plan, const void* x_host, int64_t tokens, void* blob_host,
                              size_t blob_bytes, uint64_t* payload_bytes, void* x_dev, void* blob_dev, void* ws_dev,
                              size_t ws_bytes, void* cuda_stream) {
@@ -481,6 +712,16 @@ tsq_status_t tsq_encode_host(const tsq_plan_t* plan, const void* x_host, int64_t
   const BlobLayout L = layout_for(plan, static_cast<unsigned long long>(tokens));
   if (blob_bytes < L.total) return TSQ_ERR_BUFFER_TOO_SMALL;
   const size_t x_bytes = static_cast<size_t>(tokens) * plan->hidden * 2u;
+  const int64_t part = part_rows(plan, tokens);
+  if (part < tokens) {
+    const tsq_status_t ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
+    if (ok != TSQ_OK) return ok;
+    HostPipe* pipe = plan->host_pipes.take();
+    if (!pipe) return TSQ_ERR_CUDA;
+    const tsq_status_t s = encode_host_parts(plan, *pipe, x_host, tokens, part, static_cast<unsigned char*>(blob_host), payload_bytes, x_dev, blob_dev, ws_dev, st);
+    plan->host_pipes.give_back(pipe);
+    return s;
+  }
   if (x_bytes && cudaMemcpyAsync(x_dev, x_host, x_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return TSQ_ERR_CUDA;
   const tsq_status_t s = tsq_encode(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes, cuda_stream);
   if (s != TSQ_OK) return s;
@@ -521,6 +762,16 @@ tsq_status_t tsq_decode_host(const tsq_plan_t* plan, const void* blob_host, size
     return TSQ_ERR_CORRUPT_BLOB;
   const unsigned long long stored = h.total_outliers < L.outlier_capacity ? h.total_outliers : L.outlier_capacity;
   const unsigned char* bh = static_cast<const unsigned char*>(blob_host);
+  const int64_t part = part_rows(plan, tokens);
+  if (part < tokens && parts_in_order(L, bh, tokens, part, h.total_words, stored)) {
+    if (!aligned16(y_dev) || !aligned16(blob_dev) || !aligned16(ws_dev)) return TSQ_ERR_INVALID_ARG;
+    if (ws_bytes < plan->workspace_bytes) return TSQ_ERR_BUFFER_TOO_SMALL;
+    HostPipe* pipe = plan->host_pipes.take();
+    if (!pipe) return TSQ_ERR_CUDA;
+    const tsq_status_t s = decode_host_parts(plan, *pipe, bh, blob_bytes, tokens, part, y_host, blob_dev, y_dev, ws_dev, st);
+    plan->host_pipes.give_back(pipe);
+    return s;
+  }
   unsigned char* bd = static_cast<unsigned char*>(blob_dev);
   if (cudaMemcpyAsync(bd, bh, static_cast<size_t>(L.off_words), cudaMemcpyHostToDevice, st) != cudaSuccess) return TSQ_ERR_CUDA;
   if (h.total_words && cudaMemcpyAsync(bd + L.off_words, bh + L.off_words, static_cast<size_t>(4 * h.total_words),

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kMaxThreads) decode_kernel(const __grid_consta
     if (tid == 0) record_decode_error(p, h->status);
     return;
   }
-  const bool header_ok = h->dtype == p.dtype && h->hidden == p.hidden && h->tokens == p.tokens && h->n_bits >= 1u &&
+  const bool header_ok = h->dtype == p.dtype && h->hidden == p.hidden && h->tokens == p.header_tokens && h->n_bits >= 1u &&
                          h->n_bits <= static_cast<uint32_t>(kMaxCand) && h->bits[(h->n_bits - 1u) & 7u] == p.bmax &&
                          h->bits[7] == p.variant &&
                          h->outlier_capacity == static_cast<uint32_t>(p.lay.outlier_capacity) &&

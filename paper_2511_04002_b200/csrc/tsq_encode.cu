@@ -377,12 +377,12 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
           planes_of_bytes(tb, r);
           bool passed = false;
           if (KIND == kKind84) {
-            const uint32_t sum = __reduce_add_sync(kFull, distortion_8_to_4(r));
+            const uint32_t sum = __reduce_add_sync(kFull, certain_distortion_8_to_4(r));
             if (lane == 0 && sum != 0u) atomicAdd(&m.S[ci], static_cast<int>(sum));
             compute_barrier(nt);
             // usually the certain differences alone exceed the tolerance; when they do not, the exact sum is formed (its
             // codes are needed anyway if the candidate passes)
-            if (static_cast<int>(static_cast<uint32_t>(m.S[ci]) & 0xffffu) <= p.s_max) {
+            if (m.S[ci] <= p.s_max) {
               uint32_t y[16];
 #pragma unroll
               for (uint32_t j = 0; j < 4; ++j) {
@@ -548,7 +548,8 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
       float one = 0.0f;
       if (KIND == kKind84) {
         const Level top = m.lv[p.n_bits - 1];
-        if (divide == 0u) one = one_fma_factor<BF16>(m.lo, m.hi, top, lane);
+        float s = 0.0f;
+        if (divide == 0u) one = m.lo == 0.0f ? quick_level(m.hi, &s) : one_fma_factor<BF16>(m.lo, m.hi, top, lane);
         if (lane == 0) m.S[kExactSlot] = 0;
       }
       if (lane == 0) {
@@ -722,7 +723,7 @@ static PipeKernel pipe_kernel_of(bool bf16, bool full) {
 }
 static PipeKernel pipe_kernel(const EncodeParams& p, bool full, int* index) {
   const bool bf16 = p.dtype == TSQ_BF16;
-  const int kind = p.variant != 0u ? kKindSigned : p.n_bits >= 2 && p.bits[p.n_bits - 1] == 8 && p.bits[p.n_bits - 2] == 4 ? kKind84 : kKindExact;
+  const int kind = p.variant != 0u ? kKindSigned : ends_in_4_and_8(p) ? kKind84 : kKindExact;
   *index = kind * 4 + (bf16 ? 2 : 0) + (full ? 1 : 0);
   return kind == kKindSigned ? pipe_kernel_of<kKindSigned>(bf16, full) : kind == kKind84 ? pipe_kernel_of<kKind84>(bf16, full) : pipe_kernel_of<kKindExact>(bf16, full);
 }

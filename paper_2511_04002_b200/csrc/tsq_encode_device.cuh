@@ -342,17 +342,30 @@ __device__ __forceinline__ float one_fma_factor(float lo, float hi, const Level&
   return __all_sync(kFull, same) ? top.r : 0.0f;
 }
 
-// Distortion of a group between the 8-bit level (7 code bits) and the 4-bit level, from the 8-bit codes' bit-planes alone
-// (r[k] = bit k of the codes).  Both levels round the same magnitude m, q = rint(m 127 / R) and low = rint(m 7 / R) up to
-// binary32 rounding, so |(q >> 4) - low| is 0 or 1 and is fixed by q except for the codes whose rounding interval contains
-// one of the low level's boundaries (k + 1/2) 127 / 7 = 9.07, 27.2, 45.4, 63.5, 81.6, 99.8, 117.9.  With q folded to
-// q' = min(q, 127 - q), j = q' >> 4 and n = q' & 15: the difference is 1 for n > 9 + 2j, 0 for n < 9 + 2j, open for
-// n = 9 + 2j.  Returns the number of certain differences, and of open codes in the upper half of the word.
-__device__ __forceinline__ uint32_t distortion_8_to_4(const uint32_t (&r)[8]) {
-  const uint32_t f = r[6], j1 = r[5] ^ f, j0 = r[4] ^ f, n3 = r[3] ^ f, n2 = r[2] ^ f, n1 = r[1] ^ f, n0 = r[0] ^ f;
-  const uint32_t one = n3 & ((~j1 & (n2 | (~j0 & n1))) | (j1 & ~j0 & n2 & n1));
-  const uint32_t open = n3 & n0 & ~(n2 ^ j1) & ~(n1 ^ j0);
-  return mad_u32(static_cast<uint32_t>(__popc(open)), 65536u, static_cast<uint32_t>(__popc(one)));
+// A lower bound of a group's distortion between the 8-bit level (7 code bits) and the 4-bit level, from the 8-bit codes'
+// bit-planes alone (r[k] = bit k of the codes).  Both levels round the same magnitude m, q = rint(m 127 / R) and
+// low = rint(m 7 / R) up to binary32 rounding, so |(q >> 4) - low| is 0 or 1 and is fixed by q except for the codes whose
+// rounding interval contains one of the low level's boundaries (k + 1/2) 127 / 7 = 9.07, 27.2, 45.4, 63.5, 81.6, 99.8, 117.9.
+// With q folded to q' = min(q, 127 - q), j = q' >> 4 and n = q' & 15: the difference is 1 for n > 9 + 2j, 0 for n < 9 + 2j and
+// open for n = 9 + 2j.  Returns the number of certain differences.
+__device__ __forceinline__ uint32_t certain_distortion_8_to_4(const uint32_t (&r)[8]) {
+  const uint32_t f = r[6], j1 = r[5] ^ f, j0 = r[4] ^ f, n3 = r[3] ^ f, n2 = r[2] ^ f, n1 = r[1] ^ f;
+  return __popc(n3 & ((~j1 & (n2 | (~j0 & n1))) | (j1 & ~j0 & n2 & n1)));
+}
+
+// The 8-bit level's scale of a row whose smallest magnitude is 0, as make_level gives it, and the factor of the one-FMA
+// codes (one_fma_factor), in about 20 instructions: s = fl(hi / 127) by a multiplication and two FMAs; 127 divides hi's
+// significand iff 127 s = hi exactly; and fl((hi / 2) / s) >= 63.5 iff (hi / 2) - 63.5 s (exact) >= -2^-19 s.  (A host-side
+// test compares all of it for every 16-bit hi.)  The factor is 0 when the row has to go the general way.
+__device__ __forceinline__ float quick_level(float hi, float* s_out) {
+  constexpr float kInv127 = 1.0f / 127.0f;
+  const float q0 = __fmul_rn(hi, kInv127), s = __fmaf_rn(__fmaf_rn(-127.0f, q0, hi), kInv127, q0);
+  const float rem = __fmaf_rn(-127.0f, s, hi), side = __fmaf_rn(-63.5f, s, 0.5f * hi);
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(s));
+  *s_out = s;
+  const float f = __fmul_rn(r, side >= -0x1p-19f * s ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
+  return s >= 0x1p-60f && s <= 0x1p60f && rem != 0.0f ? f : 0.0f;
 }
 
 // Pass C on one group of a row whose chosen level is plain: codes as bytes (code | sign << 7), transposed into
@@ -691,7 +704,7 @@ __device__ void write_header(const EncodeParams& p, unsigned long long total_wor
   h->version = kVersion;
   h->dtype = p.dtype;
   h->hidden = p.hidden;
-  h->tokens = p.tokens;
+  h->tokens = p.header_tokens;
   h->n_bits = static_cast<uint32_t>(p.n_bits);
 #pragma unroll
   for (int i = 0; i < 7; ++i) h->bits[i] = (i < p.n_bits) ? static_cast<uint8_t>(p.bits[i]) : 0;
@@ -701,6 +714,20 @@ __device__ void write_header(const EncodeParams& p, unsigned long long total_wor
   h->total_words = total_words;
   h->total_outliers = total_outliers;
   h->outlier_capacity = static_cast<uint32_t>(p.lay.outlier_capacity);
+}
+
+// Ends a call, or a part of one: header, status, end offsets.
+__device__ void end_part(const EncodeParams& p, uint32_t status, unsigned long long total_words, unsigned long long total_outliers) {
+  if (p.totals) {
+    p.totals[0] = total_words;
+    p.totals[1] = total_outliers;
+    p.totals[2] = status;
+    __threadfence_system();
+  }
+  if (p.write_header != 0u) {
+    write_header(p, total_words, total_outliers);
+    reinterpret_cast<BlobHeader*>(p.blob)->status = status;
+  }
 }
 
 // The CTA that finishes last publishes the totals and the status, and re-arms the workspace.  `direct`: the descriptors
@@ -728,8 +755,11 @@ __device__ void finish_call(const EncodeParams& p, uint32_t gen4, bool direct = 
       to = static_cast<uint32_t>(dout);
     }
   }
-  write_header(p, tw, to);
-  reinterpret_cast<BlobHeader*>(p.blob)->status = e;
+  if (p.chained != 0u) {
+    tw += reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_word_off)[0];
+    to += reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_out_ptr)[0];
+  }
+  end_part(p, e, tw, to);
   if (p.tokens == 0u) {  // no row writes the leading zeros of the two prefix-sum sections
     reinterpret_cast<uint32_t*>(p.blob + p.lay.off_word_off)[0] = 0u;
     reinterpret_cast<uint32_t*>(p.blob + p.lay.off_out_ptr)[0] = 0u;
@@ -755,7 +785,7 @@ __device__ __forceinline__ void write_token_fields(const EncodeParams& p, uint32
   reinterpret_cast<int32_t*>(p.blob + p.lay.off_zp)[tile] = zp;
   uint32_t* o_word_off = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_word_off);
   uint32_t* o_out_ptr = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_out_ptr);
-  if (tile == 0) {
+  if (tile == 0 && p.chained == 0u) {
     o_word_off[0] = 0;
     o_out_ptr[0] = 0;
   }

@@ -11,6 +11,7 @@ namespace {
 struct RowShared {
   Level lv[kMaxCand];  // lv[i]: AIQ parameters of candidate bits[i]
   int S[kMaxCand];     // distortion sum of candidate i against the top level
+  int certain;         // TOP84: certain differences between the 8-bit and the 4-bit codes
   RowPartials<32> part;
   uint32_t tile;
   uint32_t divide;     // some level of the row needs the division instruction
@@ -56,8 +57,7 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
 __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t gen4, uint32_t status, uint32_t total_w, uint32_t total_o) {
   if (status == TSQ_OK && total_o > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
   const bool ok = status != TSQ_ERR_TIMEOUT;
-  write_header(p, ok ? total_w : 0ull, ok ? total_o : 0ull);
-  reinterpret_cast<BlobHeader*>(p.blob)->status = status;
+  end_part(p, status, ok ? total_w : 0ull, ok ? total_o : 0ull);
   if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
   p.ws->ticket = 0u;  // every CTA has taken its own
   p.ws->gen = gen4 >> 2;
@@ -68,7 +68,9 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
 // DIRECT: calls of a few rows per SM: a row's offsets are read straight from the sizes of the rows before it
 // (direct_offsets) instead of walked back to.  With at most one row per SM every CTA is resident, so row = CTA index needs
 // no ticket.
-template <bool BF16, int UPT, int MAXT, bool SV, bool DIRECT>
+// TOP84: the candidates end in 4 and 8 bits (magnitudes): codes and planes at 8 bits first, and the 4-bit candidate decided from
+// the planes where they suffice (certain_distortion_8_to_4), else everything the general way.
+template <bool BF16, int UPT, int MAXT, bool SV, bool TOP84, bool DIRECT>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
   __shared__ RowShared sh;
@@ -76,6 +78,14 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
   launch_dependents();
   wait_for_prior_grids();
   const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
+  uint32_t part_w = 0u, part_o = 0u;  // where a later part of a call starts
+  if (DIRECT && p.chained != 0u) {
+    part_w = *reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_word_off);
+    part_o = *reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_out_ptr);
+    // never past the planes, whatever a part that has failed has left there
+    const unsigned long long most = static_cast<unsigned long long>(p.tokens) * static_cast<uint32_t>(p.bits[p.n_bits - 1]) * p.lay.wpp;
+    if (part_w + most > p.lay.words_capacity) part_w = 0u;
+  }
 
   uint32_t tile = blockIdx.x;
   if (!DIRECT || p.direct_tiles == 2u) {
@@ -142,21 +152,62 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
         sh.part.warp_cnt[warp] = wcnt;
       }
     }
+    if (TOP84 && tid == 0) sh.certain = 0;
     __syncthreads();
 
-    // ---- AIQ parameters of every candidate level (lane i of warp 0 takes candidate i) ----
     const int bmax = p.bits[p.n_bits - 1];
+    uint32_t r[UPT][8];
+    Level best;
+    int bstar = bmax;
+    uint32_t row_cnt = 0u, cnt_before = 0u;  // outliers of the row, of the warps before this one
+    bool settled = false, divide = false;
+    if (TOP84) {
+      // ---- every thread forms the row's extremes and its top level for itself (a few dozen instructions for the usual row) ----
+      const uint32_t pmin = __reduce_min_sync(kFull, lane < nwarps ? sh.part.warp_min[lane] : 0xffffu);
+      const uint32_t pmax = __reduce_max_sync(kFull, lane < nwarps ? sh.part.warp_max[lane] : 0u);
+      const uint32_t wc = lane < nwarps ? sh.part.warp_cnt[lane] : 0u;
+      row_cnt = __reduce_add_sync(kFull, wc);
+      cnt_before = __reduce_add_sync(kFull, lane < warp ? wc : 0u);
+      const float lo = E::pattern_f32(pmin), hi = E::pattern_f32(pmax);
+      best.zp = 0;
+      best.qmax = 127;
+      float one = pmin == 0u ? quick_level(hi, &best.s) : 0.0f;
+      bool plain = true;
+      if (one == 0.0f) {
+        best = make_level(lo, hi, 8, &plain);
+        if (plain) one = one_fma_factor<BF16>(lo, hi, best, lane);
+      }
+      if (plain) {
+        uint32_t S = 0u;
+#pragma unroll
+        for (int k = 0; k < UPT; ++k) {
+          uint32_t tb[8];
+          if (one != 0.0f) {
+            top_bytes_one_fma<BF16>(x[k], pack2f(one, one), tb);
+          } else {
+            top_bytes<BF16>(x[k], make_level2(best), tb);
+          }
+          planes_of_bytes(tb, r[k]);
+          S += certain_distortion_8_to_4(r[k]);
+        }
+        S = __reduce_add_sync(kFull, S);
+        if (lane == 0 && S != 0u) atomicAdd(&sh.certain, static_cast<int>(S));
+        __syncthreads();
+        settled = sh.certain > p.s_max;
+      }
+    }
+    if (!settled) {
+    // ---- AIQ parameters of every candidate level (lane i of warp 0 takes candidate i) ----
     if (warp == 0) {
       const uint32_t divide = row_levels<BF16, 32, SV>(p, sh.part, nwarps, lane, sh.lv, sh.S, &sh.row_cnt);
       if (lane == 0) sh.divide = divide;
     }
     __syncthreads();
-    const bool divide = sh.divide != 0u;
+    divide = sh.divide != 0u;
 
     // ---- Algorithm 1: descend the candidate list while the distortion stays within tolerance ----
     const Level top = sh.lv[p.n_bits - 1];
-    Level best = top;
-    int bstar = bmax;
+    best = top;
     for (int ci = p.n_bits - 2; ci >= 0; --ci) {
       const Level low = sh.lv[ci];
       const int shn = bmax - p.bits[ci];
@@ -176,7 +227,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
       bstar = p.bits[ci];
       best = low;
     }
-    const uint32_t row_cnt = sh.row_cnt;
+    row_cnt = sh.row_cnt;
+    cnt_before = sh.part.warp_cnt[warp];
+    }
     const uint32_t agg_w = static_cast<uint32_t>(bstar) * p.lay.wpp;
 
     // ---- this row's sizes are known: let the rows behind it see them, then pack ----
@@ -187,9 +240,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
         publish_aggregate(p, gen4, tile, agg_w, row_cnt);
       }
     }
-    uint32_t r[UPT][8];
 #pragma unroll
     for (int k = 0; k < UPT; ++k) {
+      if (settled) continue;
       if (divide) {
         divide_pack_regs<BF16, SV>(x[k], best, r[k]);
         if (SV && nvalid[k] < 4u) {  // pad bits stay 0: the zeros past the end of the row got the code of the value 0
@@ -221,7 +274,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
     __syncthreads();
     uint32_t word_off = sh.word_off, out_base = sh.out_base, status = sh.status;
     if (DIRECT) {
-      word_off = out_base = status = 0u;
+      word_off = part_w;
+      out_base = part_o;
+      status = 0u;
       for (uint32_t w = 0; w < nwarps; ++w) {
         word_off += sh.warp_w[w];
         out_base += sh.warp_o[w];
@@ -250,7 +305,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
         if (cnt != 0u) {
           uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
           const uint16_t* x16 = p.x + static_cast<size_t>(tile) * p.hidden;
-          unsigned long long at = static_cast<unsigned long long>(out_base) + sh.part.warp_cnt[warp] + (incl - cnt);
+          unsigned long long at = static_cast<unsigned long long>(out_base) + cnt_before + (incl - cnt);
           bool overflow = false;
 #pragma unroll
           for (int k = 0; k < UPT; ++k) {
@@ -280,23 +335,29 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
 
 }  // namespace
 
-template <bool SV, bool DIRECT>
+template <bool SV, bool TOP84, bool DIRECT>
 static cudaError_t launch_rows_variant(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
   const bool bf16 = p.dtype == TSQ_BF16;
   if (upt == 1 && threads <= 256) {
-    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 256, SV, DIRECT> : encode_rows_kernel<false, 1, 256, SV, DIRECT>, grid, threads, 0, stream, p);
+    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 256, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, SV, TOP84, DIRECT>, grid, threads, 0, stream, p);
   }
+  if (TOP84) return cudaErrorInvalidValue;
   if (upt == 1) {
-    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 1024, SV, DIRECT> : encode_rows_kernel<false, 1, 1024, SV, DIRECT>, grid, threads, 0, stream, p);
+    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 1024, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, SV, false, DIRECT>, grid, threads, 0, stream, p);
   }
-  return launch_overlapped(bf16 ? encode_rows_kernel<true, 2, 1024, SV, DIRECT> : encode_rows_kernel<false, 2, 1024, SV, DIRECT>, grid, threads, 0, stream, p);
+  return launch_overlapped(bf16 ? encode_rows_kernel<true, 2, 1024, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, SV, false, DIRECT>, grid, threads, 0, stream, p);
+}
+
+template <bool DIRECT>
+static cudaError_t launch_rows_of(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
+  if (p.variant != 0u) return launch_rows_variant<true, false, DIRECT>(p, grid, threads, upt, stream);
+  // (in the CTAs of more than 256 threads, 64 registers each, the extra path costs more than it saves)
+  if (ends_in_4_and_8(p) && upt == 1 && threads <= 256) return launch_rows_variant<false, true, DIRECT>(p, grid, threads, upt, stream);
+  return launch_rows_variant<false, false, DIRECT>(p, grid, threads, upt, stream);
 }
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
-  if (p.direct_tiles != 0u) {
-    return p.variant != 0u ? launch_rows_variant<true, true>(p, grid, threads, upt, stream) : launch_rows_variant<false, true>(p, grid, threads, upt, stream);
-  }
-  return p.variant != 0u ? launch_rows_variant<true, false>(p, grid, threads, upt, stream) : launch_rows_variant<false, false>(p, grid, threads, upt, stream);
+  return p.direct_tiles != 0u ? launch_rows_of<true>(p, grid, threads, upt, stream) : launch_rows_of<false>(p, grid, threads, upt, stream);
 }
 
 }  // namespace tsq

@@ -94,7 +94,17 @@ struct EncodeParams {
   uint32_t dtype;
   uint32_t variant;                          // 0: sign + magnitude codes; 1: codes of the signed values
   float tau, delta;
+  // A call may be encoded in parts, in order, by direct calls (direct_tiles != 0): `tokens`, x and the layout's per-token
+  // sections are then those of the part.
+  uint32_t chained;                          // 1: a later part: its offsets start at the last entries of the part before
+  uint32_t write_header, header_tokens;      // 1: the last part (or the only one); tokens of the whole call
+  unsigned long long* totals;                // where the part's end offsets go (host memory), or null
 };
+
+// The two widest candidates are 4 and 8 bits of a magnitude plan: the first decision can be taken on the 8-bit planes.
+inline bool ends_in_4_and_8(const EncodeParams& p) {
+  return p.variant == 0u && p.n_bits >= 2 && p.bits[p.n_bits - 1] == 8 && p.bits[p.n_bits - 2] == 4;
+}
 
 struct DecodeParams {
   const unsigned char* blob;
@@ -104,6 +114,7 @@ struct DecodeParams {
   uint32_t tokens, hidden, units, chunks;
   uint32_t bmax, dtype;
   uint32_t variant;
+  uint32_t header_tokens;                    // tokens of the whole call, when `tokens` is those of a part
   uint32_t overlap_next;                     // 1: the stream's next grid may be set up while this one runs
   unsigned long long blob_bytes;
 };

@@ -1,0 +1,55 @@
+"""Calls of a few rows per SM (offsets read directly, last row's CTA ends the call) at the edges of their range, several on one
+workspace, mixed with calls of the other kernels."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import tsq_ref as R
+from paper_2511_04002_b200 import binding as B
+from paper_2511_04002_b200 import synth
+from tests._parity import assert_blobs_equal, gpu_decode, gpu_encode
+from tests.test_gpu_parity import rand16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hidden", [8, 1032, 4096, 16384])
+def test_edges_of_the_range_on_one_workspace(hidden):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sizes = [1, 2, sms - 1, sms, sms + 1, 2 * sms + 1, 6 * sms, 6 * sms + 1, 3]
+    plan = B.Plan(torch.float16, hidden, max(sizes), 6.0, [2, 4, 8], 0.2)
+    ws = plan.alloc(1)[1]
+    for k, T in enumerate(sizes):
+        x = rand16((T, hidden), torch.float16, seed=hidden + k, scale=2.0, outlier_rate=0.01)
+        x[::3] = (x[::3].float().abs() * 0.2).to(torch.float16)          # rows without outliers
+        x[1::5] = (x[1::5].float().abs() ** 3 * 0.05).to(torch.float16)  # rows that descend
+        blob = torch.zeros(plan.sizes(T)[0], dtype=torch.uint8, device="cuda")
+        _, got, _ = gpu_encode(plan, x, ws=ws, blob=blob)
+        ref = R.encode(synth.raw_u16(x), R.F16, 6.0, [2, 4, 8], 0.2)
+        assert_blobs_equal(got, ref)
+        assert np.array_equal(gpu_decode(plan, blob, T, ws), R.decode(ref))
+    assert plan.workspace_status(ws) == (0, 0)
+
+
+def test_many_calls_back_to_back_on_one_stream():
+    # launches overlap their predecessors: every call reads what the one before it wrote
+    T, H = 64, 4096
+    plan = B.Plan(torch.bfloat16, H, T, 6.0, [2, 4, 8], 0.2)
+    blob, ws = plan.alloc(T)
+    x = rand16((T, H), torch.bfloat16, seed=1, scale=2.0, outlier_rate=0.01).cuda()
+    y = torch.empty_like(x)
+    want = None
+    for i in range(300):
+        plan.encode(x if i == 0 else y, blob, ws)        # encodes what the last call decoded
+        plan.decode(blob, T, y, ws)
+        if i == 0:
+            want = y.clone()
+    torch.cuda.synchronize()
+    assert plan.workspace_status(ws) == (0, 0)
+    cpu = want.cpu()
+    for _ in range(299):
+        nxt = synth.from_raw_u16(R.decode(R.encode(synth.raw_u16(cpu), R.BF16, 6.0, [2, 4, 8], 0.2)), "bf16")
+        if torch.equal(nxt.view(torch.int16), cpu.view(torch.int16)):
+            break
+        cpu = nxt
+    assert torch.equal(y.cpu().view(torch.int16), cpu.view(torch.int16))
