@@ -574,14 +574,17 @@ tsq_status_t tsq_workspace_status(const void* ws_dev, uint32_t* encode_status, u
 
 // Host-buffer calls of more than a few megabytes go in parts of consecutive rows, so that the link is busy in both directions
 // while the kernels run: a part is copied in, encoded (or decoded) and copied out, each on its own stream.  The copies are what
-// such a call costs (2048 x 4096 fp16: 16.8 MB one way and 8.5 MB the other at about 55 GB/s, against 30 us of kernels).  Rows
-// of a part: an eighth of the call, at least 1 MB and at most what direct calls take.
+// such a call costs (2048 x 4096 fp16: 16.8 MB one way and 8.5 MB the other at about 55 GB/s, against 30 us of kernels).  Every
+// further part costs both directions about 5 us, more when they run at once (16 MB each way at once: 381 us in 2 parts, 421 in
+// 4, 473 in 8, 627 in 16, against 614 one after the other): three parts (encode + decode of the tensor above 1016 us in one part,
+// 926 in two, 915 in three, 957 in four), or as many as direct calls need.
 static int64_t part_rows(const tsq_plan_t* plan, int64_t tokens) {
   int device = -1;
   if (cudaGetDevice(&device) != cudaSuccess || device != plan->device) return tokens;  // the copy streams belong to the plan's device
-  const int64_t row = static_cast<int64_t>(plan->row_bytes), least = ((1 << 20) + row - 1) / row;
-  const int64_t rows = std::min(std::max((tokens + 7) / 8, least), direct_rows(plan));
-  return rows * row < (1 << 20) || tokens * row < (4 << 20) ? tokens : rows;
+  const int64_t row = static_cast<int64_t>(plan->row_bytes), parts = std::min<int64_t>(3, tokens * row / (4 << 20));
+  if (parts < 2) return tokens;
+  const int64_t rows = std::min((tokens + parts - 1) / parts, direct_rows(plan));
+  return rows * row < (1 << 20) ? tokens : rows;
 }
 
 // The per-token sections of a part that starts at row t0.
