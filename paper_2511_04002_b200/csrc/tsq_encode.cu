@@ -99,6 +99,7 @@ struct RowMeta {
   int zp;
   float lo, hi;    // smallest and largest magnitude
   float one_fma;   // kKind84: the factor of the one-FMA codes (one_fma_factor), 0: the three-operation quotient
+  OneFma top_one, low_one;  // kKindSigned: both levels' one-FMA codes; one_fma = 0: not for this row
   uint32_t heavy;  // 1: the side buffer holds the row's outlier bitmaps (more outliers than a list holds)
 };
 
@@ -253,19 +254,6 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
         }
         bitmap_cur = split_group<BF16>(x, nvalid, p.thr16 * 0x10001u, mn2, mx2);
         cnt_cur = __popc(bitmap_cur);
-        if (SV) {
-          // min / max of the signed values of T_below instead (outlier slots are +0 by now): as order keys
-          mn2 = 0xffffffffu;
-          mx2 = 0u;
-#pragma unroll
-          for (uint32_t i = 0; i < 16; ++i) {
-            if (FULL || (i >> 2) < nvalid) {
-              const uint32_t key2 = order_keys2(x[i]);
-              mn2 = __vminu2(mn2, key2);
-              mx2 = __vmaxu2(mx2, key2);
-            }
-          }
-        }
         if (bitmap_cur != 0u) {
           // the original pattern of the group's first outlier, from the parked row while it still holds it:
           // the CSR entry is written an iteration later, and most groups with an outlier have just one
@@ -276,8 +264,13 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
 #pragma unroll
           for (uint32_t j = 0; j < 4; ++j) xp[park_index(nt, u, j)] = make_uint4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
         }
-        const uint32_t mnv = __reduce_min_sync(kFull, min(mn2 & 0xffffu, mn2 >> 16));
-        const uint32_t mxv = __reduce_max_sync(kFull, max(mx2 & 0xffffu, mx2 >> 16));
+        uint32_t mnv, mxv;
+        if (SV) {  // of the signed values of T_below instead (outlier slots are +0 by now), as order keys
+          warp_keys(signed_extremes(x, FULL ? 4u : nvalid), &mnv, &mxv);
+        } else {
+          mnv = __reduce_min_sync(kFull, min(mn2 & 0xffffu, mn2 >> 16));
+          mxv = __reduce_max_sync(kFull, max(mx2 & 0xffffu, mx2 >> 16));
+        }
         const uint32_t wcnt = __reduce_add_sync(kFull, cnt_cur);
         if (lane == 0) {
           m.part.warp_min[warp] = mnv;
@@ -364,8 +357,13 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
             } else {
               const int c0 = ci >= 0 ? ci : 0;
               const Level low = m.lv[c0];
-              uint32_t S = distortion_first<BF16, SV>(y, make_level2(top), make_level2(low), bmax - p.bits[c0], tb, lb,
-                                                      (FULL || !SV) ? 4u : group_chunks(p, u));
+              uint32_t S;
+              if (SV && m.one_fma != 0.0f) {
+                S = distortion_first_one_fma<BF16>(y, m.top_one, m.low_one, bmax - p.bits[c0], tb, lb, FULL ? 4u : group_chunks(p, u));
+              } else {
+                S = distortion_first<BF16, SV>(y, make_level2(top), make_level2(low), bmax - p.bits[c0], tb, lb,
+                                               (FULL || !SV) ? 4u : group_chunks(p, u));
+              }
               if (ci >= 0) {
                 S = __reduce_add_sync(kFull, S);
                 if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
@@ -551,6 +549,19 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
         float s = 0.0f;
         if (divide == 0u) one = m.lo == 0.0f ? quick_level(m.hi, &s) : one_fma_factor<BF16>(m.lo, m.hi, top, lane);
         if (lane == 0) m.S[kExactSlot] = 0;
+      }
+      if (KIND == kKindSigned) {
+        const int low = p.n_bits >= 2 ? p.n_bits - 2 : 0;
+        OneFma t{0.0f, 0.0f}, l{0.0f, 0.0f};
+        if (divide == 0u) {
+          t = one_fma_signed<BF16>(m.lv[p.n_bits - 1], lane);
+          if (t.r != 0.0f) l = one_fma_signed<BF16>(m.lv[low], lane);
+        }
+        one = l.r;
+        if (lane == 0) {
+          m.top_one = t;
+          m.low_one = l;
+        }
       }
       if (lane == 0) {
         m.divide = divide;

@@ -282,6 +282,77 @@ __device__ __forceinline__ void planes_of_bytes(const uint32_t (&tb)[8], uint32_
   transpose8x32_select(r);
 }
 
+// ---- signed-values variant: codes by one FMA -----------------------------------------------------------------------
+
+// A level whose codes rint(fl(v / s)) - zp one FMA gives for every 16-bit value v of the row: code = low byte of
+// fma(v, r, add), add = 2^23 + 2^22 - zp.
+struct OneFma {
+  float r, add;  // r = 0: not known to hold for the level
+};
+// Tries the 16-bit value next to each of the level's boundaries zp + k + 1/2 (between any other value and a boundary lies at
+// least half a unit of the 16-bit type, thousands of times what the two computations can differ by); run by one full warp.
+template <bool BF16>
+__device__ __forceinline__ OneFma one_fma_signed(const Level& c, uint32_t lane) {
+  const float add = kRoundMagicSigned - static_cast<float>(c.zp);
+  bool same = c.zp > -(1 << 21) && c.zp < (1 << 21);
+  for (int k = static_cast<int>(lane); k < c.qmax; k += 32) {
+    const float b = __fmul_rn(static_cast<float>(c.zp + k) + 0.5f, c.s);
+    const float v = Elem<BF16>::lo_f32(Elem<BF16>::pack_rn(b, 0.0f));
+    const float q0 = __fmul_rn(v, c.r), q = __fmaf_rn(__fmaf_rn(q0, -c.s, v), c.r, q0);
+    same = same && __fadd_rn(q, kRoundMagicSigned) - static_cast<float>(c.zp) == __fmaf_rn(v, c.r, add);
+  }
+  return OneFma{__all_sync(kFull, same) ? c.r : 0.0f, add};
+}
+
+// distortion_first<BF16, true> with both levels' codes by one FMA.
+template <bool BF16>
+__device__ __forceinline__ uint32_t distortion_first_one_fma(const uint32_t (&x)[16], const OneFma& top, const OneFma& low, int sh,
+                                                             uint32_t (&tb)[8], uint32_t (&ql)[8], uint32_t nvalid) {
+  const uint32_t shmask = (0xffu >> sh) * 0x01010101u;
+  const uint64_t rt = pack2f(top.r, top.r), at = pack2f(top.add, top.add), rl = pack2f(low.r, low.r), al = pack2f(low.add, low.add);
+  uint32_t S = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint64_t va = values2<BF16>(x[8 * h + i]), vb = values2<BF16>(x[8 * h + 4 + i]);
+      const uint32_t ct4 = bytes4(fma2(va, rt, at), fma2(vb, rt, at)) & inside, q4 = bytes4(fma2(va, rl, al), fma2(vb, rl, al)) & inside;
+      S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
+      tb[4 * h + i] = ct4;
+      ql[4 * h + i] = q4;
+    }
+  }
+  return S;
+}
+
+// Extremes of a group's signed values: as signed and as unsigned 16-bit patterns.
+struct SignedExtremes {
+  uint32_t smax, umax, umin;
+};
+__device__ __forceinline__ SignedExtremes signed_extremes(const uint32_t (&x)[16], uint32_t nvalid) {
+  SignedExtremes e{0x80008000u, 0u, 0xffffffffu};
+#pragma unroll
+  for (uint32_t i = 0; i < 16; i += 2) {
+    if ((i >> 2) < nvalid) {
+      e.smax = __vimax3_s16x2(e.smax, x[i], x[i + 1]);
+      e.umax = __vimax3_u16x2(e.umax, x[i], x[i + 1]);
+      e.umin = __vimin3_u16x2(e.umin, x[i], x[i + 1]);
+    }
+  }
+  return e;
+}
+// The warp's smallest and largest value as order keys (in every lane).  Patterns of non-negative values order like the values,
+// those of negative ones the other way round: the largest value is the largest signed pattern if that is non-negative, else
+// the smallest unsigned one; the smallest is the largest unsigned pattern if that is negative, else the smallest.
+__device__ __forceinline__ void warp_keys(const SignedExtremes& e, uint32_t* min_key, uint32_t* max_key) {
+  const int smax = __reduce_max_sync(kFull, max(static_cast<int>(static_cast<short>(e.smax & 0xffffu)), static_cast<int>(e.smax) >> 16));
+  const uint32_t umax = __reduce_max_sync(kFull, max(e.umax & 0xffffu, e.umax >> 16)), umin = __reduce_min_sync(kFull, min(e.umin & 0xffffu, e.umin >> 16));
+  const bool none = umin > umax;  // no value in the warp's groups
+  *max_key = none ? 0u : order_keys2(smax >= 0 ? static_cast<uint32_t>(smax) : umin) & 0xffffu;
+  *min_key = none ? 0xffffu : order_keys2(umax >= 0x8000u ? umax : umin) & 0xffffu;
+}
+
 // ---- 8-bit top level: codes by one FMA, and the distortion from the codes' bit-planes ----------------------------
 
 // Top-level codes of a group as bytes (grouping and signs as in distortion_first) when one FMA per element gets them right
