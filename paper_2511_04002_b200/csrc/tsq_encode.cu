@@ -306,7 +306,8 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
       if (have_prev) {
         const uint32_t n = n_a - 1u;
         RowMeta& m = sh.meta[n % kMetaRing];
-        const bool divide = m.divide != 0u;
+        const bool clamp = KIND == kKindSigned && m.divide != 0u && m.one_fma != 0.0f;  // fast steps with the clamp, as far as the first candidate
+        const bool divide = m.divide != 0u && !clamp;
         const int bmax = p.bits[p.n_bits - 1];
         const uint32_t tile_prev = m.tile;
         const uint4* xp = xpark + (n % 3u) * (p.park_stride / 16u);
@@ -359,7 +360,9 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
               const Level low = m.lv[c0];
               uint32_t S;
               if (SV && m.one_fma != 0.0f) {
-                S = distortion_first_one_fma<BF16>(y, m.top_one, m.low_one, bmax - p.bits[c0], tb, lb, FULL ? 4u : group_chunks(p, u));
+                const uint32_t nv = FULL ? 4u : group_chunks(p, u);
+                S = clamp ? distortion_first_one_fma<BF16, true>(y, m.top_one, m.low_one, bmax - p.bits[c0], tb, lb, nv, top.qmax, low.qmax)
+                          : distortion_first_one_fma<BF16, false>(y, m.top_one, m.low_one, bmax - p.bits[c0], tb, lb, nv, top.qmax, low.qmax);
               } else {
                 S = distortion_first<BF16, SV>(y, make_level2(top), make_level2(low), bmax - p.bits[c0], tb, lb,
                                                (FULL || !SV) ? 4u : group_chunks(p, u));
@@ -400,7 +403,24 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
             compute_barrier(nt);
             passed = m.S[ci] <= p.s_max;
           }
-          if (passed) {
+          if (passed && clamp) {
+            // such a row that goes lower: the further candidates with the division instruction (see above)
+            bstar = p.bits[ci];
+            best_ci = ci;
+            const uint32_t* xw = reinterpret_cast<const uint32_t*>(xp);
+            for (--ci; ci >= 0; --ci) {
+              uint32_t S = rolled_distortion<BF16, SV>(xw, nt, u, top, m.lv[ci], bmax - p.bits[ci], 4u * (FULL ? 4u : group_chunks(p, u)));
+              S = __reduce_add_sync(kFull, S);
+              if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
+              compute_barrier(nt);
+              if (m.S[ci] > p.s_max) break;
+              bstar = p.bits[ci];
+              best_ci = ci;
+            }
+            const Planes8 pl = rolled_pack<BF16, SV>(xw, nt, u, m.lv[best_ci], 4u * (FULL ? 4u : group_chunks(p, u)));
+#pragma unroll
+            for (int k = 0; k < 8; ++k) r[k] = pl.v[k];
+          } else if (passed) {
             bstar = p.bits[ci];
             best_ci = ci;
             for (--ci; ci >= 0; --ci) {
@@ -553,7 +573,11 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
       if (KIND == kKindSigned) {
         const int low = p.n_bits >= 2 ? p.n_bits - 2 : 0;
         OneFma t{0.0f, 0.0f}, l{0.0f, 0.0f};
-        if (divide == 0u) {
+        // a row that needs the division instruction for its clamps alone (every scale in range) may still take the one-FMA
+        // codes, with the clamp, for its first candidate
+        bool in_range = true;
+        for (int i = 0; i < p.n_bits; ++i) in_range = in_range && m.lv[i].s >= 0x1p-60f && m.lv[i].s <= 0x1p60f;
+        if (in_range) {
           t = one_fma_signed<BF16>(m.lv[p.n_bits - 1], lane);
           if (t.r != 0.0f) l = one_fma_signed<BF16>(m.lv[low], lane);
         }

@@ -304,10 +304,19 @@ __device__ __forceinline__ OneFma one_fma_signed(const Level& c, uint32_t lane) 
   return OneFma{__all_sync(kFull, same) ? c.r : 0.0f, add};
 }
 
-// distortion_first<BF16, true> with both levels' codes by one FMA.
-template <bool BF16>
+// Patterns 2^23 + 2^22 + code: codes above qmax become qmax.
+__device__ __forceinline__ uint64_t clamp_codes2(uint64_t t, int qmax) {
+  uint32_t lo, hi;
+  unpack2u(t, lo, hi);
+  const uint32_t most = __float_as_uint(kRoundMagicSigned) + static_cast<uint32_t>(qmax);
+  return pack2u(min(lo, most), min(hi, most));
+}
+
+// distortion_first<BF16, true> with both levels' codes by one FMA.  CLAMP: the largest values' codes may be qmax + 1 and are
+// clamped (rows whose extremes both lie half-way between codes, as when both touch the threshold).
+template <bool BF16, bool CLAMP>
 __device__ __forceinline__ uint32_t distortion_first_one_fma(const uint32_t (&x)[16], const OneFma& top, const OneFma& low, int sh,
-                                                             uint32_t (&tb)[8], uint32_t (&ql)[8], uint32_t nvalid) {
+                                                             uint32_t (&tb)[8], uint32_t (&ql)[8], uint32_t nvalid, int qtop, int qlow) {
   const uint32_t shmask = (0xffu >> sh) * 0x01010101u;
   const uint64_t rt = pack2f(top.r, top.r), at = pack2f(top.add, top.add), rl = pack2f(low.r, low.r), al = pack2f(low.add, low.add);
   uint32_t S = 0;
@@ -317,7 +326,14 @@ __device__ __forceinline__ uint32_t distortion_first_one_fma(const uint32_t (&x)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const uint64_t va = values2<BF16>(x[8 * h + i]), vb = values2<BF16>(x[8 * h + 4 + i]);
-      const uint32_t ct4 = bytes4(fma2(va, rt, at), fma2(vb, rt, at)) & inside, q4 = bytes4(fma2(va, rl, al), fma2(vb, rl, al)) & inside;
+      uint64_t ta = fma2(va, rt, at), tb2 = fma2(vb, rt, at), la = fma2(va, rl, al), lb2 = fma2(vb, rl, al);
+      if (CLAMP) {
+        ta = clamp_codes2(ta, qtop);
+        tb2 = clamp_codes2(tb2, qtop);
+        la = clamp_codes2(la, qlow);
+        lb2 = clamp_codes2(lb2, qlow);
+      }
+      const uint32_t ct4 = bytes4(ta, tb2) & inside, q4 = bytes4(la, lb2) & inside;
       S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
       tb[4 * h + i] = ct4;
       ql[4 * h + i] = q4;
