@@ -257,7 +257,8 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
   // decoder CTA: one 32-element group per thread, or two when the call has rows enough to fill the device
   // several times over with the smaller CTAs (a thread's fixed work, checking the header and the token's
   // fields, is then spread over 64 elements: 8 % faster at 8192 x 8192 and 32768 x 4096; with fewer rows
-  // the smaller CTAs leave the device short of threads and are slower); never fewer than 64 threads while
+  // the smaller CTAs leave the device short of threads and are slower: 4096 x 4096 20.2 against 15.6 us,
+  // 2048 x 5120 12.6 against 10.6); never fewer than 64 threads while
   // the row has that many groups
   p->threads = static_cast<int>(((p->units + 31u) / 32u) * 32u);
   if (p->threads > kMaxThreads) p->threads = kMaxThreads;
