@@ -165,6 +165,13 @@ struct HostPipes {
 }  // namespace
 }  // namespace tsq
 
+// Resident CTAs, ring depth and CSR lists of the pipelined encoder.
+struct PipeShape {
+  int ctas_per_sm;  // 0: rows too long for it
+  uint32_t ring, csr_cap;
+  size_t smem;
+};
+
 struct tsq_plan {
   int device;
   tsq_dtype_t dtype;
@@ -181,10 +188,10 @@ struct tsq_plan {
   int threads_half, dec_blocks_half; // the same with two groups per thread, and its resident CTAs per SM
   int enc_threads, enc_upt;         // row-at-a-time encoder: CTA size and 32-element groups per thread
   // pipelined encoder: 0 CTAs per SM when the row does not fit its shared memory
-  int pipe_threads, pipe_ctas_per_sm;
+  int pipe_threads;
   bool pipe_full;
-  uint32_t pipe_compute, pipe_park, pipe_planes, pipe_csr_cap, pipe_ring;
-  size_t pipe_smem;
+  uint32_t pipe_compute, pipe_park, pipe_planes;
+  PipeShape pipe, pipe_many;        // for calls below many_rows(), and from there on
   int sms;
   size_t dec_smem;
   size_t workspace_bytes;
@@ -210,6 +217,44 @@ const char* tsq_status_string(tsq_status_t status) {
 }
 
 uint64_t tsq_kernel_launch_count(void) { return g_launches.load(); }
+
+static bool pipe_shape(const tsq_plan_t* p, const EncodeParams& kernel_of, bool many, size_t smem_optin, PipeShape* out) {
+  // A CSR list per ring slot: four entries per group (one outlier in eight elements; rows above that take
+  // a slower path that holds up their CTA's placement) when that costs neither a resident CTA nor ring
+  // depth below 6 (or below what two entries per group give), else two entries per group.
+  *out = PipeShape{0, 4u, 2u * p->pipe_compute, 0};
+  int base_blocks = 0;
+  uint32_t base_ring = 0;
+  for (uint32_t per_group = 2u; per_group <= 4u && p->pipe_threads <= kPipeMaxThreads; per_group += 2u) {
+    const uint32_t cap = per_group * p->pipe_compute;
+    const auto smem_for = [&](uint32_t ring) {
+      return 3u * static_cast<size_t>(p->pipe_park) + ring * (static_cast<size_t>(p->pipe_planes) + 4u * static_cast<size_t>(cap));
+    };
+    if (smem_for(4u) + 8192 > smem_optin) break;
+    int blocks = 0;
+    if (encode_pipe_attrs(kernel_of, p->pipe_full, many, p->pipe_threads, smem_for(4u), &blocks) != cudaSuccess) return false;
+    if (blocks < 1) break;
+    // the deepest ring that leaves the number of resident CTAs as it is
+    uint32_t ring = 4u;
+    for (uint32_t r = static_cast<uint32_t>(kMaxRing); r > 4u; --r) {
+      if (smem_for(r) + 8192 > smem_optin) continue;
+      int b = 0;
+      if (encode_pipe_attrs(kernel_of, p->pipe_full, many, p->pipe_threads, smem_for(r), &b) != cudaSuccess) return false;
+      if (b == blocks) {
+        ring = r;
+        break;
+      }
+    }
+    if (per_group == 2u) {
+      base_blocks = blocks;
+      base_ring = ring;
+    } else if (blocks != base_blocks || ring < (base_ring < 6u ? base_ring : 6u)) {
+      break;  // the longer lists cost too much: keep the shorter ones
+    }
+    *out = PipeShape{blocks, ring, cap, smem_for(ring)};
+  }
+  return true;
+}
 
 tsq_status_t tsq_plan(tsq_plan_t** out, int device, tsq_dtype_t dtype, int32_t hidden, int64_t max_tokens, float tau,
                       const int32_t* bits, int32_t n_bits, float delta, int64_t max_outliers) {
@@ -296,53 +341,14 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     p->pipe_threads = static_cast<int>(p->pipe_compute) + 64;
     p->pipe_park = p->pipe_compute * 64u;
     p->pipe_planes = (static_cast<uint32_t>(p->bmax) * p->units * 4u + 127u) & ~127u;
-    // A CSR list per ring slot: four entries per group (one outlier in eight elements; rows above that take
-    // a slower path that holds up their CTA's placement) when that costs neither a resident CTA nor ring
-    // depth below 6 (or below what two entries per group give), else two entries per group.
-    p->pipe_ctas_per_sm = 0;
-    p->pipe_ring = 4u;
-    p->pipe_csr_cap = 2u * p->pipe_compute;
-    p->pipe_smem = 0;
-    int base_blocks = 0;
-    uint32_t base_ring = 0;
     EncodeParams kernel_of;  // what selects the kernel instance
     std::memset(&kernel_of, 0, sizeof kernel_of);
     kernel_of.dtype = static_cast<uint32_t>(dtype);
     kernel_of.variant = p->variant;
     kernel_of.n_bits = n_bits;
     for (int i = 0; i < 8; ++i) kernel_of.bits[i] = p->bits[i];
-    for (uint32_t per_group = 2u; ok && per_group <= 4u && p->pipe_threads <= kPipeMaxThreads; per_group += 2u) {
-      const uint32_t cap = per_group * p->pipe_compute;
-      const auto smem_for = [&](uint32_t ring) {
-        return 3u * static_cast<size_t>(p->pipe_park) + ring * (static_cast<size_t>(p->pipe_planes) + 4u * static_cast<size_t>(cap));
-      };
-      if (smem_for(4u) + 8192 > static_cast<size_t>(smem_optin)) break;
-      int blocks = 0;
-      ok = encode_pipe_attrs(kernel_of, p->pipe_full, p->pipe_threads, smem_for(4u), &blocks) == cudaSuccess;
-      if (!ok || blocks < 1) break;
-      // the deepest ring that leaves the number of resident CTAs as it is
-      uint32_t ring = 4u;
-      for (uint32_t r = static_cast<uint32_t>(kMaxRing); ok && r > 4u; --r) {
-        if (smem_for(r) + 8192 > static_cast<size_t>(smem_optin)) continue;
-        int b = 0;
-        ok = encode_pipe_attrs(kernel_of, p->pipe_full, p->pipe_threads, smem_for(r), &b) == cudaSuccess;
-        if (ok && b == blocks) {
-          ring = r;
-          break;
-        }
-      }
-      if (!ok) break;
-      if (per_group == 2u) {
-        base_blocks = blocks;
-        base_ring = ring;
-      } else if (blocks != base_blocks || ring < (base_ring < 6u ? base_ring : 6u)) {
-        break;  // the longer lists cost too much: keep the shorter ones
-      }
-      p->pipe_ctas_per_sm = blocks;
-      p->pipe_ring = ring;
-      p->pipe_csr_cap = cap;
-      p->pipe_smem = smem_for(ring);
-    }
+    ok = ok && pipe_shape(p, kernel_of, false, static_cast<size_t>(smem_optin), &p->pipe);
+    ok = ok && pipe_shape(p, kernel_of, true, static_cast<size_t>(smem_optin), &p->pipe_many);
   }
   cudaSetDevice(prev_dev);
   if (!ok || dec_blocks < 1 || sms < 1) {
@@ -435,22 +441,30 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 // it, so the work of that grows with the square.
 static int64_t direct_rows(const tsq_plan_t* plan) { return 6 * static_cast<int64_t>(plan->sms); }
 
+// Rows from which a call of the pipelined kernel takes the instance with one more CTA per SM: a CTA more keeps more warps at
+// hand for the same issue slots (32768 x 4096 fp16 183.5 against 174.7 us, 10240 x 4096 65.7 against 58.7, 8192 x 5120 72.7
+// against 66.9), but all CTAs start and end at once, and fewer rows per CTA do not pay for that (4800 x 4096 39.0 against
+// 40.2 us, 6000 x 4096 45.8 against 46.1, 2048 x 5120 34.7 against 38.6).
+static int64_t many_rows(const tsq_plan_t* plan) { return 48 * static_cast<int64_t>(plan->sms); }
+
 tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, size_t blob_bytes,
                         void* ws_dev, size_t ws_bytes, void* cuda_stream) {
   const tsq_status_t args_ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
   if (args_ok != TSQ_OK) return args_ok;
   EncodeParams p = encode_params(plan, x_dev, tokens, blob_dev, ws_dev);
   cudaError_t e;
-  if (plan->pipe_ctas_per_sm > 0 && tokens > direct_rows(plan)) {
+  const bool many = tokens >= many_rows(plan);
+  const PipeShape& shape = many ? plan->pipe_many : plan->pipe;
+  if (shape.ctas_per_sm > 0 && tokens > direct_rows(plan)) {
     // many rows: persistent CTAs that overlap the stages of consecutive rows
     p.compute_threads = plan->pipe_compute;
     p.park_stride = plan->pipe_park;
     p.planes_stride = plan->pipe_planes;
-    p.csr_cap = plan->pipe_csr_cap;
-    p.ring = plan->pipe_ring;
-    const long long resident = static_cast<long long>(plan->sms) * plan->pipe_ctas_per_sm;
+    p.csr_cap = shape.csr_cap;
+    p.ring = shape.ring;
+    const long long resident = static_cast<long long>(plan->sms) * shape.ctas_per_sm;
     const int grid = static_cast<int>(tokens < resident ? tokens : resident);
-    e = launch_encode_pipe(p, plan->pipe_full, grid, plan->pipe_threads, plan->pipe_smem, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_pipe(p, plan->pipe_full, many, grid, plan->pipe_threads, shape.smem, static_cast<cudaStream_t>(cuda_stream));
   } else {
     // few rows (or rows too long for the pipeline): one CTA per row; a call without rows still launches
     // one CTA, which writes the header

@@ -748,29 +748,38 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_co
 
 }  // namespace
 
-// The pipelined kernel is built for CTAs of up to kPipeMaxThreads threads (rows of up to 8192 elements)
-// and may use up to 102 registers per thread; longer rows take encode_rows_kernel.
+// The pipelined kernel is built for CTAs of up to kPipeMaxThreads threads (rows of up to 8192 elements) and may use up to 102
+// registers per thread; longer rows take encode_rows_kernel.  What bounds it is the chain of dependent instructions of an
+// iteration, so with many rows a further CTA per SM pays: the instance for those is kept to 80 registers, with which CTAs of up
+// to kPipeManyThreads threads (rows of up to 5120 elements) number three (5120) or four (4096) per SM.  Longer rows lose more
+// by the shallower ring than they gain (10000 x 6144 fp16: 93.1 us with two CTAs, 98.0 with three).
 using PipeKernel = void (*)(EncodeParams);
-template <int KIND>
+template <int KIND, int MAXT, int MINB>
 static PipeKernel pipe_kernel_of(bool bf16, bool full) {
-  if (full) return bf16 ? encode_pipe_kernel<true, true, kPipeMaxThreads, 2, KIND> : encode_pipe_kernel<false, true, kPipeMaxThreads, 2, KIND>;
-  return bf16 ? encode_pipe_kernel<true, false, kPipeMaxThreads, 2, KIND> : encode_pipe_kernel<false, false, kPipeMaxThreads, 2, KIND>;
+  if (full) return bf16 ? encode_pipe_kernel<true, true, MAXT, MINB, KIND> : encode_pipe_kernel<false, true, MAXT, MINB, KIND>;
+  return bf16 ? encode_pipe_kernel<true, false, MAXT, MINB, KIND> : encode_pipe_kernel<false, false, MAXT, MINB, KIND>;
 }
-static PipeKernel pipe_kernel(const EncodeParams& p, bool full, int* index) {
+template <int KIND>
+static PipeKernel pipe_kernel_of(bool bf16, bool full, bool many) {
+  return many ? pipe_kernel_of<KIND, 256, 3>(bf16, full) : pipe_kernel_of<KIND, kPipeMaxThreads, 2>(bf16, full);
+}
+static PipeKernel pipe_kernel(const EncodeParams& p, bool full, bool many, int* index) {
   const bool bf16 = p.dtype == TSQ_BF16;
   const int kind = p.variant != 0u ? kKindSigned : ends_in_4_and_8(p) ? kKind84 : kKindExact;
-  *index = kind * 4 + (bf16 ? 2 : 0) + (full ? 1 : 0);
-  return kind == kKindSigned ? pipe_kernel_of<kKindSigned>(bf16, full) : kind == kKind84 ? pipe_kernel_of<kKind84>(bf16, full) : pipe_kernel_of<kKindExact>(bf16, full);
+  *index = kind * 8 + (many ? 4 : 0) + (bf16 ? 2 : 0) + (full ? 1 : 0);
+  return kind == kKindSigned ? pipe_kernel_of<kKindSigned>(bf16, full, many)
+         : kind == kKind84   ? pipe_kernel_of<kKind84>(bf16, full, many)
+                             : pipe_kernel_of<kKindExact>(bf16, full, many);
 }
 
-cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, int threads, size_t smem, int* blocks_per_sm) {
+cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, bool many, int threads, size_t smem, int* blocks_per_sm) {
   if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
   int index = 0;
-  const void* fn = reinterpret_cast<const void*>(pipe_kernel(p, full, &index));
+  const void* fn = reinterpret_cast<const void*>(pipe_kernel(p, full, many && threads <= kPipeManyThreads, &index));
   // the attribute belongs to the kernel on the current device, not to a plan: it only ever grows, so
   // that every plan can launch
   static std::mutex mu;
-  static size_t granted[kMaxDevices][12] = {};
+  static size_t granted[kMaxDevices][24] = {};
   {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -787,10 +796,10 @@ cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, int threads, siz
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
-cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream) {
+cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, bool many, int grid, int threads, size_t smem, cudaStream_t stream) {
   if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
   int index = 0;
-  return launch_overlapped(pipe_kernel(p, full, &index), grid, threads, smem, stream, p);
+  return launch_overlapped(pipe_kernel(p, full, many && threads <= kPipeManyThreads, &index), grid, threads, smem, stream, p);
 }
 
 }  // namespace tsq

@@ -15,6 +15,7 @@ constexpr uint32_t kVersion = 1u;
 constexpr int kMaxCand = 7;
 constexpr int kMaxThreads = 256;          // decoder: threads per CTA, one 32-element unit per thread per pass
 constexpr int kPipeMaxThreads = 320;      // pipelined encoder: compute threads (<= 256 groups) + two service warps
+constexpr int kPipeManyThreads = 224;     // longest CTA of its instance for calls of many rows
 constexpr int kMaxDevices = 64;           // devices per process that the library keeps per-device state for
 constexpr int kMaxRing = 8;               // pipelined encoder: most rows a CTA holds between packing and placement
 constexpr int kEncMaxThreads = 1024;      // encoder: one CTA per row, one or two 32-element groups per thread
@@ -138,8 +139,8 @@ cudaError_t launch_overlapped(void (*kernel)(Args...), int grid, int threads, si
 }
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int groups_per_thread, cudaStream_t stream);
-cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, int grid, int threads, size_t smem, cudaStream_t stream);
-cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, int threads, size_t smem, int* blocks_per_sm);
+cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, bool many, int grid, int threads, size_t smem, cudaStream_t stream);
+cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, bool many, int threads, size_t smem, int* blocks_per_sm);
 cudaError_t launch_decode(const DecodeParams& p, int grid, int threads, size_t smem, cudaStream_t stream);
 cudaError_t decode_kernel_attrs(bool bf16, int threads, size_t smem, int* blocks_per_sm);
 size_t decode_smem_bytes(uint32_t row_bytes);

@@ -1,0 +1,43 @@
+"""The pipelined encoder's instance for calls of many rows: both sides of the line where it starts, each way of deciding the first
+lower candidate, whole and ragged groups, the longest rows it takes."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import tsq_ref as R
+from paper_2511_04002_b200 import binding as B
+from paper_2511_04002_b200 import synth
+from tests._parity import assert_blobs_equal, full_parity, gpu_decode, gpu_encode
+from tests.test_gpu_parity import rand16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits", [[2, 4, 8], [2, 3, 6]])
+@pytest.mark.parametrize("dtype,hidden", [(torch.float16, 8), (torch.bfloat16, 1032), (torch.float16, 2048), (torch.bfloat16, 5120)])
+def test_both_sides_of_the_line(dtype, hidden, bits):
+    line = 48 * torch.cuda.get_device_properties(0).multi_processor_count
+    plan = B.Plan(dtype, hidden, line + 3, 6.0, bits, 0.2)
+    ws = plan.alloc(1)[1]
+    x = rand16((line + 3, hidden), dtype, seed=hidden, scale=2.0, outlier_rate=0.002)
+    x[::3] = (x[::3].float().abs() * 0.2).to(dtype)           # rows without outliers
+    x[1::17] = (x[1::17].float().abs() ** 3 * 0.05).to(dtype)  # rows that descend
+    x[5::301] = (x[5::301].float() * 4.0).to(dtype)            # rows that are mostly outliers
+    x[7::299] = (x[7::299].float().abs() * 0.1 + 3.0).to(dtype)  # rows that need the division instruction
+    for T in (line - 1, line, line + 3):
+        blob = torch.zeros(plan.sizes(T)[0], dtype=torch.uint8, device="cuda")
+        _, got, _ = gpu_encode(plan, x[:T], ws=ws, blob=blob)
+        ref = R.encode(synth.raw_u16(x[:T]), R.F16 if dtype == torch.float16 else R.BF16, 6.0, bits, 0.2)
+        assert_blobs_equal(got, ref)
+        if T == line:
+            assert np.array_equal(gpu_decode(plan, blob, T, ws), R.decode(ref))
+    assert plan.workspace_status(ws) == (0, 0)
+
+
+@pytest.mark.parametrize("dtype,hidden", [(torch.float16, 2048), (torch.bfloat16, 1032)])
+def test_signed_values(dtype, hidden):
+    line = 48 * torch.cuda.get_device_properties(0).multi_processor_count
+    x = rand16((line + 1, hidden), dtype, seed=hidden, scale=2.0, outlier_rate=0.002)
+    x[::3] = (x[::3].float().abs() * 0.2).to(dtype)
+    x[7::299] = (x[7::299].float().abs() * 0.1 + 3.0).to(dtype)
+    full_parity(x, 6.0, [2, 4, 8], 0.2, check_cross=False, variant=1)
