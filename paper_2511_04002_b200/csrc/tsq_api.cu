@@ -437,9 +437,13 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 
 // Rows up to which a call goes through the one-CTA-per-row kernel with direct offsets.  It has no pipeline to fill, and up to
 // six rows per SM that is worth more than overlapping the stages of a row (4096 fp16: 300 rows 9.1 us against 14.5, 900 rows
-// 15.3 against 18.9, 1300 rows 20.1 against 21.7, 2048 rows 29.7 against 26.6).  Each row reads the sizes of all rows before
-// it, so the work of that grows with the square.
-static int64_t direct_rows(const tsq_plan_t* plan) { return 6 * static_cast<int64_t>(plan->sms); }
+// 15.3 against 18.9), up to eight for rows of middle length (1180 x 2048 12.5 against 17.3, 1150 x 4096 15.7 against 18.3,
+// 1000 x 5120 17.9 against 19.2; 1300 x 4096 19.1 against 19.3).  Each row reads the sizes of all rows before it, so the work of
+// that grows with the square, and the few threads of a short row make it many rounds (1200 x 1024 18.0 against 16.2); long rows
+// are few to an SM (1000 x 6144 21.9 against 20.9).
+static int64_t direct_rows(const tsq_plan_t* plan) {
+  return (plan->enc_threads >= 64 && plan->enc_threads <= 160 ? 8 : 6) * static_cast<int64_t>(plan->sms);
+}
 
 // Rows from which a call of the pipelined kernel takes the instance with one more CTA per SM: a CTA more keeps more warps at
 // hand for the same issue slots (32768 x 4096 fp16 183.5 against 174.7 us, 10240 x 4096 65.7 against 58.7, 8192 x 5120 72.7

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("hidden", [8, 1032, 4096, 16384])
 def test_edges_of_the_range_on_one_workspace(hidden):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    sizes = [1, 2, sms - 1, sms, sms + 1, 2 * sms + 1, 6 * sms, 6 * sms + 1, 3]
+    sizes = [1, 2, sms - 1, sms, sms + 1, 2 * sms + 1, 6 * sms, 6 * sms + 1, 8 * sms, 8 * sms + 1, 3]
     plan = B.Plan(torch.float16, hidden, max(sizes), 6.0, [2, 4, 8], 0.2)
     ws = plan.alloc(1)[1]
     for k, T in enumerate(sizes):
