@@ -191,6 +191,8 @@ struct tsq_plan {
   int pipe_threads;
   bool pipe_full;
   uint32_t pipe_compute, pipe_park, pipe_planes;
+  bool ends_in_4_and_8;
+  int rows_ctas[3];                 // resident CTAs per SM of the row-at-a-time encoder's instances (rows_instance)
   PipeShape pipe, pipe_many;        // for calls below many_rows(), and from there on
   int sms;
   size_t dec_smem;
@@ -347,6 +349,8 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     kernel_of.variant = p->variant;
     kernel_of.n_bits = n_bits;
     for (int i = 0; i < 8; ++i) kernel_of.bits[i] = p->bits[i];
+    p->ends_in_4_and_8 = ends_in_4_and_8(kernel_of);
+    for (int i = 0; i < 3; ++i) ok = ok && encode_rows_attrs(kernel_of, p->enc_threads, p->enc_upt, i, &p->rows_ctas[i]) == cudaSuccess;
     ok = ok && pipe_shape(p, kernel_of, false, static_cast<size_t>(smem_optin), &p->pipe);
     ok = ok && pipe_shape(p, kernel_of, true, static_cast<size_t>(smem_optin), &p->pipe_many);
   }
@@ -435,14 +439,16 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
   return p;
 }
 
-// Rows up to which a call goes through the one-CTA-per-row kernel with direct offsets.  It has no pipeline to fill, and up to
-// six rows per SM that is worth more than overlapping the stages of a row (4096 fp16: 300 rows 9.1 us against 14.5, 900 rows
-// 15.3 against 18.9), up to eight for rows of middle length (1180 x 2048 12.5 against 17.3, 1150 x 4096 15.7 against 18.3,
-// 1000 x 5120 17.9 against 19.2; 1300 x 4096 19.1 against 19.3).  Each row reads the sizes of all rows before it, so the work of
-// that grows with the square, and the few threads of a short row make it many rounds (1200 x 1024 18.0 against 16.2); long rows
-// are few to an SM (1000 x 6144 21.9 against 20.9).
+// Rows up to which a call goes through the one-CTA-per-row kernel with direct offsets.  It has no pipeline to fill, which is
+// worth more than overlapping the stages of a row for the first ten to fourteen rows per SM of the magnitude variant (direct
+// against pipelined: 2048 x 1024 16.4 / 19.3 us, 2048 x 2048 16.4 / 19.8, 1500 x 4096 17.6 / 19.8, 2048 x 5120 30.5 / 34.7, but
+// 2400 x 5120 31.7 / 30.5; 1500 x 6144 24.1 / 26.4, 1500 x 8192 29.3 / 30.3; with the exact sum 1500 x 4096 22.2 / 22.1).  The
+// signed values have more arithmetic to overlap (1500 x 4096 42.8 / 38.7), and rows longer than 8192 elements have no pipelined
+// kernel, but few CTAs to an SM.  Each row reads the sizes of all rows before it, so the work of that grows with the square.
 static int64_t direct_rows(const tsq_plan_t* plan) {
-  return (plan->enc_threads >= 64 && plan->enc_threads <= 160 ? 8 : 6) * static_cast<int64_t>(plan->sms);
+  const int64_t sms = plan->sms;
+  if (plan->variant != 0u || plan->enc_threads > 256 || plan->enc_upt > 1) return 6 * sms;
+  return (plan->ends_in_4_and_8 && plan->enc_threads <= 160 ? 14 : 10) * sms;
 }
 
 // Rows from which a call of the pipelined kernel takes the instance with one more CTA per SM: a CTA more keeps more warps at
@@ -450,6 +456,23 @@ static int64_t direct_rows(const tsq_plan_t* plan) {
 // against 66.9), but all CTAs start and end at once, and fewer rows per CTA do not pay for that (4800 x 4096 39.0 against
 // 40.2 us, 6000 x 4096 45.8 against 46.1, 2048 x 5120 34.7 against 38.6).
 static int64_t many_rows(const tsq_plan_t* plan) { return 48 * static_cast<int64_t>(plan->sms); }
+
+// Instance of the row-at-a-time encoder for a direct call: 128, 80 or 64 registers, so more CTAs per SM with each.  The one
+// that takes the rows in the fewest turns (a sixteenth of a turn more does not count), of those the one with the most registers:
+// 2048 x 5120 37.1, 33.2 and 30.5 us, 1500 x 4096 19.7, 17.6 and 19.6 us, 600 x 4096 10.2, 12.3 and 12.3 us.
+static int rows_instance(const tsq_plan_t* plan, int64_t tokens) {
+  int best = 0;
+  int64_t fewest = INT64_MAX;
+  for (int i = 0; i < 3; ++i) {
+    const int64_t at_once = static_cast<int64_t>(plan->sms) * std::max(plan->rows_ctas[i], 1);
+    const int64_t turns = (tokens - at_once / 16 + at_once - 1) / at_once;
+    if (turns < fewest) {
+      fewest = turns;
+      best = i;
+    }
+  }
+  return best;
+}
 
 tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, size_t blob_bytes,
                         void* ws_dev, size_t ws_bytes, void* cuda_stream) {
@@ -476,7 +499,7 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
     // up to one CTA per SM is resident whatever the CTA's size: such a call needs no tickets
     const int64_t sms = plan->sms;
     p.direct_tiles = tokens < 1 || tokens > direct_rows(plan) ? 0u : tokens <= sms ? 1u : 2u;
-    e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, rows_instance(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
   }
   g_launches.fetch_add(1);
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
@@ -602,7 +625,7 @@ static int64_t part_rows(const tsq_plan_t* plan, int64_t tokens) {
   if (cudaGetDevice(&device) != cudaSuccess || device != plan->device) return tokens;  // the copy streams belong to the plan's device
   const int64_t row = static_cast<int64_t>(plan->row_bytes), parts = std::min<int64_t>(3, tokens * row / (4 << 20));
   if (parts < 2) return tokens;
-  const int64_t rows = std::min((tokens + parts - 1) / parts, direct_rows(plan));
+  const int64_t rows = std::min((tokens + parts - 1) / parts, std::min(direct_rows(plan), 6 * static_cast<int64_t>(plan->sms)));
   return rows * row < (1 << 20) ? tokens : rows;
 }
 
@@ -645,7 +668,7 @@ static tsq_status_t encode_host_parts(const tsq_plan_t* plan, HostPipe& pipe, co
       p.chained = t0 > 0 ? 1u : 0u;
       p.write_header = queued == parts - 1 ? 1u : 0u;
       p.totals = pipe.totals + 4 * slot;
-      e = launch_encode_rows(p, static_cast<int>(n), plan->enc_threads, plan->enc_upt, st);
+      e = launch_encode_rows(p, static_cast<int>(n), plan->enc_threads, plan->enc_upt, rows_instance(plan, n), st);
       g_launches.fetch_add(1);
       if (e == cudaSuccess) e = cudaEventRecord(pipe.ready[slot], st);
     }

@@ -25,11 +25,31 @@ struct RowShared {
 // i + blockDim, ... until they carry the call's tag (payload: plane words << 17 | outliers, 15 and 17 bits for any row),
 // so the wait is one round trip past the last predecessor's store.  The sums are left by warp; the caller adds them up
 // behind its barrier.  (A walk back by one warp took 3600 of the 10100 cycles of a 64 x 4096 call: its first look found
-// nothing published, and every retry was another round trip.)
+// nothing published, and every retry was another round trip.)  With many rows a thread's polls go out in batches, so that they
+// share a round trip: short rows have few threads to share them (2048 x 1024: 16.4 us, 19.3 in the pipelined kernel).
+constexpr uint32_t kPollBatch = 4u;
 __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared& sh) {
   const uint32_t limit = lookback_limit(p), tag = gen4 | kFlagAggregate;
   uint32_t w = 0u, o = 0u, status = TSQ_OK;
-  for (uint32_t i = threadIdx.x; i < tile; i += blockDim.x) {
+  uint32_t i = threadIdx.x;
+  for (; i + (kPollBatch - 1u) * blockDim.x < tile; i += kPollBatch * blockDim.x) {  // many rows: their loads in one round trip
+    unsigned long long v[kPollBatch];
+#pragma unroll
+    for (uint32_t k = 0; k < kPollBatch; ++k) v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x);
+#pragma unroll
+    for (uint32_t k = 0; k < kPollBatch; ++k) {
+      for (uint32_t polls = 0; static_cast<uint32_t>(v[k] >> 32) != tag; v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x)) {
+        if (++polls > limit) {
+          status = TSQ_ERR_TIMEOUT;
+          break;
+        }
+        if (polls > 32u) __nanosleep(1000u);
+      }
+      w += static_cast<uint32_t>(v[k]) >> 17;
+      o += static_cast<uint32_t>(v[k]) & 0x1ffffu;
+    }
+  }
+  for (; i < tile; i += blockDim.x) {
     unsigned long long v = ld_relaxed_u64(p.desc + i);
     for (uint32_t polls = 0; static_cast<uint32_t>(v >> 32) != tag; v = ld_relaxed_u64(p.desc + i)) {
       if (++polls > limit) {
@@ -63,15 +83,16 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
   p.ws->gen = gen4 >> 2;
 }
 
-// MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instance,
-// which may use four times the registers of the 1024-thread one).  SV: the signed-values variant.
+// MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instances).  MINB: 2, 3 or
+// 4 such CTAs' worth of registers, 128, 80 or 64 to a thread: a CTA spends most of its time waiting (its row, its barriers,
+// the rows before it), so a call of more rows than fit at once runs faster the more of them do.  SV: the signed-values variant.
 // DIRECT: calls of a few rows per SM: a row's offsets are read straight from the sizes of the rows before it
 // (direct_offsets) instead of walked back to.  With at most one row per SM every CTA is resident, so row = CTA index needs
 // no ticket.
 // TOP84: the candidates end in 4 and 8 bits (magnitudes): codes and planes at 8 bits first, and the 4-bit candidate decided from
 // the planes where they suffice (certain_distortion_8_to_4), else everything the general way.
-template <bool BF16, int UPT, int MAXT, bool SV, bool TOP84, bool DIRECT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
+template <bool BF16, int UPT, int MAXT, int MINB, bool SV, bool TOP84, bool DIRECT>
+__global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
   __shared__ RowShared sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -386,29 +407,33 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) encode_rows_kernel(
 
 }  // namespace
 
+using RowsKernel = void (*)(EncodeParams);
 template <bool SV, bool TOP84, bool DIRECT>
-static cudaError_t launch_rows_variant(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
-  const bool bf16 = p.dtype == TSQ_BF16;
+static RowsKernel rows_kernel_of(bool bf16, int threads, int upt, int dense) {
   if (upt == 1 && threads <= 256) {
-    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 256, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, SV, TOP84, DIRECT>, grid, threads, 0, stream, p);
+    if (DIRECT && !SV && dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
+    if (DIRECT && !SV && dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
+    return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
   }
-  if (TOP84) return cudaErrorInvalidValue;
-  if (upt == 1) {
-    return launch_overlapped(bf16 ? encode_rows_kernel<true, 1, 1024, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, SV, false, DIRECT>, grid, threads, 0, stream, p);
-  }
-  return launch_overlapped(bf16 ? encode_rows_kernel<true, 2, 1024, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, SV, false, DIRECT>, grid, threads, 0, stream, p);
+  if (upt == 1) return bf16 ? encode_rows_kernel<true, 1, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, 1, SV, false, DIRECT>;
+  return bf16 ? encode_rows_kernel<true, 2, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, 1, SV, false, DIRECT>;
 }
 
 template <bool DIRECT>
-static cudaError_t launch_rows_of(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
-  if (p.variant != 0u) return launch_rows_variant<true, false, DIRECT>(p, grid, threads, upt, stream);
+static RowsKernel rows_kernel(const EncodeParams& p, int threads, int upt, int dense) {
+  const bool bf16 = p.dtype == TSQ_BF16;
+  if (p.variant != 0u) return rows_kernel_of<true, false, DIRECT>(bf16, threads, upt, dense);
   // (in the CTAs of more than 256 threads, 64 registers each, the extra path costs more than it saves)
-  if (ends_in_4_and_8(p) && upt == 1 && threads <= 256) return launch_rows_variant<false, true, DIRECT>(p, grid, threads, upt, stream);
-  return launch_rows_variant<false, false, DIRECT>(p, grid, threads, upt, stream);
+  if (ends_in_4_and_8(p) && upt == 1 && threads <= 256) return rows_kernel_of<false, true, DIRECT>(bf16, threads, upt, dense);
+  return rows_kernel_of<false, false, DIRECT>(bf16, threads, upt, dense);
 }
 
-cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, cudaStream_t stream) {
-  return p.direct_tiles != 0u ? launch_rows_of<true>(p, grid, threads, upt, stream) : launch_rows_of<false>(p, grid, threads, upt, stream);
+cudaError_t encode_rows_attrs(const EncodeParams& p, int threads, int upt, int dense, int* blocks_per_sm) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, reinterpret_cast<const void*>(rows_kernel<true>(p, threads, upt, dense)), threads, 0);
+}
+
+cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, int dense, cudaStream_t stream) {
+  return launch_overlapped(p.direct_tiles != 0u ? rows_kernel<true>(p, threads, upt, dense) : rows_kernel<false>(p, threads, upt, dense), grid, threads, 0, stream, p);
 }
 
 }  // namespace tsq

@@ -53,3 +53,21 @@ def test_many_calls_back_to_back_on_one_stream():
             break
         cpu = nxt
     assert torch.equal(y.cpu().view(torch.int16), cpu.view(torch.int16))
+
+
+@pytest.mark.parametrize("bits", [[2, 4, 8], [2, 3, 6]])
+@pytest.mark.parametrize("dtype,hidden", [(torch.float16, 1032), (torch.bfloat16, 5120)])
+def test_every_instance_and_the_line_to_the_pipelined_kernel(dtype, hidden, bits):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sizes = [3 * sms + 5, 4 * sms + 9, 9 * sms, 10 * sms, 10 * sms + 1, 14 * sms, 14 * sms + 1]
+    plan = B.Plan(dtype, hidden, max(sizes), 6.0, bits, 0.2)
+    ws = plan.alloc(1)[1]
+    x = rand16((max(sizes), hidden), dtype, seed=hidden, scale=2.0, outlier_rate=0.01)
+    x[::3] = (x[::3].float().abs() * 0.2).to(dtype)              # rows without outliers
+    x[1::5] = (x[1::5].float().abs() ** 3 * 0.05).to(dtype)      # rows that descend
+    x[7::29] = (x[7::29].float().abs() * 0.1 + 3.0).to(dtype)    # rows that need the division instruction
+    for T in sizes:
+        blob = torch.zeros(plan.sizes(T)[0], dtype=torch.uint8, device="cuda")
+        _, got, _ = gpu_encode(plan, x[:T], ws=ws, blob=blob)
+        assert_blobs_equal(got, R.encode(synth.raw_u16(x[:T]), R.F16 if dtype == torch.float16 else R.BF16, 6.0, bits, 0.2))
+    assert plan.workspace_status(ws) == (0, 0)
