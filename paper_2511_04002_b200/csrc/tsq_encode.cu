@@ -12,11 +12,11 @@
 // Between the passes sits scalar work per row (the AIQ parameters of every candidate: a few
 // divisions) and the placement of the row's output, which has to wait for every earlier row.
 //
-// Two kernels share the passes:
-//   encode_rows_kernel  one CTA per row, the group in registers from load to store, everything in
-//                       order; used for few rows (lowest latency per call) and for rows longer
-//                       than the pipelined kernel takes.
-//   encode_pipe_kernel  persistent CTAs that keep several rows in different stages at once, so that
+// Two kernels share the passes (tsq_encode_device.cuh):
+//   encode_rows_kernel  (tsq_encode_rows.cu) one CTA per row, the group in registers from load to store,
+//                       everything in order; used up to some rows per SM (no pipeline to fill) and for
+//                       rows longer than the pipelined kernel takes.
+//   encode_pipe_kernel  (here) persistent CTAs that keep several rows in different stages at once, so that
 //                       the vector passes never wait for the scalar work or for the placement.
 //                       Each compute thread copies its group of the next row into shared memory
 //                       asynchronously (no registers held), runs pass A on row n in place there,
@@ -25,19 +25,23 @@
 //                       offsets of rows packed earlier, ships their planes with one bulk
 //                       asynchronous store each and writes their CSR entries.  When the first
 //                       lower candidate fails (the usual case) pass C reuses the top-level bytes
-//                       that pass B already formed.
+//                       that pass B already formed; with 4 and 8 bits as the last two candidates pass B
+//                       forms only those, and decides the 4-bit candidate from their planes
+//                       (certain_distortion_8_to_4) unless the codes it leaves open matter.
 //
-// The binding resource is the integer / logic pipe, which issues at half the rate of the FMA pipe:
-// the passes work on two 16-bit elements per 32-bit register wherever they can (four codes as bytes
-// in the distortion sum and on the way to the bit transpose), and some shifts and merges are written
-// as integer multiply-adds so that they go to the FMA pipe instead.
+// What binds: the chain of dependent instructions of an iteration (about 6000 cycles at hidden 8192 with two CTAs per
+// SM, 30 to 50 % of the issue slots used), and within it the integer / logic pipe, which issues at half the rate of the
+// FMA pipe: the passes work on two 16-bit elements per 32-bit register wherever they can (four codes as bytes in the
+// distortion sum and on the way to the bit transpose), and some shifts and merges are written as integer
+// multiply-adds so that they go to the FMA pipe instead.  8192 x 8192 bf16: 98.5 us with the three-operation quotient
+// and the exact distortion sum for every row, 86.7 us (2.34 TB/s) with one FMA per code and the sum from the planes.
 //
 // Variable-length placement: where a token's planes and CSR entries start is an exclusive prefix
 // sum over all earlier tokens.  It is resolved with a decoupled look-back over per-token
 // descriptors in the workspace.  Rows are numbered by an atomic ticket taken by a running CTA,
 // so a row only ever waits for rows whose CTAs are already running, and a row publishes its own
-// sizes before it waits for anything.  A look-back step reads 256 descriptor pairs at once (eight
-// independent loads per lane) in the one-CTA-per-row kernel and 32 in the pipelined kernel.  Every wait
+// sizes before it waits for anything.  A look-back step reads 32 descriptor pairs at once (256 in the
+// one-CTA-per-row kernel, whose calls of few rows read all predecessors directly instead).  Every wait
 // is bounded and fails into a status word.
 //
 // Arithmetic contract: the codes equal  clamp(rint(m / s) - zp, 0, Qmax)  with the IEEE binary32
@@ -52,8 +56,9 @@
 // checks the three-operation sequence in exact arithmetic against the true quotient for every
 // 16-bit pattern over many ranges and levels, and the GPU parity tests compare every code.  (A
 // single fl(m * r) is not enough: 16-bit inputs put m / s on or next to a rounding boundary
-// k + 1/2 in almost every row, and there the two can round differently.)  Every other row goes
-// through the division instruction in compact loops.
+// k + 1/2 in almost every row, and there the two can round differently.  At 8 bits a factor per row that
+// has been tried out against all its rounding boundaries, one_fma_factor, does make it enough.)  Every other
+// row goes through the division instruction in compact loops.
 
 #include <mutex>
 

@@ -8,6 +8,9 @@ namespace {
 // encode_rows_kernel: one CTA per row, everything in order.
 // =====================================================================================================
 
+// EncodeParams::direct_tiles
+constexpr int kLookBack = 0, kByIndex = 1, kByTicket = 2;
+
 struct RowShared {
   Level lv[kMaxCand];  // lv[i]: AIQ parameters of candidate bits[i]
   int S[kMaxCand];     // distortion sum of candidate i against the top level
@@ -28,11 +31,12 @@ struct RowShared {
 // nothing published, and every retry was another round trip.)  With many rows a thread's polls go out in batches, so that they
 // share a round trip: short rows have few threads to share them (2048 x 1024: 16.4 us, 19.3 in the pipelined kernel).
 constexpr uint32_t kPollBatch = 4u;
+template <bool BATCHES>
 __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared& sh) {
   const uint32_t limit = lookback_limit(p), tag = gen4 | kFlagAggregate;
   uint32_t w = 0u, o = 0u, status = TSQ_OK;
   uint32_t i = threadIdx.x;
-  for (; i + (kPollBatch - 1u) * blockDim.x < tile; i += kPollBatch * blockDim.x) {  // many rows: their loads in one round trip
+  for (; BATCHES && i + (kPollBatch - 1u) * blockDim.x < tile; i += kPollBatch * blockDim.x) {  // many rows: their loads in one round trip
     unsigned long long v[kPollBatch];
 #pragma unroll
     for (uint32_t k = 0; k < kPollBatch; ++k) v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x);
@@ -86,12 +90,12 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
 // MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instances).  MINB: 2, 3 or
 // 4 such CTAs' worth of registers, 128, 80 or 64 to a thread: a CTA spends most of its time waiting (its row, its barriers,
 // the rows before it), so a call of more rows than fit at once runs faster the more of them do.  SV: the signed-values variant.
-// DIRECT: calls of a few rows per SM: a row's offsets are read straight from the sizes of the rows before it
-// (direct_offsets) instead of walked back to.  With at most one row per SM every CTA is resident, so row = CTA index needs
-// no ticket.
+// DIRECT: calls of a few rows per SM (kByIndex, kByTicket): a row's offsets are read straight from the sizes of the rows before
+// it (direct_offsets) instead of walked back to.  With at most one row per SM (kByIndex) every CTA is resident, so row = CTA
+// index needs no ticket.
 // TOP84: the candidates end in 4 and 8 bits (magnitudes): codes and planes at 8 bits first, and the 4-bit candidate decided from
 // the planes where they suffice (certain_distortion_8_to_4), else everything the general way.
-template <bool BF16, int UPT, int MAXT, int MINB, bool SV, bool TOP84, bool DIRECT>
+template <bool BF16, int UPT, int MAXT, int MINB, bool SV, bool TOP84, int DIRECT>
 __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
   __shared__ RowShared sh;
@@ -100,7 +104,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
   wait_for_prior_grids();
   const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
   uint32_t part_w = 0u, part_o = 0u;  // where a later part of a call starts
-  if (DIRECT && p.chained != 0u) {
+  if (DIRECT != kLookBack && p.chained != 0u) {
     part_w = *reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_word_off);
     part_o = *reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_out_ptr);
     // never past the planes, whatever a part that has failed has left there
@@ -109,7 +113,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
   }
 
   uint32_t tile = blockIdx.x;
-  if (!DIRECT || p.direct_tiles == 2u) {
+  if (DIRECT != kByIndex) {
     if (tid == 0) {
       sh.tile = atomicAdd(&p.ws->ticket, 1u);
       sh.status = TSQ_OK;
@@ -215,7 +219,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
         }
         // With a row or less per SM the call ends with its slowest row, and in most calls some row's open codes decide: the
         // exact sum for all rows then, one barrier for every row (64 x 4096: 5.6 us against 6.7).
-        if (p.direct_tiles != 1u) {
+        if (DIRECT != kByIndex) {
 #pragma unroll
           for (int k = 0; k < UPT; ++k) S += certain_distortion_8_to_4(r[k]);
           S = __reduce_add_sync(kFull, S);
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
 
     // ---- placement: exclusive prefix sums over the tokens before this one ----
     if (DIRECT) {
-      direct_offsets(p, gen4, tile, sh);
+      direct_offsets<DIRECT == kByTicket>(p, gen4, tile, sh);
     } else if (warp == 0) {
       uint32_t word_off = 0, out_base = 0;
       const int st = resolve_prefix<8>(p, gen4, tile, agg_w, row_cnt, lane, &word_off, &out_base, lookback_limit(p));
@@ -408,18 +412,18 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
 }  // namespace
 
 using RowsKernel = void (*)(EncodeParams);
-template <bool SV, bool TOP84, bool DIRECT>
+template <bool SV, bool TOP84, int DIRECT>
 static RowsKernel rows_kernel_of(bool bf16, int threads, int upt, int dense) {
   if (upt == 1 && threads <= 256) {
-    if (DIRECT && !SV && dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
-    if (DIRECT && !SV && dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
+    if (DIRECT == kByTicket && !SV && dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
+    if (DIRECT == kByTicket && !SV && dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
     return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
   }
   if (upt == 1) return bf16 ? encode_rows_kernel<true, 1, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, 1, SV, false, DIRECT>;
   return bf16 ? encode_rows_kernel<true, 2, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, 1, SV, false, DIRECT>;
 }
 
-template <bool DIRECT>
+template <int DIRECT>
 static RowsKernel rows_kernel(const EncodeParams& p, int threads, int upt, int dense) {
   const bool bf16 = p.dtype == TSQ_BF16;
   if (p.variant != 0u) return rows_kernel_of<true, false, DIRECT>(bf16, threads, upt, dense);
@@ -429,11 +433,14 @@ static RowsKernel rows_kernel(const EncodeParams& p, int threads, int upt, int d
 }
 
 cudaError_t encode_rows_attrs(const EncodeParams& p, int threads, int upt, int dense, int* blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, reinterpret_cast<const void*>(rows_kernel<true>(p, threads, upt, dense)), threads, 0);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, reinterpret_cast<const void*>(rows_kernel<kByTicket>(p, threads, upt, dense)), threads, 0);
 }
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, int dense, cudaStream_t stream) {
-  return launch_overlapped(p.direct_tiles != 0u ? rows_kernel<true>(p, threads, upt, dense) : rows_kernel<false>(p, threads, upt, dense), grid, threads, 0, stream, p);
+  const RowsKernel fn = p.direct_tiles == kByIndex    ? rows_kernel<kByIndex>(p, threads, upt, dense)
+                        : p.direct_tiles == kByTicket ? rows_kernel<kByTicket>(p, threads, upt, dense)
+                                                      : rows_kernel<kLookBack>(p, threads, upt, dense);
+  return launch_overlapped(fn, grid, threads, 0, stream, p);
 }
 
 }  // namespace tsq
