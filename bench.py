@@ -48,10 +48,10 @@ FALLBACK_HBM_GBS = 6650.0
 # under profiles/, keyed by kernel; each entry is valid only for the kernel source it was taken on
 # (sha256 of the .cu file) and is scaled by tokens when the capture ran a smaller case.
 NCU_TRAFFIC = {
-    "encode": {"sha256": "9f369b6f8da4de1c72cb24bcbfb7c5107516207da5c4a319645bfc4adce7f0c5",
-               "bytes_per_token": (134320896 + 35652096) / 8192, "hidden": 8192, "dtype": "bf16"},
-    "decode": {"sha256": "3c9060c47b64da8ccfe6b7343d305c20c49b4fd14c9beccf2be4a0df2b8ceb1a",
-               "bytes_per_token": (68654336 + 79920128) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "encode": {"sha256": "589752b7d2249be1d5d3969065098ebcf508b7eee762bc566a7aa8cca0fc6e83",
+               "bytes_per_token": (134317824 + 35507968) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "decode": {"sha256": "5509cf08304cd8aa933495ec35e8df502b9fd4f7de02aaf38b226b78fe36422c",
+               "bytes_per_token": (68657664 + 72382464) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
 KERNEL_NAMES = {"encode": "encode_pipe_kernel (encode_rows_kernel for few or very long rows)", "decode": "decode_kernel"}
 
