@@ -220,6 +220,9 @@ const char* tsq_status_string(tsq_status_t status) {
 
 uint64_t tsq_kernel_launch_count(void) { return g_launches.load(); }
 
+static int64_t direct_rows(const tsq_plan_t* plan);
+static int64_t many_rows(const tsq_plan_t* plan);
+
 static bool pipe_shape(const tsq_plan_t* p, const EncodeParams& kernel_of, bool many, size_t smem_optin, PipeShape* out) {
   // A CSR list per ring slot: four entries per group (one outlier in eight elements; rows above that take
   // a slower path that holds up their CTA's placement) when that costs neither a resident CTA nor ring
@@ -350,9 +353,18 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     kernel_of.n_bits = n_bits;
     for (int i = 0; i < 8; ++i) kernel_of.bits[i] = p->bits[i];
     p->ends_in_4_and_8 = ends_in_4_and_8(kernel_of);
-    for (int i = 0; i < 3; ++i) ok = ok && encode_rows_attrs(kernel_of, p->enc_threads, p->enc_upt, i, &p->rows_ctas[i]) == cudaSuccess;
-    ok = ok && pipe_shape(p, kernel_of, false, static_cast<size_t>(smem_optin), &p->pipe);
-    ok = ok && pipe_shape(p, kernel_of, true, static_cast<size_t>(smem_optin), &p->pipe_many);
+    // only what calls of max_tokens can take: the occupancy queries are most of what a plan costs
+    p->sms = sms;
+    p->pipe = p->pipe_many = PipeShape{0, 0u, 0u, 0};
+    const int64_t rows = static_cast<int64_t>(T);
+    for (int i = 0; i < 3; ++i) {
+      p->rows_ctas[i] = i > 0 ? p->rows_ctas[i - 1] : 0;
+      if (i == 0 || rows > static_cast<int64_t>(sms) * p->rows_ctas[i]) {
+        ok = ok && encode_rows_attrs(kernel_of, p->enc_threads, p->enc_upt, i, &p->rows_ctas[i]) == cudaSuccess;
+      }
+    }
+    if (rows > direct_rows(p)) ok = ok && pipe_shape(p, kernel_of, false, static_cast<size_t>(smem_optin), &p->pipe);
+    if (rows >= many_rows(p)) ok = ok && pipe_shape(p, kernel_of, true, static_cast<size_t>(smem_optin), &p->pipe_many);
   }
   cudaSetDevice(prev_dev);
   if (!ok || dec_blocks < 1 || sms < 1) {
@@ -360,7 +372,6 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     delete p;
     return TSQ_ERR_CUDA;
   }
-  p->sms = sms;
   *out = p;
   return TSQ_OK;
 }
