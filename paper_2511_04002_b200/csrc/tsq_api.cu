@@ -454,11 +454,14 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 // worth more than overlapping the stages of a row for the first ten to fourteen rows per SM of the magnitude variant (direct
 // against pipelined: 2048 x 1024 16.4 / 19.3 us, 2048 x 2048 16.4 / 19.8, 1500 x 4096 17.6 / 19.8, 2048 x 5120 30.5 / 34.7, but
 // 2400 x 5120 31.7 / 30.5; 1500 x 6144 24.1 / 26.4, 1500 x 8192 29.3 / 30.3; with the exact sum 1500 x 4096 22.2 / 22.1).  The
-// signed values have more arithmetic to overlap (1500 x 4096 42.8 / 38.7), and rows longer than 8192 elements have no pipelined
-// kernel, but few CTAs to an SM.  Each row reads the sizes of all rows before it, so the work of that grows with the square.
+// signed values have more arithmetic to overlap (1500 x 4096 42.8 / 38.7).  Rows longer than 8192 elements have no pipelined
+// kernel and threads enough to read many sizes each round trip (against the look-back 1000 x 10240 27.9 / 33.1, 4096 x 16384
+// 130.5 / 147.5, 10000 x 12288 270 / 313 us).  Each row reads the sizes of all rows before it, so the work of that grows with the
+// square: an end at 64 rows per SM.
 static int64_t direct_rows(const tsq_plan_t* plan) {
   const int64_t sms = plan->sms;
-  if (plan->variant != 0u || plan->enc_threads > 256 || plan->enc_upt > 1) return 6 * sms;
+  if (plan->enc_threads > 256 || plan->enc_upt > 1) return 64 * sms;
+  if (plan->variant != 0u) return 6 * sms;
   return (plan->ends_in_4_and_8 && plan->enc_threads <= 160 ? 14 : 10) * sms;
 }
 

@@ -24,6 +24,18 @@ struct RowShared {
   uint32_t warp_w[32], warp_o[32], warp_status[32];  // direct_offsets: by warp
 };
 
+// Whether a poll of a descriptor is to be given up: its limit ran out, or that of another poll of the call did (a call of many
+// turns of CTAs then ends after one limit, not one for each turn).
+__device__ __forceinline__ bool given_up(const EncodeParams& p, uint32_t polls, uint32_t limit) {
+  if (polls > limit) {
+    atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
+    return true;
+  }
+  if (polls <= 32u) return false;
+  __nanosleep(1000u);
+  return *reinterpret_cast<volatile const uint32_t*>(&p.ws->err) != 0u;
+}
+
 // Offsets of a row of a call whose rows are all being encoded at once: thread i polls the descriptors of rows i,
 // i + blockDim, ... until they carry the call's tag (payload: plane words << 17 | outliers, 15 and 17 bits for any row),
 // so the wait is one round trip past the last predecessor's store.  The sums are left by warp; the caller adds them up
@@ -43,11 +55,10 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
 #pragma unroll
     for (uint32_t k = 0; k < kPollBatch; ++k) {
       for (uint32_t polls = 0; static_cast<uint32_t>(v[k] >> 32) != tag; v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x)) {
-        if (++polls > limit) {
+        if (given_up(p, ++polls, limit)) {
           status = TSQ_ERR_TIMEOUT;
           break;
         }
-        if (polls > 32u) __nanosleep(1000u);
       }
       w += static_cast<uint32_t>(v[k]) >> 17;
       o += static_cast<uint32_t>(v[k]) & 0x1ffffu;
@@ -56,11 +67,10 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
   for (; i < tile; i += blockDim.x) {
     unsigned long long v = ld_relaxed_u64(p.desc + i);
     for (uint32_t polls = 0; static_cast<uint32_t>(v >> 32) != tag; v = ld_relaxed_u64(p.desc + i)) {
-      if (++polls > limit) {
+      if (given_up(p, ++polls, limit)) {
         status = TSQ_ERR_TIMEOUT;
         break;
       }
-      if (polls > 32u) __nanosleep(1000u);
     }
     w += static_cast<uint32_t>(v) >> 17;
     o += static_cast<uint32_t>(v) & 0x1ffffu;

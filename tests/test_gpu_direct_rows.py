@@ -71,3 +71,49 @@ def test_every_instance_and_the_line_to_the_pipelined_kernel(dtype, hidden, bits
         _, got, _ = gpu_encode(plan, x[:T], ws=ws, blob=blob)
         assert_blobs_equal(got, R.encode(synth.raw_u16(x[:T]), R.F16 if dtype == torch.float16 else R.BF16, 6.0, bits, 0.2))
     assert plan.workspace_status(ws) == (0, 0)
+
+
+@pytest.mark.parametrize("hidden,signed", [(8200, False), (8200, True)])
+def test_long_rows_and_the_line_to_the_look_back(hidden, signed):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    variant = B.VARIANT_SIGNED_VALUES if signed else B.VARIANT_MAGNITUDES
+    plan = B.Plan(torch.bfloat16, hidden, 64 * sms + 1, 6.0, [2, 4, 8], 0.2, variant=variant)
+    blob, ws = plan.alloc(64 * sms + 1)
+    x = rand16((64 * sms + 1, hidden), torch.bfloat16, seed=7, scale=2.0, outlier_rate=0.01)
+    x[::3] = (x[::3].float().abs() * 0.2).to(torch.bfloat16)
+    x = x.cuda()
+    few = 7 * sms + 1
+    _, got, _ = gpu_encode(plan, x[:few].cpu(), ws=ws)
+    if not signed:
+        assert_blobs_equal(got, R.encode(synth.raw_u16(x[:few].cpu()), R.BF16, 6.0, [2, 4, 8], 0.2))
+    # both sides of the line decode to the same rows, in between to those of a short call
+    y = [torch.empty_like(x) for _ in range(2)]
+    for k, T in enumerate((64 * sms, 64 * sms + 1)):
+        plan.encode(x[:T], blob, ws)
+        plan.decode(blob, T, y[k][:T], ws)
+    plan.encode(x[:few], blob, ws)
+    short = torch.empty_like(x[:few])
+    plan.decode(blob, few, short, ws)
+    assert plan.workspace_status(ws) == (0, 0)
+    assert torch.equal(y[0][:64 * sms].view(torch.int16), y[1][:64 * sms].view(torch.int16))
+    assert torch.equal(y[0][:few].view(torch.int16), short.view(torch.int16))
+
+
+def test_a_wait_that_runs_out_ends_a_call_of_many_turns():
+    # row 0 is never produced: one limit's worth of waiting for the whole call, not one for each turn of CTAs
+    T, H = 30 * torch.cuda.get_device_properties(0).multi_processor_count, 8200
+    plan = B.Plan(torch.bfloat16, H, T, 6.0, [2, 4, 8], 0.2)
+    blob, ws = plan.alloc(T)
+    x = torch.randn((T, H), device="cuda").to(torch.bfloat16)
+    plan.workspace_set_wait_limit(ws, 3000)
+    ws.view(torch.int32)[1] = 1  # the ticket counter
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    e0.record()
+    plan.encode(x, blob, ws)
+    e1.record()
+    torch.cuda.synchronize()
+    assert plan.workspace_status(ws)[0] == 7 and plan.blob_info(blob).status == 7
+    assert e0.elapsed_time(e1) < 40.0
+    plan.workspace_init(ws)
+    _, got, _ = gpu_encode(plan, x[:5].cpu(), ws=ws)
+    assert_blobs_equal(got, R.encode(synth.raw_u16(x[:5].cpu()), R.BF16, 6.0, [2, 4, 8], 0.2))
