@@ -828,6 +828,7 @@ __device__ void finish_call(const EncodeParams& p, uint32_t gen4, bool direct = 
   // totals = the last tile's inclusive prefixes, if it got that far
   unsigned long long tw = 0ull, to = 0ull;
   if (direct) {
+    if (*reinterpret_cast<volatile const uint32_t*>(&p.ws->direct_state) == (gen4 | kWaitRanOut)) e = TSQ_ERR_TIMEOUT;
     for (uint32_t i = 0; i < p.tokens; ++i) {
       const uint32_t v = static_cast<uint32_t>(ld_relaxed_u64(p.desc + i));
       tw += v >> 17;
@@ -857,6 +858,7 @@ __device__ void finish_call(const EncodeParams& p, uint32_t gen4, bool direct = 
     // generation counter about to wrap: wipe the descriptors so that old tags cannot alias
     const uint32_t n = p.ws->desc_capacity;
     for (uint32_t i = 0; i < 2u * n; ++i) p.desc[i] = 0ull;
+    p.ws->direct_state = 0u;
     g = 0u;
   }
   p.ws->ticket = 0u;

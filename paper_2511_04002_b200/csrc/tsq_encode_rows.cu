@@ -26,14 +26,20 @@ struct RowShared {
 
 // Whether a poll of a descriptor is to be given up: its limit ran out, or that of another poll of the call did (a call of many
 // turns of CTAs then ends after one limit, not one for each turn).
-__device__ __forceinline__ bool given_up(const EncodeParams& p, uint32_t polls, uint32_t limit) {
+// A row that gives up is not written, so the call must not end with TSQ_OK.  One word decides which came first, the wait that ran
+// out or the CTA of the last row ending the call (finish_direct), and both move it by atomicMax: either that CTA finds
+// kWaitRanOut, or this poll finds kCallEnded.  Then that CTA has read the size of every row, so this one's is about to be seen:
+// the polls go on (64 at most: every wait has an end).  The word carries the generation: what a call leaves in it says nothing
+// to the next.
+__device__ __forceinline__ bool given_up(const EncodeParams& p, uint32_t gen4, uint32_t polls, uint32_t limit) {
   if (polls > limit) {
-    atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
+    if (atomicMax(&p.ws->direct_state, gen4 | kWaitRanOut) == (gen4 | kCallEnded) && polls - limit <= 64u) return false;
+    atomicCAS(&p.ws->enc_status, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
     return true;
   }
   if (polls <= 32u) return false;
   __nanosleep(1000u);
-  return *reinterpret_cast<volatile const uint32_t*>(&p.ws->err) != 0u;
+  return *reinterpret_cast<volatile const uint32_t*>(&p.ws->direct_state) == (gen4 | kWaitRanOut);
 }
 
 // Offsets of a row of a call whose rows are all being encoded at once: thread i polls the descriptors of rows i,
@@ -55,7 +61,7 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
 #pragma unroll
     for (uint32_t k = 0; k < kPollBatch; ++k) {
       for (uint32_t polls = 0; static_cast<uint32_t>(v[k] >> 32) != tag; v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x)) {
-        if (given_up(p, ++polls, limit)) {
+        if (given_up(p, gen4, ++polls, limit)) {
           status = TSQ_ERR_TIMEOUT;
           break;
         }
@@ -67,7 +73,7 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
   for (; i < tile; i += blockDim.x) {
     unsigned long long v = ld_relaxed_u64(p.desc + i);
     for (uint32_t polls = 0; static_cast<uint32_t>(v >> 32) != tag; v = ld_relaxed_u64(p.desc + i)) {
-      if (given_up(p, ++polls, limit)) {
+      if (given_up(p, gen4, ++polls, limit)) {
         status = TSQ_ERR_TIMEOUT;
         break;
       }
@@ -88,7 +94,9 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
 
 // The last row's CTA ends such a call: it knows the totals, and every other CTA has read the generation (it has published
 // under it), so nothing has to wait for the others.  (A counter of finished CTAs and the atomics around it cost 1650 cycles.)
+// Whether some row before it has given up is in direct_state (given_up).
 __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t gen4, uint32_t status, uint32_t total_w, uint32_t total_o) {
+  if (atomicMax(&p.ws->direct_state, gen4 | kCallEnded) == (gen4 | kWaitRanOut)) status = TSQ_ERR_TIMEOUT;
   if (status == TSQ_OK && total_o > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
   const bool ok = status != TSQ_ERR_TIMEOUT;
   end_part(p, status, ok ? total_w : 0ull, ok ? total_o : 0ull);

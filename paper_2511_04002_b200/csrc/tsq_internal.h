@@ -69,11 +69,13 @@ struct WsControl {
   uint32_t dec_status;   // first decode error since init (sticky)
   uint32_t desc_capacity;  // tiles the descriptor array holds (set by init)
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
-  uint32_t pad[8];
+  uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut or kCallEnded, only ever grows
+  uint32_t pad[7];
 };
 static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
 
 constexpr uint32_t kFlagAggregate = 1, kFlagPrefix = 2, kFlagAbort = 3;
+constexpr uint32_t kWaitRanOut = 1, kCallEnded = 2;  // direct_state
 constexpr uint32_t kGenWrap = (1u << 30) - 2;
 
 struct EncodeParams {

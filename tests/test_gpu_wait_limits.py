@@ -1,0 +1,62 @@
+"""Calls with direct offsets whose waits may run out at any moment: wait limits of a few polls, so that some rows give up while the
+rows they wait for are about to publish their sizes.  Either the call says TSQ_ERR_TIMEOUT or its blob is whole, and a workspace
+whose call said TSQ_OK is fit for the next call of either kernel."""
+import pytest
+import torch
+
+from oracle import tsq_ref as R
+from paper_2511_04002_b200 import binding as B
+from paper_2511_04002_b200 import synth
+from tests._parity import assert_blobs_equal
+from tests.test_gpu_parity import rand16
+
+pytestmark = pytest.mark.gpu
+OK, TIMEOUT = 0, 7
+
+
+def whole(plan, x, ws):
+    """The call's blob over a known fill (0xA5 where a call writes nothing), compared with the oracle's once."""
+    blob = torch.full((plan.sizes(x.shape[0])[0],), 0xA5, dtype=torch.uint8, device="cuda")
+    plan.encode(x, blob, ws)
+    assert_blobs_equal(blob.cpu().numpy(), R.encode(synth.raw_u16(x.cpu()), R.F16, 6.0, [2, 4, 8], 0.2))
+    return blob
+
+
+@pytest.mark.parametrize("rows_per_sm,hidden", [(1, 4096),     # row = CTA index
+                                                (6, 1024),     # rows by ticket, sizes read in batches
+                                                (6, 4096), (13, 2048),
+                                                (2, 8200)])    # CTAs of more than 256 threads
+def test_status_ok_means_a_whole_blob(rows_per_sm, hidden):
+    T = rows_per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    plan = B.Plan(torch.float16, hidden, 3000, 6.0, [2, 4, 8], 0.2)
+    ws = plan.alloc(1)[1]
+    x = rand16((T, hidden), torch.float16, seed=hidden, scale=2.0, outlier_rate=0.01)
+    x[1::5] = (x[1::5].float().abs() ** 3 * 0.05).to(torch.float16)  # rows that descend: their sizes come late
+    x = x.cuda()
+    # a longer call: up to 8192 elements in the pipelined kernel
+    more = rand16((3000, hidden), torch.float16, seed=3, scale=2.0, outlier_rate=0.01).cuda()
+    good, good_more = whole(plan, x, ws), whole(plan, more, ws)
+    blob, blob_more = torch.empty_like(good), torch.empty_like(good_more)
+    seen = set()
+    for k in range(96):
+        plan.workspace_set_wait_limit(ws, 1 + k % 32)
+        blob.fill_(0xA5)
+        plan.encode(x, blob, ws)
+        status = plan.blob_info(blob).status
+        seen.add(status)
+        assert status in (OK, TIMEOUT)
+        if status == TIMEOUT:
+            assert plan.workspace_status(ws)[0] == TIMEOUT
+            plan.workspace_init(ws)
+            continue
+        assert torch.equal(blob, good), "status 0 with a wait limit of %d, and the blob is not whole" % (1 + k % 32)
+        assert plan.workspace_status(ws)[0] == OK
+        plan.workspace_set_wait_limit(ws, 0)
+        blob.fill_(0xA5)
+        blob_more.fill_(0xA5)
+        if k % 2:                                              # the next call: the same kernel, then perhaps the other one
+            plan.encode(x, blob, ws)
+        plan.encode(more, blob_more, ws)
+        assert plan.workspace_status(ws)[0] == OK
+        assert torch.equal(blob_more, good_more) and (k % 2 == 0 or torch.equal(blob, good))
+    print("statuses seen", seen)
