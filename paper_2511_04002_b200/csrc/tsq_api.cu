@@ -682,6 +682,7 @@ static tsq_status_t encode_host_parts(const tsq_plan_t* plan, HostPipe& pipe, co
       p.chained = t0 > 0 ? 1u : 0u;
       p.write_header = queued == parts - 1 ? 1u : 0u;
       p.totals = pipe.totals + 4 * slot;
+      p.totals[2] = TSQ_ERR_TIMEOUT;  // until the part's last row says otherwise
       e = launch_encode_rows(p, static_cast<int>(n), plan->enc_threads, plan->enc_upt, rows_instance(plan, n), st);
       g_launches.fetch_add(1);
       if (e == cudaSuccess) e = cudaEventRecord(pipe.ready[slot], st);
@@ -689,9 +690,10 @@ static tsq_status_t encode_host_parts(const tsq_plan_t* plan, HostPipe& pipe, co
     if (e == cudaSuccess) e = cudaEventSynchronize(pipe.ready[c % kPipeSlots]);
     if (e != cudaSuccess) break;
     const unsigned long long* t = pipe.totals + 4 * (c % kPipeSlots);
-    if (t[2] != TSQ_OK) status = static_cast<uint32_t>(t[2]);
+    // the first part that fails decides; the offsets of one that timed out, and those after it, mean nothing
+    if (status == TSQ_OK) status = static_cast<uint32_t>(t[2]);
     const unsigned long long w1 = t[0], o1 = std::min(t[1], L.outlier_capacity);
-    if (w1 < words || w1 > L.words_capacity || o1 < outliers) break;  // a part that failed: its status says so
+    if (status == TSQ_ERR_TIMEOUT || w1 < words || w1 > L.words_capacity || o1 < outliers) break;
     if (w1 > words) e = cudaMemcpyAsync(bh + L.off_words + 4 * words, bd + L.off_words + 4 * words, 4 * (w1 - words), cudaMemcpyDeviceToHost, pipe.out);
     if (e == cudaSuccess && o1 > outliers) e = cudaMemcpyAsync(bh + L.off_outl + 4 * outliers, bd + L.off_outl + 4 * outliers, 4 * (o1 - outliers), cudaMemcpyDeviceToHost, pipe.out);
     words = w1;
@@ -704,9 +706,16 @@ static tsq_status_t encode_host_parts(const tsq_plan_t* plan, HostPipe& pipe, co
   if (e != cudaSuccess || done[0] != cudaSuccess || done[1] != cudaSuccess || done[2] != cudaSuccess) return TSQ_ERR_CUDA;
   BlobHeader h;
   std::memcpy(&h, bh, sizeof h);
-  if (h.magic != kMagic) return TSQ_ERR_CORRUPT_BLOB;
+  if (status == TSQ_OK && h.status != TSQ_OK) status = h.status;
+  if (h.magic != kMagic) return status != TSQ_OK ? static_cast<tsq_status_t>(status) : TSQ_ERR_CORRUPT_BLOB;
+  if (status != h.status) {
+    // the header is written by the last part, which knows only its own status: both copies of the blob get the call's
+    h.status = status;
+    std::memcpy(bh, &h, sizeof h);
+    if (cudaMemcpyAsync(blob_dev, &h, sizeof h, cudaMemcpyHostToDevice, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return TSQ_ERR_CUDA;
+  }
   if (payload_bytes) *payload_bytes = payload_of(h.tokens, h.total_words, std::min<unsigned long long>(h.total_outliers, L.outlier_capacity));
-  return static_cast<tsq_status_t>(h.status != TSQ_OK ? h.status : status);
+  return static_cast<tsq_status_t>(status);
 }
 
 // Whether the offsets at the parts' boundaries can be used to copy a blob in parts.

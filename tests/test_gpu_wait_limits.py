@@ -1,6 +1,7 @@
 """Calls with direct offsets whose waits may run out at any moment: wait limits of a few polls, so that some rows give up while the
 rows they wait for are about to publish their sizes.  Either the call says TSQ_ERR_TIMEOUT or its blob is whole, and a workspace
 whose call said TSQ_OK is fit for the next call of either kernel."""
+import numpy as np
 import pytest
 import torch
 
@@ -60,3 +61,53 @@ def test_status_ok_means_a_whole_blob(rows_per_sm, hidden):
         assert plan.workspace_status(ws)[0] == OK
         assert torch.equal(blob_more, good_more) and (k % 2 == 0 or torch.equal(blob, good))
     print("statuses seen", seen)
+
+
+def test_a_part_that_gives_up_shows_in_the_host_blob():
+    T, H = 2100, 4096                                          # three parts
+    plan = B.Plan(torch.float16, H, T, 6.0, [2, 4, 8], 0.2)
+    x = rand16((T, H), torch.float16, seed=11, scale=2.0, outlier_rate=0.01)
+    x[1::5] = (x[1::5].float().abs() ** 3 * 0.05).to(torch.float16)
+    ref = R.encode(synth.raw_u16(x), R.F16, 6.0, [2, 4, 8], 0.2)
+    blob, ws = plan.alloc(T)
+    x_host, x_dev = x.pin_memory(), torch.empty_like(x, device="cuda")
+    blob_host = torch.empty(blob.numel(), dtype=torch.uint8).pin_memory()
+    plan.encode_host(x_host, blob_host, x_dev, blob, ws)       # the buffers hold a good blob before every call
+    assert_blobs_equal(blob_host.numpy(), ref)
+    for k in range(48):
+        plan.workspace_set_wait_limit(ws, 1 + k % 32)
+        status = OK
+        try:
+            plan.encode_host(x_host, blob_host, x_dev, blob, ws)
+        except B.TsqError as e:
+            status = e.status
+        assert status in (OK, TIMEOUT)
+        assert R.header(blob_host.numpy())["status"] == status and plan.blob_info(blob).status == status
+        if status == OK:
+            assert_blobs_equal(blob_host.numpy(), ref)
+        else:
+            plan.workspace_init(ws)
+    plan.encode_host(x_host, blob_host, x_dev, blob, ws)
+    assert_blobs_equal(blob_host.numpy(), ref)
+
+
+def test_a_timed_out_part_among_good_ones():
+    """Only the first part's wait runs out (row 0 is never handed out); the later parts find their rows and end well."""
+    T, H = 2100, 4096
+    plan = B.Plan(torch.float16, H, T, 6.0, [2, 4, 8], 0.2)
+    x = rand16((T, H), torch.float16, seed=12, scale=2.0, outlier_rate=0.01)
+    blob, ws = plan.alloc(T)
+    x_host, x_dev = x.pin_memory(), torch.empty_like(x, device="cuda")
+    blob_host = torch.zeros(blob.numel(), dtype=torch.uint8).pin_memory()
+    plan.workspace_set_wait_limit(ws, 3000)
+    torch.cuda.synchronize()
+    ws.view(torch.int32)[1] = 1                                # the ticket counter
+    torch.cuda.synchronize()
+    with pytest.raises(B.TsqError) as e:
+        plan.encode_host(x_host, blob_host, x_dev, blob, ws)
+    assert e.value.status == TIMEOUT
+    assert R.header(blob_host.numpy())["status"] == TIMEOUT and plan.blob_info(blob).status == TIMEOUT
+    plan.workspace_init(ws)
+    plan.encode_host(x_host, blob_host, x_dev, blob, ws)
+    assert_blobs_equal(blob_host.numpy(), R.encode(synth.raw_u16(x), R.F16, 6.0, [2, 4, 8], 0.2))
+    assert np.array_equal(blob.cpu().numpy()[:64], blob_host.numpy()[:64])
