@@ -209,6 +209,11 @@ tsq_status_t tsq_workspace_status(const void *ws_dev, uint32_t *encode_status, u
  * fields and only the used part of the planes and of the CSR list; *payload_bytes (HOST) receives
  * the number of meaningful bytes.  tsq_decode_host copies a blob produced that way to the device,
  * decodes and copies y back.  Both synchronise `cuda_stream` and return the asynchronous status.
+ * Calls of 8 MB of tensor and more go in parts when the plan's device is current: the copies run on two
+ * streams of the library's own, ordered behind what `cuda_stream` holds and finished when the call
+ * returns.  Those streams, their events and 256 bytes of pinned host memory are made by the first such
+ * call on a device (calls in flight at the same time have a set each) and kept for later calls of any
+ * plan: at most four sets per device, one when the device's last plan is destroyed.
  */
 tsq_status_t tsq_encode_host(const tsq_plan_t *plan, const void *x_host, int64_t tokens, void *blob_host,
                              size_t blob_bytes, uint64_t *payload_bytes, void *x_dev, void *blob_dev,

@@ -88,9 +88,9 @@ __global__ void workspace_wait_limit_kernel(WsControl* ws, uint32_t polls) { ws-
 namespace tsq {
 namespace {
 
-// What a host-buffer call needs to overlap its copies with the kernels: two copy streams, events and a few pinned words.
-// A plan keeps up to kMaxHostPipes of them between calls (one per call in flight) and destroys them with itself.
-constexpr int kMaxHostPipes = 4;
+// What a host-buffer call needs to overlap its copies with the kernels: two copy streams, events and a few pinned words.  Making
+// them takes about 0.1 ms and giving them back as much again, half of what the call they serve takes, so they outlive the plan: a
+// program that makes a plan per request does not pay for them each time (HostPipes).
 constexpr int kPipeSlots = 8;  // parts in flight
 struct HostPipe {
   cudaStream_t in = nullptr, out = nullptr;
@@ -117,50 +117,69 @@ struct HostPipe {
     cudaGetLastError();
   }
 };
-struct HostPipes {
-  std::mutex mutex;
-  HostPipe* idle[kMaxHostPipes] = {};
-  HostPipe* take() {
+// The idle pipes of each device, whichever plan's calls made them: a call takes one for as long as it lasts, or makes one, and
+// gives it back.  At most kMaxHostPipes stay per device while it has plans, one (for the next plan) when it has none.
+constexpr int kMaxHostPipes = 4;
+class HostPipes {
+ public:
+  HostPipe* take(int device) {
     {
-      std::lock_guard<std::mutex> lock(mutex);
-      for (HostPipe*& p : idle) {
-        if (p) {
-          HostPipe* got = p;
-          p = nullptr;
-          return got;
-        }
-      }
+      std::lock_guard<std::mutex> lock(mutex_);
+      Device& d = devices_[device];
+      if (d.n_idle > 0) return d.idle[--d.n_idle];
     }
     HostPipe* p = new (std::nothrow) HostPipe();
     if (p && !p->create()) {
-      p->destroy();
-      delete p;
+      release(p);
       p = nullptr;
     }
     return p;
   }
-  void give_back(HostPipe* p) {
+  void give_back(int device, HostPipe* p) {
     {
-      std::lock_guard<std::mutex> lock(mutex);
-      for (HostPipe*& slot : idle) {
-        if (!slot) {
-          slot = p;
-          return;
-        }
+      std::lock_guard<std::mutex> lock(mutex_);
+      Device& d = devices_[device];
+      if (d.n_idle < kMaxHostPipes) {
+        d.idle[d.n_idle++] = p;
+        return;
       }
     }
+    release(p);
+  }
+  void plan_made(int device) {
+    std::lock_guard<std::mutex> lock(mutex_);
+    ++devices_[device].plans;
+  }
+  void plan_gone(int device) {
+    HostPipe* surplus[kMaxHostPipes];
+    int n = 0;
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      Device& d = devices_[device];
+      if (--d.plans == 0) {
+        while (d.n_idle > 1) surplus[n++] = d.idle[--d.n_idle];
+      }
+    }
+    while (n > 0) release(surplus[--n]);
+  }
+
+ private:
+  struct Device {
+    HostPipe* idle[kMaxHostPipes];
+    int n_idle, plans;
+  };
+  static void release(HostPipe* p) {
     p->destroy();
     delete p;
   }
-  ~HostPipes() {
-    for (HostPipe* p : idle) {
-      if (p) {
-        p->destroy();
-        delete p;
-      }
-    }
-  }
+  std::mutex mutex_;
+  Device devices_[kMaxDevices] = {};
 };
+// Never destroyed: at the end of the process the CUDA runtime may be gone before it.
+HostPipes& host_pipes() {
+  static HostPipes* const pipes = new HostPipes();
+  return *pipes;
+}
 
 }  // namespace
 }  // namespace tsq
@@ -197,7 +216,6 @@ struct tsq_plan {
   int sms;
   size_t dec_smem;
   size_t workspace_bytes;
-  mutable tsq::HostPipes host_pipes;
 };
 
 using namespace tsq;
@@ -372,11 +390,16 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     delete p;
     return TSQ_ERR_CUDA;
   }
+  host_pipes().plan_made(device);
   *out = p;
   return TSQ_OK;
 }
 
-void tsq_plan_destroy(tsq_plan_t* plan) { delete plan; }
+void tsq_plan_destroy(tsq_plan_t* plan) {
+  if (!plan) return;
+  host_pipes().plan_gone(plan->device);
+  delete plan;
+}
 
 static BlobLayout layout_for(const tsq_plan_t* plan, unsigned long long tokens) {
   unsigned long long cap = tokens * plan->hidden;
@@ -784,10 +807,10 @@ tsq_status_t tsq_encode_host(const tsq_plan_t* plan, const void* x_host, int64_t
   if (part < tokens) {
     const tsq_status_t ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
     if (ok != TSQ_OK) return ok;
-    HostPipe* pipe = plan->host_pipes.take();
+    HostPipe* pipe = host_pipes().take(plan->device);
     if (!pipe) return TSQ_ERR_CUDA;
     const tsq_status_t s = encode_host_parts(plan, *pipe, x_host, tokens, part, static_cast<unsigned char*>(blob_host), payload_bytes, x_dev, blob_dev, ws_dev, st);
-    plan->host_pipes.give_back(pipe);
+    host_pipes().give_back(plan->device, pipe);
     return s;
   }
   if (x_bytes && cudaMemcpyAsync(x_dev, x_host, x_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return TSQ_ERR_CUDA;
@@ -834,10 +857,10 @@ tsq_status_t tsq_decode_host(const tsq_plan_t* plan, const void* blob_host, size
   if (part < tokens && parts_in_order(L, bh, tokens, part, h.total_words, stored)) {
     if (!aligned16(y_dev) || !aligned16(blob_dev) || !aligned16(ws_dev)) return TSQ_ERR_INVALID_ARG;
     if (ws_bytes < plan->workspace_bytes) return TSQ_ERR_BUFFER_TOO_SMALL;
-    HostPipe* pipe = plan->host_pipes.take();
+    HostPipe* pipe = host_pipes().take(plan->device);
     if (!pipe) return TSQ_ERR_CUDA;
     const tsq_status_t s = decode_host_parts(plan, *pipe, bh, blob_bytes, tokens, part, y_host, blob_dev, y_dev, ws_dev, st);
-    plan->host_pipes.give_back(pipe);
+    host_pipes().give_back(plan->device, pipe);
     return s;
   }
   unsigned char* bd = static_cast<unsigned char*>(blob_dev);
