@@ -535,7 +535,7 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
     const int grid = tokens > 0 ? static_cast<int>(tokens) : 1;
     // up to one CTA per SM is resident whatever the CTA's size: such a call needs no tickets
     const int64_t sms = plan->sms;
-    p.direct_tiles = tokens < 1 || tokens > direct_rows(plan) ? 0u : tokens <= sms ? 1u : 2u;
+    p.direct_tiles = tokens > direct_rows(plan) ? 0u : tokens <= sms ? 1u : 2u;
     e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, rows_instance(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
   }
   g_launches.fetch_add(1);

@@ -818,7 +818,7 @@ __device__ void end_part(const EncodeParams& p, uint32_t status, unsigned long l
 }
 
 // The CTA that finishes last publishes the totals and the status, and re-arms the workspace.  `direct`: the descriptors
-// are those of a call without look-back (encode_rows_kernel), which comes here only when the generation wraps.
+// are those of a call without look-back (encode_rows_kernel), which comes here only when it has no rows or the generation wraps.
 __device__ void finish_call(const EncodeParams& p, uint32_t gen4, bool direct = false) {
   __threadfence();
   const uint32_t prev = atomicAdd(&p.ws->done, 1u);

@@ -422,20 +422,26 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
     }
   }
 
-  if (DIRECT && (gen4 >> 2) < kGenWrap) return;
+  if (DIRECT && p.tokens != 0u && (gen4 >> 2) < kGenWrap) return;  // (no last row to end a call without rows)
   __syncthreads();
   if (tid == 0) finish_call(p, gen4, DIRECT);
 }
 
 }  // namespace
 
+// Only what a call can reach is built: rows of up to 8192 elements never take the look-back (their longer calls are the pipelined
+// kernel's), and the instances of 80 and 64 registers are for calls by ticket of the magnitude variant.
 using RowsKernel = void (*)(EncodeParams);
 template <bool SV, bool TOP84, int DIRECT>
 static RowsKernel rows_kernel_of(bool bf16, int threads, int upt, int dense) {
-  if (upt == 1 && threads <= 256) {
-    if (DIRECT == kByTicket && !SV && dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
-    if (DIRECT == kByTicket && !SV && dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
-    return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
+  if constexpr (DIRECT != kLookBack) {
+    if (upt == 1 && threads <= 256) {
+      if constexpr (DIRECT == kByTicket && !SV) {
+        if (dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
+        if (dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
+      }
+      return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
+    }
   }
   if (upt == 1) return bf16 ? encode_rows_kernel<true, 1, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, 1, SV, false, DIRECT>;
   return bf16 ? encode_rows_kernel<true, 2, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, 1, SV, false, DIRECT>;
