@@ -140,13 +140,18 @@ tsq_status_t tsq_workspace_init(const tsq_plan_t *plan, void *ws_dev, size_t ws_
 
 /*
  * Set how long the encoder's device-side waits may last before they give up with TSQ_ERR_TIMEOUT.  The
- * only such wait is the placement look-back: a row's offsets are the prefix sums over every earlier
- * row, and a row polls the workspace until those rows have published theirs.  `polls` counts polls of
- * one descriptor (200 ns apart for the first 32, then 1 us apart); 0 restores the built-in limit of
- * 2^20 polls (about one second), which is also what tsq_workspace_init sets.  A wait can only run out
+ * only such wait is for placement: a row's offsets are the prefix sums over every earlier row, and a
+ * row polls the workspace until those rows have published their sizes.  `polls` counts polls of one
+ * descriptor: in calls that walk back over the descriptors (the longest calls) 200 ns apart for the
+ * first 32, in calls that read every earlier row's size directly one round trip apart for the first 32,
+ * then 1 us apart in both.  0 restores the built-in limit of 2^20 polls (about one second), which is
+ * also what tsq_workspace_init sets.  With the built-in limit a wait can only run out
  * when the workspace was not initialised, is shared by calls that overlap on the GPU, or was
- * overwritten: the limit exists so that such a mistake ends in a status instead of a hang.  The
- * setting is kept in the workspace (DEVICE) and is written on `cuda_stream`.
+ * overwritten: the limit exists so that such a mistake ends in a status instead of a hang.  With a limit
+ * of a few dozen polls a sound call may time out as well.  Whatever the limit, a call whose status
+ * is TSQ_OK has written every row; a call of which one wait has run out may end with TSQ_ERR_TIMEOUT
+ * although every row was written.  The setting is kept in the workspace (DEVICE) and is written on
+ * `cuda_stream`.
  */
 tsq_status_t tsq_workspace_set_wait_limit(void *ws_dev, uint32_t polls, void *cuda_stream);
 

@@ -474,10 +474,20 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 }
 
 // Rows up to which a call goes through the one-CTA-per-row kernel with direct offsets.  It has no pipeline to fill, which is
-// worth more than overlapping the stages of a row for the first ten to fourteen rows per SM of the magnitude variant (direct
-// against pipelined: 2048 x 1024 16.4 / 19.3 us, 2048 x 2048 16.4 / 19.8, 1500 x 4096 17.6 / 19.8, 2048 x 5120 30.5 / 34.7, but
-// 2400 x 5120 31.7 / 30.5; 1500 x 6144 24.1 / 26.4, 1500 x 8192 29.3 / 30.3; with the exact sum 1500 x 4096 22.2 / 22.1).  The
-// signed values have more arithmetic to overlap (1500 x 4096 42.8 / 38.7).  Rows longer than 8192 elements have no pipelined
+// worth more than overlapping the stages of a row for the first ten to fourteen rows per SM of the magnitude variant.  Where the
+// two cross depends on the tensor as well: rows with many outliers cost the pipelined kernel more.  us, direct / pipelined, each
+// pair on the same tensors, [A] Student-t nu = 4 with 16 outlier channels, fp16, [B] Student-t nu = 3 with 0.1 % outliers, bf16
+// (on normal values with 0.1 % to 1 % outliers the two lie between A and B):
+//   4 and 8 bits last   2048 x 1024  16.7 / 20.6 [A]  14.6 / 18.3 [B]     2800 x 1024  21.5 / 23.1 [A]  20.2 / 20.6 [B]
+//                       2048 x 5120  30.0 / 34.5      24.3 / 26.3         2400 x 5120  34.5 / 38.0      29.3 / 29.0
+//                       2800 x 5120  40.2 / 41.6      34.0 / 32.1         1480 x 6144  27.3 / 31.1      21.3 / 22.9
+//                       1800 x 6144  31.0 / 36.6      27.0 / 25.6         1480 x 8192  32.6 / 47.2      27.3 / 24.8
+//   exact sums (2,3,6)  1480 x 4096  23.4 / 24.5      20.6 / 22.0         2048 x 4096  29.6 / 29.6      28.4 / 25.8
+//                       1480 x 5120  25.9 / 30.7      24.9 / 26.0         1480 x 8192  34.8 / 36.9      33.6 / 30.3
+//   signed values       888 x 4096   35.6 / 35.7 [A]                      1500 x 4096  53.1 / 45.1 [A]
+// So 14 rows per SM for rows of up to 5120 elements lie before the crossing of every such tensor; 10 for longer rows and for exact
+// sums lie before it but for the longest rows with few outliers (B crosses at 8 rows per SM of 8192 elements); the signed values
+// have more arithmetic to overlap and cross at 6.  Rows longer than 8192 elements have no pipelined
 // kernel and threads enough to read many sizes each round trip (against the look-back 1000 x 10240 27.9 / 33.1, 4096 x 16384
 // 130.5 / 147.5, 10000 x 12288 270 / 313 us).  Each row reads the sizes of all rows before it, so the work of that grows with the
 // square: an end at 64 rows per SM.

@@ -29,12 +29,15 @@
 //                       forms only those, and decides the 4-bit candidate from their planes
 //                       (certain_distortion_8_to_4) unless the codes it leaves open matter.
 //
-// What binds: the chain of dependent instructions of an iteration (about 6000 cycles at hidden 8192 with two CTAs per
-// SM, 30 to 50 % of the issue slots used), and within it the integer / logic pipe, which issues at half the rate of the
-// FMA pipe: the passes work on two 16-bit elements per 32-bit register wherever they can (four codes as bytes in the
-// distortion sum and on the way to the bit transpose), and some shifts and merges are written as integer
-// multiply-adds so that they go to the FMA pipe instead.  8192 x 8192 bf16: 98.5 us with the three-operation quotient
-// and the exact distortion sum for every row, 86.7 us (2.34 TB/s) with one FMA per code and the sum from the planes.
+// What binds: the chain of dependent instructions of an iteration, with too few warps to hide it (two CTAs of ten warps per
+// SM by registers and shared memory, half of the issue slots used), and within it the integer / logic pipe, which issues at
+// half the rate of the FMA pipe: the passes work on two 16-bit elements per 32-bit register wherever they can (four codes as
+// bytes in the distortion sum and on the way to the bit transpose), and some shifts and merges are written as integer
+// multiply-adds so that they go to the FMA pipe instead.  Of the 5400 cycles of an iteration at hidden 8192 (clock stamps of
+// compute thread 0, whose warp the others wait for) pass B takes 2000, pass C with the CSR entries 740, pass A 700, the
+// levels of the row before 340, the decision 250, the wait for a ring slot 210, publishing the sizes 170.  8192 x 8192
+// bf16: 98.5 us with the three-operation quotient and the exact distortion sum for every row, 86.8 us (2.34 TB/s) with one FMA
+// per code and the sum from the planes.
 //
 // Variable-length placement: where a token's planes and CSR entries start is an exclusive prefix
 // sum over all earlier tokens.  It is resolved with a decoupled look-back over per-token
@@ -49,8 +52,10 @@
 // outlier or a tiny element has; no code above Qmax; scale in [2^-60, 2^60], so that no intermediate
 // leaves the normal range) form the quotient without the division instruction: r = fl(1 / s) once
 // per row and level, then per element q0 = fl(m * r), the residual m - q0 * s (one FMA) and
-// q = fl(q0 + residual * r), two elements at a time with the packed binary32 instructions (each
-// lane rounds to nearest even, as the scalar instructions do).  rint is one addition of 2^23, and
+// q = fl(q0 + residual * r) (Markstein's correction: "Computation of elementary functions on the IBM
+// RISC System/6000 processor", IBM Journal of Research and Development 34 (1), 1990), two elements at
+// a time with the packed binary32 instructions (each lane rounds to nearest even, as the scalar
+// instructions do).  rint is one addition of 2^23, and
 // the code is the low byte of the sum's pattern: no subtraction, no clamp.  What has to hold is
 // that rint(q) equals rint(fl(m / s)) for every 16-bit magnitude m of the row; a host-side test
 // checks the three-operation sequence in exact arithmetic against the true quotient for every

@@ -441,7 +441,9 @@ __device__ __forceinline__ uint32_t certain_distortion_8_to_4(const uint32_t (&r
 }
 
 // The 8-bit level's scale of a row whose smallest magnitude is 0, as make_level gives it, and the factor of the one-FMA
-// codes (one_fma_factor), in about 20 instructions: s = fl(hi / 127) by a multiplication and two FMAs; 127 divides hi's
+// codes (one_fma_factor), in about 20 instructions: s = fl(hi / 127) by a multiplication and two FMAs (correctly rounded
+// division by a constant: Brisebarre, Muller and Raina, "Accelerating correctly rounded floating-point division when the
+// divisor is known in advance", IEEE Transactions on Computers 53 (8), 2004); 127 divides hi's
 // significand iff 127 s = hi exactly; and fl((hi / 2) / s) >= 63.5 iff (hi / 2) - 63.5 s (exact) >= -2^-19 s.  (A host-side
 // test compares all of it for every 16-bit hi.)  The factor is 0 when the row has to go the general way.
 __device__ __forceinline__ float quick_level(float hi, float* s_out) {
