@@ -45,15 +45,27 @@ UNIT = "GB/s"
 FALLBACK_HBM_GBS = 6650.0
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu captures summarised
-# under profiles/, keyed by kernel; each entry is valid only for the kernel source it was taken on
-# (sha256 of the .cu file) and is scaled by tokens when the capture ran a smaller case.
+# under profiles/, keyed by kernel; each entry is valid only for the source it was taken on (sha256 over the files
+# that the kernel is compiled from) and is scaled by tokens when the capture ran a smaller case.
+KERNEL_SOURCES = {
+    "encode": ("tsq_encode.cu", "tsq_encode_device.cuh", "tsq_device.cuh", "tsq_internal.h"),
+    "decode": ("tsq_decode.cu", "tsq_device.cuh", "tsq_internal.h"),
+}
 NCU_TRAFFIC = {
-    "encode": {"sha256": "589752b7d2249be1d5d3969065098ebcf508b7eee762bc566a7aa8cca0fc6e83",
-               "bytes_per_token": (134317824 + 35507968) / 8192, "hidden": 8192, "dtype": "bf16"},
-    "decode": {"sha256": "5509cf08304cd8aa933495ec35e8df502b9fd4f7de02aaf38b226b78fe36422c",
-               "bytes_per_token": (68657664 + 72382464) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "encode": {"sha256": "1dbdc786494598ea589af55802901214c9a10a7c8ca680f5875ffa93647865a4",
+               "bytes_per_token": (134335488 + 34698496) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "decode": {"sha256": "5b81cc3ac02735ff1f807c958b25cb59be970609ac00a6114357f4bb577b1d6d",
+               "bytes_per_token": (68648960 + 73330944) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
 KERNEL_NAMES = {"encode": "encode_pipe_kernel (encode_rows_kernel for few or very long rows)", "decode": "decode_kernel"}
+
+
+def kernel_sources_sha256(kernel: str) -> str:
+    digest = hashlib.sha256()
+    for name in KERNEL_SOURCES[kernel]:
+        with open(os.path.join(ROOT, "paper_2511_04002_b200", "csrc", name), "rb") as f:
+            digest.update(f.read())
+    return digest.hexdigest()
 
 
 def workload_by_name(name: str, tokens: int | None):
@@ -464,10 +476,7 @@ def run_tsq(args, w):
     traffic = None
     rec = NCU_TRAFFIC.get(dom)
     if rec:
-        src = os.path.join(ROOT, "paper_2511_04002_b200", "csrc", "tsq_%s.cu" % dom)
-        with open(src, "rb") as f:
-            same = hashlib.sha256(f.read()).hexdigest() == rec["sha256"]
-        if same and rec["hidden"] == H and rec["dtype"] == w.recipe.dtype:
+        if kernel_sources_sha256(dom) == rec["sha256"] and rec["hidden"] == H and rec["dtype"] == w.recipe.dtype:
             traffic = rec["bytes_per_token"] * T
     roofline = {"bound": "hbm", "kernel": KERNEL_NAMES[dom], "achieved": kern[dom]["GB/s"], "peak": peak,
                 "unit": "GB/s", "frac": kern[dom]["GB/s"] / peak, "traffic": traffic, "peak_source": peak_kind,
