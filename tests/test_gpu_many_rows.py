@@ -41,3 +41,16 @@ def test_signed_values(dtype, hidden):
     x[::3] = (x[::3].float().abs() * 0.2).to(dtype)
     x[7::299] = (x[7::299].float().abs() * 0.1 + 3.0).to(dtype)
     full_parity(x, 6.0, [2, 4, 8], 0.2, check_cross=False, variant=1)
+
+
+@pytest.mark.parametrize("bits", [[2, 4, 8], [8]])
+@pytest.mark.parametrize("dtype,hidden", [(torch.float16, 1032), (torch.bfloat16, 5120)])
+def test_signed_values_ragged_fp16_and_whole_bf16_groups(dtype, hidden, bits):
+    # with the cases above: all four signed instances of 80 registers, each over every kind of row
+    line = 48 * torch.cuda.get_device_properties(0).multi_processor_count
+    x = rand16((line + 1, hidden), dtype, seed=hidden + 1, scale=2.0, outlier_rate=0.002)
+    x[::3] = (x[::3].float().abs() * 0.2).to(dtype)
+    x[1::17] = (x[1::17].float().abs() ** 3 * 0.05).to(dtype)
+    x[5::301] = (x[5::301].float() * 4.0).to(dtype)
+    x[7::299] = (x[7::299].float().abs() * 0.1 + 3.0).to(dtype)
+    full_parity(x, 6.0, bits, 0.2, check_cross=False, variant=1)
