@@ -111,3 +111,43 @@ def test_a_timed_out_part_among_good_ones():
     plan.encode_host(x_host, blob_host, x_dev, blob, ws)
     assert_blobs_equal(blob_host.numpy(), R.encode(synth.raw_u16(x), R.F16, 6.0, [2, 4, 8], 0.2))
     assert np.array_equal(blob.cpu().numpy()[:64], blob_host.numpy()[:64])
+
+
+LAST_GENERATION = (1 << 30) - 2                                # the call that runs as it wipes the descriptors and starts over
+
+
+@pytest.mark.parametrize("rows_per_sm,hidden", [(1, 1032), (6, 1024), (20, 1024), (1, 8200), (70, 8200)])
+def test_generations_start_over(rows_per_sm, hidden):
+    # direct calls by index and by ticket, the pipelined kernel, CTAs of more than 256 threads, those with look-back
+    T = rows_per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    plan = B.Plan(torch.float16, hidden, T, 6.0, [2, 4, 8], 0.2)
+    ws = plan.alloc(1)[1]
+    g = torch.Generator(device="cuda").manual_seed(hidden)
+    x = (torch.randn((T, hidden), generator=g, device="cuda") * 2.0).to(torch.float16)
+    good = whole(plan, x, ws) if rows_per_sm < 70 else torch.full((plan.sizes(T)[0],), 0xA5, dtype=torch.uint8, device="cuda")
+    if rows_per_sm == 70:
+        plan.encode(x, good, ws)
+    torch.cuda.synchronize()
+    ws.view(torch.int32)[0] = LAST_GENERATION - 3
+    blob = torch.empty_like(good)
+    for _ in range(5):                                         # two before it, the call itself, two after
+        blob.fill_(0xA5)
+        plan.encode(x, blob, ws)
+        assert torch.equal(blob, good)
+    assert plan.workspace_status(ws) == (OK, OK) and int(ws.view(torch.int32)[0]) == 2
+
+
+def test_a_wait_that_runs_out_in_the_last_generation():
+    T, H = 6 * torch.cuda.get_device_properties(0).multi_processor_count, 1024
+    plan = B.Plan(torch.float16, H, T, 6.0, [2, 4, 8], 0.2)
+    blob, ws = plan.alloc(T)
+    x = torch.randn((T, H), device="cuda").to(torch.float16)
+    plan.workspace_set_wait_limit(ws, 3000)
+    torch.cuda.synchronize()
+    ws.view(torch.int32)[0] = LAST_GENERATION - 1
+    ws.view(torch.int32)[1] = 1                                # the ticket counter: row 0 is never handed out
+    torch.cuda.synchronize()
+    plan.encode(x, blob, ws)
+    assert plan.blob_info(blob).status == TIMEOUT and plan.workspace_status(ws)[0] == TIMEOUT
+    plan.workspace_init(ws)
+    whole(plan, x, ws)
