@@ -57,7 +57,7 @@ NCU_TRAFFIC = {
     "decode": {"sha256": "5b81cc3ac02735ff1f807c958b25cb59be970609ac00a6114357f4bb577b1d6d",
                "bytes_per_token": (68648960 + 73330944) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
-KERNEL_NAMES = {"encode": "encode_pipe_kernel (encode_rows_kernel for few or very long rows)", "decode": "decode_kernel"}
+KERNEL_NAMES = {"encode": "sizes_kernel + pack_kernel (encode_rows_kernel for few rows)", "decode": "decode_kernel"}
 
 
 def kernel_sources_sha256(kernel: str) -> str:

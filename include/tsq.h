@@ -134,18 +134,17 @@ tsq_status_t tsq_plan_sizes(const tsq_plan_t *plan, int64_t tokens, tsq_sizes_t 
  * before the buffer's first use and after any TSQ_ERR_TIMEOUT; encode and decode leave it ready
  * for the next call.  One workspace serves one call at a time: calls that may overlap on the GPU
  * need separate workspaces.  (Variable-length placement, the prefix sums behind word_off and
- * out_ptr, is resolved inside the encode kernel through this buffer.)
+ * out_ptr, is resolved inside the encode kernels through this buffer.)
  */
 tsq_status_t tsq_workspace_init(const tsq_plan_t *plan, void *ws_dev, size_t ws_bytes, void *cuda_stream);
 
 /*
  * Set how long the encoder's device-side waits may last before they give up with TSQ_ERR_TIMEOUT.  The
- * only such wait is for placement: a row's offsets are the prefix sums over every earlier row, and a
- * row polls the workspace until those rows have published their sizes.  `polls` counts polls of one
- * descriptor: in calls that walk back over the descriptors (the longest calls) 200 ns apart for the
- * first 32, in calls that read every earlier row's size directly one round trip apart for the first 32,
- * then 1 us apart in both.  0 restores the built-in limit of 2^20 polls (about one second), which is
- * also what tsq_workspace_init sets.  With the built-in limit a wait can only run out
+ * only such wait is for placement in calls of few rows: a row's offsets are the sums over every earlier row, and a
+ * row polls the workspace until those rows have published their sizes.  (Calls of more rows go through two kernels that wait
+ * for nothing; they end with TSQ_ERR_TIMEOUT when the workspace is not as a finished call leaves it.)  `polls` counts polls of one
+ * row's size: one round trip apart for the first 32, then 1 us apart.  0 restores the built-in limit of 2^20 polls (about one
+ * second), which is also what tsq_workspace_init sets.  With the built-in limit a wait can only run out
  * when the workspace was not initialised, is shared by calls that overlap on the GPU, or was
  * overwritten: the limit exists so that such a mistake ends in a status instead of a hang.  With a limit
  * of a few dozen polls a sound call may time out as well.  Whatever the limit, a call whose status
@@ -158,7 +157,7 @@ tsq_status_t tsq_workspace_set_wait_limit(void *ws_dev, uint32_t polls, void *cu
 /*
  * Encode x (DEVICE, [tokens x hidden]) into blob (DEVICE, >= blob_bytes from tsq_plan_sizes,
  * 16-byte aligned): TS (Eq. "ts") + TAB-Q (Algorithm 1, token-wise) + bit-plane packing, one
- * kernel launch.  tokens == 0 writes an empty, valid blob.  Returns argument errors before
+ * kernel launch, or two for calls of more than a few rows per SM.  tokens == 0 writes an empty, valid blob.  Returns argument errors before
  * anything is enqueued.
  */
 tsq_status_t tsq_encode(const tsq_plan_t *plan, const void *x_dev, int64_t tokens, void *blob_dev,
@@ -169,7 +168,7 @@ tsq_status_t tsq_encode(const tsq_plan_t *plan, const void *x_dev, int64_t token
  * counterpart: this is a convenience of the library.)  Some hosts of this codec are not allowed to
  * allocate device memory where they call it: code running inside a region that forbids allocation
  * (a latency-critical serving loop with a frozen memory pool, a plug-in whose embedding runtime owns
- * all device memory, a thread that must never take the allocator's lock).  For them the look-back
+ * all device memory, a thread that must never take the allocator's lock).  For them the placement
  * scratch lives in a fixed array inside the library image instead of in a caller-allocated workspace;
  * x_dev and blob_dev are still the caller's.
  *   - Limit: the plan's max_tokens must be <= 16384 (the array is 256 KiB + 256 B per device, held

@@ -184,13 +184,6 @@ HostPipes& host_pipes() {
 }  // namespace
 }  // namespace tsq
 
-// Resident CTAs, ring depth and CSR lists of the pipelined encoder.
-struct PipeShape {
-  int ctas_per_sm;  // 0: rows too long for it
-  uint32_t ring, csr_cap;
-  size_t smem;
-};
-
 struct tsq_plan {
   int device;
   tsq_dtype_t dtype;
@@ -205,14 +198,10 @@ struct tsq_plan {
   uint32_t variant;                 // 0: sign + magnitude codes; 1: codes of the signed values
   int threads;                      // decoder CTA size, one group per thread
   int threads_half, dec_blocks_half; // the same with two groups per thread, and its resident CTAs per SM
-  int enc_threads, enc_upt;         // row-at-a-time encoder: CTA size and 32-element groups per thread
-  // pipelined encoder: 0 CTAs per SM when the row does not fit its shared memory
-  int pipe_threads;
-  bool pipe_full;
-  uint32_t pipe_compute, pipe_park, pipe_planes;
+  int enc_threads, enc_upt;         // one-kernel encoder: CTA size and 32-element groups per thread
   bool ends_in_4_and_8;
-  int rows_ctas[3];                 // resident CTAs per SM of the row-at-a-time encoder's instances (rows_instance)
-  PipeShape pipe, pipe_many;        // for calls below many_rows(), and from there on
+  int rows_ctas[3];                 // resident CTAs per SM of the one-kernel encoder's instances (rows_instance)
+  tsq::TwoPassShape two_pass;            // two-kernel encoder, for calls of more rows than direct_rows()
   int sms;
   size_t dec_smem;
   size_t workspace_bytes;
@@ -239,46 +228,6 @@ const char* tsq_status_string(tsq_status_t status) {
 uint64_t tsq_kernel_launch_count(void) { return g_launches.load(); }
 
 static int64_t direct_rows(const tsq_plan_t* plan);
-static int64_t many_rows(const tsq_plan_t* plan);
-
-static bool pipe_shape(const tsq_plan_t* p, const EncodeParams& kernel_of, bool many, size_t smem_optin, PipeShape* out) {
-  // A CSR list per ring slot: four entries per group (one outlier in eight elements; rows above that take
-  // a slower path that holds up their CTA's placement) when that costs neither a resident CTA nor ring
-  // depth below 6 (or below what two entries per group give), else two entries per group.
-  *out = PipeShape{0, 4u, 2u * p->pipe_compute, 0};
-  int base_blocks = 0;
-  uint32_t base_ring = 0;
-  for (uint32_t per_group = 2u; per_group <= 4u && p->pipe_threads <= kPipeMaxThreads; per_group += 2u) {
-    const uint32_t cap = per_group * p->pipe_compute;
-    const auto smem_for = [&](uint32_t ring) {
-      return 3u * static_cast<size_t>(p->pipe_park) + ring * (static_cast<size_t>(p->pipe_planes) + 4u * static_cast<size_t>(cap));
-    };
-    if (smem_for(4u) + 8192 > smem_optin) break;
-    int blocks = 0;
-    if (encode_pipe_attrs(kernel_of, p->pipe_full, many, p->pipe_threads, smem_for(4u), &blocks) != cudaSuccess) return false;
-    if (blocks < 1) break;
-    // the deepest ring that leaves the number of resident CTAs as it is
-    uint32_t ring = 4u;
-    for (uint32_t r = static_cast<uint32_t>(kMaxRing); r > 4u; --r) {
-      if (smem_for(r) + 8192 > smem_optin) continue;
-      int b = 0;
-      if (encode_pipe_attrs(kernel_of, p->pipe_full, many, p->pipe_threads, smem_for(r), &b) != cudaSuccess) return false;
-      if (b == blocks) {
-        ring = r;
-        break;
-      }
-    }
-    if (per_group == 2u) {
-      base_blocks = blocks;
-      base_ring = ring;
-    } else if (blocks != base_blocks || ring < (base_ring < 6u ? base_ring : 6u)) {
-      break;  // the longer lists cost too much: keep the shorter ones
-    }
-    *out = PipeShape{blocks, ring, cap, smem_for(ring)};
-  }
-  return true;
-}
-
 tsq_status_t tsq_plan(tsq_plan_t** out, int device, tsq_dtype_t dtype, int32_t hidden, int64_t max_tokens, float tau,
                       const int32_t* bits, int32_t n_bits, float delta, int64_t max_outliers) {
   return tsq_plan_variant(out, device, dtype, hidden, max_tokens, tau, bits, n_bits, delta, max_outliers, TSQ_VARIANT_MAGNITUDES);
@@ -356,24 +305,17 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
   ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, p->threads, p->dec_smem, &dec_blocks) == cudaSuccess;
   ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, p->threads_half, p->dec_smem, &p->dec_blocks_half) == cudaSuccess;
   {
-    // pipelined encoder: three parked rows and a ring of rows of planes and of CSR entries per CTA
-    int smem_optin = 0;
-    ok = ok && cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) == cudaSuccess;
-    p->pipe_compute = (p->units + 31u) / 32u * 32u;
-    p->pipe_full = (p->hidden % 32u == 0u) && (p->units == p->pipe_compute);  // every compute thread owns a whole group
-    p->pipe_threads = static_cast<int>(p->pipe_compute) + 64;
-    p->pipe_park = p->pipe_compute * 64u;
-    p->pipe_planes = (static_cast<uint32_t>(p->bmax) * p->units * 4u + 127u) & ~127u;
-    EncodeParams kernel_of;  // what selects the kernel instance
+    EncodeParams kernel_of;  // what selects the kernel instances
     std::memset(&kernel_of, 0, sizeof kernel_of);
     kernel_of.dtype = static_cast<uint32_t>(dtype);
     kernel_of.variant = p->variant;
+    kernel_of.units = p->units;
+    kernel_of.chunks = p->chunks;
     kernel_of.n_bits = n_bits;
     for (int i = 0; i < 8; ++i) kernel_of.bits[i] = p->bits[i];
     p->ends_in_4_and_8 = ends_in_4_and_8(kernel_of);
     // only what calls of max_tokens can take: the occupancy queries are most of what a plan costs
     p->sms = sms;
-    p->pipe = p->pipe_many = PipeShape{0, 0u, 0u, 0};
     const int64_t rows = static_cast<int64_t>(T);
     for (int i = 0; i < 3; ++i) {
       p->rows_ctas[i] = i > 0 ? p->rows_ctas[i - 1] : 0;
@@ -381,8 +323,8 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
         ok = ok && encode_rows_attrs(kernel_of, p->enc_threads, p->enc_upt, i, &p->rows_ctas[i]) == cudaSuccess;
       }
     }
-    if (rows > direct_rows(p)) ok = ok && pipe_shape(p, kernel_of, false, static_cast<size_t>(smem_optin), &p->pipe);
-    if (rows >= many_rows(p)) ok = ok && pipe_shape(p, kernel_of, true, static_cast<size_t>(smem_optin), &p->pipe_many);
+    p->two_pass = two_pass_shape(kernel_of);
+    if (rows > direct_rows(p)) ok = ok && two_pass_attrs(kernel_of, p->two_pass) == cudaSuccess;
   }
   cudaSetDevice(prev_dev);
   if (!ok || dec_blocks < 1 || sms < 1) {
@@ -473,38 +415,25 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
   return p;
 }
 
-// Rows up to which a call goes through the one-CTA-per-row kernel with direct offsets.  It has no pipeline to fill, which is
-// worth more than overlapping the stages of a row for the first ten to fourteen rows per SM of the magnitude variant.  Where the
-// two cross depends on the tensor as well: rows with many outliers cost the pipelined kernel more.  us, direct / pipelined, each
-// pair on the same tensors, [A] Student-t nu = 4 with 16 outlier channels, fp16, [B] Student-t nu = 3 with 0.1 % outliers, bf16
-// (on normal values with 0.1 % to 1 % outliers the two lie between A and B):
-//   4 and 8 bits last   2048 x 1024  16.7 / 20.6 [A]  14.6 / 18.3 [B]     2800 x 1024  21.5 / 23.1 [A]  20.2 / 20.6 [B]
-//                       2048 x 5120  30.0 / 34.5      24.3 / 26.3         2400 x 5120  34.5 / 38.0      29.3 / 29.0
-//                       2800 x 5120  40.2 / 41.6      34.0 / 32.1         1480 x 6144  27.3 / 31.1      21.3 / 22.9
-//                       1800 x 6144  31.0 / 36.6      27.0 / 25.6         1480 x 8192  32.6 / 47.2      27.3 / 24.8
-//   exact sums (2,3,6)  1480 x 4096  23.4 / 24.5      20.6 / 22.0         2048 x 4096  29.6 / 29.6      28.4 / 25.8
-//                       1480 x 5120  25.9 / 30.7      24.9 / 26.0         1480 x 8192  34.8 / 36.9      33.6 / 30.3
-//   signed values       888 x 4096   35.6 / 35.7 [A]                      1500 x 4096  53.1 / 45.1 [A]
-// So 14 rows per SM for rows of up to 5120 elements lie before the crossing of every such tensor; 10 for longer rows and for exact
-// sums lie before it but for the longest rows with few outliers (B crosses at 8 rows per SM of 8192 elements); the signed values
-// have more arithmetic to overlap and cross at 6.  Rows longer than 8192 elements have no pipelined
-// kernel and threads enough to read many sizes each round trip (against the look-back 1000 x 10240 27.9 / 33.1, 4096 x 16384
-// 130.5 / 147.5, 10000 x 12288 270 / 313 us).  Each row reads the sizes of all rows before it, so the work of that grows with the
-// square: an end at 64 rows per SM.
+// Rows up to which a call goes through one kernel, whose rows read the sizes of the rows before them directly, instead of two.  The
+// second kernel costs a launch and a second read of the input; in the one kernel every row waits for the slowest row before it, and
+// the more rows do not fit at once the more that costs.  us, one kernel / two, each pair on the same tensors (n: normal values with 0.1 %
+// outliers, n0: none, n1: 1 %, t3: Student-t nu = 3 with 0.1 %, t4: nu = 4 with 16 outlier channels):
+//   up to 2048 elements  1042 x 1976 fp16, 8 outlier channels  11.6 / 12.6                     2048 x 1024 bf16 t3  14.9 / 11.9
+//   up to 5120            300 x 4096 fp16 n   7.8 / 11.0     600 x 4096 bf16 n   10.1 / 11.4    777 x 3000 bf16 n   11.4 / 12.5
+//                        1000 x 4096 fp16 n0 13.8 / 13.7    1500 x 4096 fp16 n1 18.0 / 14.5   2048 x 5120 fp16 t4  29.8 / 24.1
+//   up to 8192            300 x 8192 bf16 t3  9.4 / 9.7      600 x 8192 fp16 n   13.2 / 12.4   1000 x 8192 fp16 t4  22.1 / 14.6
+//   longer                300 x 12288 fp16 n 12.9 / 12.6     600 x 12288 fp16 n  19.8 / 13.7    600 x 16384 fp16 t4 26.0 / 17.5
+//   signed values          64 x 4096 fp16 n  12.6 / 8.6      300 x 4096 fp16 n   20.9 / 12.0    600 x 5120 fp16 t4  35.6 / 17.0
+// (Signed values: one row in ten has a code that needs the clamp, which the one kernel forms by the division instruction; 1 x 4096 4.1 / 7.4.)
 static int64_t direct_rows(const tsq_plan_t* plan) {
   const int64_t sms = plan->sms;
-  if (plan->enc_threads > 256 || plan->enc_upt > 1) return 64 * sms;
-  if (plan->variant != 0u) return 6 * sms;
-  return (plan->ends_in_4_and_8 && plan->enc_threads <= 160 ? 14 : 10) * sms;
+  if (plan->variant != 0u) return 8;
+  if (plan->enc_upt > 1 || plan->enc_threads > 256) return 2 * sms;
+  return (plan->enc_threads <= 64 ? 8 : plan->enc_threads <= 160 ? 6 : 4) * sms;
 }
 
-// Rows from which a call of the pipelined kernel takes the instance with one more CTA per SM: a CTA more keeps more warps at
-// hand for the same issue slots (32768 x 4096 fp16 183.5 against 174.7 us, 10240 x 4096 65.7 against 58.7, 8192 x 5120 72.7
-// against 66.9), but all CTAs start and end at once, and fewer rows per CTA do not pay for that (4800 x 4096 39.0 against
-// 40.2 us, 6000 x 4096 45.8 against 46.1, 2048 x 5120 34.7 against 38.6).
-static int64_t many_rows(const tsq_plan_t* plan) { return 48 * static_cast<int64_t>(plan->sms); }
-
-// Instance of the row-at-a-time encoder for a direct call: 128, 80 or 64 registers, so more CTAs per SM with each.  The one
+// Instance of the one-kernel encoder: 128, 80 or 64 registers, so more CTAs per SM with each.  The one
 // that takes the rows in the fewest turns (a sixteenth of a turn more does not count), of those the one with the most registers:
 // 2048 x 5120 37.1, 33.2 and 30.5 us, 1500 x 4096 19.7, 17.6 and 19.6 us, 600 x 4096 10.2, 12.3 and 12.3 us.
 static int rows_instance(const tsq_plan_t* plan, int64_t tokens) {
@@ -526,28 +455,16 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
   const tsq_status_t args_ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
   if (args_ok != TSQ_OK) return args_ok;
   EncodeParams p = encode_params(plan, x_dev, tokens, blob_dev, ws_dev);
-  cudaError_t e;
-  const bool many = tokens >= many_rows(plan);
-  const PipeShape& shape = many ? plan->pipe_many : plan->pipe;
-  if (shape.ctas_per_sm > 0 && tokens > direct_rows(plan)) {
-    // many rows: persistent CTAs that overlap the stages of consecutive rows
-    p.compute_threads = plan->pipe_compute;
-    p.park_stride = plan->pipe_park;
-    p.planes_stride = plan->pipe_planes;
-    p.csr_cap = shape.csr_cap;
-    p.ring = shape.ring;
-    const long long resident = static_cast<long long>(plan->sms) * shape.ctas_per_sm;
-    const int grid = static_cast<int>(tokens < resident ? tokens : resident);
-    e = launch_encode_pipe(p, plan->pipe_full, many, grid, plan->pipe_threads, shape.smem, static_cast<cudaStream_t>(cuda_stream));
-  } else {
-    // few rows (or rows too long for the pipeline): one CTA per row; a call without rows still launches
-    // one CTA, which writes the header
-    const int grid = tokens > 0 ? static_cast<int>(tokens) : 1;
-    // up to one CTA per SM is resident whatever the CTA's size: such a call needs no tickets
-    const int64_t sms = plan->sms;
-    p.direct_tiles = tokens > direct_rows(plan) ? 0u : tokens <= sms ? 1u : 2u;
-    e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, rows_instance(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
+  if (tokens > direct_rows(plan)) {
+    const cudaError_t e = launch_encode_two_pass(p, plan->two_pass, static_cast<cudaStream_t>(cuda_stream));
+    g_launches.fetch_add(2);
+    return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
   }
+  // few rows: one CTA per row (a call without rows still launches one CTA, which writes the header).  Up to one CTA per SM is
+  // resident whatever the CTA's size: such a call needs no tickets.
+  const int grid = tokens > 0 ? static_cast<int>(tokens) : 1;
+  p.direct_tiles = tokens <= plan->sms ? 1u : 2u;
+  const cudaError_t e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, rows_instance(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
   g_launches.fetch_add(1);
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
 }
@@ -672,7 +589,7 @@ static int64_t part_rows(const tsq_plan_t* plan, int64_t tokens) {
   if (cudaGetDevice(&device) != cudaSuccess || device != plan->device) return tokens;  // the copy streams belong to the plan's device
   const int64_t row = static_cast<int64_t>(plan->row_bytes), parts = std::min<int64_t>(3, tokens * row / (4 << 20));
   if (parts < 2) return tokens;
-  const int64_t rows = std::min((tokens + parts - 1) / parts, std::min(direct_rows(plan), 6 * static_cast<int64_t>(plan->sms)));
+  const int64_t rows = std::min((tokens + parts - 1) / parts, 6 * static_cast<int64_t>(plan->sms));
   return rows * row < (1 << 20) ? tokens : rows;
 }
 

@@ -27,18 +27,13 @@ __device__ __forceinline__ void bulk_s2g(void* gmem_dst, const void* smem_src, u
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// all bulk groups of this thread but the latest have finished reading their source
-__device__ __forceinline__ void bulk_wait_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Per-thread asynchronous 16-byte copies global -> shared (no registers hold the data in flight).  The
-// lines are kept in L1 as well: the encoder reads the patterns of a group's further outliers from the
-// input a second time (measured 1 to 2 % faster than bypassing L1).
+// Per-thread asynchronous 16-byte copies global -> shared (no registers hold the data in flight), past L1.
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(smem_dst)), "l"(gmem_src) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(smem_dst)), "l"(gmem_src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
@@ -47,10 +42,6 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
-}
-// two adjacent 64-bit words in one request (16-byte aligned); nothing is assumed about the pair being read atomically
-__device__ __forceinline__ void ld_relaxed_u64x2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
 }
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
@@ -89,6 +80,7 @@ struct Elem<false> {  // IEEE binary16
   }
   // 0xffff in each half where a >= b or the pair is unordered
   static __device__ __forceinline__ uint32_t geu_mask(uint32_t a, uint32_t b) { return __hgeu2_mask(as2(a), as2(b)); }
+  static __device__ __forceinline__ uint32_t eq_mask(uint32_t a, uint32_t b) { return __heq2_mask(as2(a), as2(b)); }
   static __device__ __forceinline__ float lo_f32(uint32_t v) { return __low2float(as2(v)); }
   static __device__ __forceinline__ float hi_f32(uint32_t v) { return __high2float(as2(v)); }
   static __device__ __forceinline__ float pattern_f32(uint32_t p) {
@@ -112,6 +104,7 @@ struct Elem<true> {  // bfloat16
     return u;
   }
   static __device__ __forceinline__ uint32_t geu_mask(uint32_t a, uint32_t b) { return __hgeu2_mask(as2(a), as2(b)); }
+  static __device__ __forceinline__ uint32_t eq_mask(uint32_t a, uint32_t b) { return __heq2_mask(as2(a), as2(b)); }
   static __device__ __forceinline__ float lo_f32(uint32_t v) { return __uint_as_float(mad_u32(v, 65536u, 0u)); }
   static __device__ __forceinline__ float hi_f32(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
   static __device__ __forceinline__ float pattern_f32(uint32_t p) { return __uint_as_float(p << 16); }

@@ -1,54 +1,26 @@
 // tsq encode kernels: threshold splitting (Eq. "ts") + token-wise TAB-Q (Algorithm 1 on AIQ,
-// Eq. "Proposed") + bit-plane packing + CSR emission, fused into one kernel.
+// Eq. "Proposed") + bit-plane packing + CSR emission.
 //
-// One CTA encodes one token row at a time, one thread per group of 32 elements (64 bytes), and every
-// thread only ever touches its own group: the input is read from HBM exactly once.  The passes:
-//   A  threshold split: outlier bitmap, outlier slots set to +0 (what T_below holds there), and
-//      the row's min / max of the inlier magnitudes (CTA reduction);
-//   B  Algorithm 1: AIQ codes at the top level and at each lower candidate, distortion sums
-//      (CTA reduction, one candidate at a time, stopping at the first failure);
-//   C  codes at the chosen level -> bytes (code | sign << 7) -> 8 x 32 bit transpose -> the
-//      group's b* plane words, one contiguous run per thread.
-// Between the passes sits scalar work per row (the AIQ parameters of every candidate: a few
-// divisions) and the placement of the row's output, which has to wait for every earlier row.
+// Variable-length placement: where a token's planes and CSR entries start is an exclusive prefix sum over all earlier
+// tokens, and a token's sizes are known only after Algorithm 1 has run on it.  Calls of many rows therefore go through two
+// kernels that wait for nothing (here); calls of few rows through one that reads the sizes of the rows before it directly
+// (tsq_encode_rows.cu).
+//   sizes_kernel   one CTA per row: threshold, extremes, outlier count, Algorithm 1; leaves the row's bit-width, scale and
+//                  zero-point in the blob, its sizes and how its codes are formed in the workspace, and adds the sizes to cells for
+//                  the row's block of 32, 1024 and 32768 rows.
+//   pack_kernel    one CTA per row: its offsets from the cells (three loads per lane of one warp), codes -> bytes
+//                  (code | sign << 7) -> 8 x 32 bit transpose -> plane words, outlier entries.
+// x is read twice.  The forms that read it once (rows in shared memory or in registers, placement at once, by look-back, or put
+// off by a row's time) were all slower: in token order every row waits for the slowest of the rows before it, and a few rows in a
+// hundred take Algorithm 1 further than the first candidate (8192 x 8192 bf16 / 32768 x 4096 bf16 with 1 % outliers, us: persistent CTAs with a
+// ring of packed rows 87 / 190, one CTA per row 104 / 281, placement a row later 87 / 349, these kernels 65 / 126).
 //
-// Two kernels share the passes (tsq_encode_device.cuh):
-//   encode_rows_kernel  (tsq_encode_rows.cu) one CTA per row, the group in registers from load to store,
-//                       everything in order; used up to some rows per SM (no pipeline to fill) and for
-//                       rows longer than the pipelined kernel takes.
-//   encode_pipe_kernel  (here) persistent CTAs that keep several rows in different stages at once, so that
-//                       the vector passes never wait for the scalar work or for the placement.
-//                       Each compute thread copies its group of the next row into shared memory
-//                       asynchronously (no registers held), runs pass A on row n in place there,
-//                       then passes B and C of row n - 1 from its copy; a "levels" warp turns row
-//                       n's min / max into AIQ parameters meanwhile; a "placement" warp resolves the
-//                       offsets of rows packed earlier, ships their planes with one bulk
-//                       asynchronous store each and writes their CSR entries.  When the first
-//                       lower candidate fails (the usual case) pass C reuses the top-level bytes
-//                       that pass B already formed; with 4 and 8 bits as the last two candidates pass B
-//                       forms only those, and decides the 4-bit candidate from their planes
-//                       (certain_distortion_8_to_4) unless the codes it leaves open matter.
-//
-// What binds: the chain of dependent instructions of an iteration, with too few warps to hide it (two CTAs of ten warps per
-// SM by registers and shared memory, half of the issue slots used), and within it the integer / logic pipe, which issues at
-// half the rate of the FMA pipe: the passes work on two 16-bit elements per 32-bit register wherever they can (four codes as
-// bytes in the distortion sum and on the way to the bit transpose), and some shifts and merges are written as integer
-// multiply-adds so that they go to the FMA pipe instead.  Of the 5400 cycles of an iteration at hidden 8192 (clock stamps of
-// compute thread 0, whose warp the others wait for) pass B takes 2000, pass C with the CSR entries 740, pass A 700, the
-// levels of the row before 340, the decision 250, the wait for a ring slot 210, publishing the sizes 170.  8192 x 8192
-// bf16: 98.5 us with the three-operation quotient and the exact distortion sum for every row, 86.8 us (2.34 TB/s) with one FMA
-// per code and the sum from the planes.
-//
-// Variable-length placement: where a token's planes and CSR entries start is an exclusive prefix
-// sum over all earlier tokens.  It is resolved with a decoupled look-back over per-token
-// descriptors in the workspace.  Rows are numbered by an atomic ticket taken by a running CTA,
-// so a row only ever waits for rows whose CTAs are already running, and a row publishes its own
-// sizes before it waits for anything.  A look-back step reads 32 descriptor pairs at once (256 in the
-// one-CTA-per-row kernel, whose calls of few rows read all predecessors directly instead).  Every wait
-// is bounded and fails into a status word.
+// What binds: DRAM and instruction issue about equally.  The two kernels move 332 MB at 8192 x 8192 bf16 (x twice, 8 % of the
+// second time from L2; 51 us at the copy rate) and issue every other to two cycles out of three.  So the passes work on two 16-bit elements
+// per 32-bit register and on two binary32 values per 64-bit register wherever they can, and what a row costs once is kept short.
 //
 // Arithmetic contract: the codes equal  clamp(rint(m / s) - zp, 0, Qmax)  with the IEEE binary32
-// quotient m / s.  "Plain" rows (nearly every row of real data: zero-point 0, which any row with an
+// quotient m / s.  "Plain" levels (zero-point 0, which any row with an
 // outlier or a tiny element has; no code above Qmax; scale in [2^-60, 2^60], so that no intermediate
 // leaves the normal range) form the quotient without the division instruction: r = fl(1 / s) once
 // per row and level, then per element q0 = fl(m * r), the residual m - q0 * s (one FMA) and
@@ -61,755 +33,857 @@
 // checks the three-operation sequence in exact arithmetic against the true quotient for every
 // 16-bit pattern over many ranges and levels, and the GPU parity tests compare every code.  (A
 // single fl(m * r) is not enough: 16-bit inputs put m / s on or next to a rounding boundary
-// k + 1/2 in almost every row, and there the two can round differently.  At 8 bits a factor per row that
-// has been tried out against all its rounding boundaries, one_fma_factor, does make it enough.)  Every other
-// row goes through the division instruction in compact loops.
-
-#include <mutex>
+// k + 1/2 in almost every row, and there the two can round differently.  A factor per row that is moved off the one
+// boundary that can be hit, or has been tried out against all of them, does make it enough: kOneUp, kOneDown, kOneTried.)  Every other
+// row goes through the division instruction.
 
 #include "tsq_encode_device.cuh"
 
 namespace tsq {
 namespace {
 
-// =====================================================================================================
-// encode_pipe_kernel: persistent CTAs, rows in several stages at once.
-// =====================================================================================================
-// Threads: `compute` threads (one per 32-element group of a row, a multiple of 32), then the levels
-// warp, then the placement warp.  Row n of a CTA (n = 0, 1, ... in the order it takes them):
-//   compute warps, iteration n - 1  asynchronous copies of the row into xpark[n % 3], 64 bytes per thread
-//   compute warps, iteration n      pass A on the thread's own 64 bytes, thresholded values written back in
-//                                   place; per-warp partial results in meta[n % kMetaRing]
-//   levels warp                     meta[..].lv = AIQ parameters of every candidate (after a_ready > n)
-//   compute warps, iteration n + 1  passes B and C from the parked copy (after lv_ready > n), planes
-//                                   into planes[n % ring], CSR entries into csr[n % ring]
-//   placement warp                  offsets by look-back, bulk store of the planes, token fields, CSR
-//                                   entries (after packed > n); then placed = n + 1 frees the slots.
-// Each thread copies, thresholds and re-reads only its own group, so the parked rows need no barrier.  All counters
-// only grow; every wait on them is bounded and raises `abort`.
+// How the levels of a row are decided
+constexpr int kKind84 = 0;      // magnitudes, candidates end in 4 and 8 bits: bounds, exact sums where they leave it open
+constexpr int kKindExact = 1;   // any other candidates of the magnitudes: exact sums
+constexpr int kKindSigned = 2;  // signed values: exact sums
 
-// Rows a CTA may hold between packing and placement: p.ring (2 .. kMaxRing) slots of planes and CSR entries,
-// as many as fit beside the parked rows.  Placement waits for the rows before it, so a deep ring is what
-// keeps the compute warps busy while a slow predecessor (a row whose descent goes on) holds everybody up.
-constexpr int kMetaRing = kMaxRing + 2;  // row records: one row in pass A and one being packed on top of those
+// How pack_kernel forms a row's codes
+constexpr uint32_t kDivide = 0;    // by the division instruction
+constexpr uint32_t kPlain = 1;     // three-operation quotient
+constexpr uint32_t kOneUp = 2;     // one FMA, factor 1/s moved up (half the largest magnitude rounds up), zero-point 0
+constexpr uint32_t kOneDown = 3;   // one FMA, factor 1/s moved down
+constexpr uint32_t kOneTried = 4;  // one FMA with fl(1/s), tried out against every boundary
+constexpr uint32_t kCapped = 5;    // signed values: three-operation quotient, the largest value's code clamped
 
-// How the pipelined kernel decides the first lower candidate:
-constexpr int kKind84 = 0;      // 8 bits against 4: from the 8-bit codes' planes, the exact sum only when the open codes matter
-constexpr int kKindExact = 1;   // any other candidates: the exact distortion sum
-constexpr int kKindSigned = 2;  // signed-values variant, exact sum
-constexpr int kExactSlot = kMaxCand - 1;  // kKind84 (at most four candidates): the distortion slot of the exact first sum
-
-struct RowMeta {
-  Level lv[kMaxCand];
-  int S[kMaxCand];
-  RowPartials<(kPipeMaxThreads - 64) / 32> part;
-  uint32_t tile, row_cnt, divide;
-  uint32_t bstar, agg_w;
-  float scale;
-  int zp;
-  float lo, hi;    // smallest and largest magnitude
-  float one_fma;   // kKind84: the factor of the one-FMA codes (one_fma_factor), 0: the three-operation quotient
-  OneFma top_one, low_one;  // kKindSigned: both levels' one-FMA codes; one_fma = 0: not for this row
-  uint32_t heavy;  // 1: the side buffer holds the row's outlier bitmaps (more outliers than a list holds)
-};
-
-struct PipeShared {
-  RowMeta meta[kMetaRing];
-  volatile uint32_t a_ready;   // rows whose pass A results are in their record
-  volatile uint32_t lv_ready;  // rows whose levels are computed
-  volatile uint32_t packed;    // rows packed and parked
-  volatile uint32_t placed;    // rows placed
-  volatile uint32_t finished;  // the compute warps are done: a_ready and packed are final
-  volatile uint32_t abort;     // a wait inside the CTA ran out
-  volatile uint32_t stop[2];   // abort as thread 0 saw it before the iteration's barrier, by iteration parity: what the
-                               // compute threads act on, so that all of them leave the row loop in the same iteration
-  uint32_t wait_limit;         // polls before a handshake gives up
-  uint32_t next_tile[2];       // ticket of the row after the current one, by iteration parity
-  // Rows with more outliers than a ring slot's list holds: the compute threads leave the groups' bitmaps in a side
-  // buffer, the placement warp posts the row's CSR offset there once it is resolved, and the compute threads write
-  // the entries themselves, all at once, at the top of a later iteration.  (One buffer: a second one would cost
-  // the ring a slot at hidden 8192.  A row that finds it taken leaves its bitmaps in the list instead.)
-  uint32_t heavy_bm[kPipeMaxThreads - 64];
-  uint32_t heavy_wcnt[(kPipeMaxThreads - 64) / 32];  // exclusive scan of the warps' outlier counts
-  uint32_t heavy_tile;
-  volatile uint32_t heavy_base;      // out_ptr[tile], from the placement warp
-  volatile uint32_t heavy_posted;    // such rows whose offset has been posted
-  volatile uint32_t heavy_seen[2];   // heavy_posted as thread 0 saw it before the iteration's barrier, by iteration parity
-};
-
-__device__ __forceinline__ void compute_barrier(uint32_t nthreads) {
-  asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
+// A row's size in its slot: outliers | bits << 17 | mode << 21 (the upper half stays 0: no tag of a direct call)
+__device__ __forceinline__ unsigned long long row_entry(uint32_t outliers, int b, uint32_t mode) {
+  return outliers | static_cast<uint32_t>(b) << 17 | mode << 21;
 }
 
-// Wait until *counter > n.  Returns false when the wait is to be given up: `finished` is set and the
-// counter will not grow any more, or the CTA aborted, or the limit ran out (which raises abort).
-__device__ __forceinline__ bool wait_beyond(volatile uint32_t* counter, uint32_t n, PipeShared& sh, bool may_finish,
-                                            uint32_t nap_ns) {
-  for (uint32_t polls = 0;; ++polls) {
-    if (*counter > n) return true;
-    if (sh.abort != 0u) return false;
-    if (may_finish && sh.finished != 0u) return *counter > n;
-    if (polls > sh.wait_limit) {
-      sh.abort = 1u;
-      return false;
-    }
-    __nanosleep(nap_ns);
+__device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ uint4 load_once(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void store32(uint32_t* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f, uint32_t g, uint32_t h) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h) : "memory");
+}
+// top bits of the halves of ta, tb as bytes 0xff / 0: a.lo, b.lo, a.hi, b.hi
+__device__ __forceinline__ uint32_t top_bits4(uint32_t ta, uint32_t tb) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, 0xfbd9;" : "=r"(r) : "r"(ta), "r"(tb));
+  return r;
+}
+// min(|x|, m) of the two elements of a pair
+template <bool BF16>
+__device__ __forceinline__ uint32_t min_abs2(uint32_t x, uint32_t m) {
+  uint32_t r;
+  if (BF16) {
+    asm("{.reg .b32 t; abs.bf16x2 t, %1; min.bf16x2 %0, t, %2;}" : "=r"(r) : "r"(x), "r"(m));
+  } else {
+    asm("{.reg .b32 t; abs.f16x2 t, %1; min.f16x2 %0, t, %2;}" : "=r"(r) : "r"(x), "r"(m));
   }
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2_rm(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
-// FULL: every compute thread owns a whole 32-element group (hidden is a multiple of 1024), so none of the
-// checks for short or missing groups is needed.
-// SV: the signed-values variant.
-// KIND: how the first lower candidate is decided (see the kKind constants).
-template <bool BF16, bool FULL, int MAXT, int MINB, int KIND>
-__global__ void __launch_bounds__(MAXT, MINB) encode_pipe_kernel(const __grid_constant__ EncodeParams p) {
+template <int NW>
+struct __align__(16) SizesShared {
+  static constexpr int kSlots = NW < 4 ? 4 : NW;
+  // by warp; the entries past the last warp are neutral
+  uint32_t warp_min[kSlots], warp_cnt[kSlots];
+  int warp_max[kSlots];
+  int warp_sum[2][kSlots];
+  Level lv[kMaxCand];
+  uint32_t divide;
+};
+
+struct RowChoice {
+  int b, zp;
+  float s;
+  uint32_t mode;
+};
+
+// The sum of v over the CTA, in every thread; `turn` alternates between calls that follow one another.
+template <int NW>
+__device__ __forceinline__ int cta_sum(SizesShared<NW>& sh, int v, uint32_t turn, uint32_t nwarps) {
+  v = __reduce_add_sync(kFull, v);
+  if (nwarps == 1u) return v;
+  if ((threadIdx.x & 31u) == 0u) sh.warp_sum[turn][threadIdx.x >> 5] = v;
+  __syncthreads();
+  int sum = 0;
+#pragma unroll
+  for (int w = 0; w < SizesShared<NW>::kSlots; w += 4) {
+    const int4 a = *reinterpret_cast<const int4*>(&sh.warp_sum[turn][w]);
+    sum += a.x + a.y + a.z + a.w;
+  }
+  return sum;
+}
+
+// Algorithm 1 with exact sums for one row, by the whole CTA, from the row's extremes (patterns of magnitudes, or order keys).
+// The thread's chunks are read again (C chunks, 32 per warp and step, as in sizes_kernel).
+template <bool BF16, int C, bool SV, int NW>
+__device__ __noinline__ RowChoice settle_exactly(const EncodeParams& p, const uint4* xrow, uint32_t pmin, uint32_t pmax, SizesShared<NW>& sh) {
+  using E = Elem<BF16>;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const uint32_t thr2 = p.thr16 * 0x10001u;
+  __syncthreads();
+  if (warp == 0) {
+    const int b = p.bits[min(lane, static_cast<uint32_t>(p.n_bits - 1))];
+    bool plain = false;
+    const Level lv = SV ? make_level_signed(E::pattern_f32(pattern_of_key(pmin)), E::pattern_f32(pattern_of_key(pmax)), b, &plain)
+                        : make_level(E::pattern_f32(pmin), E::pattern_f32(pmax), b, &plain);
+    if (lane < static_cast<uint32_t>(p.n_bits)) sh.lv[lane] = lv;
+    const bool all = __all_sync(kFull, plain);
+    if (lane == 0) sh.divide = all ? 0u : 1u;
+  }
+  __syncthreads();
+  const bool divide = sh.divide != 0u;
+  const Level top = sh.lv[p.n_bits - 1];
+  const int bmax = p.bits[p.n_bits - 1];
+  RowChoice best{bmax, top.zp, top.s, divide ? kDivide : kPlain};
+  for (int ci = p.n_bits - 2; ci >= 0; --ci) {
+    const Level low = sh.lv[ci];
+    const int shn = bmax - p.bits[ci];
+    uint32_t S = 0;
+#pragma unroll 1
+    for (uint32_t k = 0; k < (C + 3u) / 4u; ++k) {
+      uint32_t x[16];
+      uint32_t nvalid = 0u;
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) {
+        const uint32_t idx = (warp * C + 4u * k + j) * 32u + lane;
+        uint4 c = make_uint4(0u, 0u, 0u, 0u);
+        if (4u * k + j < static_cast<uint32_t>(C) && idx < p.chunks) {
+          c = xrow[idx];
+          nvalid = j + 1u;
+        }
+        x[4 * j + 0] = c.x;
+        x[4 * j + 1] = c.y;
+        x[4 * j + 2] = c.z;
+        x[4 * j + 3] = c.w;
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) x[i] &= ~E::geu_mask(x[i] & 0x7fff7fffu, thr2);
+      if (divide) {
+        S += divide_distortion_regs<BF16, SV>(x, top, low, shn, 4u * nvalid);
+      } else {
+        S += distortion_group<BF16, SV>(x, make_level2(top), make_level2(low), shn, nvalid);
+      }
+    }
+    if (cta_sum(sh, static_cast<int>(S), static_cast<uint32_t>(ci) & 1u, nwarps) > p.s_max) break;  // keep the last level that passed
+    best.b = p.bits[ci];
+    best.s = low.s;
+    best.zp = low.zp;
+  }
+  return best;
+}
+
+// hi / Q, correctly rounded for every 16-bit hi (as in quick_level); *tie: Q divides hi's significand.
+template <int Q>
+__device__ __forceinline__ float divide_by(float hi, bool* tie) {
+  constexpr float kInv = 1.0f / static_cast<float>(Q);
+  const float q0 = __fmul_rn(hi, kInv), s = __fmaf_rn(__fmaf_rn(-static_cast<float>(Q), q0, hi), kInv, q0);
+  *tie = __fmaf_rn(-static_cast<float>(Q), s, hi) == 0.0f;
+  return s;
+}
+// Whether rint(fl((hi / 2) / s)) is the upper of the two codes that hi / 2 lies between (k and k + 1, k + 1/2 = Q / 2): the quotient
+// rounds to k + 1/2 or more iff (hi / 2) - (k + 1/2) s (exact) is not below -2^-half s, half an ulp below k + 1/2; ties go to
+// k + 1 there (k = 63, 3 and 1 are odd).
+__device__ __forceinline__ bool middle_up(float hi, float s, float middle, float half) { return __fmaf_rn(-middle, s, 0.5f * hi) >= -half * s; }
+
+// The distortion sum between the 8-bit level and a lower one, for rows with zero-point 0, without forming codes.  In ideal arithmetic the lower
+// level (Q codes above 0) rounds y = Q m / range up at y = k + 1/2 and q >> sh steps at y = (2^sh j - 1/2) Q / 127; both are even about Q / 2, and
+// with v = |y - Q / 2| they lie at v = k and at v = k / ratio, ratio = 127 / (2^sh Q), k = 1, 2, ...  So the difference of an element is 1 between
+// k / ratio and k and 0 elsewhere: with w = y - Q / 2 it is floor(ratio w) - floor(w), negative for w < 0.  kMargin moves both steps inwards, further
+// than the rounding of all of this and of the codes goes: the sum is a lower bound, and exact but for elements that lie next to a step.
+constexpr float kMargin = 0x1p-19f;
+struct Steps {
+  uint64_t per2, mid2, ratio2, one2;
+};
+__device__ __forceinline__ Steps steps_of(float q, float ratio, float range) {
+  const float c = q * rcp_approx(range), ka = ratio - kMargin * ratio, kb = 1.0f + kMargin;
+  return Steps{pack2f(c, c), pack2f(-0.5f * q, -0.5f * q), pack2f(ka, ka), pack2f(kb, kb)};
+}
+template <bool BF16>
+__device__ __forceinline__ uint64_t add_differences(uint32_t x, uint32_t hi2, const Steps& t, uint64_t acc) {
+  const uint64_t magic2 = pack2f(kRoundMagicSigned, kRoundMagicSigned), neg2 = pack2f(-1.0f, -1.0f);
+  const uint64_t w = fma2(values2<BF16>(min_abs2<BF16>(x, hi2)), t.per2, t.mid2);  // an outlier counts as hi: 0
+  const uint64_t d = fma2(fma2_rm(w, t.one2, magic2), neg2, fma2_rm(w, t.ratio2, magic2));
+  return fma2(d, d, acc);
+}
+__device__ __forceinline__ int sum_of(uint64_t acc) {
+  float a, b;
+  unpack2f(acc, a, b);
+  return __float2int_rn(a + b);
+}
+
+// The same sum over a row's chunks read again, for a further candidate.
+template <bool BF16, int C, int NW>
+__device__ __noinline__ int sum_again(const EncodeParams& p, const uint4* xrow, uint32_t hi2, float q, float ratio, float range, uint32_t turn, SizesShared<NW>& sh) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  uint4 v[C];
+#pragma unroll
+  for (uint32_t j = 0; j < static_cast<uint32_t>(C); ++j) {
+    const uint32_t idx = (warp * C + j) * 32u + lane;
+    v[j] = idx < p.chunks ? xrow[idx] : make_uint4(0u, 0u, 0u, 0u);
+  }
+  const Steps t = steps_of(q, ratio, range);
+  uint64_t acc = 0ull;
+#pragma unroll
+  for (uint32_t j = 0; j < static_cast<uint32_t>(C); ++j) {
+    acc = add_differences<BF16>(v[j].x, hi2, t, acc);
+    acc = add_differences<BF16>(v[j].y, hi2, t, acc);
+    acc = add_differences<BF16>(v[j].z, hi2, t, acc);
+    acc = add_differences<BF16>(v[j].w, hi2, t, acc);
+  }
+  return cta_sum(sh, sum_of(acc), turn, nwarps);
+}
+
+// By the whole warp: the 16-bit magnitude next to each step (one per lane), and by how much the sum is off for an element of that magnitude.
+template <bool BF16>
+__device__ __forceinline__ int step_error(float q, float ratio, float range, int sh, uint32_t lane, uint32_t* pattern) {
+  using E = Elem<BF16>;
+  const uint32_t k = lane & 15u;
+  const bool of_low = lane < 16u;
+  const float at = (of_low ? static_cast<float>(k) + 0.5f : (static_cast<float>((k + 1u) << sh) - 0.5f) * q * (1.0f / 127.0f)) / q * range;
+  *pattern = E::pack_rn(at, 0.0f) & 0xffffu;
+  const float m = E::pattern_f32(*pattern);
+  const bool middle_again = !of_low && static_cast<float>(2u * k + 1u) == q;  // both have a step there
+  if (static_cast<float>(k) >= q || middle_again || fabsf(m - at) > 0x1p-14f * at) return 0;
+  const int code = __float2int_rn(__fdiv_rn(m, __fdiv_rn(range, 127.0f))), low = __float2int_rn(__fdiv_rn(m, __fdiv_rn(range, q)));
+  const float w = __fmaf_rn(m, q * rcp_approx(range), -0.5f * q);
+  const float d = __fmaf_rd(w, ratio - kMargin * ratio, kRoundMagicSigned) - __fmaf_rd(w, 1.0f + kMargin, kRoundMagicSigned);
+  return abs((code >> sh) - low) - static_cast<int>(fabsf(d));
+}
+
+template <bool BF16, int C, int KIND, bool FULL, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
   constexpr bool SV = KIND == kKindSigned;
+  using Shared = SizesShared<MAXT / 32>;
+  __shared__ Shared sh;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  launch_dependents();
+  if (tid >= nwarps && tid < static_cast<uint32_t>(Shared::kSlots)) {
+    sh.warp_min[tid] = 0xffffu;
+    sh.warp_max[tid] = KIND == kKind84 ? -32768 : 0;
+    sh.warp_cnt[tid] = 0u;
+    sh.warp_sum[0][tid] = sh.warp_sum[1][tid] = 0;
+  }
+  wait_for_prior_grids();
+  const uint32_t tile = blockIdx.x;
+  const uint4* xrow = reinterpret_cast<const uint4*>(p.x) + static_cast<size_t>(tile) * p.chunks;
+  uint32_t x[C][4];
+  uint32_t nv = FULL ? C : 0u;
+#pragma unroll
+  for (uint32_t j = 0; j < C; ++j) {
+    const uint32_t idx = (warp * C + j) * 32u + lane;
+    uint4 c = make_uint4(0u, 0u, 0u, 0u);
+    if (FULL || idx < p.chunks) {
+      c = load_once(xrow + idx);
+      if (!FULL) nv = j + 1u;
+    }
+    x[j][0] = c.x;
+    x[j][1] = c.y;
+    x[j][2] = c.z;
+    x[j][3] = c.w;
+  }
+  const uint32_t turn = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn) & 1u;
+  if (tile == 0u && tid == 0u) p.ws->sums_turn_next = turn ^ 1u;
+  const uint32_t thr2 = p.thr16 * 0x10001u;
+
+  uint32_t mn, cnt = 0u;
+  int mx;
+  if (KIND == kKind84) {
+    uint32_t mxt = 0x80008000u, mnt = 0xffffffffu;
+    int c1 = 0;
+#pragma unroll
+    for (int j = 0; j < C; j += 2) {
+      const uint32_t in = FULL ? 0xffffffffu : (j < static_cast<int>(nv) ? 0x00ff00ffu : 0u) | (j + 1 < static_cast<int>(nv) ? 0xff00ff00u : 0u);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t ta = (x[j][i] | 0x80008000u) - thr2, tb = (x[j + 1][i] | 0x80008000u) - thr2;
+        mxt = __vimax3_s16x2(mxt, ta, tb);
+        if (FULL) {
+          mnt = __vimin3_u16x2(mnt, ta, tb);
+        } else {
+          if (j < static_cast<int>(nv)) mnt = __vminu2(mnt, ta);
+          if (j + 1 < static_cast<int>(nv)) mnt = __vminu2(mnt, tb);
+        }
+        const uint32_t f = FULL ? top_bits4(ta, tb) : top_bits4(ta, tb) & in;
+        c1 = __dp4a(static_cast<int>(f), static_cast<int>(f), c1);
+      }
+    }
+    mn = __reduce_min_sync(kFull, min(mnt & 0xffffu, mnt >> 16));
+    mx = __reduce_max_sync(kFull, max(static_cast<int>(static_cast<short>(mxt & 0xffffu)), static_cast<int>(mxt) >> 16));
+    cnt = static_cast<uint32_t>(__reduce_add_sync(kFull, c1));
+  } else {
+    // outlier slots become +0, as T_below has it; extremes of the magnitudes, or of the signed values: their patterns as signed (smax) and as
+    // unsigned numbers (umax, umin)
+    uint32_t smax = 0x80008000u, umax = 0u, umin = 0xffffffffu;
+    int c1 = 0;
+#pragma unroll
+    for (int j = 0; j < C; j += 2) {
+      const bool in_a = FULL || j < static_cast<int>(nv), in_b = FULL || j + 1 < static_cast<int>(nv);
+      const uint32_t in = (in_a ? 0x00ff00ffu : 0u) | (in_b ? 0xff00ff00u : 0u);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t f = top_bits4((x[j][i] | 0x80008000u) - thr2, (x[j + 1][i] | 0x80008000u) - thr2) & in;
+        c1 = __dp4a(static_cast<int>(f), static_cast<int>(f), c1);
+        x[j][i] &= ~__byte_perm(f, 0u, 0x2200);
+        x[j + 1][i] &= ~__byte_perm(f, 0u, 0x3311);
+        const uint32_t va = SV ? x[j][i] : x[j][i] & 0x7fff7fffu, vb = SV ? x[j + 1][i] : x[j + 1][i] & 0x7fff7fffu;
+        if (in_a) {  // (a row's chunks end with those of a thread: b inside means a inside)
+          const uint32_t v2 = in_b ? vb : va;
+          if (SV) smax = __vimax3_s16x2(smax, va, v2);
+          umax = __vimax3_u16x2(umax, va, v2);
+          umin = __vimin3_u16x2(umin, va, v2);
+        }
+      }
+    }
+    cnt = static_cast<uint32_t>(__reduce_add_sync(kFull, c1));
+    const uint32_t most = __reduce_max_sync(kFull, max(umax & 0xffffu, umax >> 16)), least = __reduce_min_sync(kFull, min(umin & 0xffffu, umin >> 16));
+    mn = least;
+    mx = static_cast<int>(most);
+    if (SV) {
+      // As order keys.  Patterns of non-negative values order like the values, those of negative ones the other way round: the
+      // largest value is the largest signed pattern if that is non-negative, else the smallest unsigned one; the smallest is the largest
+      // unsigned pattern if that is negative, else the smallest.  (A warp without values: the neutral keys.)
+      const int top = __reduce_max_sync(kFull, max(static_cast<int>(static_cast<short>(smax & 0xffffu)), static_cast<int>(smax) >> 16));
+      const bool none = least > most;
+      mx = none ? 0 : static_cast<int>(order_keys2(top >= 0 ? static_cast<uint32_t>(top) : least) & 0xffffu);
+      mn = none ? 0xffffu : order_keys2(most >= 0x8000u ? most : least) & 0xffffu;
+    }
+  }
+  uint32_t pmin = mn, row_cnt = cnt;
+  int mxr = mx;
+  if (nwarps > 1u) {
+    if (lane == 0) {
+      sh.warp_min[warp] = mn;
+      sh.warp_max[warp] = mx;
+      sh.warp_cnt[warp] = cnt;
+    }
+    __syncthreads();
+    row_cnt = 0u;
+#pragma unroll
+    for (int w = 0; w < Shared::kSlots; w += 4) {
+      const uint4 a = *reinterpret_cast<const uint4*>(&sh.warp_min[w]), c = *reinterpret_cast<const uint4*>(&sh.warp_cnt[w]);
+      const int4 b = *reinterpret_cast<const int4*>(&sh.warp_max[w]);
+      pmin = min(pmin, min(min(a.x, a.y), min(a.z, a.w)));
+      mxr = max(mxr, max(max(b.x, b.y), max(b.z, b.w)));
+      row_cnt += c.x + c.y + c.z + c.w;
+    }
+  }
+  uint32_t pmax = static_cast<uint32_t>(mxr);
+  RowChoice best{0, 0, 0.0f, kPlain};
+  if (KIND == kKind84) {
+    pmin = row_cnt != 0u ? 0u : (pmin + p.thr16) & 0x7fffu;
+    pmax = mxr < 0 ? 0u : (pmax + p.thr16) & 0x7fffu;
+    const float lo = E::pattern_f32(pmin), hi = E::pattern_f32(pmax), range = hi - lo;
+    if (hi >= 0x1p-50f && hi <= 0x1p60f && 256.0f * lo <= hi) {
+      const uint32_t hi2 = pmax * 0x10001u;
+      int S;
+      {
+        const Steps t = steps_of(7.0f, 127.0f / 112.0f, range);
+        uint64_t acc = 0ull;
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc = add_differences<BF16>(x[j][i], hi2, t, acc);
+        }
+        S = cta_sum(sh, sum_of(acc), 0u, nwarps);
+      }
+      best.b = 8;
+      if (S <= p.s_max) {  // the 4-bit candidate may pass: exact sums from here on, candidate by candidate
+        uint32_t turn_of_sum = 1u;
+#pragma unroll 1
+        for (int ci = p.n_bits - 2; ci >= 0; --ci) {
+          const int b = p.bits[ci];
+          const float q = static_cast<float>((1 << (b - 1)) - 1), ratio = b == 4 ? 127.0f / 112.0f : b == 3 ? 127.0f / 96.0f : 127.0f / 64.0f;
+          if (b == 3) {
+            S = sum_again<BF16, C>(p, xrow, hi2, q, ratio, range, turn_of_sum, sh);
+            turn_of_sum ^= 1u;
+          }
+          if (b == 2) S = 0;  // (one step for both, in the middle)
+          uint32_t pattern;
+          const int error = step_error<BF16>(q, ratio, range, 8 - b, lane, &pattern);
+#pragma unroll 1
+          for (uint32_t open = __ballot_sync(kFull, error != 0); open != 0u; open &= open - 1u) {
+            const int l = __ffs(open) - 1;
+            const uint32_t m2 = __shfl_sync(kFull, pattern, l) * 0x10001u;
+            uint32_t same = 0u;  // minus the elements of that magnitude, by half
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) same = __vadd2(same, E::eq_mask(x[j][i] & 0x7fff7fffu, m2));
+            }
+            const int n = -(static_cast<int>(static_cast<short>(same & 0xffffu)) + (static_cast<int>(same) >> 16));
+            S += __shfl_sync(kFull, error, l) * cta_sum(sh, n, turn_of_sum, nwarps);
+            turn_of_sum ^= 1u;
+          }
+          if (S > p.s_max) break;  // keep the last level that passed
+          best.b = b;
+        }
+      }
+      if (best.b != 0 && warp == 0u) {
+        const int b = best.b;
+        if (pmin == 0u && b == 8) {
+          bool tie;
+          best.s = divide_by<127>(hi, &tie);
+          if (!tie) best.mode = middle_up(hi, best.s, 63.5f, 0x1p-19f) ? kOneUp : kOneDown;
+        } else if (pmin == 0u) {
+          bool tie = false;
+          best.s = b == 4 ? divide_by<7>(hi, &tie) : b == 3 ? divide_by<3>(hi, &tie) : hi;
+          const bool up = b == 4 ? middle_up(hi, best.s, 3.5f, 0x1p-23f) : b == 3 ? middle_up(hi, best.s, 1.5f, 0x1p-24f) : false;
+          if (!tie || b == 2) best.mode = up ? kOneUp : kOneDown;
+        } else {
+          const float q = static_cast<float>((1 << (b - 1)) - 1);
+          best.s = __fdiv_rn(range, q);
+          const float r = __frcp_rn(best.s);
+          bool same = true;
+#pragma unroll 1
+          for (uint32_t i = lane; i < static_cast<uint32_t>(q); i += 32u) {
+            const float m = E::lo_f32(E::pack_rn(__fmul_rn(static_cast<float>(i) + 0.5f, best.s), 0.0f));
+            const float q0 = __fmul_rn(m, r), qt = __fmaf_rn(__fmaf_rn(q0, -best.s, m), r, q0);
+            same = same && __fadd_rn(qt, kRoundMagic) == __fmaf_rn(m, r, kRoundMagic);
+          }
+          if (__all_sync(kFull, same)) best.mode = kOneTried;
+        }
+      }
+    }
+  }
+  if (KIND != kKind84) {
+    // The exact sums, candidate by candidate, while every level has the packed steps (lane i takes candidate i).  Signed values: a code
+    // that needs the clamp is one that a tie has rounded up against the smallest value's, which only the largest value's can be (its quotient lies
+    // qmax above the smallest one's): its elements are counted, and what they add to the sum is taken out of it again.
+    const int mine = static_cast<int>(min(lane, static_cast<uint32_t>(p.n_bits - 1)));
+    const float largest = E::pattern_f32(SV ? pattern_of_key(pmax) : pmax);
+    bool plain, packed;
+    Level lv;
+    if (SV) {
+      lv = make_level_signed(E::pattern_f32(pattern_of_key(pmin)), largest, p.bits[mine], &plain, &packed);
+    } else {
+      lv = make_level(E::pattern_f32(pmin), largest, p.bits[mine], &plain);
+      packed = plain;
+    }
+    if (__all_sync(kFull, packed)) {
+      const bool all_plain = !SV || __all_sync(kFull, plain);
+      const auto level_of = [&](int i) {
+        return Level{__shfl_sync(kFull, lv.s, i), __shfl_sync(kFull, lv.r, i), __shfl_sync(kFull, lv.zp, i), __shfl_sync(kFull, lv.qmax, i)};
+      };
+      const Level top = level_of(p.n_bits - 1);
+      const int bmax = p.bits[p.n_bits - 1];
+      best = RowChoice{bmax, top.zp, top.s, all_plain ? kPlain : kCapped};
+      int n_largest = 0;
+      if (!all_plain) {
+        const uint32_t m2 = pattern_of_key(pmax) * 0x10001u;
+        uint32_t same = 0u;  // minus the elements of that value, by half
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+          if (j < static_cast<int>(nv)) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) same = __vadd2(same, E::eq_mask(x[j][i], m2));
+          }
+        }
+        n_largest = cta_sum(sh, -(static_cast<int>(static_cast<short>(same & 0xffffu)) + (static_cast<int>(same) >> 16)), static_cast<uint32_t>(p.n_bits - 1) & 1u, nwarps);
+      }
+#pragma unroll 1
+      for (int ci = p.n_bits - 2; ci >= 0; --ci) {
+        const Level low = level_of(ci);
+        const int shn = bmax - p.bits[ci];
+        uint32_t sum = 0u;
+#pragma unroll
+        for (int j = 0; j < C; j += 4) {
+          uint32_t g[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) g[i] = x[j + i / 4][i & 3];
+          const int left = static_cast<int>(nv) - j;
+          sum += distortion_group<BF16, SV>(g, make_level2(top), make_level2(low), shn, FULL ? 4u : left <= 0 ? 0u : static_cast<uint32_t>(min(left, 4)));
+        }
+        int S = cta_sum(sh, static_cast<int>(sum), static_cast<uint32_t>(ci) & 1u, nwarps);
+        if (!all_plain) {  // as the packed steps have it for the largest value, whose difference is 0
+          const int code = (__float2int_rn(__fdiv_rn(largest, top.s)) - top.zp) & 0xff, lower = (__float2int_rn(__fdiv_rn(largest, low.s)) - low.zp) & 0xff;
+          S -= n_largest * abs((code >> shn) - lower);
+        }
+        if (S > p.s_max) break;  // keep the last level that passed
+        best.b = p.bits[ci];
+        best.s = low.s;
+        best.zp = low.zp;
+      }
+    }
+  }
+  if (best.b == 0) best = settle_exactly<BF16, C, SV>(p, xrow, pmin, pmax, sh);
+  if (tid == 0) {
+    unsigned long long* cells = p.desc + 1;
+    const unsigned long long size = (static_cast<unsigned long long>(static_cast<uint32_t>(best.b) * p.lay.wpp) << 32) | row_cnt;
+    if ((tile | 31u) < p.tokens) red_add_u64(cells + 2u * ((tile & ~31u) + turn), size);
+    if ((tile | 1023u) < p.tokens) red_add_u64(cells + 2u * ((tile & ~1023u) + 2u + turn), size);
+    if ((tile | 32767u) < p.tokens) red_add_u64(cells + 2u * ((tile & ~32767u) + 4u + turn), size);
+    p.desc[2u * tile] = row_entry(row_cnt, best.b, best.mode);
+    reinterpret_cast<uint8_t*>(p.blob + p.lay.off_bits)[tile] = static_cast<uint8_t>(best.b);
+    reinterpret_cast<float*>(p.blob + p.lay.off_scale)[tile] = best.s;
+    reinterpret_cast<int32_t*>(p.blob + p.lay.off_zp)[tile] = best.zp;
+  }
+}
+
+constexpr uint32_t kListCap = 512u;  // entries of a warp's outlier list
+template <int NW>
+struct PackShared {
+  uint32_t cnt[NW];  // outliers by warp
+  uint32_t word_off, out_base;
+};
+
+// Words and outliers before row `tile`, by one warp (lane 0's result counts): the rows of its block of 32, the blocks of 32 before it in
+// its block of 1024, those of 1024 in its block of 32768, those of 32768 before it: three loads per lane, all in one round trip.
+__device__ __forceinline__ void sums_before(const EncodeParams& p, uint32_t next_turn, uint32_t tile, uint32_t lane, uint32_t* words, uint32_t* outliers) {
+  const unsigned long long* cells = p.desc + 1;
+  const uint32_t row = (tile & ~31u) + lane, g = (tile & ~1023u) + 32u * lane, q = (tile & ~32767u) + 1024u * lane;
+  unsigned long long part = 0ull, g0 = 0ull, g1 = 0ull, q0 = 0ull, q1 = 0ull;
+  if (row < tile) {
+    const uint32_t e = static_cast<uint32_t>(p.desc[2u * row]);
+    part = (static_cast<unsigned long long>(((e >> 17) & 15u) * p.lay.wpp) << 32) | (e & 0x1ffffu);
+  }
+  if (g + 31u < tile) {  // both turns' cells: which one counts arrives in the same round trip
+    g0 = cells[2u * g];
+    g1 = cells[2u * (g + 1u)];
+  }
+  if (q + 1023u < tile) {
+    q0 = cells[2u * (q + 2u)];
+    q1 = cells[2u * (q + 3u)];
+  }
+  const uint32_t turn = (next_turn & 1u) ^ 1u;
+  part += turn ? g1 + q1 : g0 + q0;
+  for (unsigned long long c = 32768ull * lane; c + 32767ull < tile; c += 32ull * 32768ull) part += cells[2u * (c + 4u + turn)];
+  *words = __reduce_add_sync(kFull, static_cast<uint32_t>(part >> 32));
+  *outliers = __reduce_add_sync(kFull, static_cast<uint32_t>(part));
+}
+
+template <bool BF16, int G, bool SV, bool FULL, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant__ EncodeParams p) {
+  using E = Elem<BF16>;
+  __shared__ PackShared<MAXT / 32> sh;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
-  __shared__ PipeShared sh;
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-  const uint32_t nt = p.compute_threads, nwarps = nt >> 5;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nt = blockDim.x, nwarps = nt >> 5;
   launch_dependents();
   wait_for_prior_grids();
-  const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
-  uint4* const xpark = reinterpret_cast<uint4*>(smem_dyn);
-  uint32_t* const planes = reinterpret_cast<uint32_t*>(smem_dyn + 3u * p.park_stride);
-  uint32_t* const csr = reinterpret_cast<uint32_t*>(smem_dyn + 3u * p.park_stride + p.ring * p.planes_stride);  // p.ring lists of p.csr_cap entries
-
-  if (tid == 0) {
-    sh.a_ready = 0u;
-    sh.lv_ready = 0u;
-    sh.packed = 0u;
-    sh.placed = 0u;
-    sh.finished = 0u;
-    sh.abort = 0u;
-    sh.stop[0] = sh.stop[1] = 0u;
-    sh.heavy_posted = 0u;
-    sh.heavy_seen[0] = sh.heavy_seen[1] = 0u;
-    {
-      const uint32_t lim = lookback_limit(p);
-      sh.wait_limit = lim > 0xffffffffu / kHandshakeFactor ? 0xffffffffu : lim * kHandshakeFactor;
+  const uint32_t tile = p.tokens - 1u - blockIdx.x;  // from the end: what sizes_kernel has read last is still in L2
+  const uint4* xrow = reinterpret_cast<const uint4*>(p.x) + static_cast<size_t>(tile) * p.chunks;
+  uint4* const park = reinterpret_cast<uint4*>(smem_dyn) + warp * (128u * G);
+  uint16_t* const list = reinterpret_cast<uint16_t*>(smem_dyn + nwarps * (2048u * G)) + warp * kListCap;
+  const uint32_t u0 = warp * (32u * G) + lane;  // the lane's group in the warp's first segment
+  {
+    uint4* dst = park + 4u * (lane >> 2) + (((lane & 3u) + (lane >> 3)) & 3u);
+    const uint32_t c0 = warp * (128u * G) + lane;
+#pragma unroll
+    for (uint32_t i = 0; i < 4u * G; ++i) {
+      if (FULL || c0 + 32u * i < p.chunks) cp_async16(dst + 32u * i, xrow + c0 + 32u * i);
     }
-    sh.next_tile[0] = atomicAdd(&p.ws->ticket, 1u);
+    cp_async_commit();
   }
-  __syncthreads();
-
-  if (tid < nt) {
-    // ================================ compute warps ================================
-    const uint32_t u = tid;  // this thread's group in every row
-    uint32_t tile_cur = sh.next_tile[0];
-    bool have_prev = false;  // row n_a - 1 has been through pass A and is not packed yet
-    uint32_t n_a = 0u;       // rows of this CTA that finished pass A; n_a - have_prev of them are packed
-    uint32_t bitmap_prev = 0u, cnt_prev = 0u, first_prev = 0u;  // outliers of the thread's group in row n_a - 1
-    uint32_t slot = 0u;      // ring slot of the next row to be packed: (rows packed so far) mod p.ring
-    uint32_t heavy_filled = 0u, heavy_done = 0u;  // rows put into / written out of the side buffer (the same in every thread)
-    // The CSR entries of the row in the side buffer, to their place in the blob: every thread takes its own group.
-    const auto emit_heavy = [&]() {
-      const uint32_t bm = sh.heavy_bm[u];
-      const uint32_t wbase = sh.heavy_wcnt[warp];
-      const uint32_t tile_h = sh.heavy_tile;
-      const uint32_t base = sh.heavy_base;
-      const uint32_t cnt = __popc(bm);
-      uint32_t incl = cnt;
+  const uint32_t next = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn_next);
+  const bool sound = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket) == 0u;
+  const uint32_t entry = static_cast<uint32_t>(p.desc[2u * tile]);
+  const float s = reinterpret_cast<const float*>(p.blob + p.lay.off_scale)[tile];
+  if (warp == nwarps - 1u) {
+    uint32_t w, o;
+    sums_before(p, next, tile, lane, &w, &o);
+    if (lane == 0) {
+      sh.word_off = w;
+      sh.out_base = o;
+    }
+  }
+  const uint32_t thr2 = p.thr16 * 0x10001u;
+  const int b = static_cast<int>((entry >> 17) & 15u);
+  const uint32_t mode = entry >> 21, row_cnt = entry & 0x1ffffu;
+  const uint32_t agg_w = static_cast<uint32_t>(b) * p.lay.wpp;
+  uint32_t x[G][16], bitmap[G];
+  cp_async_wait_all();
+  __syncwarp();
+  const uint4* own = park + 4u * lane;
+  const uint32_t rot = lane >> 1;
+#pragma unroll
+  for (uint32_t j = 0; j < 4; ++j) {
+    const uint4* from = own + ((j + rot) & 3u);
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const uint4 v = FULL || 4u * (u0 + 32u * k) + j < p.chunks ? from[128 * k] : make_uint4(0u, 0u, 0u, 0u);
+      x[k][4 * j + 0] = v.x;
+      x[k][4 * j + 1] = v.y;
+      x[k][4 * j + 2] = v.z;
+      x[k][4 * j + 3] = v.w;
+    }
+  }
+  // ---- outliers: bitmap of each group; where they are in the warp's part of the row, in order, into its list ----
+  uint32_t all = 0u;
+#pragma unroll
+  for (int k = 0; k < G; ++k) bitmap[k] = 0u;
+  const auto pattern_at = [&](int k, uint32_t e) {  // of element e of the lane's group in segment k, from the parked row
+    return static_cast<uint32_t>(reinterpret_cast<const uint16_t*>(own + 128 * k)[8u * (((e >> 3) + rot) & 3u) + (e & 7u)]);
+  };
+  if (row_cnt != 0u) {
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      uint32_t nat = 0u;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t acc = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t ta = (x[k][8 * h + i] | 0x80008000u) - thr2, tb = (x[k][8 * h + 4 + i] | 0x80008000u) - thr2;
+          acc |= top_bits4(ta, tb) & (0x01010101u << (2 * i));
+        }
+        nat |= ((acc & 0xffffu) | ((acc >> 16) << 1)) << (16 * h);
+      }
+      if (!FULL) {
+        const uint32_t u = u0 + 32u * k;
+        const uint32_t chunks = 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
+        if (chunks < 4u) nat &= (1u << (8u * chunks)) - 1u;
+      }
+      bitmap[k] = nat;
+    }
+    // how many come before the lane's in each segment, two segments to a register
+    uint32_t at[G];
+#pragma unroll
+    for (int k = 0; k < G; k += 2) {
+      const uint32_t own2 = __popc(bitmap[k]) | (k + 1 < G ? __popc(bitmap[k + 1 < G ? k + 1 : k]) << 16 : 0u);
+      uint32_t incl = own2;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t v = __shfl_up_sync(kFull, incl, d);
-        if (lane >= static_cast<uint32_t>(d)) incl += v;
+        const uint32_t up = __shfl_up_sync(kFull, incl, d);
+        if (lane >= static_cast<uint32_t>(d)) incl += up;
       }
-      if (bm != 0u) {
-        unsigned long long at = static_cast<unsigned long long>(base) + wbase + (incl - cnt);
-        const uint4* g = reinterpret_cast<const uint4*>(p.x + static_cast<size_t>(tile_h) * p.hidden) + 4u * u;
-        const uint32_t nv = FULL ? 4u : group_chunks(p, u);
-        uint4 v[4];
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) v[j] = j < nv ? g[j] : make_uint4(0u, 0u, 0u, 0u);
-        uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
-        bool overflow = false;
-        for_each_flagged(bm, v, 32u * u, [&](uint32_t entry) {
-          if (at < p.lay.outlier_capacity) {
-            o_outl[at] = entry;
-          } else {
-            overflow = true;
-          }
-          ++at;
-        });
-        if (overflow) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_OUTLIER_OVERFLOW));
-      }
-    };
-    if (tile_cur < p.tokens) fetch_group(p, xpark, tile_cur, 0u, u, FULL ? 4u : group_chunks(p, u));
-    // thread 0: the ticket of the row after tile_cur, asked for a whole iteration before it is needed
-    // (the round trip of the atomic is longer than pass A)
-    uint32_t ticket_ahead = 0xffffffffu;
-    if (tid == 0 && tile_cur < p.tokens) ticket_ahead = atomicAdd(&p.ws->ticket, 1u);
-
-    for (uint32_t it = 0u;; ++it) {
-      const bool have_cur = tile_cur < p.tokens;
-      if (!have_cur && !have_prev) break;
-      uint32_t bitmap_cur = 0u, cnt_cur = 0u, first_cur = 0u;
-      if (have_cur) {
-        // ---- pass A of row n_a: threshold split in registers, park the row, per-warp partial results ----
-        RowMeta& m = sh.meta[n_a % kMetaRing];
-        const uint32_t nvalid = FULL ? 4u : group_chunks(p, u);
-        uint32_t mn2 = E::kInfPattern * 0x10001u, mx2 = 0u;
-        uint4* xp = xpark + (n_a % 3u) * (p.park_stride / 16u);
-        cp_async_wait_all();  // this thread's own copies: nobody else touches these 64 bytes
-        uint32_t x[16];
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) {
-          const uint4 c = j < nvalid ? xp[park_index(nt, u, j)] : make_uint4(0u, 0u, 0u, 0u);
-          x[4 * j + 0] = c.x;
-          x[4 * j + 1] = c.y;
-          x[4 * j + 2] = c.z;
-          x[4 * j + 3] = c.w;
-        }
-        bitmap_cur = split_group<BF16>(x, nvalid, p.thr16 * 0x10001u, mn2, mx2);
-        cnt_cur = __popc(bitmap_cur);
-        if (bitmap_cur != 0u) {
-          // the original pattern of the group's first outlier, from the parked row while it still holds it:
-          // the CSR entry is written an iteration later, and most groups with an outlier have just one
-          const uint32_t b = static_cast<uint32_t>(__ffs(bitmap_cur) - 1);
-          first_cur = reinterpret_cast<const uint16_t*>(xp)[8u * park_index(nt, u, b >> 3) + (b & 7u)];
-        }
-        if (bitmap_cur != 0u || nvalid < 4u) {  // outlier slots become +0 (and the chunks past the end of the row)
-#pragma unroll
-          for (uint32_t j = 0; j < 4; ++j) xp[park_index(nt, u, j)] = make_uint4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
-        }
-        uint32_t mnv, mxv;
-        if (SV) {  // of the signed values of T_below instead (outlier slots are +0 by now), as order keys
-          warp_keys(signed_extremes(x, FULL ? 4u : nvalid), &mnv, &mxv);
-        } else {
-          mnv = __reduce_min_sync(kFull, min(mn2 & 0xffffu, mn2 >> 16));
-          mxv = __reduce_max_sync(kFull, max(mx2 & 0xffffu, mx2 >> 16));
-        }
-        const uint32_t wcnt = __reduce_add_sync(kFull, cnt_cur);
-        if (lane == 0) {
-          m.part.warp_min[warp] = mnv;
-          m.part.warp_max[warp] = mxv;
-          m.part.warp_cnt[warp] = wcnt;
-        }
-      }
-      if (tid == 0) {
-        if (have_cur) {
-          sh.meta[n_a % kMetaRing].tile = tile_cur;
-          sh.next_tile[(n_a + 1u) & 1u] = ticket_ahead;
-        }
-        if (have_prev) {
-          // pass B of row n_a - 1 needs its levels
-          wait_beyond(&sh.lv_ready, n_a - 1u, sh, false, 100u);
-        }
-        // The levels and placement warps may raise abort at any moment.  Thread 0 alone samples it, before the
-        // barrier, into a word that nobody else writes: every compute thread then takes the same branch.
-        sh.stop[it & 1u] = sh.abort;
-        if (heavy_filled != heavy_done) sh.heavy_seen[it & 1u] = sh.heavy_posted;
-      }
-      compute_barrier(nt);
-      if (sh.stop[it & 1u] != 0u) break;
-      if (tid == 0) {
-        __threadfence_block();
-        if (have_cur) sh.a_ready = n_a + 1u;
-        sh.packed = n_a - (have_prev ? 1u : 0u);
-        if (have_cur && ticket_ahead < p.tokens) ticket_ahead = atomicAdd(&p.ws->ticket, 1u);  // for the row after the next
-      }
-      const uint32_t tile_next = have_cur ? sh.next_tile[(n_a + 1u) & 1u] : 0xffffffffu;
-      if (tile_next < p.tokens) fetch_group(p, xpark, tile_next, (n_a + 1u) % 3u, u, FULL ? 4u : group_chunks(p, u));  // in flight during passes B and C below
-
-      if (have_prev) {
-        const uint32_t n = n_a - 1u;
-        RowMeta& m = sh.meta[n % kMetaRing];
-        const bool clamp = KIND == kKindSigned && m.divide != 0u && m.one_fma != 0.0f;  // fast steps with the clamp, as far as the first candidate
-        const bool divide = m.divide != 0u && !clamp;
-        const int bmax = p.bits[p.n_bits - 1];
-        const uint32_t tile_prev = m.tile;
-        const uint4* xp = xpark + (n % 3u) * (p.park_stride / 16u);
-        uint32_t r[8];
-        int best_ci = p.n_bits - 1;  // the chosen candidate: its level is read again where it is needed
-        int bstar = bmax;
-        const Level top = m.lv[p.n_bits - 1];
-        if (divide) {
-          // ---- a row whose scale or zero-point is outside the range of the FMA quotient and of the packed
-          //      integer steps (rare): Algorithm 1 with the division instruction, in loops that are not unrolled ----
-          const uint32_t* xw = reinterpret_cast<const uint32_t*>(xp);
-          for (int ci = p.n_bits - 2; ci >= 0; --ci) {
-            const Level low = m.lv[ci];
-            uint32_t S = rolled_distortion<BF16, SV>(xw, nt, u, top, low, bmax - p.bits[ci], 4u * (FULL ? 4u : group_chunks(p, u)));
-            S = __reduce_add_sync(kFull, S);
-            if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
-            compute_barrier(nt);
-            if (m.S[ci] > p.s_max) break;  // keep the last level that passed
-            bstar = p.bits[ci];
-            best_ci = ci;
-          }
-          const Planes8 pl = rolled_pack<BF16, SV>(xw, nt, u, m.lv[best_ci], 4u * (FULL ? 4u : group_chunks(p, u)));
-#pragma unroll
-          for (int k = 0; k < 8; ++k) r[k] = pl.v[k];
-        } else {
-          // ---- Algorithm 1, one candidate per turn.  The first turn also leaves the top-level bytes (what pass C
-          //      packs when the first lower candidate fails, the usual case, and where later turns take the
-          //      top-level codes from); every turn leaves its candidate's codes, which become the planes when
-          //      that candidate is the last to pass.  With one candidate only, the turn runs for its bytes alone. ----
-          uint32_t tb[8], lb[8];
-          int ci = p.n_bits - 2;
-          {
-            uint32_t y[16];
-#pragma unroll
-            for (uint32_t j = 0; j < 4; ++j) {
-              const uint4 c = xp[park_index(nt, u, j)];
-              y[4 * j + 0] = c.x;
-              y[4 * j + 1] = c.y;
-              y[4 * j + 2] = c.z;
-              y[4 * j + 3] = c.w;
-            }
-            if (KIND == kKind84) {
-              if (m.one_fma != 0.0f) {
-                top_bytes_one_fma<BF16>(y, pack2f(m.one_fma, m.one_fma), tb);
-              } else {
-                top_bytes<BF16>(y, make_level2(top), tb);
-              }
-            } else {
-              const int c0 = ci >= 0 ? ci : 0;
-              const Level low = m.lv[c0];
-              uint32_t S;
-              if (SV && m.one_fma != 0.0f) {
-                const uint32_t nv = FULL ? 4u : group_chunks(p, u);
-                S = clamp ? distortion_first_one_fma<BF16, true>(y, m.top_one, m.low_one, bmax - p.bits[c0], tb, lb, nv, top.qmax, low.qmax)
-                          : distortion_first_one_fma<BF16, false>(y, m.top_one, m.low_one, bmax - p.bits[c0], tb, lb, nv, top.qmax, low.qmax);
-              } else {
-                S = distortion_first<BF16, SV>(y, make_level2(top), make_level2(low), bmax - p.bits[c0], tb, lb,
-                                               (FULL || !SV) ? 4u : group_chunks(p, u));
-              }
-              if (ci >= 0) {
-                S = __reduce_add_sync(kFull, S);
-                if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
-              }
-            }
-          }
-          // pass C at the top level right away: the usual outcome, and work to do while the other warps
-          // arrive at the barrier (a row that goes lower transposes once more, below)
-          planes_of_bytes(tb, r);
-          bool passed = false;
-          if (KIND == kKind84) {
-            const uint32_t sum = __reduce_add_sync(kFull, certain_distortion_8_to_4(r));
-            if (lane == 0 && sum != 0u) atomicAdd(&m.S[ci], static_cast<int>(sum));
-            compute_barrier(nt);
-            // usually the certain differences alone exceed the tolerance; when they do not, the exact sum is formed (its
-            // codes are needed anyway if the candidate passes)
-            if (m.S[ci] <= p.s_max) {
-              uint32_t y[16];
-#pragma unroll
-              for (uint32_t j = 0; j < 4; ++j) {
-                const uint4 c = xp[park_index(nt, u, j)];
-                y[4 * j + 0] = c.x;
-                y[4 * j + 1] = c.y;
-                y[4 * j + 2] = c.z;
-                y[4 * j + 3] = c.w;
-              }
-              uint32_t S = distortion_next<BF16, false>(y, tb, make_level2(m.lv[ci]), bmax - p.bits[ci], lb);
-              S = __reduce_add_sync(kFull, S);
-              if (lane == 0 && S != 0u) atomicAdd(&m.S[kExactSlot], static_cast<int>(S));
-              compute_barrier(nt);
-              passed = m.S[kExactSlot] <= p.s_max;
-            }
-          } else if (ci >= 0) {
-            compute_barrier(nt);
-            passed = m.S[ci] <= p.s_max;
-          }
-          if (passed && clamp) {
-            // such a row that goes lower: the further candidates with the division instruction (see above)
-            bstar = p.bits[ci];
-            best_ci = ci;
-            const uint32_t* xw = reinterpret_cast<const uint32_t*>(xp);
-            for (--ci; ci >= 0; --ci) {
-              uint32_t S = rolled_distortion<BF16, SV>(xw, nt, u, top, m.lv[ci], bmax - p.bits[ci], 4u * (FULL ? 4u : group_chunks(p, u)));
-              S = __reduce_add_sync(kFull, S);
-              if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
-              compute_barrier(nt);
-              if (m.S[ci] > p.s_max) break;
-              bstar = p.bits[ci];
-              best_ci = ci;
-            }
-            const Planes8 pl = rolled_pack<BF16, SV>(xw, nt, u, m.lv[best_ci], 4u * (FULL ? 4u : group_chunks(p, u)));
-#pragma unroll
-            for (int k = 0; k < 8; ++k) r[k] = pl.v[k];
-          } else if (passed) {
-            bstar = p.bits[ci];
-            best_ci = ci;
-            for (--ci; ci >= 0; --ci) {
-              uint32_t y[16], ql[8];
-#pragma unroll
-              for (uint32_t j = 0; j < 4; ++j) {
-                const uint4 c = xp[park_index(nt, u, j)];
-                y[4 * j + 0] = c.x;
-                y[4 * j + 1] = c.y;
-                y[4 * j + 2] = c.z;
-                y[4 * j + 3] = c.w;
-              }
-              const Level low = m.lv[ci];
-              uint32_t S = distortion_next<BF16, SV>(y, tb, make_level2(low), bmax - p.bits[ci], ql,
-                                                     (FULL || !SV) ? 4u : group_chunks(p, u));
-              S = __reduce_add_sync(kFull, S);
-              if (lane == 0 && S != 0u) atomicAdd(&m.S[ci], static_cast<int>(S));
-              compute_barrier(nt);
-              if (m.S[ci] > p.s_max) break;  // keep the last level that passed
-              bstar = p.bits[ci];
-              best_ci = ci;
-#pragma unroll
-              for (int k = 0; k < 8; ++k) lb[k] = ql[k];
-            }
-            // the chosen candidate's codes with the signs of the top-level bytes
-#pragma unroll
-            for (int k = 0; k < 8; ++k) tb[k] = SV ? lb[k] : (lb[k] | (tb[k] & 0x80808080u));
-            planes_of_bytes(tb, r);
-          }
-        }
-        const uint32_t row_cnt = m.row_cnt;
-        const uint32_t agg_w = static_cast<uint32_t>(bstar) * p.lay.wpp;
-        // more outliers than the slot's list holds: into a side buffer when one is free
-        const bool to_heavy = row_cnt > p.csr_cap && heavy_filled == heavy_done;
-        if (tid == 0) {
-          // the row's sizes are known: let the rows behind it see them
-          publish_aggregate(p, gen4, tile_prev, agg_w, row_cnt);
-          m.heavy = to_heavy ? 1u : 0u;
-          m.bstar = static_cast<uint32_t>(bstar);
-          m.agg_w = agg_w;
-          m.scale = m.lv[best_ci].s;
-          m.zp = m.lv[best_ci].zp;
-        }
-        // ---- the slot that the row's planes and CSR entries go to must have been emptied by the placement of
-        //      row n - p.ring.  Every thread looks for itself, and only now: the row's sizes are published
-        //      already, so a CTA whose ring is full does not keep the rows behind it (in other CTAs) waiting
-        //      for this row's sizes on top of its own wait. ----
-        const bool slot_free = n < p.ring || wait_beyond(&sh.placed, n - p.ring, sh, false, 100u);
-        // ---- planes of the chosen level into the row's slot, in blob order ----
-        if (slot_free && (FULL || u < p.units)) store_planes<SV>(planes + slot * (p.planes_stride / 4u) + u * static_cast<uint32_t>(bstar), r, bstar, true);
-        // ---- a row with more outliers than the list holds leaves its groups' bitmaps in a side buffer, or, when
-        //      both are taken, in the list itself (it has room for at least two words per compute thread), where
-        //      the placement warp makes the entries from them ----
-        if (to_heavy) {
-          sh.heavy_bm[u] = bitmap_prev;
-          if (lane == 0) sh.heavy_wcnt[warp] = m.part.warp_cnt[warp];
-          if (tid == 0) sh.heavy_tile = tile_prev;
-          ++heavy_filled;
-        } else if (slot_free && row_cnt > p.csr_cap) {
-          csr[slot * p.csr_cap + u] = bitmap_prev;
-        }
-        // ---- CSR entries of T_above into the row's list: ascending columns, original patterns ----
-        const uint32_t flagged = __ballot_sync(kFull, cnt_prev != 0u);
-        if (flagged != 0u) {
-          uint32_t before;  // outliers in the lanes below this one
-          if (__ballot_sync(kFull, cnt_prev > 1u) == 0u) {
-            before = __popc(flagged & ((1u << lane) - 1u));  // one per flagged lane: its rank among them
-          } else {
-            uint32_t incl = cnt_prev;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-              const uint32_t v = __shfl_up_sync(kFull, incl, d);
-              if (lane >= static_cast<uint32_t>(d)) incl += v;
-            }
-            before = incl - cnt_prev;
-          }
-          if (slot_free && cnt_prev != 0u && row_cnt <= p.csr_cap) {
-            uint32_t* list = csr + slot * p.csr_cap;
-            const uint16_t* x16 = p.x + static_cast<size_t>(tile_prev) * p.hidden;
-            uint32_t at = m.part.warp_cnt[warp] + before;
-            uint32_t bm = bitmap_prev;
-            list[at++] = ((32u * u + static_cast<uint32_t>(__ffs(bm) - 1)) << 16) | first_prev;
-            bm &= bm - 1u;
-            if (__popc(bm) <= 5) {
-              while (bm != 0u) {  // further outliers of the group: read from the input again
-                const uint32_t e = 32u * u + static_cast<uint32_t>(__ffs(bm) - 1);
-                bm &= bm - 1u;
-                list[at++] = (e << 16) | x16[e];
-              }
-            } else {
-              // many: the group's 64 bytes in one round trip instead of one dependent load per outlier
-              const uint4* g = reinterpret_cast<const uint4*>(x16) + 4u * u;
-              const uint32_t nv = FULL ? 4u : group_chunks(p, u);
-              uint4 v[4];
-#pragma unroll
-              for (uint32_t j = 0; j < 4; ++j) v[j] = j < nv ? g[j] : make_uint4(0u, 0u, 0u, 0u);
-              for_each_flagged(bm, v, 32u * u, [&](uint32_t entry) { list[at++] = entry; });
-            }
-          }
-        }
-        fence_proxy_async_smem();  // the planes are about to be read by the bulk-copy engine
-        slot = slot + 1u == p.ring ? 0u : slot + 1u;
-      }
-      // the row in the side buffer, once the placement warp has posted its offset (as thread 0 saw it before this
-      // iteration's barrier).  Here, after pass C, so that the buffer is not refilled in the iteration that empties it:
-      // the next pass C comes after the next barrier.
-      if (heavy_filled != heavy_done && sh.heavy_seen[it & 1u] > heavy_done) {
-        emit_heavy();
-        ++heavy_done;
-      }
-      have_prev = have_cur;
-      bitmap_prev = bitmap_cur;
-      cnt_prev = cnt_cur;
-      first_prev = first_cur;
-      if (have_cur) ++n_a;
-      tile_cur = tile_next;
-    }
-    compute_barrier(nt);
-    if (tid == 0) {
-      __threadfence_block();
-      sh.packed = n_a - (have_prev ? 1u : 0u);  // have_prev is still set only when the loop was left by an abort
-      __threadfence_block();
-      sh.finished = 1u;
-    }
-    // rows still in the side buffers: wait for the placement warp to post their offsets
-    while (heavy_done < heavy_filled) {
-      if (tid == 0) sh.heavy_seen[0] = wait_beyond(&sh.heavy_posted, heavy_done, sh, false, 200u) ? 1u : 0u;
-      compute_barrier(nt);
-      const bool posted = sh.heavy_seen[0] != 0u;
-      if (posted) emit_heavy();
-      ++heavy_done;
-      compute_barrier(nt);  // before thread 0 writes heavy_seen[0] again
-      if (!posted) break;   // the CTA aborted
-    }
-  } else if (warp == nwarps) {
-    // ================================ levels warp ================================
-    for (uint32_t n = 0;; ++n) {
-      if (!wait_beyond(&sh.a_ready, n, sh, true, 500u)) break;
-      __threadfence_block();
-      RowMeta& m = sh.meta[n % kMetaRing];
-      const uint32_t divide = row_levels<BF16, (kPipeMaxThreads - 64) / 32, SV>(p, m.part, nwarps, lane, m.lv, m.S, &m.row_cnt, &m.lo, &m.hi);
-      __syncwarp();
-      float one = 0.0f;
-      if (KIND == kKind84) {
-        const Level top = m.lv[p.n_bits - 1];
-        float s = 0.0f;
-        if (divide == 0u) one = m.lo == 0.0f ? quick_level(m.hi, &s) : one_fma_factor<BF16>(m.lo, m.hi, top, lane);
-        if (lane == 0) m.S[kExactSlot] = 0;
-      }
-      if (KIND == kKindSigned) {
-        const int low = p.n_bits >= 2 ? p.n_bits - 2 : 0;
-        OneFma t{0.0f, 0.0f}, l{0.0f, 0.0f};
-        // a row that needs the division instruction for its clamps alone (every scale in range) may still take the one-FMA
-        // codes, with the clamp, for its first candidate
-        bool in_range = true;
-        for (int i = 0; i < p.n_bits; ++i) in_range = in_range && m.lv[i].s >= 0x1p-60f && m.lv[i].s <= 0x1p60f;
-        if (in_range) {
-          t = one_fma_signed<BF16>(m.lv[p.n_bits - 1], lane);
-          if (t.r != 0.0f) l = one_fma_signed<BF16>(m.lv[low], lane);
-        }
-        one = l.r;
-        if (lane == 0) {
-          m.top_one = t;
-          m.low_one = l;
-        }
-      }
-      if (lane == 0) {
-        m.divide = divide;
-        m.one_fma = one;
-      }
-      __syncwarp();
-      if (lane == 0) {
-        __threadfence_block();
-        sh.lv_ready = n + 1u;
+      const uint32_t sum2 = __shfl_sync(kFull, incl, 31), before2 = incl - own2;
+      at[k] = all + (before2 & 0xffffu);
+      all += sum2 & 0xffffu;
+      if (k + 1 < G) {
+        at[k + 1 < G ? k + 1 : k] = all + (before2 >> 16);
+        all += sum2 >> 16;
       }
     }
-  } else {
-    // ================================ placement warp ================================
-    uint32_t slot = 0u;  // n mod p.ring
-    for (uint32_t n = 0;; ++n, slot = slot + 1u == p.ring ? 0u : slot + 1u) {
-      if (!wait_beyond(&sh.packed, n, sh, true, 1500u)) break;
-      __threadfence_block();
-      const RowMeta& m = sh.meta[n % kMetaRing];
-      const uint32_t tile = m.tile, agg_w = m.agg_w, row_cnt = m.row_cnt;
-      // Everything the stores below need from shared memory is read before the look-back, whose round trips it then
-      // overlaps with: the token's fields (one per lane: a lone warp pays for every divergent branch, so each lane
-      // selects its field's address and value and one store serves them all) and, for the usual row, whose CSR
-      // entries number 64 at most, the entries themselves, two per lane.
-      const uint32_t heavy = m.heavy;
-      const bool short_list = heavy == 0u && row_cnt <= 64u && row_cnt <= p.csr_cap;
-      uint32_t e0 = 0u, e1 = 0u;
-      if (short_list) {
-        const uint32_t* list = csr + slot * p.csr_cap;
-        if (lane < row_cnt) e0 = list[lane];
-        if (lane + 32u < row_cnt) e1 = list[lane + 32u];
-      }
-      // lanes 1 .. 4: scale, zero-point, word_off[tile + 1], out_ptr[tile + 1]; lanes 5, 6 (first token only): the two leading zeros
-      unsigned long long field_off = 0ull;
-      uint32_t field_val = 0u;
-      bool field = false;
-      if (lane == 1u) { field_off = p.lay.off_scale + 4ull * tile; field_val = __float_as_uint(m.scale); field = true; }
-      if (lane == 2u) { field_off = p.lay.off_zp + 4ull * tile; field_val = static_cast<uint32_t>(m.zp); field = true; }
-      if (lane == 3u) { field_off = p.lay.off_word_off + 4ull * (tile + 1u); field_val = agg_w; field = true; }
-      if (lane == 4u) { field_off = p.lay.off_out_ptr + 4ull * (tile + 1u); field_val = row_cnt; field = true; }
-      if (lane == 5u && tile == 0u) { field_off = p.lay.off_word_off; field = true; }
-      if (lane == 6u && tile == 0u) { field_off = p.lay.off_out_ptr; field = true; }
-      const uint32_t bstar8 = m.bstar;
-      uint32_t word_off = 0, out_base = 0;
-      const int st = resolve_prefix<1>(p, gen4, tile, agg_w, row_cnt, lane, &word_off, &out_base, lookback_limit(p));
-      if (st != TSQ_OK) {
-        if (lane == 0) {
-          publish(p, gen4 | kFlagAbort, tile, 0u, 0u);
-          if (st > 0) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(st));
-        }
-      } else {
-        uint32_t* wdst = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
-        const uint32_t* src = planes + slot * (p.planes_stride / 4u);
-        if (p.vec_store != 0u) {
-          if (lane == 0) {
-            bulk_s2g(wdst, src, agg_w * 4u);
-            bulk_commit();
-          }
-        } else {  // runs of words that are not multiples of 16 bytes: plain stores
-          for (uint32_t w = lane; w < agg_w; w += 32) wdst[w] = src[w];
-        }
-        // the token's fields
-        if (lane == 3u) field_val += word_off;
-        if (lane == 4u) field_val += out_base;
-        if (field) *reinterpret_cast<uint32_t*>(p.blob + field_off) = field_val;
-        if (lane == 0) reinterpret_cast<uint8_t*>(p.blob + p.lay.off_bits)[tile] = static_cast<uint8_t>(bstar8);
-        if (row_cnt != 0u) {
-          uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
-          bool overflow = false;
-          if (short_list) {
-            const unsigned long long at0 = static_cast<unsigned long long>(out_base) + lane, at1 = at0 + 32ull;
-            if (lane < row_cnt) {
-              if (at0 < p.lay.outlier_capacity) {
-                o_outl[at0] = e0;
-              } else {
-                overflow = true;
-              }
-            }
-            if (lane + 32u < row_cnt) {
-              if (at1 < p.lay.outlier_capacity) {
-                o_outl[at1] = e1;
-              } else {
-                overflow = true;
-              }
-            }
-          } else if (heavy != 0u) {
-            // the compute threads write this row's entries: tell them where
-            if (lane == 0) {
-              sh.heavy_base = out_base;
-              __threadfence_block();
-              sh.heavy_posted = sh.heavy_posted + 1u;
-            }
-          } else if (row_cnt <= p.csr_cap) {
-            const uint32_t* list = csr + slot * p.csr_cap;
-            for (uint32_t i = lane; i < row_cnt; i += 32) {
-              const unsigned long long at = static_cast<unsigned long long>(out_base) + i;
-              if (at < p.lay.outlier_capacity) {
-                o_outl[at] = list[i];
-              } else {
-                overflow = true;
-              }
-            }
-          } else {
-            // more outliers than the list holds: the list holds the groups' bitmaps instead.  32 groups per turn:
-            // a scan of the counts, then every lane reads its group's 64 bytes from the input again (one round
-            // trip for the whole turn) and writes its entries
-            const uint32_t* bms = csr + slot * p.csr_cap;
-            const uint4* xrow4 = reinterpret_cast<const uint4*>(p.x + static_cast<size_t>(tile) * p.hidden);
-            unsigned long long pos = out_base;
-            for (uint32_t g0 = 0; g0 < nt; g0 += 32u) {
-              const uint32_t g = g0 + lane;
-              const uint32_t bm = bms[g];
-              const uint32_t cnt = __popc(bm);
-              uint32_t incl = cnt;
+    if (all <= kListCap) {
 #pragma unroll
-              for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t up = __shfl_up_sync(kFull, incl, d);
-                if (lane >= static_cast<uint32_t>(d)) incl += up;
-              }
-              unsigned long long at = pos + (incl - cnt);
-              pos += __shfl_sync(kFull, incl, 31);
-              if (bm != 0u) {
-                uint4 v[4];
-#pragma unroll
-                for (uint32_t j = 0; j < 4; ++j) v[j] = 4u * g + j < p.chunks ? xrow4[4u * g + j] : make_uint4(0u, 0u, 0u, 0u);
-                for_each_flagged(bm, v, 32u * g, [&](uint32_t entry) {
-                  if (at < p.lay.outlier_capacity) {
-                    o_outl[at] = entry;
-                  } else {
-                    overflow = true;
-                  }
-                  ++at;
-                });
-              }
-            }
-          }
-          if (__any_sync(kFull, overflow) && lane == 0) {
-            atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_OUTLIER_OVERFLOW));
-          }
+      for (int k = 0; k < G; ++k) {
+        for (uint32_t rest = bitmap[k], i = at[k]; rest != 0u; rest &= rest - 1u, ++i) {
+          list[i] = static_cast<uint16_t>(32u * (32u * k + lane) + static_cast<uint32_t>(__ffs(rest) - 1));
         }
-      }
-      __syncwarp();
-      if (lane == 0) {
-        // A slot may be refilled once the bulk store has read it.  The wait is for the store of the row
-        // before this one, which has had a whole row's time to finish: this row's store is left in flight
-        // and its slot is given back one row later (plain stores have read their slot already).
-        if (p.vec_store != 0u) bulk_wait_read_but_one();
-        __threadfence_block();
-        sh.placed = p.vec_store != 0u ? n : n + 1u;
       }
     }
-    if (lane == 0) bulk_wait_all();  // shared memory must outlive the stores that read it
+    __syncwarp();
+    if (lane == 0u) sh.cnt[warp] = all;
   }
-
   __syncthreads();
+  const uint32_t word_off = sh.word_off, out_base = sh.out_base, word_end = word_off + agg_w, out_end = out_base + row_cnt;
+  uint32_t status = sound && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
+  if (status == TSQ_OK) {
+    uint32_t* wrow = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
+    const uint32_t align = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(wrow));
+    const bool vec = (align & 15u) == 0u;
+    if (!SV && mode >= kOneUp) {
+      const float r = mode == kOneTried ? __frcp_rn(s) : __fmul_rn(rcp_approx(s), mode == kOneUp ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
+      const bool vec32 = b == 8 && (align & 31u) == 0u;
+      const uint64_t r2 = pack2f(r, r), magic2 = pack2f(kRoundMagicSigned + 128.0f, kRoundMagicSigned + 128.0f);
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        uint32_t tb[8], pl[8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t xa = x[k][8 * h + i], xb = x[k][8 * h + 4 + i];
+            // (an outlier's pattern has bits above the low byte: byte permutes)
+            const uint32_t c4 = __vabsdiffu4(bytes4_any(fma2(values2<BF16>(xa), r2, magic2), fma2(values2<BF16>(xb), r2, magic2)), 0x80808080u);
+            tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
+          }
+        }
+        planes_of_bytes(tb, pl);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pl[i] &= ~bitmap[k];
+        const uint32_t u = u0 + 32u * k;
+        if (FULL || u < p.units) {
+          if (vec32) {
+            store32(wrow + 8u * u, pl[7], pl[0], pl[1], pl[2], pl[3], pl[4], pl[5], pl[6]);
+          } else {
+            store_planes<false>(wrow + u * static_cast<uint32_t>(b), pl, b, vec);
+          }
+        }
+      }
+    } else {
+      Level best;
+      best.s = s;
+      best.r = __frcp_rn(s);
+      best.zp = reinterpret_cast<const int32_t*>(p.blob + p.lay.off_zp)[tile];
+      best.qmax = SV ? (1 << b) - 1 : (1 << (b - 1)) - 1;
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        const uint32_t u = u0 + 32u * k;
+        const uint32_t chunks = 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
+        uint32_t pl[8];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[k][i] &= ~E::geu_mask(x[k][i] & 0x7fff7fffu, thr2);
+        if (mode == kDivide) {
+          divide_pack_regs<BF16, SV>(x[k], best, pl);
+          if (SV && chunks < 4u) {
+            const uint32_t inside = (1u << (8u * chunks)) - 1u;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) pl[q] &= inside;
+          }
+        } else if (SV && mode == kCapped) {
+          pack_group<BF16, SV, true>(x[k], make_level2(best), pl, chunks, kRoundMagicSigned + static_cast<float>(best.zp + best.qmax));
+        } else {
+          pack_group<BF16, SV>(x[k], make_level2(best), pl, chunks);
+        }
+        if (FULL || u < p.units) store_planes<SV>(wrow + u * static_cast<uint32_t>(b), pl, b, vec);
+      }
+    }
+    if (all != 0u) {  // the warp has outliers
+      uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
+      uint32_t base = out_base + __reduce_add_sync(kFull, lane < warp ? sh.cnt[lane] : 0u);
+      if (all <= kListCap) {
+        const uint16_t* parked = reinterpret_cast<const uint16_t*>(park);
+        const uint32_t col0 = warp * (1024u * G);
+        for (uint32_t i = lane; i < all; i += 32u) {
+          const uint32_t c = list[i];  // element c & 7 of chunk (c >> 3) & 3 of group c >> 5
+          const uint32_t v = parked[(c & ~31u) + 8u * (((c >> 3) + (c >> 6)) & 3u) + (c & 7u)];
+          if (base + i < p.lay.outlier_capacity) o_outl[base + i] = (col0 + c) << 16 | v;
+        }
+      } else {  // too many for the list: each lane its own
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+          uint32_t bm = bitmap[k], pos = base, rest = bm;
+          for (uint32_t m = __ballot_sync(kFull, rest != 0u); m != 0u; m = __ballot_sync(kFull, rest != 0u)) {
+            pos += __popc(m & ((1u << lane) - 1u));
+            base += __popc(m);
+            rest &= rest - 1u;
+          }
+          const uint32_t col0 = 32u * (u0 + 32u * k);
+          for (; bm != 0u; bm &= bm - 1u, ++pos) {
+            const uint32_t e = static_cast<uint32_t>(__ffs(bm) - 1);
+            if (pos < p.lay.outlier_capacity) o_outl[pos] = (col0 + e) << 16 | pattern_at(k, e);
+          }
+        }
+      }
+    }
+  }
   if (tid == 0) {
-    if (sh.abort != 0u) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
-    finish_call(p, gen4);
+    uint32_t* o_word_off = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_word_off);
+    uint32_t* o_out_ptr = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_out_ptr);
+    if (status == TSQ_OK) {
+      if (tile == 0u) {
+        o_word_off[0] = 0u;
+        o_out_ptr[0] = 0u;
+      }
+      o_word_off[tile + 1u] = word_end;
+      o_out_ptr[tile + 1u] = out_end;
+    }
+    if (tile == p.tokens - 1u) {
+      if (status == TSQ_OK && out_end > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
+      const bool ok = status != TSQ_ERR_TIMEOUT;
+      end_part(p, status, ok ? word_end : 0u, ok ? out_end : 0u);
+      if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
+      // (the slots of this call's rows carry no tag, and the other CTAs are still reading them)
+      next_generation(p, *reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u, p.tokens);
+      p.ws->sums_turn = next;
+    }
+  }
+  // ---- the cells that the next call adds to ----
+  if (blockIdx.x < 32u) {
+    const uint32_t blocks = max(p.ws->desc_capacity, p.tokens) >> 5;
+    for (uint32_t i = blockIdx.x * nt + tid; i < blocks; i += min(gridDim.x, 32u) * nt) {
+      unsigned long long* c = p.desc + 64ull * i + 1u + 2u * (next & 1u);
+      c[0] = 0ull;
+      if ((i & 31u) == 0u) c[4] = 0ull;
+      if ((i & 1023u) == 0u) c[8] = 0ull;
+    }
   }
 }
 
 }  // namespace
 
-// The pipelined kernel is built for CTAs of up to kPipeMaxThreads threads (rows of up to 8192 elements) and may use up to 102
-// registers per thread; longer rows take encode_rows_kernel.  What bounds it is the chain of dependent instructions of an
-// iteration, so with many rows a further CTA per SM pays: the instance for those is kept to 80 registers, with which CTAs of up
-// to kPipeManyThreads threads (rows of up to 5120 elements) number three (5120) or four (4096) per SM.  Longer rows lose more
-// by the shallower ring than they gain (10000 x 6144 fp16: 93.1 us with two CTAs, 98.0 with three).
-using PipeKernel = void (*)(EncodeParams);
-template <int KIND, int MAXT, int MINB>
-static PipeKernel pipe_kernel_of(bool bf16, bool full) {
-  if (full) return bf16 ? encode_pipe_kernel<true, true, MAXT, MINB, KIND> : encode_pipe_kernel<false, true, MAXT, MINB, KIND>;
-  return bf16 ? encode_pipe_kernel<true, false, MAXT, MINB, KIND> : encode_pipe_kernel<false, false, MAXT, MINB, KIND>;
+// Only what a call can reach is built.  CTAs of up to 128 threads (rows of up to 10240 elements) get the instances of 64 to 80
+// registers, longer rows those of 256 and 512 threads.
+using EncodeKernel = void (*)(EncodeParams);
+template <int KIND, int C, int MAXT, int MINB>
+static EncodeKernel sizes_instance(bool bf16, bool full) {
+  if (full) return bf16 ? sizes_kernel<true, C, KIND, true, MAXT, MINB> : sizes_kernel<false, C, KIND, true, MAXT, MINB>;
+  return bf16 ? sizes_kernel<true, C, KIND, false, MAXT, MINB> : sizes_kernel<false, C, KIND, false, MAXT, MINB>;
 }
 template <int KIND>
-static PipeKernel pipe_kernel_of(bool bf16, bool full, bool many) {
-  return many ? pipe_kernel_of<KIND, 256, 3>(bf16, full) : pipe_kernel_of<KIND, kPipeMaxThreads, 2>(bf16, full);
+static EncodeKernel sizes_longer(bool bf16, bool full, int per_thread) {
+  if (per_thread == 16) return bf16 ? sizes_kernel<true, 16, KIND, false, 512, 1> : sizes_kernel<false, 16, KIND, false, 512, 1>;
+  return sizes_instance<KIND, 8, 256, KIND == kKind84 ? 3 : 2>(bf16, full);
 }
-static PipeKernel pipe_kernel(const EncodeParams& p, bool full, bool many, int* index) {
-  const bool bf16 = p.dtype == TSQ_BF16;
-  const int kind = p.variant != 0u ? kKindSigned : ends_in_4_and_8(p) ? kKind84 : kKindExact;
-  *index = kind * 8 + (many ? 4 : 0) + (bf16 ? 2 : 0) + (full ? 1 : 0);
-  return kind == kKindSigned ? pipe_kernel_of<kKindSigned>(bf16, full, many)
-         : kind == kKind84   ? pipe_kernel_of<kKind84>(bf16, full, many)
-                             : pipe_kernel_of<kKindExact>(bf16, full, many);
+static EncodeKernel sizes_of(const EncodeParams& p, const TwoPassShape& s) {
+  const bool bf16 = p.dtype == TSQ_BF16, full = s.sizes_full;
+  const int c = s.sizes_chunks;
+  if (p.variant != 0u) return sizes_longer<kKindSigned>(bf16, full, c);
+  if (!ends_in_4_and_8(p)) return sizes_longer<kKindExact>(bf16, full, c);
+  if (s.sizes_threads > 128) return sizes_longer<kKind84>(bf16, full, c);
+  return c == 4   ? sizes_instance<kKind84, 4, 128, 10>(bf16, full)
+         : c == 6 ? sizes_instance<kKind84, 6, 128, 8>(bf16, full)
+         : c == 8 ? sizes_instance<kKind84, 8, 128, 7>(bf16, full)
+                  : sizes_instance<kKind84, 10, 128, 6>(bf16, full);
+}
+template <bool SV, int G, int MAXT, int MINB>
+static EncodeKernel pack_instance(bool bf16, bool full) {
+  if (full) return bf16 ? pack_kernel<true, G, SV, true, MAXT, MINB> : pack_kernel<false, G, SV, true, MAXT, MINB>;
+  return bf16 ? pack_kernel<true, G, SV, false, MAXT, MINB> : pack_kernel<false, G, SV, false, MAXT, MINB>;
+}
+static EncodeKernel pack_of(const EncodeParams& p, const TwoPassShape& s) {
+  const bool bf16 = p.dtype == TSQ_BF16, full = s.pack_full, sv = p.variant != 0u;
+  if (s.pack_groups == 4) {
+    if (sv) return bf16 ? pack_kernel<true, 4, true, false, 512, 1> : pack_kernel<false, 4, true, false, 512, 1>;
+    return bf16 ? pack_kernel<true, 4, false, false, 512, 1> : pack_kernel<false, 4, false, false, 512, 1>;
+  }
+  if (sv) return pack_instance<true, 2, 256, 3>(bf16, full);
+  return s.pack_threads > 128 ? pack_instance<false, 2, 256, 3>(bf16, full) : pack_instance<false, 2, 128, 7>(bf16, full);
 }
 
-cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, bool many, int threads, size_t smem, int* blocks_per_sm) {
-  if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
-  int index = 0;
-  const void* fn = reinterpret_cast<const void*>(pipe_kernel(p, full, many && threads <= kPipeManyThreads, &index));
-  // the attribute belongs to the kernel on the current device, not to a plan: it only ever grows, so
-  // that every plan can launch
-  static std::mutex mu;
-  static size_t granted[kMaxDevices][24] = {};
-  {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(mu);
-    size_t& have = granted[dev][index];
-    if (smem > have) {
-      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-      if (e != cudaSuccess) return e;
-      have = smem;
+// Threads and elements per thread for the plan's rows.  sizes_kernel: chunks of 8 elements per thread, 8 where it makes no
+// difference, else as many as leave the fewest threads idle (5120 elements: 64 threads with 10 chunks instead of 96 with 8).  pack_kernel: 64
+// elements per thread (32: 154 us against 126 at 32768 x 4096, a row's own work is spread over too few elements).
+TwoPassShape two_pass_shape(const EncodeParams& p) {
+  TwoPassShape s{};
+  const int chunks = static_cast<int>(p.chunks), segs = static_cast<int>((p.units + 31u) / 32u);
+  const auto warps = [&](int per_thread) { return (chunks + 32 * per_thread - 1) / (32 * per_thread); };
+  if (ends_in_4_and_8(p)) {
+    for (const int c : {8, 10, 6, 4}) {
+      if (warps(c) <= 4 && (s.sizes_chunks == 0 || warps(c) * c < warps(s.sizes_chunks) * s.sizes_chunks)) s.sizes_chunks = c;
     }
   }
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
+  if (s.sizes_chunks == 0) s.sizes_chunks = warps(8) <= 8 ? 8 : 16;
+  s.sizes_threads = 32 * warps(s.sizes_chunks);
+  s.sizes_full = s.sizes_threads * s.sizes_chunks == chunks;
+  s.pack_groups = segs <= 16 ? 2 : 4;
+  const int pack_warps = (segs + s.pack_groups - 1) / s.pack_groups;
+  s.pack_threads = 32 * pack_warps;
+  s.pack_full = pack_warps * s.pack_groups * 128 == chunks;
+  s.pack_smem = static_cast<size_t>(pack_warps) * (2048u * static_cast<size_t>(s.pack_groups) + sizeof(uint16_t) * kListCap);
+  return s;
 }
 
-cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, bool many, int grid, int threads, size_t smem, cudaStream_t stream) {
-  if (threads > kPipeMaxThreads) return cudaErrorInvalidValue;
-  int index = 0;
-  return launch_overlapped(pipe_kernel(p, full, many && threads <= kPipeManyThreads, &index), grid, threads, smem, stream, p);
+cudaError_t two_pass_attrs(const EncodeParams& p, const TwoPassShape& s) {
+  if (s.pack_smem <= 48u * 1024u) return cudaSuccess;
+  // the attribute belongs to the kernel on the current device, not to a plan: always what the longest row needs
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(pack_of(p, s)), cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * (8192 + 2 * static_cast<int>(kListCap)));
+}
+
+cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, cudaStream_t stream) {
+  const int grid = static_cast<int>(p.tokens);
+  const cudaError_t e = launch_overlapped(sizes_of(p, s), grid, s.sizes_threads, 0, stream, p);
+  return e != cudaSuccess ? e : launch_overlapped(pack_of(p, s), grid, s.pack_threads, s.pack_smem, stream, p);
 }
 
 }  // namespace tsq

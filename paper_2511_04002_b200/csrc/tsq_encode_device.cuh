@@ -1,5 +1,5 @@
 // Device code shared by the encode kernels: AIQ parameters of a level, the vector passes over a 32-element group,
-// the placement look-back and the blob's header and per-token fields.  Included by one .cu file per kernel.
+// the end of a call and the blob's header and per-token fields.  Included by one .cu file per kernel.
 #ifndef TSQ_ENCODE_DEVICE_CUH_
 #define TSQ_ENCODE_DEVICE_CUH_
 
@@ -10,8 +10,7 @@ namespace tsq {
 namespace {
 
 constexpr float kRoundMagic = 8388608.0f;  // 2^23: adding it to 0 <= y < 2^23 rounds y to an integer, ties to even
-constexpr uint32_t kLookbackPollLimit = 1u << 20;  // polls of one descriptor (200 ns to 1 us apart): about a second
-constexpr uint32_t kHandshakeFactor = 4u;          // handshakes inside a CTA poll faster: four times as many polls
+constexpr uint32_t kPollLimit = 1u << 20;  // polls of one slot (a round trip to 1 us apart): about a second
 
 // AIQ parameters of one candidate level for one row (Eq. "Proposed").
 struct __align__(16) Level {
@@ -41,7 +40,7 @@ __device__ __forceinline__ Level make_level(float mmin, float mmax, int b, bool*
 // negative, a constant row takes its own magnitude as the scale.  *plain: the fast steps apply: the FMA quotient is
 // safe and no code needs a clamp (codes grow with the value, the smallest is 0 by construction, so the largest
 // value's code decides); the zero-point is then subtracted byte-wise, modulo 256.
-__device__ __forceinline__ Level make_level_signed(float vmin, float vmax, int b, bool* plain) {
+__device__ __forceinline__ Level make_level_signed(float vmin, float vmax, int b, bool* plain, bool* in_range = nullptr) {
   Level c;
   c.qmax = (1 << b) - 1;
   // two finite values of opposite sign can lie further apart than binary32 holds: the largest finite value then
@@ -50,7 +49,9 @@ __device__ __forceinline__ Level make_level_signed(float vmin, float vmax, int b
   c.s = range > 0.0f ? __fdiv_rn(range, static_cast<float>(c.qmax)) : (a > 0.0f ? a : 1.0f);
   c.zp = __float2int_rn(__fdiv_rn(vmin, c.s));
   c.r = __frcp_rn(c.s);
-  *plain = (c.s >= 0x1p-60f) && (c.s <= 0x1p60f) && (__float2int_rn(__fdiv_rn(vmax, c.s)) - c.zp <= c.qmax);
+  const bool in = (c.s >= 0x1p-60f) && (c.s <= 0x1p60f);
+  *plain = in && (__float2int_rn(__fdiv_rn(vmax, c.s)) - c.zp <= c.qmax);
+  if (in_range) *in_range = in && c.zp > -(1 << 21) && c.zp < (1 << 21);
   return c;
 }
 
@@ -205,43 +206,6 @@ __device__ __forceinline__ uint32_t distortion_group(const uint32_t (&x)[16], co
   return S;
 }
 
-// Pass B for the first lower candidate, keeping what pass C needs if that candidate fails: on return tb[4h + i]
-// holds the top-level bytes (code | sign << 7) of elements 16h + 2i, 16h + 8 + 2i, 16h + 2i + 1, 16h + 8 + 2i + 1 (pair i
-// of chunks 2h and 2h + 1, low elements first) and ql the candidate's own codes in the same grouping, no signs.
-// (Any grouping of four serves the sum; this one costs the byte assembly least, and two byte permutes per i
-// turn it into the input of the bit transpose.)
-// SV: bytes are the 8-bit codes of the signed values, no signs; bytes of chunks at and past `nvalid` are 0.
-template <bool BF16, bool SV = false>
-__device__ __forceinline__ uint32_t distortion_first(const uint32_t (&x)[16], const Level2& top, const Level2& low, int sh,
-                                                     uint32_t (&tb)[8], uint32_t (&ql)[8], uint32_t nvalid = 4u) {
-  const uint32_t shmask = ((SV ? 0xffu : 0x7fu) >> sh) * 0x01010101u;
-  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
-  uint32_t S = 0;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    // bytes 0 and 2 of a word belong to chunk 2h, bytes 1 and 3 to chunk 2h + 1
-    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];  // pairs i of chunks 2h and 2h + 1
-      if (SV) {
-        const uint32_t ct4 = codes4<BF16, true>(xa, xb, top) & inside, q4 = codes4<BF16, true>(xa, xb, low) & inside;
-        S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
-        tb[4 * h + i] = ct4;
-        ql[4 * h + i] = q4;
-        continue;
-      }
-      const uint64_t ma = magnitudes2<BF16>(xa), mb = magnitudes2<BF16>(xb);
-      const uint32_t ct4 = bytes4(quotient2(ma, top, magic2), quotient2(mb, top, magic2));
-      const uint32_t q4 = bytes4(quotient2(ma, low, magic2), quotient2(mb, low, magic2));
-      S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
-      tb[4 * h + i] = ct4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);  // the sign bits sit in bytes 1 and 3 of a pair
-      ql[4 * h + i] = q4;
-    }
-  }
-  return S;
-}
-
 // Pass B for a further candidate: the top-level codes come from the bytes the first turn left.
 template <bool BF16, bool SV = false>
 __device__ __forceinline__ uint32_t distortion_next(const uint32_t (&x)[16], const uint32_t (&tb)[8], const Level2& low, int sh,
@@ -280,93 +244,6 @@ __device__ __forceinline__ void planes_of_bytes(const uint32_t (&tb)[8], uint32_
     r[2 * i + 1] = __byte_perm(tb[i], tb[4 + i], 0x7632);  // byte c = element 8c + 2i + 1
   }
   transpose8x32_select(r);
-}
-
-// ---- signed-values variant: codes by one FMA -----------------------------------------------------------------------
-
-// A level whose codes rint(fl(v / s)) - zp one FMA gives for every 16-bit value v of the row: code = low byte of
-// fma(v, r, add), add = 2^23 + 2^22 - zp.
-struct OneFma {
-  float r, add;  // r = 0: not known to hold for the level
-};
-// Tries the 16-bit value next to each of the level's boundaries zp + k + 1/2 (between any other value and a boundary lies at
-// least half a unit of the 16-bit type, thousands of times what the two computations can differ by); run by one full warp.
-template <bool BF16>
-__device__ __forceinline__ OneFma one_fma_signed(const Level& c, uint32_t lane) {
-  const float add = kRoundMagicSigned - static_cast<float>(c.zp);
-  bool same = c.zp > -(1 << 21) && c.zp < (1 << 21);
-  for (int k = static_cast<int>(lane); k < c.qmax; k += 32) {
-    const float b = __fmul_rn(static_cast<float>(c.zp + k) + 0.5f, c.s);
-    const float v = Elem<BF16>::lo_f32(Elem<BF16>::pack_rn(b, 0.0f));
-    const float q0 = __fmul_rn(v, c.r), q = __fmaf_rn(__fmaf_rn(q0, -c.s, v), c.r, q0);
-    same = same && __fadd_rn(q, kRoundMagicSigned) - static_cast<float>(c.zp) == __fmaf_rn(v, c.r, add);
-  }
-  return OneFma{__all_sync(kFull, same) ? c.r : 0.0f, add};
-}
-
-// Patterns 2^23 + 2^22 + code: codes above qmax become qmax.
-__device__ __forceinline__ uint64_t clamp_codes2(uint64_t t, int qmax) {
-  uint32_t lo, hi;
-  unpack2u(t, lo, hi);
-  const uint32_t most = __float_as_uint(kRoundMagicSigned) + static_cast<uint32_t>(qmax);
-  return pack2u(min(lo, most), min(hi, most));
-}
-
-// distortion_first<BF16, true> with both levels' codes by one FMA.  CLAMP: the largest values' codes may be qmax + 1 and are
-// clamped (rows whose extremes both lie half-way between codes, as when both touch the threshold).
-template <bool BF16, bool CLAMP>
-__device__ __forceinline__ uint32_t distortion_first_one_fma(const uint32_t (&x)[16], const OneFma& top, const OneFma& low, int sh,
-                                                             uint32_t (&tb)[8], uint32_t (&ql)[8], uint32_t nvalid, int qtop, int qlow) {
-  const uint32_t shmask = (0xffu >> sh) * 0x01010101u;
-  const uint64_t rt = pack2f(top.r, top.r), at = pack2f(top.add, top.add), rl = pack2f(low.r, low.r), al = pack2f(low.add, low.add);
-  uint32_t S = 0;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint64_t va = values2<BF16>(x[8 * h + i]), vb = values2<BF16>(x[8 * h + 4 + i]);
-      uint64_t ta = fma2(va, rt, at), tb2 = fma2(vb, rt, at), la = fma2(va, rl, al), lb2 = fma2(vb, rl, al);
-      if (CLAMP) {
-        ta = clamp_codes2(ta, qtop);
-        tb2 = clamp_codes2(tb2, qtop);
-        la = clamp_codes2(la, qlow);
-        lb2 = clamp_codes2(lb2, qlow);
-      }
-      const uint32_t ct4 = bytes4(ta, tb2) & inside, q4 = bytes4(la, lb2) & inside;
-      S = __vsadu4((ct4 >> sh) & shmask, q4) + S;
-      tb[4 * h + i] = ct4;
-      ql[4 * h + i] = q4;
-    }
-  }
-  return S;
-}
-
-// Extremes of a group's signed values: as signed and as unsigned 16-bit patterns.
-struct SignedExtremes {
-  uint32_t smax, umax, umin;
-};
-__device__ __forceinline__ SignedExtremes signed_extremes(const uint32_t (&x)[16], uint32_t nvalid) {
-  SignedExtremes e{0x80008000u, 0u, 0xffffffffu};
-#pragma unroll
-  for (uint32_t i = 0; i < 16; i += 2) {
-    if ((i >> 2) < nvalid) {
-      e.smax = __vimax3_s16x2(e.smax, x[i], x[i + 1]);
-      e.umax = __vimax3_u16x2(e.umax, x[i], x[i + 1]);
-      e.umin = __vimin3_u16x2(e.umin, x[i], x[i + 1]);
-    }
-  }
-  return e;
-}
-// The warp's smallest and largest value as order keys (in every lane).  Patterns of non-negative values order like the values,
-// those of negative ones the other way round: the largest value is the largest signed pattern if that is non-negative, else
-// the smallest unsigned one; the smallest is the largest unsigned pattern if that is negative, else the smallest.
-__device__ __forceinline__ void warp_keys(const SignedExtremes& e, uint32_t* min_key, uint32_t* max_key) {
-  const int smax = __reduce_max_sync(kFull, max(static_cast<int>(static_cast<short>(e.smax & 0xffffu)), static_cast<int>(e.smax) >> 16));
-  const uint32_t umax = __reduce_max_sync(kFull, max(e.umax & 0xffffu, e.umax >> 16)), umin = __reduce_min_sync(kFull, min(e.umin & 0xffffu, e.umin >> 16));
-  const bool none = umin > umax;  // no value in the warp's groups
-  *max_key = none ? 0u : order_keys2(smax >= 0 ? static_cast<uint32_t>(smax) : umin) & 0xffffu;
-  *min_key = none ? 0xffffu : order_keys2(umax >= 0x8000u ? umax : umin) & 0xffffu;
 }
 
 // ---- 8-bit top level: codes by one FMA, and the distortion from the codes' bit-planes ----------------------------
@@ -458,10 +335,16 @@ __device__ __forceinline__ float quick_level(float hi, float* s_out) {
 }
 
 // Pass C on one group of a row whose chosen level is plain: codes as bytes (code | sign << 7), transposed into
-// bit-planes: on return r[k] = bit k of every byte, k < 7 code bits, k = 7 signs.
-template <bool BF16, bool SV = false>
-__device__ __forceinline__ void pack_group(const uint32_t (&x)[16], const Level2& lv, uint32_t (&r)[8], uint32_t nvalid = 4u) {
-  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
+// bit-planes: on return r[k] = bit k of every byte, k < 7 code bits, k = 7 signs.  SV with CAP: the largest value's code may be qmax + 1
+// and is clamped.
+template <bool BF16, bool SV = false, bool CAP = false>
+__device__ __forceinline__ void pack_group(const uint32_t (&x)[16], const Level2& lv, uint32_t (&r)[8], uint32_t nvalid = 4u, float cap = 0.0f) {
+  const uint64_t magic2 = SV ? pack2f(kRoundMagicSigned, kRoundMagicSigned) : pack2f(kRoundMagic, kRoundMagic);
+  const auto capped = [&](uint64_t t) {
+    float lo, hi;
+    unpack2f(t, lo, hi);
+    return pack2f(fminf(lo, cap), fminf(hi, cap));
+  };
   uint32_t tb[8];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -470,7 +353,12 @@ __device__ __forceinline__ void pack_group(const uint32_t (&x)[16], const Level2
     for (int i = 0; i < 4; ++i) {
       const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
       if (SV) {
-        tb[4 * h + i] = codes4<BF16, true>(xa, xb, lv) & inside;
+        uint64_t ta = quotient2(values2<BF16>(xa), lv, magic2), tc = quotient2(values2<BF16>(xb), lv, magic2);
+        if (CAP) {
+          ta = capped(ta);
+          tc = capped(tc);
+        }
+        tb[4 * h + i] = __vsub4(bytes4_any(ta, tc), lv.zp4) & inside;
         continue;
       }
       const uint32_t c4 = bytes4(quotient2(magnitudes2<BF16>(xa), lv, magic2), quotient2(magnitudes2<BF16>(xb), lv, magic2));
@@ -499,9 +387,6 @@ __device__ __forceinline__ uint32_t divide_distortion_regs(const uint32_t (&x)[1
   return S;
 }
 
-struct Planes8 {
-  uint32_t v[8];
-};
 template <bool BF16, bool SV = false>
 __device__ __forceinline__ void divide_pack_regs(const uint32_t (&x)[16], const Level& lv, uint32_t (&r)[8]) {
 #pragma unroll
@@ -512,84 +397,6 @@ __device__ __forceinline__ void divide_pack_regs(const uint32_t (&x)[16], const 
     const uint32_t b2 = codes2_divide<BF16, SV>(x[i], lv) | (SV ? 0u : ((x[i] >> 8) & 0x00800080u));
 #pragma unroll
     for (int k = 0; k < 8; ++k) r[k] |= (((b2 >> k) & 1u) << (2 * i)) | (((b2 >> (16 + k)) & 1u) << (2 * i + 1));
-  }
-}
-
-// The same two steps for rows that need the division instruction, written as loops over the parked
-// row's words (xw: the row as 32-bit words) so that they take little room in the instruction stream.
-__device__ __forceinline__ uint32_t park_index(uint32_t nt, uint32_t u, uint32_t j);
-// (SV: only the first `pairs` words, the ones inside the row, count: see divide_distortion_regs.)
-template <bool BF16, bool SV = false>
-__device__ __noinline__ uint32_t rolled_distortion(const uint32_t* xw, uint32_t nt, uint32_t u, Level top, Level low, int sh,
-                                                   uint32_t pairs = 16u) {
-  const uint32_t shmask = (0xffffu >> sh) * 0x10001u;
-  uint32_t S = 0;
-#pragma unroll 1
-  for (uint32_t i = 0; i < (SV ? pairs : 16u); ++i) {
-    const uint32_t x = xw[4u * park_index(nt, u, i >> 2) + (i & 3u)];
-    const uint32_t a = (codes2_divide<BF16, SV>(x, top) >> sh) & shmask;
-    const uint32_t q = codes2_divide<BF16, SV>(x, low);
-    const uint32_t d = max_s16x2(a, q) - min_s16x2(a, q);
-    S += (d & 0xffffu) + (d >> 16);
-  }
-  return S;
-}
-template <bool BF16, bool SV = false>
-__device__ __noinline__ Planes8 rolled_pack(const uint32_t* xw, uint32_t nt, uint32_t u, Level lv, uint32_t pairs = 16u) {
-  uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // r[k] bit e = bit k of the byte (code | sign << 7; SV: the 8-bit code) of element e
-#pragma unroll 1
-  for (uint32_t i = 0; i < (SV ? pairs : 16u); ++i) {
-    const uint32_t x = xw[4u * park_index(nt, u, i >> 2) + (i & 3u)];
-    // elements 2i (byte 0) and 2i + 1 (byte 2)
-    const uint32_t b2 = codes2_divide<BF16, SV>(x, lv) | (SV ? 0u : ((x >> 8) & 0x00800080u));
-#pragma unroll
-    for (int k = 0; k < 8; ++k) r[k] |= (((b2 >> k) & 1u) << (2u * i)) | (((b2 >> (16 + k)) & 1u) << (2u * i + 1u));
-  }
-  Planes8 out;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) out.v[k] = r[k];
-  return out;
-}
-
-// Shared-memory index (in 16-byte chunks) of chunk j of group u inside a parked row of nt groups: a group's
-// four chunks stay together, rotated so that the 16-byte accesses of neighbouring threads fall into
-// different banks.  (Keeping the chunks with the same j side by side instead measured 8 % slower while the
-// copies bypassed L1, and no faster than this since they do not.)
-__device__ __forceinline__ uint32_t park_index(uint32_t /*nt*/, uint32_t u, uint32_t j) { return 4u * u + ((j + (u >> 1)) & 3u); }
-
-// Number of 16-byte chunks of group u that lie inside the row (4, fewer in the last group, 0 beyond it).
-// Recomputed where it is needed: a value kept alive across the whole row loop costs a register there.
-__device__ __forceinline__ uint32_t group_chunks(const EncodeParams& p, uint32_t u) {
-  return 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
-}
-
-// Asynchronous copy of the 64 bytes of group u of row `tile` into parked row `slot` (chunks
-// j >= nvalid lie past the end of the row and are not copied).
-__device__ __forceinline__ void fetch_group(const EncodeParams& p, uint4* xpark, uint32_t tile, uint32_t slot, uint32_t u,
-                                            uint32_t nvalid) {
-  const uint4* xrow = reinterpret_cast<const uint4*>(p.x + static_cast<size_t>(tile) * p.hidden);
-  uint4* xp = xpark + slot * (p.park_stride / 16u);
-#pragma unroll
-  for (uint32_t j = 0; j < 4; ++j) {
-    if (j < nvalid) cp_async16(&xp[park_index(p.compute_threads, u, j)], &xrow[4u * u + j]);
-  }
-  cp_async_commit();
-}
-
-// The CSR entries (column << 16 | original pattern) of the elements of one group that `bm` flags, in
-// ascending column order, from the group's 64 bytes as they stand in the input (v[j] = chunk j): f(entry) is
-// called once per flagged element.  All 32 positions are visited under a predicate: no data-dependent loads.
-template <typename F>
-__device__ __forceinline__ void for_each_flagged(uint32_t bm, const uint4 (&v)[4], uint32_t col0, F&& f) {
-#pragma unroll
-  for (uint32_t j = 0; j < 4; ++j) {
-    const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
-#pragma unroll
-    for (uint32_t i = 0; i < 4; ++i) {
-      const uint32_t e = 8u * j + 2u * i;
-      if ((bm >> e) & 1u) f(((col0 + e) << 16) | (w[i] & 0xffffu));
-      if ((bm >> (e + 1u)) & 1u) f(((col0 + e + 1u) << 16) | (w[i] >> 16));
-    }
   }
 }
 
@@ -668,123 +475,13 @@ __device__ __forceinline__ uint32_t row_levels(const EncodeParams& p, RowPartial
 }
 
 // The limit on device-side waits: the workspace's setting, else the built-in one.
-__device__ __forceinline__ uint32_t lookback_limit(const EncodeParams& p) {
+__device__ __forceinline__ uint32_t poll_limit_of(const EncodeParams& p) {
   const uint32_t set = *reinterpret_cast<volatile const uint32_t*>(&p.ws->poll_limit);
-  return set != 0u ? set : kLookbackPollLimit;
+  return set != 0u ? set : kPollLimit;
 }
 
 __device__ __forceinline__ unsigned long long pack_desc(uint32_t tag, uint32_t value) {
   return (static_cast<unsigned long long>(tag) << 32) | value;
-}
-
-// Decoupled look-back over the tile descriptors.
-// Tile t owns two adjacent descriptors, desc[2t] for plane words and desc[2t + 1] for outliers, each
-// (generation * 4 + flag) << 32 | payload: an AGGREGATE payload is the tile's own size, a PREFIX
-// payload the inclusive prefix sum up to and including the tile.  Both are read in the same round
-// trip; a tile counts as published once both carry the same flag of the current generation.
-__device__ __forceinline__ void publish(const EncodeParams& p, uint32_t tag, uint32_t tile, uint32_t w, uint32_t o) {
-  st_relaxed_u64(p.desc + 2 * static_cast<size_t>(tile), pack_desc(tag, w));
-  st_relaxed_u64(p.desc + 2 * static_cast<size_t>(tile) + 1, pack_desc(tag, o));
-}
-
-__device__ __forceinline__ void publish_aggregate(const EncodeParams& p, uint32_t gen4, uint32_t tile, uint32_t agg_w,
-                                                  uint32_t agg_o) {
-  if (tile > 0) publish(p, gen4 | kFlagAggregate, tile, agg_w, agg_o);
-}
-
-// State of a tile from its two descriptors: 0 = not (consistently) published yet, else the common flag.
-__device__ __forceinline__ uint32_t tile_state(uint32_t gen4, unsigned long long vw, unsigned long long vo) {
-  const uint32_t tw = static_cast<uint32_t>(vw >> 32), to = static_cast<uint32_t>(vo >> 32);
-  const uint32_t fw = ((tw & ~3u) == gen4) ? (tw & 3u) : 0u, fo = ((to & ~3u) == gen4) ? (to & 3u) : 0u;
-  if (fw == kFlagAbort || fo == kFlagAbort) return kFlagAbort;
-  return fw == fo ? fw : 0u;
-}
-
-// Run by one full warp for its tile, after publish_aggregate: walk back to the nearest published
-// prefix, then publish this tile's own.
-// Returns TSQ_OK, TSQ_ERR_TIMEOUT (gave up) or -1 when a predecessor has aborted.
-// DEPTH = descriptor pairs each lane reads per step (32 * DEPTH tiles per round trip).  The one-CTA-per-row
-// kernel, whose rows all finish at about the same time, looks back 256 tiles at once; the pipelined
-// kernel, where the nearest finished prefix is rarely more than a few dozen tiles away and the look-back
-// runs in a lone warp that issues slowly, takes 32 (measured: 6 % faster at hidden 8192 and 20 % at
-// 1024 than with 256).
-template <int DEPTH>
-__device__ int resolve_prefix(const EncodeParams& p, uint32_t gen4, uint32_t tile, uint32_t agg_w, uint32_t agg_o,
-                              uint32_t lane, uint32_t* excl_w, uint32_t* excl_o, uint32_t poll_limit) {
-  uint32_t base_w = 0, base_o = 0;  // prefix found at the end of the walk
-  uint32_t part_w = 0, part_o = 0;  // this lane's share of the aggregates walked over
-  if (tile > 0) {
-    int pos = static_cast<int>(tile) - 1;  // nearest tile not yet accounted for
-    uint32_t polls = 0;
-    bool done = false;
-    while (!done) {
-      unsigned long long vw[DEPTH], vo[DEPTH];
-#pragma unroll
-      for (int k = 0; k < DEPTH; ++k) {
-        const int j = pos - (32 * k + static_cast<int>(lane));
-        // before tile 0: prefix 0
-        vw[k] = vo[k] = pack_desc(gen4 | kFlagPrefix, 0u);
-        if (j >= 0) ld_relaxed_u64x2(p.desc + 2 * static_cast<size_t>(j), vw[k], vo[k]);
-      }
-      int consumed = 32 * DEPTH;
-      bool stopped = false;
-      int verdict = TSQ_OK;
-#pragma unroll
-      for (int k = 0; k < DEPTH; ++k) {
-        if (stopped) continue;
-        // the usual window: 32 aggregates
-        const uint32_t agg_tag = gen4 | kFlagAggregate;
-        if (__all_sync(kFull, static_cast<uint32_t>(vw[k] >> 32) == agg_tag && static_cast<uint32_t>(vo[k] >> 32) == agg_tag)) {
-          part_w += static_cast<uint32_t>(vw[k]);
-          part_o += static_cast<uint32_t>(vo[k]);
-          continue;
-        }
-        const uint32_t state = tile_state(gen4, vw[k], vo[k]);
-        const uint32_t stop = __ballot_sync(kFull, state != kFlagAggregate);
-        const uint32_t first = stop ? static_cast<uint32_t>(__ffs(stop) - 1) : 32u;
-        if (lane < first) {
-          part_w += static_cast<uint32_t>(vw[k]);
-          part_o += static_cast<uint32_t>(vo[k]);
-        }
-        if (stop == 0u) continue;
-        stopped = true;
-        const uint32_t first_state = __shfl_sync(kFull, state, first);
-        if (first_state == kFlagAbort) {
-          verdict = -1;
-        } else if (first_state == kFlagPrefix) {
-          base_w = __shfl_sync(kFull, static_cast<uint32_t>(vw[k]), first);
-          base_o = __shfl_sync(kFull, static_cast<uint32_t>(vo[k]), first);
-          done = true;
-        } else {  // not published yet: keep what was walked over, poll again from there
-          consumed = 32 * k + static_cast<int>(first);
-        }
-      }
-      if (verdict != TSQ_OK) return verdict;
-      if (!done) {
-        pos -= consumed;
-        if (consumed == 0) {
-          // tile `pos` has published nothing yet: watch its two descriptors alone until it has
-          for (;;) {
-            uint32_t state = 0u;
-            if (lane == 0) {
-              unsigned long long w0, w1;
-              ld_relaxed_u64x2(p.desc + 2 * static_cast<size_t>(pos), w0, w1);
-              state = tile_state(gen4, w0, w1);
-            }
-            if (__shfl_sync(kFull, state, 0) != 0u) break;
-            if (++polls > poll_limit) return TSQ_ERR_TIMEOUT;
-            __nanosleep(polls < 32u ? 200u : 1000u);
-          }
-        }
-      }
-    }
-    base_w += __reduce_add_sync(kFull, part_w);
-    base_o += __reduce_add_sync(kFull, part_o);
-  }
-  if (lane == 0) publish(p, gen4 | kFlagPrefix, tile, base_w + agg_w, base_o + agg_o);
-  *excl_w = base_w;
-  *excl_o = base_o;
-  return TSQ_OK;
 }
 
 __device__ void write_header(const EncodeParams& p, unsigned long long total_words, unsigned long long total_outliers) {
@@ -819,53 +516,46 @@ __device__ void end_part(const EncodeParams& p, uint32_t status, unsigned long l
   }
 }
 
-// The CTA that finishes last publishes the totals and the status, and re-arms the workspace.  `direct`: the descriptors
-// are those of a call without look-back (encode_rows_kernel), which comes here only when it has no rows or the generation wraps.
-__device__ void finish_call(const EncodeParams& p, uint32_t gen4, bool direct = false) {
+// The generation of the call that ends; after the last one they start over, and the slots from `first` on are wiped so that old tags
+// cannot alias.
+__device__ void next_generation(const EncodeParams& p, uint32_t g, uint32_t first) {
+  if (g >= kGenWrap) {
+    const uint32_t n = max(p.ws->desc_capacity, p.tokens);
+    for (uint32_t i = first; i < n; ++i) p.desc[2ull * i] = 0ull;
+    p.ws->direct_state = 0u;
+    g = 0u;
+  }
+  p.ws->gen = g;
+}
+
+// Ends a call of encode_rows_kernel that its last row's CTA does not end: one without rows, or one whose generation is the last before they
+// start over.  The CTA that finishes last publishes the totals and the status, and re-arms the workspace.
+__device__ void finish_call(const EncodeParams& p, uint32_t gen4) {
   __threadfence();
   const uint32_t prev = atomicAdd(&p.ws->done, 1u);
   if (prev != gridDim.x - 1u) return;
   __threadfence();
-  uint32_t e = atomicExch(&p.ws->err, 0u);
-  // totals = the last tile's inclusive prefixes, if it got that far
+  uint32_t e = *reinterpret_cast<volatile const uint32_t*>(&p.ws->direct_state) == (gen4 | kWaitRanOut) ? TSQ_ERR_TIMEOUT : TSQ_OK;
   unsigned long long tw = 0ull, to = 0ull;
-  if (direct) {
-    if (*reinterpret_cast<volatile const uint32_t*>(&p.ws->direct_state) == (gen4 | kWaitRanOut)) e = TSQ_ERR_TIMEOUT;
-    for (uint32_t i = 0; i < p.tokens; ++i) {
-      const uint32_t v = static_cast<uint32_t>(ld_relaxed_u64(p.desc + i));
-      tw += v >> 17;
-      to += v & 0x1ffffu;
-    }
-    if (e == 0u && to > p.lay.outlier_capacity) e = TSQ_ERR_OUTLIER_OVERFLOW;
-  } else if (p.tokens != 0u) {
-    const unsigned long long dw = ld_relaxed_u64(p.desc + 2 * static_cast<size_t>(p.tokens - 1u));
-    const unsigned long long dout = ld_relaxed_u64(p.desc + 2 * static_cast<size_t>(p.tokens - 1u) + 1);
-    if (tile_state(gen4, dw, dout) == kFlagPrefix) {
-      tw = static_cast<uint32_t>(dw);
-      to = static_cast<uint32_t>(dout);
-    }
+  for (uint32_t i = 0; i < p.tokens; ++i) {
+    const uint32_t v = static_cast<uint32_t>(ld_relaxed_u64(p.desc + 2ull * i));
+    tw += v >> 17;
+    to += v & 0x1ffffu;
   }
   if (p.chained != 0u) {
     tw += reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_word_off)[0];
     to += reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_out_ptr)[0];
   }
+  if (e == TSQ_OK && to > p.lay.outlier_capacity) e = TSQ_ERR_OUTLIER_OVERFLOW;
   end_part(p, e, tw, to);
   if (p.tokens == 0u) {  // no row writes the leading zeros of the two prefix-sum sections
     reinterpret_cast<uint32_t*>(p.blob + p.lay.off_word_off)[0] = 0u;
     reinterpret_cast<uint32_t*>(p.blob + p.lay.off_out_ptr)[0] = 0u;
   }
-  if (e != 0u) atomicCAS(&p.ws->enc_status, 0u, e);
-  uint32_t g = (gen4 >> 2);
-  if (g >= kGenWrap) {
-    // generation counter about to wrap: wipe the descriptors so that old tags cannot alias
-    const uint32_t n = p.ws->desc_capacity;
-    for (uint32_t i = 0; i < 2u * n; ++i) p.desc[i] = 0ull;
-    p.ws->direct_state = 0u;
-    g = 0u;
-  }
+  if (e != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, e);
   p.ws->ticket = 0u;
   p.ws->done = 0u;
-  p.ws->gen = g;
+  next_generation(p, gen4 >> 2, 0u);
 }
 
 // The per-token fields of the blob, written by one thread.

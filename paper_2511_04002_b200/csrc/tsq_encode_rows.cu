@@ -9,7 +9,7 @@ namespace {
 // =====================================================================================================
 
 // EncodeParams::direct_tiles
-constexpr int kLookBack = 0, kByIndex = 1, kByTicket = 2;
+constexpr int kByIndex = 1, kByTicket = 2;
 
 struct RowShared {
   Level lv[kMaxCand];  // lv[i]: AIQ parameters of candidate bits[i]
@@ -19,8 +19,6 @@ struct RowShared {
   uint32_t tile;
   uint32_t divide;     // some level of the row needs the division instruction
   uint32_t row_cnt;    // outliers of the row
-  uint32_t word_off, out_base;
-  uint32_t status;     // TSQ_OK, or why the row is not written
   uint32_t warp_w[32], warp_o[32], warp_status[32];  // direct_offsets: by warp
 };
 
@@ -51,16 +49,16 @@ __device__ __forceinline__ bool given_up(const EncodeParams& p, uint32_t gen4, u
 constexpr uint32_t kPollBatch = 4u;
 template <bool BATCHES>
 __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared& sh) {
-  const uint32_t limit = lookback_limit(p), tag = gen4 | kFlagAggregate;
+  const uint32_t limit = poll_limit_of(p), tag = gen4 | kFlagAggregate;
   uint32_t w = 0u, o = 0u, status = TSQ_OK;
   uint32_t i = threadIdx.x;
   for (; BATCHES && i + (kPollBatch - 1u) * blockDim.x < tile; i += kPollBatch * blockDim.x) {  // many rows: their loads in one round trip
     unsigned long long v[kPollBatch];
 #pragma unroll
-    for (uint32_t k = 0; k < kPollBatch; ++k) v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x);
+    for (uint32_t k = 0; k < kPollBatch; ++k) v[k] = ld_relaxed_u64(p.desc + 2ull * (i + k * blockDim.x));
 #pragma unroll
     for (uint32_t k = 0; k < kPollBatch; ++k) {
-      for (uint32_t polls = 0; static_cast<uint32_t>(v[k] >> 32) != tag; v[k] = ld_relaxed_u64(p.desc + i + k * blockDim.x)) {
+      for (uint32_t polls = 0; static_cast<uint32_t>(v[k] >> 32) != tag; v[k] = ld_relaxed_u64(p.desc + 2ull * (i + k * blockDim.x))) {
         if (given_up(p, gen4, ++polls, limit)) {
           status = TSQ_ERR_TIMEOUT;
           break;
@@ -71,8 +69,8 @@ __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t g
     }
   }
   for (; i < tile; i += blockDim.x) {
-    unsigned long long v = ld_relaxed_u64(p.desc + i);
-    for (uint32_t polls = 0; static_cast<uint32_t>(v >> 32) != tag; v = ld_relaxed_u64(p.desc + i)) {
+    unsigned long long v = ld_relaxed_u64(p.desc + 2ull * i);
+    for (uint32_t polls = 0; static_cast<uint32_t>(v >> 32) != tag; v = ld_relaxed_u64(p.desc + 2ull * i)) {
       if (given_up(p, gen4, ++polls, limit)) {
         status = TSQ_ERR_TIMEOUT;
         break;
@@ -122,7 +120,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
   wait_for_prior_grids();
   const uint32_t gen4 = (*reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u) << 2;
   uint32_t part_w = 0u, part_o = 0u;  // where a later part of a call starts
-  if (DIRECT != kLookBack && p.chained != 0u) {
+  if (p.chained != 0u) {
     part_w = *reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_word_off);
     part_o = *reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_out_ptr);
     // never past the planes, whatever a part that has failed has left there
@@ -132,10 +130,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
 
   uint32_t tile = blockIdx.x;
   if (DIRECT != kByIndex) {
-    if (tid == 0) {
-      sh.tile = atomicAdd(&p.ws->ticket, 1u);
-      sh.status = TSQ_OK;
-    }
+    if (tid == 0) sh.tile = atomicAdd(&p.ws->ticket, 1u);
     __syncthreads();
     tile = sh.tile;
   }
@@ -327,13 +322,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
     const uint32_t agg_w = static_cast<uint32_t>(bstar) * p.lay.wpp;
 
     // ---- this row's sizes are known: let the rows behind it see them, then pack ----
-    if (tid == 0) {
-      if (DIRECT) {
-        st_relaxed_u64(p.desc + tile, pack_desc(gen4 | kFlagAggregate, agg_w << 17 | row_cnt));
-      } else {
-        publish_aggregate(p, gen4, tile, agg_w, row_cnt);
-      }
-    }
+    if (tid == 0) st_relaxed_u64(p.desc + 2ull * tile, pack_desc(gen4 | kFlagAggregate, agg_w << 17 | row_cnt));
 #pragma unroll
     for (int k = 0; k < UPT; ++k) {
       if (settled) continue;
@@ -350,34 +339,15 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
     }
 
     // ---- placement: exclusive prefix sums over the tokens before this one ----
-    if (DIRECT) {
-      direct_offsets<DIRECT == kByTicket>(p, gen4, tile, sh);
-    } else if (warp == 0) {
-      uint32_t word_off = 0, out_base = 0;
-      const int st = resolve_prefix<8>(p, gen4, tile, agg_w, row_cnt, lane, &word_off, &out_base, lookback_limit(p));
-      if (lane == 0) {
-        sh.word_off = word_off;
-        sh.out_base = out_base;
-        if (st != TSQ_OK) {
-          publish(p, gen4 | kFlagAbort, tile, 0u, 0u);
-          sh.status = st < 0 ? 0xffffffffu : static_cast<uint32_t>(st);
-          if (st > 0) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(st));
-        }
-      }
-    }
+    direct_offsets<DIRECT == kByTicket>(p, gen4, tile, sh);
     __syncthreads();
-    uint32_t word_off = sh.word_off, out_base = sh.out_base, status = sh.status;
-    if (DIRECT) {
-      word_off = part_w;
-      out_base = part_o;
-      status = 0u;
-      for (uint32_t w = 0; w < nwarps; ++w) {
-        word_off += sh.warp_w[w];
-        out_base += sh.warp_o[w];
-        status |= sh.warp_status[w];
-      }
-      if (tile == p.tokens - 1u && tid == blockDim.x - 1u && (gen4 >> 2) < kGenWrap) finish_direct(p, gen4, status, word_off + agg_w, out_base + row_cnt);
+    uint32_t word_off = part_w, out_base = part_o, status = TSQ_OK;
+    for (uint32_t w = 0; w < nwarps; ++w) {
+      word_off += sh.warp_w[w];
+      out_base += sh.warp_o[w];
+      status |= sh.warp_status[w];
     }
+    if (tile == p.tokens - 1u && tid == blockDim.x - 1u && (gen4 >> 2) < kGenWrap) finish_direct(p, gen4, status, word_off + agg_w, out_base + row_cnt);
 
     if (status == TSQ_OK) {
       // ---- plane words: group u owns words u * b* .. u * b* + b* - 1 ----
@@ -400,7 +370,6 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
           uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
           const uint16_t* x16 = p.x + static_cast<size_t>(tile) * p.hidden;
           unsigned long long at = static_cast<unsigned long long>(out_base) + cnt_before + (incl - cnt);
-          bool overflow = false;
 #pragma unroll
           for (int k = 0; k < UPT; ++k) {
             uint32_t bm = bitmap[k];
@@ -408,40 +377,32 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
             while (bm != 0u) {
               const uint32_t e = 32u * u + static_cast<uint32_t>(__ffs(bm) - 1);
               bm &= bm - 1u;
-              if (at < p.lay.outlier_capacity) {
-                o_outl[at] = (e << 16) | x16[e];
-              } else {
-                overflow = true;
-              }
+              if (at < p.lay.outlier_capacity) o_outl[at] = (e << 16) | x16[e];  // (finish_direct reports what does not fit)
               ++at;
             }
           }
-          if (overflow && !DIRECT) atomicCAS(&p.ws->err, 0u, static_cast<uint32_t>(TSQ_ERR_OUTLIER_OVERFLOW));
         }
       }
     }
   }
 
-  if (DIRECT && p.tokens != 0u && (gen4 >> 2) < kGenWrap) return;  // (no last row to end a call without rows)
+  if (p.tokens != 0u && (gen4 >> 2) < kGenWrap) return;  // (no last row to end a call without rows)
   __syncthreads();
-  if (tid == 0) finish_call(p, gen4, DIRECT);
+  if (tid == 0) finish_call(p, gen4);
 }
 
 }  // namespace
 
-// Only what a call can reach is built: rows of up to 8192 elements never take the look-back (their longer calls are the pipelined
-// kernel's), and the instances of 80 and 64 registers are for calls by ticket of the magnitude variant.
+// Only what a call can reach is built: the instances of 80 and 64 registers are for calls by ticket of the magnitude variant.
 using RowsKernel = void (*)(EncodeParams);
 template <bool SV, bool TOP84, int DIRECT>
 static RowsKernel rows_kernel_of(bool bf16, int threads, int upt, int dense) {
-  if constexpr (DIRECT != kLookBack) {
-    if (upt == 1 && threads <= 256) {
-      if constexpr (DIRECT == kByTicket && !SV) {
-        if (dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
-        if (dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
-      }
-      return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
+  if (upt == 1 && threads <= 256) {
+    if constexpr (DIRECT == kByTicket && !SV) {
+      if (dense == 1) return bf16 ? encode_rows_kernel<true, 1, 256, 3, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 3, SV, TOP84, DIRECT>;
+      if (dense == 2) return bf16 ? encode_rows_kernel<true, 1, 256, 4, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 4, SV, TOP84, DIRECT>;
     }
+    return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
   }
   if (upt == 1) return bf16 ? encode_rows_kernel<true, 1, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, 1, SV, false, DIRECT>;
   return bf16 ? encode_rows_kernel<true, 2, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, 1, SV, false, DIRECT>;
@@ -461,9 +422,7 @@ cudaError_t encode_rows_attrs(const EncodeParams& p, int threads, int upt, int d
 }
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, int dense, cudaStream_t stream) {
-  const RowsKernel fn = p.direct_tiles == kByIndex    ? rows_kernel<kByIndex>(p, threads, upt, dense)
-                        : p.direct_tiles == kByTicket ? rows_kernel<kByTicket>(p, threads, upt, dense)
-                                                      : rows_kernel<kLookBack>(p, threads, upt, dense);
+  const RowsKernel fn = p.direct_tiles == kByIndex ? rows_kernel<kByIndex>(p, threads, upt, dense) : rows_kernel<kByTicket>(p, threads, upt, dense);
   return launch_overlapped(fn, grid, threads, 0, stream, p);
 }
 

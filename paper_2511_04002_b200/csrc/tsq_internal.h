@@ -14,11 +14,8 @@ constexpr uint32_t kMagic = 0x31515354u;  // 'T','S','Q','1'
 constexpr uint32_t kVersion = 1u;
 constexpr int kMaxCand = 7;
 constexpr int kMaxThreads = 256;          // decoder: threads per CTA, one 32-element unit per thread per pass
-constexpr int kPipeMaxThreads = 320;      // pipelined encoder: compute threads (<= 256 groups) + two service warps
-constexpr int kPipeManyThreads = 224;     // longest CTA of its instance for calls of many rows
 constexpr int kMaxDevices = 64;           // devices per process that the library keeps per-device state for
-constexpr int kMaxRing = 8;               // pipelined encoder: most rows a CTA holds between packing and placement
-constexpr int kEncMaxThreads = 1024;      // encoder: one CTA per row, one or two 32-element groups per thread
+constexpr int kEncMaxThreads = 1024;      // one-kernel encoder: one CTA per row, one or two 32-element groups per thread
 
 struct BlobHeader {
   uint32_t magic, version, dtype, hidden, tokens, n_bits;
@@ -57,9 +54,14 @@ __host__ __device__ inline BlobLayout make_layout(uint32_t hidden, unsigned long
   return L;
 }
 
-// Workspace: a 64-byte control block and two adjacent 64-bit descriptors per token (plane words,
-// outliers).  A descriptor is (tag << 32) | value with tag = generation * 4 + flag; stale
-// generations read as "not yet published", so the array never needs clearing between calls.
+// Workspace: a 64-byte control block and, per token t, two adjacent 64-bit words:
+//   desc[2 t]      the slot of row t.  Calls of one kernel: (tag << 32) | plane words << 17 | outliers, tag = generation * 4 + flag; stale
+//                  generations read as "not yet published", so nothing needs clearing between calls.  Calls of two kernels:
+//                  outliers | bits << 17 | mode << 21, upper half 0 (no tag: generations start at 1).
+//   desc[2 t + 1]  cells of calls of two kernels: plane words << 32 | outliers of a whole block of rows, two of each, used in turn.  Block of 32
+//                  rows that starts at row t: cells t and t + 1; of 1024 rows: t + 2, t + 3; of 32768 rows: t + 4, t + 5.  A call
+//                  adds to the cells of its turn, which the call before it has left at 0, and clears those of the other.
+// (Where a word is does not depend on the number of tokens, so a workspace may serve plans of different sizes.)
 struct WsControl {
   uint32_t gen;          // generation of the last finished encode
   uint32_t ticket;       // next tile to hand out (self-resetting)
@@ -70,11 +72,13 @@ struct WsControl {
   uint32_t desc_capacity;  // tiles the descriptor array holds (set by init)
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
   uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut or kCallEnded, only ever grows
-  uint32_t pad[7];
+  uint32_t sums_turn;      // calls of two kernels: whose turn the cells are, read by the first and written by the second kernel
+  uint32_t sums_turn_next; // the same for the next call, written by the first kernel and read by the second
+  uint32_t pad[5];
 };
 static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
 
-constexpr uint32_t kFlagAggregate = 1, kFlagPrefix = 2, kFlagAbort = 3;
+constexpr uint32_t kFlagAggregate = 1;
 constexpr uint32_t kWaitRanOut = 1, kCallEnded = 2;  // direct_state
 constexpr uint32_t kGenWrap = (1u << 30) - 2;
 
@@ -82,7 +86,7 @@ struct EncodeParams {
   const uint16_t* x;
   unsigned char* blob;
   WsControl* ws;
-  unsigned long long* desc;                  // [2 * max_tokens] tile descriptors
+  unsigned long long* desc;                  // [2 * max_tokens] slots and cells
   BlobLayout lay;
   uint32_t tokens, hidden, units, chunks;   // units = ceil(H/32), chunks = H/8
   uint32_t thr16;                            // smallest non-negative 16-bit pattern with value >= tau
@@ -90,10 +94,7 @@ struct EncodeParams {
   int32_t bits[8];
   int32_t s_max;                             // floor(delta * H), clamped to [-1, INT32_MAX]
   uint32_t vec_store;                        // 1: every token's plane words start on a 16-byte boundary
-  uint32_t direct_tiles;                     // one-CTA-per-row kernel: 0 = look-back, 1 = direct offsets and row index = CTA index
-                                             // (every CTA resident), 2 = direct offsets, rows by ticket
-  // pipelined kernel only: thread split, shared-memory strides (bytes; csr_cap in entries), ring depth in rows
-  uint32_t compute_threads, park_stride, planes_stride, csr_cap, ring;
+  uint32_t direct_tiles;                     // one-kernel encoder: 1 = row index = CTA index (every CTA resident), 2 = rows by ticket
   uint32_t dtype;
   uint32_t variant;                          // 0: sign + magnitude codes; 1: codes of the signed values
   float tau, delta;
@@ -142,8 +143,16 @@ cudaError_t launch_overlapped(void (*kernel)(Args...), int grid, int threads, si
 
 cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int upt, int dense, cudaStream_t stream);
 cudaError_t encode_rows_attrs(const EncodeParams& p, int threads, int upt, int dense, int* blocks_per_sm);
-cudaError_t launch_encode_pipe(const EncodeParams& p, bool full, bool many, int grid, int threads, size_t smem, cudaStream_t stream);
-cudaError_t encode_pipe_attrs(const EncodeParams& p, bool full, bool many, int threads, size_t smem, int* blocks_per_sm);
+// The two-kernel encoder: threads, chunks of 8 elements per thread (sizes) and 32-element groups per thread (pack); full: no thread
+// has a short or missing share.
+struct TwoPassShape {
+  int sizes_threads, sizes_chunks, pack_threads, pack_groups;
+  bool sizes_full, pack_full;
+  size_t pack_smem;
+};
+TwoPassShape two_pass_shape(const EncodeParams& p);
+cudaError_t two_pass_attrs(const EncodeParams& p, const TwoPassShape& s);
+cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeParams& p, int grid, int threads, size_t smem, cudaStream_t stream);
 cudaError_t decode_kernel_attrs(bool bf16, int threads, size_t smem, int* blocks_per_sm);
 size_t decode_smem_bytes(uint32_t row_bytes);
