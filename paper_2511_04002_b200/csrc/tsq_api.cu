@@ -405,7 +405,6 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
   p.n_bits = plan->n_bits;
   for (int i = 0; i < 8; ++i) p.bits[i] = plan->bits[i];
   p.s_max = plan->s_max;
-  p.vec_store = (plan->units % 4u == 0u) ? 1u : 0u;
   p.dtype = static_cast<uint32_t>(plan->dtype);
   p.variant = plan->variant;
   p.tau = plan->tau;
@@ -416,21 +415,30 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 }
 
 // Rows up to which a call goes through one kernel, whose rows read the sizes of the rows before them directly, instead of two.  The
-// second kernel costs a launch and a second read of the input; in the one kernel every row waits for the slowest row before it, and
-// the more rows do not fit at once the more that costs.  us, one kernel / two, each pair on the same tensors (n: normal values with 0.1 %
-// outliers, n0: none, n1: 1 %, t3: Student-t nu = 3 with 0.1 %, t4: nu = 4 with 16 outlier channels):
-//   up to 2048 elements  1042 x 1976 fp16, 8 outlier channels  11.6 / 12.6                     2048 x 1024 bf16 t3  14.9 / 11.9
-//   up to 5120            300 x 4096 fp16 n   7.8 / 11.0     600 x 4096 bf16 n   10.1 / 11.4    777 x 3000 bf16 n   11.4 / 12.5
-//                        1000 x 4096 fp16 n0 13.8 / 13.7    1500 x 4096 fp16 n1 18.0 / 14.5   2048 x 5120 fp16 t4  29.8 / 24.1
-//   up to 8192            300 x 8192 bf16 t3  9.4 / 9.7      600 x 8192 fp16 n   13.2 / 12.4   1000 x 8192 fp16 t4  22.1 / 14.6
-//   longer                300 x 12288 fp16 n 12.9 / 12.6     600 x 12288 fp16 n  19.8 / 13.7    600 x 16384 fp16 t4 26.0 / 17.5
-//   signed values          64 x 4096 fp16 n  12.6 / 8.6      300 x 4096 fp16 n   20.9 / 12.0    600 x 5120 fp16 t4  35.6 / 17.0
+// second kernel costs a launch and a second read of the input; in the one kernel every row waits for the slowest row before it, which
+// is cheap while all rows are in flight at once (rows_ctas) and they are few enough to read each other's sizes (8 per SM).  us, one kernel /
+// two, each pair on the same tensors (n: normal values with 0.1 % outliers, n0: none, t3: Student-t nu = 3 with 0.1 %, t4: nu = 4 with 16
+// outlier channels):
+//   up to 2048 elements  1042 x 1976 fp16, 8 channels  9.4 / 11.5    1184 x 1024 bf16 t3   9.1 / 10.2    1500 x 1024 fp16 n   13.6 / 10.7
+//   up to 5120            300 x 4096 fp16 n            7.7 / 9.0      777 x 3000 bf16 n   10.2 / 12.4    1000 x 4096 fp16 n0  13.2 / 13.6
+//                        1500 x 4096 fp16 n1          18.0 / 14.5    2048 x 5120 fp16 t4  29.8 / 22.0
+//   up to 8192            300 x 8192 bf16 t3           9.1 / 9.9      600 x 8192 fp16 n   11.8 / 12.8    1000 x 8192 fp16 t4  22.1 / 14.8
+//   longer                300 x 12288 fp16 n          11.2 / 13.5     600 x 12288 fp16 n  19.8 / 13.7     600 x 16384 fp16 t4 26.0 / 17.5
+//   signed values          64 x 4096 fp16 n           12.6 / 8.6      300 x 4096 fp16 n   20.9 / 10.4     600 x 5120 fp16 t4  35.6 / 17.0
 // (Signed values: one row in ten has a code that needs the clamp, which the one kernel forms by the division instruction; 1 x 4096 4.1 / 7.4.)
 static int64_t direct_rows(const tsq_plan_t* plan) {
-  const int64_t sms = plan->sms;
   if (plan->variant != 0u) return 8;
-  if (plan->enc_upt > 1 || plan->enc_threads > 256) return 2 * sms;
-  return (plan->enc_threads <= 64 ? 8 : plan->enc_threads <= 160 ? 6 : 4) * sms;
+  const int64_t at_once = static_cast<int64_t>(plan->sms) * std::min(std::max(plan->rows_ctas[2], 1), 8);
+  return at_once + at_once / 16;  // (a sixteenth of a turn more does not count)
+}
+
+// Rows up to which the second of the two kernels takes 32 elements per thread instead of 64, for rows of up to 5120 elements: more warps share
+// a row while they do not fill the device several times over, and rows of one segment of 1024 elements leave half of the wider threads
+// idle.  us, 32 / 64 elements: 300 x 4096 9.0 / 9.9, 2048 x 4096 16.3 / 16.4, 2048 x 5120 22.0 / 22.6, 4096 x 4096 28.4 / 27.3, 8192 x 4096 45.6 / 40.4,
+// 8192 x 1024 22.5 / 24.0, 1000 x 8192 16.8 / 14.8.
+static bool few_rows(const tsq_plan_t* plan, int64_t tokens) {
+  const int64_t segments = (plan->units + 31u) / 32u;
+  return segments <= 5 && (segments == 1 || tokens * segments <= 80 * static_cast<int64_t>(plan->sms));
 }
 
 // Instance of the one-kernel encoder: 128, 80 or 64 registers, so more CTAs per SM with each.  The one
@@ -456,7 +464,7 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
   if (args_ok != TSQ_OK) return args_ok;
   EncodeParams p = encode_params(plan, x_dev, tokens, blob_dev, ws_dev);
   if (tokens > direct_rows(plan)) {
-    const cudaError_t e = launch_encode_two_pass(p, plan->two_pass, static_cast<cudaStream_t>(cuda_stream));
+    const cudaError_t e = launch_encode_two_pass(p, plan->two_pass, few_rows(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
     g_launches.fetch_add(2);
     return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
   }

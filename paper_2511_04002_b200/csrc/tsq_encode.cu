@@ -47,14 +47,6 @@ constexpr int kKind84 = 0;      // magnitudes, candidates end in 4 and 8 bits: b
 constexpr int kKindExact = 1;   // any other candidates of the magnitudes: exact sums
 constexpr int kKindSigned = 2;  // signed values: exact sums
 
-// How pack_kernel forms a row's codes
-constexpr uint32_t kDivide = 0;    // by the division instruction
-constexpr uint32_t kPlain = 1;     // three-operation quotient
-constexpr uint32_t kOneUp = 2;     // one FMA, factor 1/s moved up (half the largest magnitude rounds up), zero-point 0
-constexpr uint32_t kOneDown = 3;   // one FMA, factor 1/s moved down
-constexpr uint32_t kOneTried = 4;  // one FMA with fl(1/s), tried out against every boundary
-constexpr uint32_t kCapped = 5;    // signed values: three-operation quotient, the largest value's code clamped
-
 // A row's size in its slot: outliers | bits << 17 | mode << 21 (the upper half stays 0: no tag of a direct call)
 __device__ __forceinline__ unsigned long long row_entry(uint32_t outliers, int b, uint32_t mode) {
   return outliers | static_cast<uint32_t>(b) << 17 | mode << 21;
@@ -68,37 +60,6 @@ __device__ __forceinline__ uint4 load_once(const uint4* p) {
   asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void store32(uint32_t* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f, uint32_t g, uint32_t h) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h) : "memory");
-}
-// top bits of the halves of ta, tb as bytes 0xff / 0: a.lo, b.lo, a.hi, b.hi
-__device__ __forceinline__ uint32_t top_bits4(uint32_t ta, uint32_t tb) {
-  uint32_t r;
-  asm("prmt.b32 %0, %1, %2, 0xfbd9;" : "=r"(r) : "r"(ta), "r"(tb));
-  return r;
-}
-// min(|x|, m) of the two elements of a pair
-template <bool BF16>
-__device__ __forceinline__ uint32_t min_abs2(uint32_t x, uint32_t m) {
-  uint32_t r;
-  if (BF16) {
-    asm("{.reg .b32 t; abs.bf16x2 t, %1; min.bf16x2 %0, t, %2;}" : "=r"(r) : "r"(x), "r"(m));
-  } else {
-    asm("{.reg .b32 t; abs.f16x2 t, %1; min.f16x2 %0, t, %2;}" : "=r"(r) : "r"(x), "r"(m));
-  }
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2_rm(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 template <int NW>
 struct __align__(16) SizesShared {
   static constexpr int kSlots = NW < 4 ? 4 : NW;
@@ -191,45 +152,6 @@ __device__ __noinline__ RowChoice settle_exactly(const EncodeParams& p, const ui
   return best;
 }
 
-// hi / Q, correctly rounded for every 16-bit hi (as in quick_level); *tie: Q divides hi's significand.
-template <int Q>
-__device__ __forceinline__ float divide_by(float hi, bool* tie) {
-  constexpr float kInv = 1.0f / static_cast<float>(Q);
-  const float q0 = __fmul_rn(hi, kInv), s = __fmaf_rn(__fmaf_rn(-static_cast<float>(Q), q0, hi), kInv, q0);
-  *tie = __fmaf_rn(-static_cast<float>(Q), s, hi) == 0.0f;
-  return s;
-}
-// Whether rint(fl((hi / 2) / s)) is the upper of the two codes that hi / 2 lies between (k and k + 1, k + 1/2 = Q / 2): the quotient
-// rounds to k + 1/2 or more iff (hi / 2) - (k + 1/2) s (exact) is not below -2^-half s, half an ulp below k + 1/2; ties go to
-// k + 1 there (k = 63, 3 and 1 are odd).
-__device__ __forceinline__ bool middle_up(float hi, float s, float middle, float half) { return __fmaf_rn(-middle, s, 0.5f * hi) >= -half * s; }
-
-// The distortion sum between the 8-bit level and a lower one, for rows with zero-point 0, without forming codes.  In ideal arithmetic the lower
-// level (Q codes above 0) rounds y = Q m / range up at y = k + 1/2 and q >> sh steps at y = (2^sh j - 1/2) Q / 127; both are even about Q / 2, and
-// with v = |y - Q / 2| they lie at v = k and at v = k / ratio, ratio = 127 / (2^sh Q), k = 1, 2, ...  So the difference of an element is 1 between
-// k / ratio and k and 0 elsewhere: with w = y - Q / 2 it is floor(ratio w) - floor(w), negative for w < 0.  kMargin moves both steps inwards, further
-// than the rounding of all of this and of the codes goes: the sum is a lower bound, and exact but for elements that lie next to a step.
-constexpr float kMargin = 0x1p-19f;
-struct Steps {
-  uint64_t per2, mid2, ratio2, one2;
-};
-__device__ __forceinline__ Steps steps_of(float q, float ratio, float range) {
-  const float c = q * rcp_approx(range), ka = ratio - kMargin * ratio, kb = 1.0f + kMargin;
-  return Steps{pack2f(c, c), pack2f(-0.5f * q, -0.5f * q), pack2f(ka, ka), pack2f(kb, kb)};
-}
-template <bool BF16>
-__device__ __forceinline__ uint64_t add_differences(uint32_t x, uint32_t hi2, const Steps& t, uint64_t acc) {
-  const uint64_t magic2 = pack2f(kRoundMagicSigned, kRoundMagicSigned), neg2 = pack2f(-1.0f, -1.0f);
-  const uint64_t w = fma2(values2<BF16>(min_abs2<BF16>(x, hi2)), t.per2, t.mid2);  // an outlier counts as hi: 0
-  const uint64_t d = fma2(fma2_rm(w, t.one2, magic2), neg2, fma2_rm(w, t.ratio2, magic2));
-  return fma2(d, d, acc);
-}
-__device__ __forceinline__ int sum_of(uint64_t acc) {
-  float a, b;
-  unpack2f(acc, a, b);
-  return __float2int_rn(a + b);
-}
-
 // The same sum over a row's chunks read again, for a further candidate.
 template <bool BF16, int C, int NW>
 __device__ __noinline__ int sum_again(const EncodeParams& p, const uint4* xrow, uint32_t hi2, float q, float ratio, float range, uint32_t turn, SizesShared<NW>& sh) {
@@ -252,23 +174,6 @@ __device__ __noinline__ int sum_again(const EncodeParams& p, const uint4* xrow, 
   return cta_sum(sh, sum_of(acc), turn, nwarps);
 }
 
-// By the whole warp: the 16-bit magnitude next to each step (one per lane), and by how much the sum is off for an element of that magnitude.
-template <bool BF16>
-__device__ __forceinline__ int step_error(float q, float ratio, float range, int sh, uint32_t lane, uint32_t* pattern) {
-  using E = Elem<BF16>;
-  const uint32_t k = lane & 15u;
-  const bool of_low = lane < 16u;
-  const float at = (of_low ? static_cast<float>(k) + 0.5f : (static_cast<float>((k + 1u) << sh) - 0.5f) * q * (1.0f / 127.0f)) / q * range;
-  *pattern = E::pack_rn(at, 0.0f) & 0xffffu;
-  const float m = E::pattern_f32(*pattern);
-  const bool middle_again = !of_low && static_cast<float>(2u * k + 1u) == q;  // both have a step there
-  if (static_cast<float>(k) >= q || middle_again || fabsf(m - at) > 0x1p-14f * at) return 0;
-  const int code = __float2int_rn(__fdiv_rn(m, __fdiv_rn(range, 127.0f))), low = __float2int_rn(__fdiv_rn(m, __fdiv_rn(range, q)));
-  const float w = __fmaf_rn(m, q * rcp_approx(range), -0.5f * q);
-  const float d = __fmaf_rd(w, ratio - kMargin * ratio, kRoundMagicSigned) - __fmaf_rd(w, 1.0f + kMargin, kRoundMagicSigned);
-  return abs((code >> sh) - low) - static_cast<int>(fabsf(d));
-}
-
 template <bool BF16, int C, int KIND, bool FULL, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
@@ -286,7 +191,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
   wait_for_prior_grids();
   const uint32_t tile = blockIdx.x;
   const uint4* xrow = reinterpret_cast<const uint4*>(p.x) + static_cast<size_t>(tile) * p.chunks;
-  uint32_t x[C][4];
+  uint32_t x[4 * C];
   uint32_t nv = FULL ? C : 0u;
 #pragma unroll
   for (uint32_t j = 0; j < C; ++j) {
@@ -296,10 +201,10 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
       c = load_once(xrow + idx);
       if (!FULL) nv = j + 1u;
     }
-    x[j][0] = c.x;
-    x[j][1] = c.y;
-    x[j][2] = c.z;
-    x[j][3] = c.w;
+    x[4 * j + 0] = c.x;
+    x[4 * j + 1] = c.y;
+    x[4 * j + 2] = c.z;
+    x[4 * j + 3] = c.w;
   }
   const uint32_t turn = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn) & 1u;
   if (tile == 0u && tid == 0u) p.ws->sums_turn_next = turn ^ 1u;
@@ -315,7 +220,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
       const uint32_t in = FULL ? 0xffffffffu : (j < static_cast<int>(nv) ? 0x00ff00ffu : 0u) | (j + 1 < static_cast<int>(nv) ? 0xff00ff00u : 0u);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t ta = (x[j][i] | 0x80008000u) - thr2, tb = (x[j + 1][i] | 0x80008000u) - thr2;
+        const uint32_t ta = (x[4 * j + i] | 0x80008000u) - thr2, tb = (x[4 * j + 4 + i] | 0x80008000u) - thr2;
         mxt = __vimax3_s16x2(mxt, ta, tb);
         if (FULL) {
           mnt = __vimin3_u16x2(mnt, ta, tb);
@@ -341,11 +246,11 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
       const uint32_t in = (in_a ? 0x00ff00ffu : 0u) | (in_b ? 0xff00ff00u : 0u);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t f = top_bits4((x[j][i] | 0x80008000u) - thr2, (x[j + 1][i] | 0x80008000u) - thr2) & in;
+        const uint32_t f = top_bits4((x[4 * j + i] | 0x80008000u) - thr2, (x[4 * j + 4 + i] | 0x80008000u) - thr2) & in;
         c1 = __dp4a(static_cast<int>(f), static_cast<int>(f), c1);
-        x[j][i] &= ~__byte_perm(f, 0u, 0x2200);
-        x[j + 1][i] &= ~__byte_perm(f, 0u, 0x3311);
-        const uint32_t va = SV ? x[j][i] : x[j][i] & 0x7fff7fffu, vb = SV ? x[j + 1][i] : x[j + 1][i] & 0x7fff7fffu;
+        x[4 * j + i] &= ~__byte_perm(f, 0u, 0x2200);
+        x[4 * j + 4 + i] &= ~__byte_perm(f, 0u, 0x3311);
+        const uint32_t va = SV ? x[4 * j + i] : x[4 * j + i] & 0x7fff7fffu, vb = SV ? x[4 * j + 4 + i] : x[4 * j + 4 + i] & 0x7fff7fffu;
         if (in_a) {  // (a row's chunks end with those of a thread: b inside means a inside)
           const uint32_t v2 = in_b ? vb : va;
           if (SV) smax = __vimax3_s16x2(smax, va, v2);
@@ -393,76 +298,30 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
     pmin = row_cnt != 0u ? 0u : (pmin + p.thr16) & 0x7fffu;
     pmax = mxr < 0 ? 0u : (pmax + p.thr16) & 0x7fffu;
     const float lo = E::pattern_f32(pmin), hi = E::pattern_f32(pmax), range = hi - lo;
-    if (hi >= 0x1p-50f && hi <= 0x1p60f && 256.0f * lo <= hi) {
+    if (steps_apply(lo, hi)) {
       const uint32_t hi2 = pmax * 0x10001u;
-      int S;
-      {
-        const Steps t = steps_of(7.0f, 127.0f / 112.0f, range);
-        uint64_t acc = 0ull;
+      const Steps t = steps_of(7.0f, 127.0f / 112.0f, range);
+      uint64_t acc = 0ull;
 #pragma unroll
-        for (int j = 0; j < C; ++j) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) acc = add_differences<BF16>(x[j][i], hi2, t, acc);
-        }
-        S = cta_sum(sh, sum_of(acc), 0u, nwarps);
-      }
+      for (int i = 0; i < 4 * C; ++i) acc = add_differences<BF16>(x[i], hi2, t, acc);
+      const int S = cta_sum(sh, sum_of(acc), 0u, nwarps);
       best.b = 8;
-      if (S <= p.s_max) {  // the 4-bit candidate may pass: exact sums from here on, candidate by candidate
+      if (S <= p.s_max) {  // the 4-bit candidate may pass (3 to 7 % of the rows)
         uint32_t turn_of_sum = 1u;
-#pragma unroll 1
-        for (int ci = p.n_bits - 2; ci >= 0; --ci) {
-          const int b = p.bits[ci];
-          const float q = static_cast<float>((1 << (b - 1)) - 1), ratio = b == 4 ? 127.0f / 112.0f : b == 3 ? 127.0f / 96.0f : 127.0f / 64.0f;
-          if (b == 3) {
-            S = sum_again<BF16, C>(p, xrow, hi2, q, ratio, range, turn_of_sum, sh);
-            turn_of_sum ^= 1u;
-          }
-          if (b == 2) S = 0;  // (one step for both, in the middle)
-          uint32_t pattern;
-          const int error = step_error<BF16>(q, ratio, range, 8 - b, lane, &pattern);
-#pragma unroll 1
-          for (uint32_t open = __ballot_sync(kFull, error != 0); open != 0u; open &= open - 1u) {
-            const int l = __ffs(open) - 1;
-            const uint32_t m2 = __shfl_sync(kFull, pattern, l) * 0x10001u;
-            uint32_t same = 0u;  // minus the elements of that magnitude, by half
-#pragma unroll
-            for (int j = 0; j < C; ++j) {
-#pragma unroll
-              for (int i = 0; i < 4; ++i) same = __vadd2(same, E::eq_mask(x[j][i] & 0x7fff7fffu, m2));
-            }
-            const int n = -(static_cast<int>(static_cast<short>(same & 0xffffu)) + (static_cast<int>(same) >> 16));
-            S += __shfl_sync(kFull, error, l) * cta_sum(sh, n, turn_of_sum, nwarps);
-            turn_of_sum ^= 1u;
-          }
-          if (S > p.s_max) break;  // keep the last level that passed
-          best.b = b;
-        }
+        best.b = descend<BF16>(
+            p, x, range, S,
+            [&](int v) {
+              const int sum = cta_sum(sh, v, turn_of_sum, nwarps);
+              turn_of_sum ^= 1u;
+              return sum;
+            },
+            [&](float q, float ratio) {
+              const int sum = sum_again<BF16, C>(p, xrow, hi2, q, ratio, range, turn_of_sum, sh);
+              turn_of_sum ^= 1u;
+              return sum;
+            });
       }
-      if (best.b != 0 && warp == 0u) {
-        const int b = best.b;
-        if (pmin == 0u && b == 8) {
-          bool tie;
-          best.s = divide_by<127>(hi, &tie);
-          if (!tie) best.mode = middle_up(hi, best.s, 63.5f, 0x1p-19f) ? kOneUp : kOneDown;
-        } else if (pmin == 0u) {
-          bool tie = false;
-          best.s = b == 4 ? divide_by<7>(hi, &tie) : b == 3 ? divide_by<3>(hi, &tie) : hi;
-          const bool up = b == 4 ? middle_up(hi, best.s, 3.5f, 0x1p-23f) : b == 3 ? middle_up(hi, best.s, 1.5f, 0x1p-24f) : false;
-          if (!tie || b == 2) best.mode = up ? kOneUp : kOneDown;
-        } else {
-          const float q = static_cast<float>((1 << (b - 1)) - 1);
-          best.s = __fdiv_rn(range, q);
-          const float r = __frcp_rn(best.s);
-          bool same = true;
-#pragma unroll 1
-          for (uint32_t i = lane; i < static_cast<uint32_t>(q); i += 32u) {
-            const float m = E::lo_f32(E::pack_rn(__fmul_rn(static_cast<float>(i) + 0.5f, best.s), 0.0f));
-            const float q0 = __fmul_rn(m, r), qt = __fmaf_rn(__fmaf_rn(q0, -best.s, m), r, q0);
-            same = same && __fadd_rn(qt, kRoundMagic) == __fmaf_rn(m, r, kRoundMagic);
-          }
-          if (__all_sync(kFull, same)) best.mode = kOneTried;
-        }
-      }
+      if (warp == 0u) best.s = scale_of<BF16>(lo, hi, best.b, lane, &best.mode);
     }
   }
   if (KIND != kKind84) {
@@ -495,7 +354,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
         for (int j = 0; j < C; ++j) {
           if (j < static_cast<int>(nv)) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) same = __vadd2(same, E::eq_mask(x[j][i], m2));
+            for (int i = 0; i < 4; ++i) same = __vadd2(same, E::eq_mask(x[4 * j + i], m2));
           }
         }
         n_largest = cta_sum(sh, -(static_cast<int>(static_cast<short>(same & 0xffffu)) + (static_cast<int>(same) >> 16)), static_cast<uint32_t>(p.n_bits - 1) & 1u, nwarps);
@@ -509,7 +368,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
         for (int j = 0; j < C; j += 4) {
           uint32_t g[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) g[i] = x[j + i / 4][i & 3];
+          for (int i = 0; i < 16; ++i) g[i] = x[4 * j + i];
           const int left = static_cast<int>(nv) - j;
           sum += distortion_group<BF16, SV>(g, make_level2(top), make_level2(low), shn, FULL ? 4u : left <= 0 ? 0u : static_cast<uint32_t>(min(left, 4)));
         }
@@ -636,17 +495,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   if (row_cnt != 0u) {
 #pragma unroll
     for (int k = 0; k < G; ++k) {
-      uint32_t nat = 0u;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t acc = 0u;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t ta = (x[k][8 * h + i] | 0x80008000u) - thr2, tb = (x[k][8 * h + 4 + i] | 0x80008000u) - thr2;
-          acc |= top_bits4(ta, tb) & (0x01010101u << (2 * i));
-        }
-        nat |= ((acc & 0xffffu) | ((acc >> 16) << 1)) << (16 * h);
-      }
+      uint32_t nat = outliers_of(x[k], thr2);
       if (!FULL) {
         const uint32_t u = u0 + 32u * k;
         const uint32_t chunks = 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
@@ -689,36 +538,14 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   uint32_t status = sound && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
   if (status == TSQ_OK) {
     uint32_t* wrow = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
-    const uint32_t align = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(wrow));
-    const bool vec = (align & 15u) == 0u;
     if (!SV && mode >= kOneUp) {
-      const float r = mode == kOneTried ? __frcp_rn(s) : __fmul_rn(rcp_approx(s), mode == kOneUp ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
-      const bool vec32 = b == 8 && (align & 31u) == 0u;
-      const uint64_t r2 = pack2f(r, r), magic2 = pack2f(kRoundMagicSigned + 128.0f, kRoundMagicSigned + 128.0f);
+      const float r = one_fma_factor(s, mode);
 #pragma unroll
       for (int k = 0; k < G; ++k) {
-        uint32_t tb[8], pl[8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint32_t xa = x[k][8 * h + i], xb = x[k][8 * h + 4 + i];
-            // (an outlier's pattern has bits above the low byte: byte permutes)
-            const uint32_t c4 = __vabsdiffu4(bytes4_any(fma2(values2<BF16>(xa), r2, magic2), fma2(values2<BF16>(xb), r2, magic2)), 0x80808080u);
-            tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
-          }
-        }
-        planes_of_bytes(tb, pl);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) pl[i] &= ~bitmap[k];
+        uint32_t pl[8];
+        planes_by_one_fma<BF16>(x[k], pack2f(r, r), bitmap[k], pl);
         const uint32_t u = u0 + 32u * k;
-        if (FULL || u < p.units) {
-          if (vec32) {
-            store32(wrow + 8u * u, pl[7], pl[0], pl[1], pl[2], pl[3], pl[4], pl[5], pl[6]);
-          } else {
-            store_planes<false>(wrow + u * static_cast<uint32_t>(b), pl, b, vec);
-          }
-        }
+        if (FULL || u < p.units) store_planes<false>(wrow, u, pl, b);
       }
     } else {
       Level best;
@@ -745,7 +572,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
         } else {
           pack_group<BF16, SV>(x[k], make_level2(best), pl, chunks);
         }
-        if (FULL || u < p.units) store_planes<SV>(wrow + u * static_cast<uint32_t>(b), pl, b, vec);
+        if (FULL || u < p.units) store_planes<SV>(wrow, u, pl, b);
       }
     }
     if (all != 0u) {  // the warp has outliers
@@ -754,6 +581,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (all <= kListCap) {
         const uint16_t* parked = reinterpret_cast<const uint16_t*>(park);
         const uint32_t col0 = warp * (1024u * G);
+#pragma unroll 2
         for (uint32_t i = lane; i < all; i += 32u) {
           const uint32_t c = list[i];  // element c & 7 of chunk (c >> 3) & 3 of group c >> 5
           const uint32_t v = parked[(c & ~31u) + 8u * (((c >> 3) + (c >> 6)) & 3u) + (c & 7u)];
@@ -841,19 +669,20 @@ static EncodeKernel pack_instance(bool bf16, bool full) {
   if (full) return bf16 ? pack_kernel<true, G, SV, true, MAXT, MINB> : pack_kernel<false, G, SV, true, MAXT, MINB>;
   return bf16 ? pack_kernel<true, G, SV, false, MAXT, MINB> : pack_kernel<false, G, SV, false, MAXT, MINB>;
 }
-static EncodeKernel pack_of(const EncodeParams& p, const TwoPassShape& s) {
-  const bool bf16 = p.dtype == TSQ_BF16, full = s.pack_full, sv = p.variant != 0u;
-  if (s.pack_groups == 4) {
+static EncodeKernel pack_of(const EncodeParams& p, const PackShape& s) {
+  const bool bf16 = p.dtype == TSQ_BF16, full = s.full, sv = p.variant != 0u;
+  if (s.groups == 4) {
     if (sv) return bf16 ? pack_kernel<true, 4, true, false, 512, 1> : pack_kernel<false, 4, true, false, 512, 1>;
     return bf16 ? pack_kernel<true, 4, false, false, 512, 1> : pack_kernel<false, 4, false, false, 512, 1>;
   }
+  if (s.groups == 1) return sv ? pack_instance<true, 1, 256, 4>(bf16, full) : pack_instance<false, 1, 256, 5>(bf16, full);
   if (sv) return pack_instance<true, 2, 256, 3>(bf16, full);
-  return s.pack_threads > 128 ? pack_instance<false, 2, 256, 3>(bf16, full) : pack_instance<false, 2, 128, 7>(bf16, full);
+  return s.threads > 128 ? pack_instance<false, 2, 256, 3>(bf16, full) : pack_instance<false, 2, 128, 7>(bf16, full);
 }
 
 // Threads and elements per thread for the plan's rows.  sizes_kernel: chunks of 8 elements per thread, 8 where it makes no
 // difference, else as many as leave the fewest threads idle (5120 elements: 64 threads with 10 chunks instead of 96 with 8).  pack_kernel: 64
-// elements per thread (32: 154 us against 126 at 32768 x 4096, a row's own work is spread over too few elements).
+// elements per thread, or 32 for few rows (few_rows in tsq_api.cu).
 TwoPassShape two_pass_shape(const EncodeParams& p) {
   TwoPassShape s{};
   const int chunks = static_cast<int>(p.chunks), segs = static_cast<int>((p.units + 31u) / 32u);
@@ -866,24 +695,27 @@ TwoPassShape two_pass_shape(const EncodeParams& p) {
   if (s.sizes_chunks == 0) s.sizes_chunks = warps(8) <= 8 ? 8 : 16;
   s.sizes_threads = 32 * warps(s.sizes_chunks);
   s.sizes_full = s.sizes_threads * s.sizes_chunks == chunks;
-  s.pack_groups = segs <= 16 ? 2 : 4;
-  const int pack_warps = (segs + s.pack_groups - 1) / s.pack_groups;
-  s.pack_threads = 32 * pack_warps;
-  s.pack_full = pack_warps * s.pack_groups * 128 == chunks;
-  s.pack_smem = static_cast<size_t>(pack_warps) * (2048u * static_cast<size_t>(s.pack_groups) + sizeof(uint16_t) * kListCap);
+  const auto pack_shape = [&](int groups) {
+    const int pack_warps = (segs + groups - 1) / groups;
+    return PackShape{32 * pack_warps, groups, pack_warps * groups * 128 == chunks,
+                     static_cast<size_t>(pack_warps) * (2048u * static_cast<size_t>(groups) + sizeof(uint16_t) * kListCap)};
+  };
+  s.pack = pack_shape(segs <= 16 ? 2 : 4);
+  s.pack_few = segs <= 8 ? pack_shape(1) : s.pack;  // (few_rows in tsq_api.cu)
   return s;
 }
 
 cudaError_t two_pass_attrs(const EncodeParams& p, const TwoPassShape& s) {
-  if (s.pack_smem <= 48u * 1024u) return cudaSuccess;
+  if (s.pack.smem <= 48u * 1024u) return cudaSuccess;
   // the attribute belongs to the kernel on the current device, not to a plan: always what the longest row needs
-  return cudaFuncSetAttribute(reinterpret_cast<const void*>(pack_of(p, s)), cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * (8192 + 2 * static_cast<int>(kListCap)));
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(pack_of(p, s.pack)), cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * (8192 + 2 * static_cast<int>(kListCap)));
 }
 
-cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, cudaStream_t stream) {
+cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, bool few, cudaStream_t stream) {
   const int grid = static_cast<int>(p.tokens);
+  const PackShape& pack = few ? s.pack_few : s.pack;
   const cudaError_t e = launch_overlapped(sizes_of(p, s), grid, s.sizes_threads, 0, stream, p);
-  return e != cudaSuccess ? e : launch_overlapped(pack_of(p, s), grid, s.pack_threads, s.pack_smem, stream, p);
+  return e != cudaSuccess ? e : launch_overlapped(pack_of(p, pack), grid, pack.threads, pack.smem, stream, p);
 }
 
 }  // namespace tsq

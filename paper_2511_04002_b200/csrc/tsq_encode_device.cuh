@@ -246,92 +246,208 @@ __device__ __forceinline__ void planes_of_bytes(const uint32_t (&tb)[8], uint32_
   transpose8x32_select(r);
 }
 
-// ---- 8-bit top level: codes by one FMA, and the distortion from the codes' bit-planes ----------------------------
+// ---- rows with zero-point 0, candidates that end in 4 and 8 bits ----------------------------------------------------------
 
-// Top-level codes of a group as bytes (grouping and signs as in distortion_first) when one FMA per element gets them right
-// (see one_fma_factor): r2 = {r, r}.  On the signed value, rounded as 128 + q: the distance of the low byte from 128 is the
-// code, which saves the absolute values.
+// top bits of the halves of ta, tb as bytes 0xff / 0: a.lo, b.lo, a.hi, b.hi
+__device__ __forceinline__ uint32_t top_bits4(uint32_t ta, uint32_t tb) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, 0xfbd9;" : "=r"(r) : "r"(ta), "r"(tb));
+  return r;
+}
+// min(|x|, m) of the two elements of a pair
 template <bool BF16>
-__device__ __forceinline__ void top_bytes_one_fma(const uint32_t (&x)[16], uint64_t r2, uint32_t (&tb)[8]) {
-  const uint64_t magic2 = pack2f(kRoundMagicSigned + 128.0f, kRoundMagicSigned + 128.0f);
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
-      const uint32_t c4 = __vabsdiffu4(bytes4(fma2(values2<BF16>(xa), r2, magic2), fma2(values2<BF16>(xb), r2, magic2)), 0x80808080u);
-      tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
-    }
+__device__ __forceinline__ uint32_t min_abs2(uint32_t x, uint32_t m) {
+  uint32_t r;
+  if (BF16) {
+    asm("{.reg .b32 t; abs.bf16x2 t, %1; min.bf16x2 %0, t, %2;}" : "=r"(r) : "r"(x), "r"(m));
+  } else {
+    asm("{.reg .b32 t; abs.f16x2 t, %1; min.f16x2 %0, t, %2;}" : "=r"(r) : "r"(x), "r"(m));
   }
+  return r;
 }
-// The same with the three-operation quotient.
-template <bool BF16>
-__device__ __forceinline__ void top_bytes(const uint32_t (&x)[16], const Level2& top, uint32_t (&tb)[8]) {
-  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
-      const uint32_t c4 = bytes4(quotient2(magnitudes2<BF16>(xa), top, magic2), quotient2(magnitudes2<BF16>(xb), top, magic2));
-      tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
-    }
-  }
+__device__ __forceinline__ uint64_t fma2_rm(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
-
-// A factor r for which fma(m, r, 2^23) rounds to the 8-bit level's code rint(fl(m / s)) of every 16-bit magnitude m of the
-// row, or 0 when none is known; run by one full warp.  The two can only disagree where m / s lies within about 2^-22
-// (relative) of a boundary k + 1/2, and a 16-bit m that close to one is rare:
-//   - lo = 0 (the usual row, s = fl(hi / 127)): m / hi is a ratio of two integers below 2^11, so that m / s is either at least
-//     2^-19 away from every boundary or, in exact arithmetic, on one.  254 m = (2k + 1) hi then, which only m = hi / 2 solves
-//     (k = 63) unless 127 divides hi's significand.  So 1 / s is moved by 2^-21 to the side that fl((hi / 2) / s) rounds to,
-//     and rows with such a significand (1 in 127) are left out.
-//   - else the 16-bit magnitude next to each of the 127 boundaries is tried, four per lane.
-template <bool BF16>
-__device__ __forceinline__ float one_fma_factor(float lo, float hi, const Level& top, uint32_t lane) {
-  if (lo == 0.0f) {
-    const uint32_t f = __float_as_uint(hi), m = (f & 0x7fffffu) | 0x800000u;  // 127 divides it iff it divides the significand
-    if (m % 127u == 0u || f < 0x00800000u) return 0.0f;
-    const float half = 0.5f * hi, q0 = __fmul_rn(half, top.r), q = __fmaf_rn(__fmaf_rn(q0, -top.s, half), top.r, q0);
-    return __fmul_rn(top.r, q >= 63.5f ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
-  }
-  bool same = true;
-#pragma unroll
-  for (uint32_t i = 0; i < 4; ++i) {
-    const float b = __fmul_rn(static_cast<float>(lane + 32u * i) + 0.5f, top.s);
-    const float m = Elem<BF16>::lo_f32(Elem<BF16>::pack_rn(b, 0.0f));
-    const float q0 = __fmul_rn(m, top.r), q = __fmaf_rn(__fmaf_rn(q0, -top.s, m), top.r, q0);
-    same = same && __fadd_rn(q, kRoundMagic) == __fmaf_rn(m, top.r, kRoundMagic);
-  }
-  return __all_sync(kFull, same) ? top.r : 0.0f;
-}
-
-// A lower bound of a group's distortion between the 8-bit level (7 code bits) and the 4-bit level, from the 8-bit codes'
-// bit-planes alone (r[k] = bit k of the codes).  Both levels round the same magnitude m, q = rint(m 127 / R) and
-// low = rint(m 7 / R) up to binary32 rounding, so |(q >> 4) - low| is 0 or 1 and is fixed by q except for the codes whose
-// rounding interval contains one of the low level's boundaries (k + 1/2) 127 / 7 = 9.07, 27.2, 45.4, 63.5, 81.6, 99.8, 117.9.
-// With q folded to q' = min(q, 127 - q), j = q' >> 4 and n = q' & 15: the difference is 1 for n > 9 + 2j, 0 for n < 9 + 2j and
-// open for n = 9 + 2j.  Returns the number of certain differences.
-__device__ __forceinline__ uint32_t certain_distortion_8_to_4(const uint32_t (&r)[8]) {
-  const uint32_t f = r[6], j1 = r[5] ^ f, j0 = r[4] ^ f, n3 = r[3] ^ f, n2 = r[2] ^ f, n1 = r[1] ^ f;
-  return __popc(n3 & ((~j1 & (n2 | (~j0 & n1))) | (j1 & ~j0 & n2 & n1)));
-}
-
-// The 8-bit level's scale of a row whose smallest magnitude is 0, as make_level gives it, and the factor of the one-FMA
-// codes (one_fma_factor), in about 20 instructions: s = fl(hi / 127) by a multiplication and two FMAs (correctly rounded
-// division by a constant: Brisebarre, Muller and Raina, "Accelerating correctly rounded floating-point division when the
-// divisor is known in advance", IEEE Transactions on Computers 53 (8), 2004); 127 divides hi's
-// significand iff 127 s = hi exactly; and fl((hi / 2) / s) >= 63.5 iff (hi / 2) - 63.5 s (exact) >= -2^-19 s.  (A host-side
-// test compares all of it for every 16-bit hi.)  The factor is 0 when the row has to go the general way.
-__device__ __forceinline__ float quick_level(float hi, float* s_out) {
-  constexpr float kInv127 = 1.0f / 127.0f;
-  const float q0 = __fmul_rn(hi, kInv127), s = __fmaf_rn(__fmaf_rn(-127.0f, q0, hi), kInv127, q0);
-  const float rem = __fmaf_rn(-127.0f, s, hi), side = __fmaf_rn(-63.5f, s, 0.5f * hi);
+__device__ __forceinline__ float rcp_approx(float x) {
   float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(s));
-  *s_out = s;
-  const float f = __fmul_rn(r, side >= -0x1p-19f * s ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
-  return s >= 0x1p-60f && s <= 0x1p60f && rem != 0.0f ? f : 0.0f;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// hi / Q, correctly rounded for every 16-bit hi (as in quick_level); *tie: Q divides hi's significand.
+template <int Q>
+__device__ __forceinline__ float divide_by(float hi, bool* tie) {
+  constexpr float kInv = 1.0f / static_cast<float>(Q);
+  const float q0 = __fmul_rn(hi, kInv), s = __fmaf_rn(__fmaf_rn(-static_cast<float>(Q), q0, hi), kInv, q0);
+  *tie = __fmaf_rn(-static_cast<float>(Q), s, hi) == 0.0f;
+  return s;
+}
+// Whether rint(fl((hi / 2) / s)) is the upper of the two codes that hi / 2 lies between (k and k + 1, k + 1/2 = Q / 2): the quotient
+// rounds to k + 1/2 or more iff (hi / 2) - (k + 1/2) s (exact) is not below -2^-half s, half an ulp below k + 1/2; ties go to
+// k + 1 there (k = 63, 3 and 1 are odd).
+__device__ __forceinline__ bool middle_up(float hi, float s, float middle, float half) { return __fmaf_rn(-middle, s, 0.5f * hi) >= -half * s; }
+
+// The distortion sum between the 8-bit level and a lower one, for rows with zero-point 0, without forming codes.  In ideal arithmetic the lower
+// level (Q codes above 0) rounds y = Q m / range up at y = k + 1/2 and q >> sh steps at y = (2^sh j - 1/2) Q / 127; both are even about Q / 2, and
+// with v = |y - Q / 2| they lie at v = k and at v = k / ratio, ratio = 127 / (2^sh Q), k = 1, 2, ...  So the difference of an element is 1 between
+// k / ratio and k and 0 elsewhere: with w = y - Q / 2 it is floor(ratio w) - floor(w), negative for w < 0.  kMargin moves both steps inwards, further
+// than the rounding of all of this and of the codes goes: the sum is a lower bound, and exact but for elements that lie next to a step.
+constexpr float kMargin = 0x1p-19f;
+struct Steps {
+  uint64_t per2, mid2, ratio2, one2;
+};
+__device__ __forceinline__ Steps steps_of(float q, float ratio, float range) {
+  const float c = q * rcp_approx(range), ka = ratio - kMargin * ratio, kb = 1.0f + kMargin;
+  return Steps{pack2f(c, c), pack2f(-0.5f * q, -0.5f * q), pack2f(ka, ka), pack2f(kb, kb)};
+}
+template <bool BF16>
+__device__ __forceinline__ uint64_t add_differences(uint32_t x, uint32_t hi2, const Steps& t, uint64_t acc) {
+  const uint64_t magic2 = pack2f(kRoundMagicSigned, kRoundMagicSigned), neg2 = pack2f(-1.0f, -1.0f);
+  const uint64_t w = fma2(values2<BF16>(min_abs2<BF16>(x, hi2)), t.per2, t.mid2);  // an outlier counts as hi: 0
+  const uint64_t d = fma2(fma2_rm(w, t.one2, magic2), neg2, fma2_rm(w, t.ratio2, magic2));
+  return fma2(d, d, acc);
+}
+__device__ __forceinline__ int sum_of(uint64_t acc) {
+  float a, b;
+  unpack2f(acc, a, b);
+  return __float2int_rn(a + b);
+}
+
+// By the whole warp: the 16-bit magnitude next to each step (one per lane), and by how much the sum is off for an element of that magnitude.
+template <bool BF16>
+__device__ __forceinline__ int step_error(float q, float ratio, float range, int sh, uint32_t lane, uint32_t* pattern) {
+  using E = Elem<BF16>;
+  const uint32_t k = lane & 15u;
+  const bool of_low = lane < 16u;
+  const float at = (of_low ? static_cast<float>(k) + 0.5f : (static_cast<float>((k + 1u) << sh) - 0.5f) * q * (1.0f / 127.0f)) / q * range;
+  *pattern = E::pack_rn(at, 0.0f) & 0xffffu;
+  const float m = E::pattern_f32(*pattern);
+  const bool middle_again = !of_low && static_cast<float>(2u * k + 1u) == q;  // both have a step there
+  if (static_cast<float>(k) >= q || middle_again || fabsf(m - at) > 0x1p-14f * at) return 0;
+  const int code = __float2int_rn(__fdiv_rn(m, __fdiv_rn(range, 127.0f))), low = __float2int_rn(__fdiv_rn(m, __fdiv_rn(range, q)));
+  const float w = __fmaf_rn(m, q * rcp_approx(range), -0.5f * q);
+  const float d = __fmaf_rd(w, ratio - kMargin * ratio, kRoundMagicSigned) - __fmaf_rd(w, 1.0f + kMargin, kRoundMagicSigned);
+  return abs((code >> sh) - low) - static_cast<int>(fabsf(d));
+}
+
+// The lowest candidate that passes, for a row with zero-point 0 whose distortion at 4 bits, `S` (the lower bound that add_differences gives), is within
+// the tolerance: exact sums from here on, candidate by candidate.  x: the thread's elements; cta_sum(v): the sum of v over the CTA;
+// again(q, ratio): the CTA's sum of differences at another level.
+template <bool BF16, int N, typename Sum, typename Again>
+__device__ __forceinline__ int descend(const EncodeParams& p, const uint32_t (&x)[N], float range, int S, Sum&& cta_sum, Again&& again) {
+  const uint32_t lane = threadIdx.x & 31u;
+  int best = 8;
+#pragma unroll 1
+  for (int ci = p.n_bits - 2; ci >= 0; --ci) {
+    const int b = p.bits[ci];
+    const float q = static_cast<float>((1 << (b - 1)) - 1), ratio = b == 4 ? 127.0f / 112.0f : b == 3 ? 127.0f / 96.0f : 127.0f / 64.0f;
+    if (b == 3) S = again(q, ratio);
+    if (b == 2) S = 0;  // (one step for both levels, in the middle)
+    uint32_t pattern;
+    const int error = step_error<BF16>(q, ratio, range, 8 - b, lane, &pattern);
+#pragma unroll 1
+    for (uint32_t open = __ballot_sync(kFull, error != 0); open != 0u; open &= open - 1u) {
+      const int l = __ffs(open) - 1;
+      const uint32_t m2 = __shfl_sync(kFull, pattern, l) * 0x10001u;
+      uint32_t same = 0u;  // minus the elements of that magnitude, by half
+#pragma unroll
+      for (int i = 0; i < N; ++i) same = __vadd2(same, Elem<BF16>::eq_mask(x[i] & 0x7fff7fffu, m2));
+      S += __shfl_sync(kFull, error, l) * cta_sum(-(static_cast<int>(static_cast<short>(same & 0xffffu)) + (static_cast<int>(same) >> 16)));
+    }
+    if (S > p.s_max) break;  // keep the last level that passed
+    best = b;
+  }
+  return best;
+}
+
+// Whether add_differences applies to a row with these extremes: zero-point 0 and no clamp at any level (the smallest magnitude is less than half a
+// code of the widest one: lo / s <= 127 / 255), and nothing leaves the normal range.
+__device__ __forceinline__ bool steps_apply(float lo, float hi) { return hi >= 0x1p-50f && hi <= 0x1p60f && 256.0f * lo <= hi; }
+
+// How pack_kernel, or the rest of encode_rows_kernel, forms a row's codes
+constexpr uint32_t kDivide = 0;    // by the division instruction
+constexpr uint32_t kPlain = 1;     // three-operation quotient
+constexpr uint32_t kOneUp = 2;     // one FMA, factor 1/s moved up (half the largest magnitude rounds up), zero-point 0
+constexpr uint32_t kOneDown = 3;   // one FMA, factor 1/s moved down
+constexpr uint32_t kOneTried = 4;  // one FMA with fl(1/s), tried out against every boundary
+constexpr uint32_t kCapped = 5;    // signed values: three-operation quotient, the largest value's code clamped
+
+// Scale of the level of b bits (2, 3, 4 or 8) of such a row, and how its codes may be formed; run by one full warp.
+template <bool BF16>
+__device__ __forceinline__ float scale_of(float lo, float hi, int b, uint32_t lane, uint32_t* mode) {
+  using E = Elem<BF16>;
+  float s;
+  *mode = kPlain;
+  if (lo == 0.0f) {
+    bool tie = false, up = false;  // (2 bits: s = hi, and (hi / 2) / hi = 1/2 rounds to 0)
+    s = hi;
+    if (b == 8) {
+      s = divide_by<127>(hi, &tie);
+      up = middle_up(hi, s, 63.5f, 0x1p-19f);
+    } else if (b == 4) {
+      s = divide_by<7>(hi, &tie);
+      up = middle_up(hi, s, 3.5f, 0x1p-23f);
+    } else if (b == 3) {
+      s = divide_by<3>(hi, &tie);
+      up = middle_up(hi, s, 1.5f, 0x1p-24f);
+    }
+    if (!tie) *mode = up ? kOneUp : kOneDown;
+    return s;
+  }
+  const float q = static_cast<float>((1 << (b - 1)) - 1);
+  s = __fdiv_rn(hi - lo, q);
+  const float r = __frcp_rn(s);
+  bool same = true;
+#pragma unroll 1
+  for (uint32_t i = lane; i < static_cast<uint32_t>(q); i += 32u) {
+    const float m = E::lo_f32(E::pack_rn(__fmul_rn(static_cast<float>(i) + 0.5f, s), 0.0f));
+    const float q0 = __fmul_rn(m, r), qt = __fmaf_rn(__fmaf_rn(q0, -s, m), r, q0);
+    same = same && __fadd_rn(qt, kRoundMagic) == __fmaf_rn(m, r, kRoundMagic);
+  }
+  if (__all_sync(kFull, same)) *mode = kOneTried;
+  return s;
+}
+__device__ __forceinline__ float one_fma_factor(float s, uint32_t mode) {
+  return mode == kOneTried ? __frcp_rn(s) : __fmul_rn(rcp_approx(s), mode == kOneUp ? 1.0f + 0x1p-21f : 1.0f - 0x1p-21f);
+}
+
+// Planes of a group whose codes take one FMA per element: r2 = {r, r} (one_fma_factor), nat = the group's outliers, whose slots become 0.  The codes are
+// formed on the signed value and rounded as 128 + q: the distance of the low byte from 128 is the code, which saves the absolute values.  (An outlier's
+// pattern has bits above the low byte: byte permutes, where a multiply-add would carry them into its neighbour.)
+template <bool BF16>
+__device__ __forceinline__ void planes_by_one_fma(const uint32_t (&x)[16], uint64_t r2, uint32_t nat, uint32_t (&pl)[8]) {
+  const uint64_t magic2 = pack2f(kRoundMagicSigned + 128.0f, kRoundMagicSigned + 128.0f);
+  uint32_t tb[8];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t xa = x[8 * h + i], xb = x[8 * h + 4 + i];
+      const uint32_t c4 = __vabsdiffu4(bytes4_any(fma2(values2<BF16>(xa), r2, magic2), fma2(values2<BF16>(xb), r2, magic2)), 0x80808080u);
+      tb[4 * h + i] = c4 | (__byte_perm(xa, xb, 0x7351) & 0x80808080u);
+    }
+  }
+  planes_of_bytes(tb, pl);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) pl[i] &= ~nat;
+}
+
+// Outliers of a group, bit e = element e, from t = (x | sign) - threshold: the top bit of each half of t is set for |x| >= tau, NaN included, and among the
+// others t orders like the magnitude.
+__device__ __forceinline__ uint32_t outliers_of(const uint32_t (&x)[16], uint32_t thr2) {
+  uint32_t nat = 0u;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t acc = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc |= top_bits4((x[8 * h + i] | 0x80008000u) - thr2, (x[8 * h + 4 + i] | 0x80008000u) - thr2) & (0x01010101u << (2 * i));
+    }
+    nat |= ((acc & 0xffffu) | ((acc >> 16) << 1)) << (16 * h);
+  }
+  return nat;
 }
 
 // Pass C on one group of a row whose chosen level is plain: codes as bytes (code | sign << 7), transposed into
@@ -400,34 +516,28 @@ __device__ __forceinline__ void divide_pack_regs(const uint32_t (&x)[16], const 
   }
 }
 
-// The b* plane words of one group, in blob order (plane 0 = sign, plane 1 + k = code bit k), to dst.
-// SV: plane k = code bit k, no sign plane.
+__device__ __forceinline__ void store32(uint32_t* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f, uint32_t g, uint32_t h) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h) : "memory");
+}
+
+// The b* plane words of group u of a row, in blob order (plane 0 = sign, plane 1 + k = code bit k; SV: plane k = code bit k, no sign plane), by
+// the widest stores that the row's start allows: rows of 94 groups, say, start on multiples of 32 bytes at 8 bits and of 16 at 4.
 template <bool SV = false>
-__device__ __forceinline__ void store_planes(uint32_t* dst, const uint32_t (&r)[8], int bstar, bool vec) {
-  if (SV) {
-    if (vec && bstar == 8) {
-      reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[0], r[1], r[2], r[3]);
-      reinterpret_cast<uint4*>(dst)[1] = make_uint4(r[4], r[5], r[6], r[7]);
-    } else if (vec && bstar == 4) {
-      reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[0], r[1], r[2], r[3]);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (q < bstar) dst[q] = r[q];
-      }
-    }
-    return;
-  }
-  if (vec && bstar == 8) {
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[7], r[0], r[1], r[2]);
-    reinterpret_cast<uint4*>(dst)[1] = make_uint4(r[3], r[4], r[5], r[6]);
-  } else if (vec && bstar == 4) {
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(r[7], r[0], r[1], r[2]);
+__device__ __forceinline__ void store_planes(uint32_t* row, uint32_t u, const uint32_t (&r)[8], int bstar) {
+  const uint32_t start = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(row));
+  uint32_t* dst = row + u * static_cast<uint32_t>(bstar);
+  const uint32_t w[8] = {SV ? r[0] : r[7], SV ? r[1] : r[0], SV ? r[2] : r[1], SV ? r[3] : r[2], SV ? r[4] : r[3], SV ? r[5] : r[4], SV ? r[6] : r[5], SV ? r[7] : r[6]};
+  if (bstar == 8 && (start & 31u) == 0u) {
+    store32(dst, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+  } else if ((bstar == 8 || bstar == 4) && (start & 15u) == 0u) {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    if (bstar == 8) reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  } else if (bstar == 2 && (start & 7u) == 0u) {
+    reinterpret_cast<uint2*>(dst)[0] = make_uint2(w[0], w[1]);
   } else {
-    dst[0] = r[7];
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-      if (q < bstar - 1) dst[1 + q] = r[q];
+    for (int q = 0; q < 8; ++q) {
+      if (q < bstar) dst[q] = w[q];
     }
   }
 }

@@ -11,15 +11,19 @@ namespace {
 // EncodeParams::direct_tiles
 constexpr int kByIndex = 1, kByTicket = 2;
 
+constexpr uint32_t kListCap = 256u;  // entries of a warp's outlier list
+
+template <int NW>
 struct RowShared {
   Level lv[kMaxCand];  // lv[i]: AIQ parameters of candidate bits[i]
   int S[kMaxCand];     // distortion sum of candidate i against the top level
-  int certain;         // TOP84: certain differences between the 8-bit and the 4-bit codes
   RowPartials<32> part;
+  int warp_sum[2][32]; // TOP84: distortion sums by warp, two sets in turn
   uint32_t tile;
   uint32_t divide;     // some level of the row needs the division instruction
   uint32_t row_cnt;    // outliers of the row
   uint32_t warp_w[32], warp_o[32], warp_status[32];  // direct_offsets: by warp
+  uint16_t list[NW][kListCap];  // where a warp's outliers are in its part of the row
 };
 
 // Whether a poll of a descriptor is to be given up: its limit ran out, or that of another poll of the call did (a call of many
@@ -47,8 +51,8 @@ __device__ __forceinline__ bool given_up(const EncodeParams& p, uint32_t gen4, u
 // nothing published, and every retry was another round trip.)  With many rows a thread's polls go out in batches, so that they
 // share a round trip: short rows have few threads to share them (2048 x 1024: 16.4 us, 19.3 in the pipelined kernel).
 constexpr uint32_t kPollBatch = 4u;
-template <bool BATCHES>
-__device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared& sh) {
+template <bool BATCHES, int NW>
+__device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared<NW>& sh) {
   const uint32_t limit = poll_limit_of(p), tag = gen4 | kFlagAggregate;
   uint32_t w = 0u, o = 0u, status = TSQ_OK;
   uint32_t i = threadIdx.x;
@@ -109,12 +113,12 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
 // DIRECT: calls of a few rows per SM (kByIndex, kByTicket): a row's offsets are read straight from the sizes of the rows before
 // it (direct_offsets) instead of walked back to.  With at most one row per SM (kByIndex) every CTA is resident, so row = CTA
 // index needs no ticket.
-// TOP84: the candidates end in 4 and 8 bits (magnitudes): codes and planes at 8 bits first, and the 4-bit candidate decided from
-// the planes where they suffice (certain_distortion_8_to_4), else everything the general way.
+// TOP84: the candidates end in 4 and 8 bits (magnitudes): the 4-bit candidate decided without forming codes (add_differences), so that a row's
+// sizes are published before its planes are formed, and the rows behind it find them when theirs are.
 template <bool BF16, int UPT, int MAXT, int MINB, bool SV, bool TOP84, int DIRECT>
 __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_constant__ EncodeParams p) {
   using E = Elem<BF16>;
-  __shared__ RowShared sh;
+  __shared__ RowShared<MAXT / 32> sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarps = blockDim.x >> 5;
   launch_dependents();
   wait_for_prior_grids();
@@ -156,43 +160,56 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
 
     // ---- pass A: threshold split, min / max of the inlier magnitudes, outlier counts ----
     const uint32_t thr2 = p.thr16 * 0x10001u;
-    uint32_t mn2 = E::kInfPattern * 0x10001u, mx2 = 0u;
     uint32_t bitmap[UPT];
-    uint32_t cnt = 0u;
-#pragma unroll
-    for (int k = 0; k < UPT; ++k) {
-      bitmap[k] = split_group<BF16>(x[k], nvalid[k], thr2, mn2, mx2);
-      cnt += __popc(bitmap[k]);
-    }
-    if (SV) {
-      // min / max of the signed values of T_below instead (outlier slots are +0 by now): as order keys
-      mn2 = 0xffffffffu;
-      mx2 = 0u;
+    uint32_t cnt = 0u, mnv, mxv;
+    if (TOP84) {
+      // (the outlier slots keep their values: see outliers_of, add_differences, planes_by_one_fma)
+      uint32_t mnt = 0xffffffffu, mxt = 0x80008000u;
 #pragma unroll
       for (int k = 0; k < UPT; ++k) {
 #pragma unroll
-        for (uint32_t i = 0; i < 16; ++i) {
-          if ((i >> 2) < nvalid[k]) {
-            const uint32_t key2 = order_keys2(x[k][i]);
-            mn2 = __vminu2(mn2, key2);
-            mx2 = __vmaxu2(mx2, key2);
+        for (uint32_t i = 0; i < 16; i += 2) {
+          const uint32_t ta = (x[k][i] | 0x80008000u) - thr2, tb = (x[k][i + 1] | 0x80008000u) - thr2;
+          mxt = __vimax3_s16x2(mxt, ta, tb);
+          if (i / 4u < nvalid[k]) mnt = __vimin3_u16x2(mnt, ta, tb);
+        }
+        bitmap[k] = outliers_of(x[k], thr2);
+        if (nvalid[k] < 4u) bitmap[k] &= (1u << (8u * nvalid[k])) - 1u;
+        cnt += __popc(bitmap[k]);
+      }
+      mnv = __reduce_min_sync(kFull, min(mnt & 0xffffu, mnt >> 16));
+      mxv = static_cast<uint32_t>(__reduce_max_sync(kFull, max(static_cast<int>(static_cast<short>(mxt & 0xffffu)), static_cast<int>(mxt) >> 16)));
+    } else {
+      uint32_t mn2 = E::kInfPattern * 0x10001u, mx2 = 0u;
+#pragma unroll
+      for (int k = 0; k < UPT; ++k) {
+        bitmap[k] = split_group<BF16>(x[k], nvalid[k], thr2, mn2, mx2);
+        cnt += __popc(bitmap[k]);
+      }
+      if (SV) {
+        // min / max of the signed values of T_below instead (outlier slots are +0 by now): as order keys
+        mn2 = 0xffffffffu;
+        mx2 = 0u;
+#pragma unroll
+        for (int k = 0; k < UPT; ++k) {
+#pragma unroll
+          for (uint32_t i = 0; i < 16; ++i) {
+            if ((i >> 2) < nvalid[k]) {
+              const uint32_t key2 = order_keys2(x[k][i]);
+              mn2 = __vminu2(mn2, key2);
+              mx2 = __vmaxu2(mx2, key2);
+            }
           }
         }
       }
+      mnv = __reduce_min_sync(kFull, min(mn2 & 0xffffu, mn2 >> 16));
+      mxv = __reduce_max_sync(kFull, max(mx2 & 0xffffu, mx2 >> 16));
     }
-    {
-      const uint32_t mnv = __reduce_min_sync(kFull, min(mn2 & 0xffffu, mn2 >> 16));
-      const uint32_t mxv = __reduce_max_sync(kFull, max(mx2 & 0xffffu, mx2 >> 16));
-      const uint32_t wcnt = __reduce_add_sync(kFull, cnt);
-      if (lane == 0) {
-        sh.part.warp_min[warp] = mnv;
-        sh.part.warp_max[warp] = mxv;
-        sh.part.warp_cnt[warp] = wcnt;
-      }
-    }
-    if (TOP84 && tid < static_cast<uint32_t>(kMaxCand)) {
-      sh.S[tid] = 0;
-      sh.certain = 0;
+    const uint32_t wcnt = __reduce_add_sync(kFull, cnt);
+    if (lane == 0) {
+      sh.part.warp_min[warp] = mnv;
+      sh.part.warp_max[warp] = mxv;
+      sh.part.warp_cnt[warp] = wcnt;
     }
     __syncthreads();
 
@@ -200,89 +217,58 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
     uint32_t r[UPT][8];
     Level best;
     int bstar = bmax;
-    uint32_t row_cnt = 0u, cnt_before = 0u;  // outliers of the row, of the warps before this one
+    uint32_t row_cnt = 0u, mode = kPlain;
+    float lo = 0.0f, hi = 0.0f;
     bool settled = false, divide = false;
     if (TOP84) {
-      // ---- every thread forms the row's extremes and its top level for itself (a few dozen instructions for the usual row) ----
-      const uint32_t pmin = __reduce_min_sync(kFull, lane < nwarps ? sh.part.warp_min[lane] : 0xffffu);
-      const uint32_t pmax = __reduce_max_sync(kFull, lane < nwarps ? sh.part.warp_max[lane] : 0u);
-      const uint32_t wc = lane < nwarps ? sh.part.warp_cnt[lane] : 0u;
-      row_cnt = __reduce_add_sync(kFull, wc);
-      cnt_before = __reduce_add_sync(kFull, lane < warp ? wc : 0u);
-      const float lo = E::pattern_f32(pmin), hi = E::pattern_f32(pmax);
-      best.zp = 0;
-      best.qmax = 127;
-      float one = pmin == 0u ? quick_level(hi, &best.s) : 0.0f;
-      bool plain = true;
-      if (one == 0.0f) {
-        best = make_level(lo, hi, 8, &plain);
-        if (plain) one = one_fma_factor<BF16>(lo, hi, best, lane);
-      }
-      if (plain) {
-        uint32_t tb[UPT][8];
-        uint32_t S = 0u;
+      // ---- every thread forms the row's extremes for itself ----
+      uint32_t pmin = __reduce_min_sync(kFull, lane < nwarps ? sh.part.warp_min[lane] : 0xffffu);
+      const int mx = __reduce_max_sync(kFull, lane < nwarps ? static_cast<int>(sh.part.warp_max[lane]) : -32768);
+      row_cnt = __reduce_add_sync(kFull, lane < nwarps ? sh.part.warp_cnt[lane] : 0u);
+      pmin = row_cnt != 0u ? 0u : (pmin + p.thr16) & 0x7fffu;
+      const uint32_t pmax = mx < 0 ? 0u : (static_cast<uint32_t>(mx) + p.thr16) & 0x7fffu;
+      lo = E::pattern_f32(pmin);
+      hi = E::pattern_f32(pmax);
+      if (steps_apply(lo, hi)) {
+        uint32_t turn = 0u;
+        const auto cta_sum = [&](int v) {
+          v = __reduce_add_sync(kFull, v);
+          if (nwarps == 1u) return v;
+          if (lane == 0) sh.warp_sum[turn][warp] = v;
+          __syncthreads();
+          const int sum = __reduce_add_sync(kFull, lane < nwarps ? sh.warp_sum[turn][lane] : 0);
+          turn ^= 1u;
+          return sum;
+        };
+        const auto differences = [&](float q, float ratio) {
+          const Steps t = steps_of(q, ratio, hi - lo);
+          uint64_t acc = 0ull;
+#pragma unroll
+          for (int k = 0; k < UPT; ++k) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc = add_differences<BF16>(x[k][i], pmax * 0x10001u, t, acc);
+          }
+          return cta_sum(sum_of(acc));
+        };
+        const int S = differences(7.0f, 127.0f / 112.0f);
+        if (S <= p.s_max) {
+          static_assert(!TOP84 || UPT == 1, "one group per thread");
+          bstar = descend<BF16>(p, x[0], hi - lo, S, cta_sum, differences);
+        }
+        settled = true;
+      } else {
+        // ---- the general way: magnitudes, outlier slots +0 ----
 #pragma unroll
         for (int k = 0; k < UPT; ++k) {
-          if (one != 0.0f) {
-            top_bytes_one_fma<BF16>(x[k], pack2f(one, one), tb[k]);
-          } else {
-            top_bytes<BF16>(x[k], make_level2(best), tb[k]);
-          }
-          planes_of_bytes(tb[k], r[k]);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) x[k][i] &= ~E::geu_mask(x[k][i] & 0x7fff7fffu, thr2);
         }
-        // With a row or less per SM the call ends with its slowest row, and in most calls some row's open codes decide: the
-        // exact sum for all rows then, one barrier for every row (64 x 4096: 5.6 us against 6.7).
-        if (DIRECT != kByIndex) {
-#pragma unroll
-          for (int k = 0; k < UPT; ++k) S += certain_distortion_8_to_4(r[k]);
-          S = __reduce_add_sync(kFull, S);
-          if (lane == 0 && S != 0u) atomicAdd(&sh.certain, static_cast<int>(S));
-          __syncthreads();
-          settled = sh.certain > p.s_max;
+        __syncthreads();
+        if (lane == 0) {
+          sh.part.warp_min[warp] = pmin;
+          sh.part.warp_max[warp] = pmax;
         }
-        // the rest of Algorithm 1, every candidate's codes against the top-level bytes
-        uint32_t lb[UPT][8];
-        bool lower = false;
-        for (int ci = p.n_bits - 2; !settled; --ci) {
-          if (ci < 0) {
-            settled = true;
-            break;
-          }
-          bool low_plain = false;
-          const Level low = make_level(lo, hi, p.bits[ci], &low_plain);
-          if (!low_plain) break;  // the general way, from the start
-          uint32_t ql[UPT][8];
-          S = 0u;
-#pragma unroll
-          for (int k = 0; k < UPT; ++k) S += distortion_next<BF16>(x[k], tb[k], make_level2(low), 8 - p.bits[ci], ql[k]);
-          S = __reduce_add_sync(kFull, S);
-          if (lane == 0 && S != 0u) atomicAdd(&sh.S[ci], static_cast<int>(S));
-          __syncthreads();
-          if (sh.S[ci] > p.s_max) {  // keep the last level that passed
-            settled = true;
-            break;
-          }
-          bstar = p.bits[ci];
-          best = low;
-          lower = true;
-#pragma unroll
-          for (int k = 0; k < UPT; ++k) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) lb[k][i] = ql[k][i];
-          }
-        }
-        if (settled && lower) {
-#pragma unroll
-          for (int k = 0; k < UPT; ++k) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) tb[k][i] = lb[k][i] | (tb[k][i] & 0x80808080u);
-            planes_of_bytes(tb[k], r[k]);
-          }
-        }
-        if (!settled) {
-          bstar = bmax;
-          __syncthreads();  // before the sums are set to 0 again
-        }
+        __syncthreads();
       }
     }
     if (!settled) {
@@ -317,15 +303,27 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
       best = low;
     }
     row_cnt = sh.row_cnt;
-    cnt_before = sh.part.warp_cnt[warp];
     }
     const uint32_t agg_w = static_cast<uint32_t>(bstar) * p.lay.wpp;
 
     // ---- this row's sizes are known: let the rows behind it see them, then pack ----
     if (tid == 0) st_relaxed_u64(p.desc + 2ull * tile, pack_desc(gen4 | kFlagAggregate, agg_w << 17 | row_cnt));
+    if (settled) {
+      best.s = scale_of<BF16>(lo, hi, bstar, lane, &mode);
+      best.zp = 0;
+      best.qmax = (1 << (bstar - 1)) - 1;
+      best.r = mode >= kOneUp ? one_fma_factor(best.s, mode) : __frcp_rn(best.s);
+    }
 #pragma unroll
     for (int k = 0; k < UPT; ++k) {
-      if (settled) continue;
+      if (settled && mode >= kOneUp) {
+        planes_by_one_fma<BF16>(x[k], pack2f(best.r, best.r), bitmap[k], r[k]);
+        continue;
+      }
+      if (settled) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[k][i] &= ~E::geu_mask(x[k][i] & 0x7fff7fffu, thr2);
+      }
       if (divide) {
         divide_pack_regs<BF16, SV>(x[k], best, r[k]);
         if (SV && nvalid[k] < 4u) {  // pad bits stay 0: the zeros past the end of the row got the code of the value 0
@@ -335,6 +333,34 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
         }
       } else {
         pack_group<BF16, SV>(x[k], make_level2(best), r[k], nvalid[k]);
+      }
+    }
+
+    // ---- where the warp's outliers are, in order, and its first 32 entries (original patterns, read again from the input) ----
+    const uint32_t col0 = 32u * UPT * (32u * warp);
+    const uint16_t* x16 = p.x + static_cast<size_t>(tile) * p.hidden;
+    uint32_t before = 0u, entry = 0u;
+    if (wcnt != 0u) {
+      uint32_t incl = cnt;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t n = __shfl_up_sync(kFull, incl, d);
+        if (lane >= static_cast<uint32_t>(d)) incl += n;
+      }
+      before = incl - cnt;
+      if (wcnt <= kListCap) {
+        uint32_t at = before;
+#pragma unroll
+        for (int k = 0; k < UPT; ++k) {
+          for (uint32_t rest = bitmap[k]; rest != 0u; rest &= rest - 1u, ++at) {
+            sh.list[warp][at] = static_cast<uint16_t>(32u * (UPT * lane + k) + static_cast<uint32_t>(__ffs(rest) - 1));
+          }
+        }
+        __syncwarp();
+        if (lane < wcnt) {
+          const uint32_t c = col0 + sh.list[warp][lane];
+          entry = c << 16 | x16[c];
+        }
       }
     }
 
@@ -355,30 +381,28 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
 #pragma unroll
       for (int k = 0; k < UPT; ++k) {
         const uint32_t u = UPT * tid + k;
-        if (u < p.units) store_planes<SV>(wrow + static_cast<size_t>(u) * bstar, r[k], bstar, p.vec_store != 0u);
+        if (u < p.units) store_planes<SV>(wrow, u, r[k], bstar);
       }
       if (tid == 0) write_token_fields(p, tile, bstar, best.s, best.zp, word_off + agg_w, out_base + row_cnt);
-      // ---- CSR entries of T_above: ascending columns, original patterns (read again from the input) ----
-      if (__ballot_sync(kFull, cnt != 0u) != 0u) {
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const uint32_t n = __shfl_up_sync(kFull, incl, d);
-          if (lane >= static_cast<uint32_t>(d)) incl += n;
-        }
-        if (cnt != 0u) {
-          uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
-          const uint16_t* x16 = p.x + static_cast<size_t>(tile) * p.hidden;
-          unsigned long long at = static_cast<unsigned long long>(out_base) + cnt_before + (incl - cnt);
+      // ---- CSR entries of T_above: ascending columns ----
+      if (wcnt != 0u) {
+        uint32_t* o_outl = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_outl);
+        // outliers of the warps before this one (warp_cnt is an exclusive scan where the levels were formed the general way)
+        const uint32_t warps_before = TOP84 && settled ? __reduce_add_sync(kFull, lane < warp ? sh.part.warp_cnt[lane] : 0u) : sh.part.warp_cnt[warp];
+        unsigned long long at = static_cast<unsigned long long>(out_base) + warps_before;  // (finish_direct reports what does not fit)
+        if (wcnt <= kListCap) {
+          if (lane < wcnt && at + lane < p.lay.outlier_capacity) o_outl[at + lane] = entry;
+          for (uint32_t i = lane + 32u; i < wcnt; i += 32u) {
+            const uint32_t c = col0 + sh.list[warp][i];
+            if (at + i < p.lay.outlier_capacity) o_outl[at + i] = c << 16 | x16[c];
+          }
+        } else {  // too many for the list: each lane its own
+          at += before;
 #pragma unroll
           for (int k = 0; k < UPT; ++k) {
-            uint32_t bm = bitmap[k];
-            const uint32_t u = UPT * tid + k;
-            while (bm != 0u) {
-              const uint32_t e = 32u * u + static_cast<uint32_t>(__ffs(bm) - 1);
-              bm &= bm - 1u;
-              if (at < p.lay.outlier_capacity) o_outl[at] = (e << 16) | x16[e];  // (finish_direct reports what does not fit)
-              ++at;
+            for (uint32_t rest = bitmap[k]; rest != 0u; rest &= rest - 1u, ++at) {
+              const uint32_t c = col0 + 32u * (UPT * lane + k) + static_cast<uint32_t>(__ffs(rest) - 1);
+              if (at < p.lay.outlier_capacity) o_outl[at] = c << 16 | x16[c];
             }
           }
         }
@@ -404,7 +428,7 @@ static RowsKernel rows_kernel_of(bool bf16, int threads, int upt, int dense) {
     }
     return bf16 ? encode_rows_kernel<true, 1, 256, 2, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 256, 2, SV, TOP84, DIRECT>;
   }
-  if (upt == 1) return bf16 ? encode_rows_kernel<true, 1, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 1, 1024, 1, SV, false, DIRECT>;
+  if (upt == 1) return bf16 ? encode_rows_kernel<true, 1, 1024, 1, SV, TOP84, DIRECT> : encode_rows_kernel<false, 1, 1024, 1, SV, TOP84, DIRECT>;
   return bf16 ? encode_rows_kernel<true, 2, 1024, 1, SV, false, DIRECT> : encode_rows_kernel<false, 2, 1024, 1, SV, false, DIRECT>;
 }
 
@@ -412,8 +436,7 @@ template <int DIRECT>
 static RowsKernel rows_kernel(const EncodeParams& p, int threads, int upt, int dense) {
   const bool bf16 = p.dtype == TSQ_BF16;
   if (p.variant != 0u) return rows_kernel_of<true, false, DIRECT>(bf16, threads, upt, dense);
-  // (in the CTAs of more than 256 threads, 64 registers each, the extra path costs more than it saves)
-  if (ends_in_4_and_8(p) && upt == 1 && threads <= 256) return rows_kernel_of<false, true, DIRECT>(bf16, threads, upt, dense);
+  if (ends_in_4_and_8(p) && upt == 1) return rows_kernel_of<false, true, DIRECT>(bf16, threads, upt, dense);
   return rows_kernel_of<false, false, DIRECT>(bf16, threads, upt, dense);
 }
 

@@ -93,7 +93,6 @@ struct EncodeParams {
   int32_t n_bits;
   int32_t bits[8];
   int32_t s_max;                             // floor(delta * H), clamped to [-1, INT32_MAX]
-  uint32_t vec_store;                        // 1: every token's plane words start on a 16-byte boundary
   uint32_t direct_tiles;                     // one-kernel encoder: 1 = row index = CTA index (every CTA resident), 2 = rows by ticket
   uint32_t dtype;
   uint32_t variant;                          // 0: sign + magnitude codes; 1: codes of the signed values
@@ -145,14 +144,19 @@ cudaError_t launch_encode_rows(const EncodeParams& p, int grid, int threads, int
 cudaError_t encode_rows_attrs(const EncodeParams& p, int threads, int upt, int dense, int* blocks_per_sm);
 // The two-kernel encoder: threads, chunks of 8 elements per thread (sizes) and 32-element groups per thread (pack); full: no thread
 // has a short or missing share.
+struct PackShape {
+  int threads, groups;
+  bool full;
+  size_t smem;
+};
 struct TwoPassShape {
-  int sizes_threads, sizes_chunks, pack_threads, pack_groups;
-  bool sizes_full, pack_full;
-  size_t pack_smem;
+  int sizes_threads, sizes_chunks;
+  bool sizes_full;
+  PackShape pack, pack_few;  // pack_few: for calls that do not fill the device several times over
 };
 TwoPassShape two_pass_shape(const EncodeParams& p);
 cudaError_t two_pass_attrs(const EncodeParams& p, const TwoPassShape& s);
-cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, cudaStream_t stream);
+cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, bool few, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeParams& p, int grid, int threads, size_t smem, cudaStream_t stream);
 cudaError_t decode_kernel_attrs(bool bf16, int threads, size_t smem, int* blocks_per_sm);
 size_t decode_smem_bytes(uint32_t row_bytes);
