@@ -197,7 +197,6 @@ struct tsq_plan {
   uint32_t thr16;
   uint32_t variant;                 // 0: sign + magnitude codes; 1: codes of the signed values
   int threads;                      // decoder CTA size, one group per thread
-  int threads_half, dec_blocks_half; // the same with two groups per thread, and its resident CTAs per SM
   int enc_threads, enc_upt;         // one-kernel encoder: CTA size and 32-element groups per thread
   bool ends_in_4_and_8;
   int rows_ctas[3];                 // resident CTAs per SM of the one-kernel encoder's instances (rows_instance)
@@ -271,24 +270,14 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
   const double smax = std::floor(static_cast<double>(delta) * static_cast<double>(hidden));
   p->s_max = smax < -1.0 ? -1 : (smax > 2147483647.0 ? 2147483647 : static_cast<int32_t>(smax));
   p->thr16 = threshold_pattern(dtype, tau);
-  // decoder CTA: one 32-element group per thread, or two when the call has rows enough to fill the device
-  // several times over with the smaller CTAs (a thread's fixed work, checking the header and the token's
-  // fields, is then spread over 64 elements: 8 % faster at 8192 x 8192 and 32768 x 4096; with fewer rows
-  // the smaller CTAs leave the device short of threads and are slower: 4096 x 4096 20.2 against 15.6 us,
-  // 2048 x 5120 12.6 against 10.6); never fewer than 64 threads while
-  // the row has that many groups
+  // decoder CTA: one 32-element group per thread, as far as a CTA goes (two per thread were slower in every size but for rows
+  // that are all 8 bits wide: 8192 x 8192 42.1 against 38.0 us, 16384 x 4096 42.0 against 37.2 us)
   p->threads = static_cast<int>(((p->units + 31u) / 32u) * 32u);
   if (p->threads > kMaxThreads) p->threads = kMaxThreads;
-  {
-    const uint32_t all = static_cast<uint32_t>(p->threads), half = (((p->units + 1u) / 2u + 31u) / 32u) * 32u;
-    const uint32_t floor64 = all < 64u ? all : 64u;
-    p->threads_half = static_cast<int>(half > floor64 ? half : floor64);
-    if (p->threads_half > p->threads) p->threads_half = p->threads;
-  }
   // encoder: one thread per 32-element group, two for rows longer than kEncMaxThreads groups
   p->enc_upt = p->units > static_cast<uint32_t>(kEncMaxThreads) ? 2 : 1;
   p->enc_threads = static_cast<int>(((p->units + p->enc_upt - 1) / p->enc_upt + 31u) / 32u * 32u);
-  p->dec_smem = decode_smem_bytes(p->row_bytes);
+  p->dec_smem = decode_smem_bytes(p->row_bytes, p->threads);
   const unsigned long long desc = T > 0 ? T : 1;
   p->workspace_bytes = static_cast<size_t>(align16(sizeof(WsControl) + 16ull * desc));
 
@@ -300,10 +289,9 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
   int prev_dev = 0;
   cudaGetDevice(&prev_dev);
   bool ok = cudaSetDevice(device) == cudaSuccess;
-  int sms = 0, dec_blocks = 0;
+  int sms = 0;
   ok = ok && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
-  ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, p->threads, p->dec_smem, &dec_blocks) == cudaSuccess;
-  ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, p->threads_half, p->dec_smem, &p->dec_blocks_half) == cudaSuccess;
+  ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, variant != 0, p->dec_smem) == cudaSuccess;
   {
     EncodeParams kernel_of;  // what selects the kernel instances
     std::memset(&kernel_of, 0, sizeof kernel_of);
@@ -327,7 +315,7 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     if (rows > direct_rows(p)) ok = ok && two_pass_attrs(kernel_of, p->two_pass) == cudaSuccess;
   }
   cudaSetDevice(prev_dev);
-  if (!ok || dec_blocks < 1 || sms < 1) {
+  if (!ok || sms < 1) {
     cudaGetLastError();
     delete p;
     return TSQ_ERR_CUDA;
@@ -499,13 +487,10 @@ static DecodeParams decode_params(const tsq_plan_t* plan, const void* blob_dev, 
 
 static tsq_status_t launch_decode_part(const tsq_plan_t* plan, DecodeParams& p, void* cuda_stream) {
   const int64_t tokens = p.tokens;
-  // A call that fills the device once lets the next grid in early (0.6 us per call at 64 rows).  A longer one does not: an
-  // encode that follows it would be set up unevenly over the SMs that become free first, which costs its persistent CTAs
-  // more than the launch (32768 x 4096 encode + decode: 312 us with, 295 us without).
+  // A call of at most a row per SM lets the next grid in early (0.6 us per call at 64 rows).  A longer one does not: the next grid's CTAs
+  // wait where its own later ones should run (600 x 8192 5.3 us without, 7.2 us with; 16384 x 1024 16.5 and 20.4 us).
   p.overlap_next = tokens <= static_cast<int64_t>(plan->sms) ? 1u : 0u;
-  const bool many_rows = tokens >= 3 * static_cast<int64_t>(plan->sms) * plan->dec_blocks_half;
-  const cudaError_t e = launch_decode(p, static_cast<int>(tokens), many_rows ? plan->threads_half : plan->threads,
-                                      plan->dec_smem, static_cast<cudaStream_t>(cuda_stream));
+  const cudaError_t e = launch_decode(p, plan->sms, plan->threads, plan->dec_smem, static_cast<cudaStream_t>(cuda_stream));
   g_launches.fetch_add(1);
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
 }
