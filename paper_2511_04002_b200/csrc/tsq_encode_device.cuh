@@ -206,36 +206,7 @@ __device__ __forceinline__ uint32_t distortion_group(const uint32_t (&x)[16], co
   return S;
 }
 
-// Pass B for a further candidate: the top-level codes come from the bytes the first turn left.
-template <bool BF16, bool SV = false>
-__device__ __forceinline__ uint32_t distortion_next(const uint32_t (&x)[16], const uint32_t (&tb)[8], const Level2& low, int sh,
-                                                    uint32_t (&ql)[8], uint32_t nvalid = 4u) {
-  // a byte of tb is code | sign << 7 (SV: an 8-bit code): shifted right by sh >= 1, the sign bit and the bits that
-  // come in from the next byte all land above the mask
-  const uint32_t shmask = ((SV ? 0xffu : 0x7fu) >> sh) * 0x01010101u;
-  const uint64_t magic2 = pack2f(kRoundMagic, kRoundMagic);
-  uint32_t S = 0;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const uint32_t inside = (2u * h < nvalid ? 0x00ff00ffu : 0u) | (2u * h + 1u < nvalid ? 0xff00ff00u : 0u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (SV) {
-        const uint32_t q4 = codes4<BF16, true>(x[8 * h + i], x[8 * h + 4 + i], low) & inside;
-        S = __vsadu4((tb[4 * h + i] >> sh) & shmask, q4) + S;
-        ql[4 * h + i] = q4;
-        continue;
-      }
-      const uint32_t q4 = bytes4(quotient2(magnitudes2<BF16>(x[8 * h + i]), low, magic2),
-                                 quotient2(magnitudes2<BF16>(x[8 * h + 4 + i]), low, magic2));
-      S = __vsadu4((tb[4 * h + i] >> sh) & shmask, q4) + S;
-      ql[4 * h + i] = q4;
-    }
-  }
-  return S;
-}
-
-// Bytes of one group as distortion_first leaves them -> bit-planes: on return r[k] = bit k of every byte,
+// Bytes of one group (code | sign << 7, element order of the callers) -> bit-planes: on return r[k] = bit k of every byte,
 // k < 7 code bits, k = 7 signs.
 __device__ __forceinline__ void planes_of_bytes(const uint32_t (&tb)[8], uint32_t (&r)[8]) {
 #pragma unroll
@@ -551,8 +522,7 @@ struct RowPartials {
 };
 template <bool BF16, int NW, bool SV = false>
 __device__ __forceinline__ uint32_t row_levels(const EncodeParams& p, RowPartials<NW>& part, uint32_t nwarps, uint32_t lane,
-                                               Level* lv_out, int* S_out, uint32_t* row_cnt, float* lo_out = nullptr,
-                                               float* hi_out = nullptr) {
+                                               Level* lv_out, int* S_out, uint32_t* row_cnt) {
   using E = Elem<BF16>;
   const uint32_t pmin = __reduce_min_sync(kFull, lane < nwarps ? part.warp_min[lane] : 0xffffu);
   const uint32_t pmax = __reduce_max_sync(kFull, lane < nwarps ? part.warp_max[lane] : 0u);
@@ -574,13 +544,7 @@ __device__ __forceinline__ uint32_t row_levels(const EncodeParams& p, RowPartial
     lv_out[lane] = lv;
     S_out[lane] = 0;
   }
-  if (lane == 0) {
-    *row_cnt = total;
-    if (lo_out) {  // magnitudes (not meant for SV)
-      *lo_out = E::pattern_f32(pmin);
-      *hi_out = E::pattern_f32(pmax);
-    }
-  }
+  if (lane == 0) *row_cnt = total;
   return __all_sync(kFull, plain) ? 0u : 1u;
 }
 
