@@ -291,7 +291,7 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
   bool ok = cudaSetDevice(device) == cudaSuccess;
   int sms = 0;
   ok = ok && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
-  ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, variant != 0, p->dec_smem) == cudaSuccess;
+  ok = ok && decode_kernel_attrs(dtype == TSQ_BF16, variant != 0, 4u * p->units == p->chunks, p->dec_smem) == cudaSuccess;
   {
     EncodeParams kernel_of;  // what selects the kernel instances
     std::memset(&kernel_of, 0, sizeof kernel_of);

@@ -3,8 +3,8 @@
 // outliers of T_above over their slots.  One CTA per token row; the row is assembled in shared
 // memory and leaves through one bulk asynchronous store.
 //
-// What bounds it: bytes, for calls of many rows (8192 x 8192 with every row at 8 bits: 35.4 us for 201 MB; a kernel that only widens as many bytes
-// to 16 bits takes 33.4 us, 32768 x 4096 with 1 % outliers 71.2 against 63 us), two dependent round trips to memory and the launch for the others.
+// What bounds it: bytes, for calls of many rows (8192 x 8192 with every row at 8 bits: 34.6 us for 201 MB; a kernel that only widens as many bytes
+// to 16 bits takes 33.4 us, 32768 x 4096 with 1 % outliers 69.5 against 63 us), two dependent round trips to memory and the launch for the others.
 // Threads in flight decide more than instructions: 32768 x 4096 took 77 us with 40 registers a thread and 302 instructions per warp and
 // group, 71.6 us with 32 and 379.  CTAs that stay and take several rows, and warps that send their 2 KB of a row by themselves, were
 // both slower (78 to 90 us at 32768 x 4096).
@@ -121,7 +121,9 @@ __device__ __forceinline__ void code_bytes(const Planes<4>& q, uint32_t (&r)[8])
 //     rounds.  Two elements per instruction, each lane rounding as the scalar instruction does;
 //   - the sign plane is not transposed: one multiplication by 2^(15 - 2i) + 2^(30 - 2i) brings bits 2i and 2i + 1 of a chunk's
 //     sign byte to bits 15 and 31 (the two images of the byte do not overlap), one logic instruction takes them over.
-template <bool BF16, int KIND, int W>
+// FULL: the row has no short last group (a comparison less per 8 elements: 2 to 3 % of a long call, 8192 x 8192 35.4 -> 34.6 us,
+// 32768 x 4096 71.2 -> 69.5 us).
+template <bool BF16, int KIND, int W, bool FULL>
 __device__ __forceinline__ void restore_groups(const DecodeParams& p, const uint32_t* words, uint32_t b, float s, int32_t zp) {
   using E = Elem<BF16>;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
@@ -150,7 +152,7 @@ __device__ __forceinline__ void restore_groups(const DecodeParams& p, const uint
         out[i] = E::pack_rn(lo, hi);
         if (KIND != kSigned) out[i] |= mad_u32(sgn, (1u << (15 - 2 * i)) + (1u << (30 - 2 * i)), 0u) & 0x80008000u;
       }
-      if (cidx < p.chunks) stage4[cidx] = make_uint4(out[0], out[1], out[2], out[3]);
+      if (FULL || cidx < p.chunks) stage4[cidx] = make_uint4(out[0], out[1], out[2], out[3]);
     }
   }
 }
@@ -158,7 +160,7 @@ __device__ __forceinline__ void restore_groups(const DecodeParams& p, const uint
 // Rare: a zero-point or a scale that the fused form cannot take.
 template <bool BF16>
 __device__ __noinline__ void restore_rare(const DecodeParams& p, const uint32_t* words, uint32_t b, float s, int32_t zp) {
-  restore_groups<BF16, kMagnitudes, 8>(p, words, b, s, zp);
+  restore_groups<BF16, kMagnitudes, 8, false>(p, words, b, s, zp);
 }
 
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
@@ -166,7 +168,7 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) 
 }
 
 // RES: threads that an SM holds, from which the registers of a thread follow (launch_decode says which is taken when).
-template <bool BF16, bool SV, int RES>
+template <bool BF16, bool SV, bool FULL, int RES>
 __global__ void __launch_bounds__(kMaxThreads, RES / kMaxThreads) decode_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ __align__(128) unsigned char smem_dyn[];  // one output row
   constexpr bool kShare = RES == 2048;
@@ -231,16 +233,16 @@ __global__ void __launch_bounds__(kMaxThreads, RES / kMaxThreads) decode_kernel(
   const uint32_t* words = reinterpret_cast<const uint32_t*>(p.blob + p.lay.off_words) + wo;
   if (SV) {
     if (b <= 4u) {
-      restore_groups<BF16, kSigned, 4>(p, words, b, s, zp);
+      restore_groups<BF16, kSigned, 4, FULL>(p, words, b, s, zp);
     } else {
-      restore_groups<BF16, kSigned, 8>(p, words, b, s, zp);
+      restore_groups<BF16, kSigned, 8, FULL>(p, words, b, s, zp);
     }
   } else if (zp != 0 || s > 0x1p100f) {  // 2^23 * s must stay finite for the fused form
     restore_rare<BF16>(p, words, b, s, zp);
   } else if (b <= 4u) {
-    restore_groups<BF16, kFused, 4>(p, words, b, s, zp);
+    restore_groups<BF16, kFused, 4, FULL>(p, words, b, s, zp);
   } else {
-    restore_groups<BF16, kFused, 8>(p, words, b, s, zp);
+    restore_groups<BF16, kFused, 8, FULL>(p, words, b, s, zp);
   }
   if (kShare) cp_async_wait_all();
   __syncthreads();
@@ -278,29 +280,35 @@ __global__ void __launch_bounds__(kMaxThreads, RES / kMaxThreads) decode_kernel(
 size_t decode_smem_bytes(uint32_t row_bytes, int threads) { return row_stage_bytes(row_bytes) + sizeof(uint32_t) * threads; }
 
 using DecodeFn = void (*)(DecodeParams);
-static DecodeFn kernel_of(bool bf16, bool signed_values, int which) {
-  static const DecodeFn fn[2][2][3] = {
-      {{decode_kernel<false, false, 1024>, decode_kernel<false, false, 1536>, decode_kernel<false, false, 2048>},
-       {decode_kernel<false, true, 1024>, decode_kernel<false, true, 1536>, decode_kernel<false, true, 2048>}},
-      {{decode_kernel<true, false, 1024>, decode_kernel<true, false, 1536>, decode_kernel<true, false, 2048>},
-       {decode_kernel<true, true, 1024>, decode_kernel<true, true, 1536>, decode_kernel<true, true, 2048>}}};
-  return fn[bf16][signed_values][which];
+template <bool BF16, bool SV, bool FULL>
+static DecodeFn instance_of(int which) {
+  return which == 0   ? decode_kernel<BF16, SV, FULL, 1024>
+         : which == 1 ? decode_kernel<BF16, SV, FULL, 1536>
+                      : decode_kernel<BF16, SV, FULL, 2048>;
+}
+static DecodeFn kernel_of(bool bf16, bool signed_values, bool full, int which) {
+  if (signed_values) {
+    if (full) return bf16 ? instance_of<true, true, true>(which) : instance_of<false, true, true>(which);
+    return bf16 ? instance_of<true, true, false>(which) : instance_of<false, true, false>(which);
+  }
+  if (full) return bf16 ? instance_of<true, false, true>(which) : instance_of<false, false, true>(which);
+  return bf16 ? instance_of<true, false, false>(which) : instance_of<false, false, false>(which);
 }
 
-cudaError_t decode_kernel_attrs(bool bf16, bool signed_values, size_t smem) {
+cudaError_t decode_kernel_attrs(bool bf16, bool signed_values, bool full, size_t smem) {
   // the attribute belongs to the kernel on the current device, not to a plan: it only ever grows, so
   // that every plan can launch
   static std::mutex mu;
-  static size_t granted[kMaxDevices][2][2] = {};
+  static size_t granted[kMaxDevices][2][2][2] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
-  size_t& now = granted[dev][bf16][signed_values];
+  size_t& now = granted[dev][bf16][signed_values][full];
   if (smem <= now) return cudaSuccess;
   for (int which = 0; which < 3; ++which) {
-    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel_of(bf16, signed_values, which)),
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel_of(bf16, signed_values, full, which)),
                              cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
@@ -316,7 +324,8 @@ cudaError_t decode_kernel_attrs(bool bf16, bool signed_values, size_t smem) {
 cudaError_t launch_decode(const DecodeParams& p, int sms, int threads, size_t smem, cudaStream_t stream) {
   const unsigned long long per_sm = static_cast<unsigned long long>(p.tokens) * threads / sms;
   const int which = per_sm <= 1060 ? 0 : per_sm <= 2560 ? 1 : 2;
-  return launch_overlapped(kernel_of(p.dtype == TSQ_BF16, p.variant != 0u, which), static_cast<int>(p.tokens), threads, smem, stream, p);
+  const DecodeFn kernel = kernel_of(p.dtype == TSQ_BF16, p.variant != 0u, 4u * p.units == p.chunks, which);
+  return launch_overlapped(kernel, static_cast<int>(p.tokens), threads, smem, stream, p);
 }
 
 }  // namespace tsq

@@ -158,7 +158,7 @@ TwoPassShape two_pass_shape(const EncodeParams& p);
 cudaError_t two_pass_attrs(const EncodeParams& p, const TwoPassShape& s);
 cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, bool few, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeParams& p, int sms, int threads, size_t smem, cudaStream_t stream);
-cudaError_t decode_kernel_attrs(bool bf16, bool signed_values, size_t smem);
+cudaError_t decode_kernel_attrs(bool bf16, bool signed_values, bool full, size_t smem);
 size_t decode_smem_bytes(uint32_t row_bytes, int threads);
 
 }  // namespace tsq
