@@ -52,10 +52,10 @@ KERNEL_SOURCES = {
     "decode": ("tsq_decode.cu", "tsq_device.cuh", "tsq_internal.h"),
 }
 NCU_TRAFFIC = {
-    "encode": {"sha256": "1dbdc786494598ea589af55802901214c9a10a7c8ca680f5875ffa93647865a4",
-               "bytes_per_token": (134335488 + 34698496) / 8192, "hidden": 8192, "dtype": "bf16"},
-    "decode": {"sha256": "5b81cc3ac02735ff1f807c958b25cb59be970609ac00a6114357f4bb577b1d6d",
-               "bytes_per_token": (68648960 + 73330944) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "encode": {"sha256": "baf9476e9d4bda9eb41f4d4afa8f16dfb920496cff71841b49f831613a60de75",  # both kernels
+               "bytes_per_token": (123747328 + 3328 + 134421504 + 63116288) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "decode": {"sha256": "07216779d4f0ba2db981a58b07c9a60216b6517b7a3d4fe69148b1ac166ae1f9",
+               "bytes_per_token": (68634112 + 119722750) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
 KERNEL_NAMES = {"encode": "sizes_kernel + pack_kernel (encode_rows_kernel for few rows)", "decode": "decode_kernel"}
 
