@@ -450,7 +450,6 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
     for (uint32_t i = 0; i < 4u * G; ++i) {
       if (FULL || c0 + 32u * i < p.chunks) cp_async16(dst + 32u * i, xrow + c0 + 32u * i);
     }
-    cp_async_commit();
   }
   const uint32_t next = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn_next);
   const bool sound = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket) == 0u;

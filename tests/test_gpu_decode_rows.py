@@ -59,3 +59,21 @@ def test_rows_of_every_width(dtype, hidden, threads_per_sm, signed):
     got = gpu_decode(plan, torch.from_numpy(blob).cuda(), tokens, ws)
     assert np.array_equal(got, want), np.argwhere(got != want)[:4]
     assert plan.workspace_status(ws) == (0, 0)
+
+
+@pytest.mark.parametrize("hidden", [1000, 4096])
+def test_first_outliers_of_long_calls_in_turn(hidden):
+    # The 32-register instance, whose threads take their first outlier through shared memory: two blobs with other lists in turn, so that
+    # an entry read too early is one of the other blob's.
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tokens = 2562 * sms // ((hidden + 1023) // 1024 * 32)
+    blobs = [blob_of_any_rows(tokens, hidden, R.F16, False, hidden + k) for k in range(2)]
+    plan = B.Plan(torch.float16, hidden, tokens, 6.0, BITS, 0.2)
+    ws = plan.alloc(1)[1]
+    on_device = [torch.from_numpy(blob).cuda() for blob, _ in blobs]
+    want = [torch.from_numpy(y.view(np.int16)).cuda() for _, y in blobs]
+    y = torch.empty((tokens, hidden), dtype=torch.float16, device="cuda")
+    for k in range(40):
+        plan.decode(on_device[k % 2], tokens, y, ws)
+        assert torch.equal(y.view(torch.int16), want[k % 2]), "call %d" % k
+    assert plan.workspace_status(ws) == (0, 0)
