@@ -327,7 +327,8 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
   if (KIND != kKind84) {
     // The exact sums, candidate by candidate, while every level has the packed steps (lane i takes candidate i).  Signed values: a code
     // that needs the clamp is one that a tie has rounded up against the smallest value's, which only the largest value's can be (its quotient lies
-    // qmax above the smallest one's): its elements are counted, and what they add to the sum is taken out of it again.
+    // qmax above the smallest one's).  Each level rounds its own scale, so the largest value may be clamped at one level and one short of
+    // qmax at another: its elements are counted, and what the packed steps have added for them is exchanged for their true difference.
     const int mine = static_cast<int>(min(lane, static_cast<uint32_t>(p.n_bits - 1)));
     const float largest = E::pattern_f32(SV ? pattern_of_key(pmax) : pmax);
     bool plain, packed;
@@ -373,9 +374,9 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
           sum += distortion_group<BF16, SV>(g, make_level2(top), make_level2(low), shn, FULL ? 4u : left <= 0 ? 0u : static_cast<uint32_t>(min(left, 4)));
         }
         int S = cta_sum(sh, static_cast<int>(sum), static_cast<uint32_t>(ci) & 1u, nwarps);
-        if (!all_plain) {  // as the packed steps have it for the largest value, whose difference is 0
-          const int code = (__float2int_rn(__fdiv_rn(largest, top.s)) - top.zp) & 0xff, lower = (__float2int_rn(__fdiv_rn(largest, low.s)) - low.zp) & 0xff;
-          S -= n_largest * abs((code >> shn) - lower);
+        if (!all_plain) {  // the largest value's difference: the packed steps' (codes modulo 256, not clamped) for the true one
+          const int code = __float2int_rn(__fdiv_rn(largest, top.s)) - top.zp, lower = __float2int_rn(__fdiv_rn(largest, low.s)) - low.zp;
+          S += n_largest * (abs((min(code, top.qmax) >> shn) - min(lower, low.qmax)) - abs(((code & 0xff) >> shn) - (lower & 0xff)));
         }
         if (S > p.s_max) break;  // keep the last level that passed
         best.b = p.bits[ci];
