@@ -133,7 +133,9 @@ tsq_status_t tsq_plan_sizes(const tsq_plan_t *plan, int64_t tokens, tsq_sizes_t 
  * Zero a workspace (DEVICE, workspace_bytes, 16-byte aligned) on `cuda_stream`.  Required once
  * before the buffer's first use and after any TSQ_ERR_TIMEOUT; encode and decode leave it ready
  * for the next call.  One workspace serves one call at a time: calls that may overlap on the GPU
- * need separate workspaces.  (Variable-length placement, the prefix sums behind word_off and
+ * need separate workspaces.  A workspace that plans of different max_tokens share is to be initialised
+ * through the plan with the most: it is cleared as far as that plan needs it, and a call of two kernels
+ * (tsq_encode) with more rows writes no row and ends with TSQ_ERR_TIMEOUT.  (Variable-length placement, the prefix sums behind word_off and
  * out_ptr, is resolved inside the encode kernels through this buffer.)
  */
 tsq_status_t tsq_workspace_init(const tsq_plan_t *plan, void *ws_dev, size_t ws_bytes, void *cuda_stream);
@@ -142,7 +144,8 @@ tsq_status_t tsq_workspace_init(const tsq_plan_t *plan, void *ws_dev, size_t ws_
  * Set how long the encoder's device-side waits may last before they give up with TSQ_ERR_TIMEOUT.  The
  * only such wait is for placement in calls of few rows: a row's offsets are the sums over every earlier row, and a
  * row polls the workspace until those rows have published their sizes.  (Calls of more rows go through two kernels that wait
- * for nothing; they end with TSQ_ERR_TIMEOUT when the workspace is not as a finished call leaves it.)  `polls` counts polls of one
+ * for nothing; they end with TSQ_ERR_TIMEOUT when the workspace is not as a finished call leaves it, or was
+ * initialised for fewer rows.)  `polls` counts polls of one
  * row's size: one round trip apart for the first 32, then 1 us apart.  0 restores the built-in limit of 2^20 polls (about one
  * second), which is also what tsq_workspace_init sets.  With the built-in limit a wait can only run out
  * when the workspace was not initialised, is shared by calls that overlap on the GPU, or was

@@ -446,11 +446,11 @@ static int rows_instance(const tsq_plan_t* plan, int64_t tokens) {
   return best;
 }
 
-tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, size_t blob_bytes,
-                        void* ws_dev, size_t ws_bytes, void* cuda_stream) {
-  const tsq_status_t args_ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
-  if (args_ok != TSQ_OK) return args_ok;
+// An encode call whose arguments have been checked.  cleared_rows: EncodeParams.
+static tsq_status_t enqueue_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, void* ws_dev, unsigned long long cleared_rows,
+                                   void* cuda_stream) {
   EncodeParams p = encode_params(plan, x_dev, tokens, blob_dev, ws_dev);
+  p.cleared_rows = static_cast<uint32_t>(cleared_rows);
   if (tokens > direct_rows(plan)) {
     const cudaError_t e = launch_encode_two_pass(p, plan->two_pass, few_rows(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
     g_launches.fetch_add(2);
@@ -463,6 +463,12 @@ tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t token
   const cudaError_t e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, rows_instance(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
   g_launches.fetch_add(1);
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
+}
+
+tsq_status_t tsq_encode(const tsq_plan_t* plan, const void* x_dev, int64_t tokens, void* blob_dev, size_t blob_bytes,
+                        void* ws_dev, size_t ws_bytes, void* cuda_stream) {
+  const tsq_status_t args_ok = check_encode_args(plan, x_dev, tokens, blob_dev, blob_bytes, ws_dev, ws_bytes);
+  return args_ok != TSQ_OK ? args_ok : enqueue_encode(plan, x_dev, tokens, blob_dev, ws_dev, 0, cuda_stream);
 }
 
 static DecodeParams decode_params(const tsq_plan_t* plan, const void* blob_dev, size_t blob_bytes, int64_t tokens, void* y_dev, void* ws_dev) {
@@ -529,12 +535,13 @@ tsq_status_t tsq_encode_noalloc(const tsq_plan_t* plan, const void* x_dev, int64
   if (args_ok != TSQ_OK) return args_ok;
   // The array keeps whatever the last call left (including an unfinished call's tickets): start clean.
   // This also zeroes the generation counter and the recorded capacity: every call through this entry
-  // point runs as generation 1, so the wrap-around path that reads the capacity is never taken here.
+  // point runs as generation 1, so the wrap-around path that reads the capacity is never taken here, and
+  // the rows that have been cleared are told with the call.
   if (cudaMemsetAsync(ws, 0, plan->workspace_bytes, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
     cudaGetLastError();
     return TSQ_ERR_CUDA;
   }
-  return tsq_encode(plan, x_dev, tokens, blob_dev, blob_bytes, ws, kStaticWsBytes, cuda_stream);
+  return enqueue_encode(plan, x_dev, tokens, blob_dev, ws, plan->max_tokens, cuda_stream);
 }
 
 static unsigned long long payload_of(unsigned long long tokens, unsigned long long words, unsigned long long outliers) {

@@ -404,6 +404,8 @@ template <int NW>
 struct PackShared {
   uint32_t cnt[NW];  // outliers by warp
   uint32_t word_off, out_base;
+  uint32_t next_turn;  // of the cells, in the next call
+  uint32_t sound;      // the workspace is as a finished call leaves it and has cells for all of this call's rows
 };
 
 // Words and outliers before row `tile`, by one warp (lane 0's result counts): the rows of its block of 32, the blocks of 32 before it in
@@ -452,16 +454,22 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (FULL || c0 + 32u * i < p.chunks) cp_async16(dst + 32u * i, xrow + c0 + 32u * i);
     }
   }
-  const uint32_t next = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn_next);
-  const bool sound = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket) == 0u;
   const uint32_t entry = static_cast<uint32_t>(p.desc[2u * tile]);
   const float s = reinterpret_cast<const float*>(p.blob + p.lay.off_scale)[tile];
   if (warp == nwarps - 1u) {
+    // The control block's words by one warp per CTA: every CTA of the call reads the same line, which takes one request after the other
+    // (us of a call with 2 words read by every warp / 3 by every warp / 3 by one warp: 2048 x 5120 22.0 / 24.5 / 18.6, 8192 x 8192 70.6 / 74.0 / 68.7,
+    // signed pair 2048 x 5120 40.8 / 44.6 / 38.3).
+    const uint32_t next = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn_next);
+    const uint32_t ticket = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket);
+    const uint32_t has_cells = *reinterpret_cast<volatile const uint32_t*>(&p.ws->desc_capacity);
     uint32_t w, o;
     sums_before(p, next, tile, lane, &w, &o);
     if (lane == 0) {
       sh.word_off = w;
       sh.out_base = o;
+      sh.next_turn = next;
+      sh.sound = ticket == 0u && p.tokens <= max(has_cells, p.cleared_rows) ? 1u : 0u;
     }
   }
   const uint32_t thr2 = p.thr16 * 0x10001u;
@@ -535,7 +543,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   }
   __syncthreads();
   const uint32_t word_off = sh.word_off, out_base = sh.out_base, word_end = word_off + agg_w, out_end = out_base + row_cnt;
-  uint32_t status = sound && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
+  uint32_t status = sh.sound != 0u && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
   if (status == TSQ_OK) {
     uint32_t* wrow = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
     if (!SV && mode >= kOneUp) {
@@ -623,14 +631,14 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
       // (the slots of this call's rows carry no tag, and the other CTAs are still reading them)
       next_generation(p, *reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u, p.tokens);
-      p.ws->sums_turn = next;
+      p.ws->sums_turn = sh.next_turn;
     }
   }
   // ---- the cells that the next call adds to ----
   if (blockIdx.x < 32u) {
     const uint32_t blocks = max(p.ws->desc_capacity, p.tokens) >> 5;
     for (uint32_t i = blockIdx.x * nt + tid; i < blocks; i += min(gridDim.x, 32u) * nt) {
-      unsigned long long* c = p.desc + 64ull * i + 1u + 2u * (next & 1u);
+      unsigned long long* c = p.desc + 64ull * i + 1u + 2u * (sh.next_turn & 1u);
       c[0] = 0ull;
       if ((i & 31u) == 0u) c[4] = 0ull;
       if ((i & 1023u) == 0u) c[8] = 0ull;

@@ -61,7 +61,9 @@ __host__ __device__ inline BlobLayout make_layout(uint32_t hidden, unsigned long
 //   desc[2 t + 1]  cells of calls of two kernels: plane words << 32 | outliers of a whole block of rows, two of each, used in turn.  Block of 32
 //                  rows that starts at row t: cells t and t + 1; of 1024 rows: t + 2, t + 3; of 32768 rows: t + 4, t + 5.  A call
 //                  adds to the cells of its turn, which the call before it has left at 0, and clears those of the other.
-// (Where a word is does not depend on the number of tokens, so a workspace may serve plans of different sizes.)
+// Where a word is does not depend on the number of tokens, so a workspace may serve plans of different sizes, as far as it has been
+// initialised: cells must be 0 when a call adds to them, and every call clears those of desc_capacity rows.  A call of two kernels with more
+// rows than that writes no row and ends with TSQ_ERR_TIMEOUT.  (Slots need no such bound: their tags tell.)
 struct WsControl {
   uint32_t gen;          // generation of the last finished encode
   uint32_t ticket;       // next tile to hand out (self-resetting)
@@ -69,7 +71,7 @@ struct WsControl {
   uint32_t err;          // first error of the running encode
   uint32_t enc_status;   // first encode error since init (sticky)
   uint32_t dec_status;   // first decode error since init (sticky)
-  uint32_t desc_capacity;  // tiles the descriptor array holds (set by init)
+  uint32_t desc_capacity;  // rows whose slots and cells init has cleared
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
   uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut or kCallEnded, only ever grows
   uint32_t sums_turn;      // calls of two kernels: whose turn the cells are, read by the first and written by the second kernel
@@ -93,6 +95,7 @@ struct EncodeParams {
   int32_t n_bits;
   int32_t bits[8];
   int32_t s_max;                             // floor(delta * H), clamped to [-1, INT32_MAX]
+  uint32_t cleared_rows;                     // rows whose slots and cells the call itself clears before its kernels (0: see desc_capacity)
   uint32_t direct_tiles;                     // one-kernel encoder: 1 = row index = CTA index (every CTA resident), 2 = rows by ticket
   uint32_t dtype;
   uint32_t variant;                          // 0: sign + magnitude codes; 1: codes of the signed values

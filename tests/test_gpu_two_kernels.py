@@ -111,3 +111,27 @@ def test_under_capture_and_on_two_streams():
     torch.cuda.synchronize()
     assert_blobs_equal(blob.cpu().numpy(), refs[1])
     assert np.array_equal(synth.raw_u16(x.cpu()), R.decode(refs[1]))
+
+
+def test_workspace_initialised_for_fewer_rows():
+    # large enough for the plan, cleared for a smaller one only: no row is written, and the status says so; calls within what was cleared, and calls
+    # of one kernel, are not concerned
+    H, bits = 256, [2, 4, 8]
+    big, small = B.Plan(torch.float16, H, 3000, 6.0, bits, 0.2), B.Plan(torch.float16, H, 1400, 6.0, bits, 0.2)
+    x = rows_of_every_kind(3000, H, torch.float16, 8)
+    ws = torch.full((big.sizes(1)[1],), 0x11, dtype=torch.uint8, device="cuda")
+    small.workspace_init(ws)
+    for T in (1400, 100, 1399):
+        check(big, x[:T], ws, bits)
+    assert big.workspace_status(ws) == (0, 0)
+    for T in (1401, 3000):
+        blob = torch.full((big.sizes(T)[0],), 0xA5, dtype=torch.uint8, device="cuda")
+        big.encode(x[:T].cuda(), blob, ws)
+        assert big.blob_info(blob).status == 7 == big.workspace_status(ws)[0]
+        lay = R.layout(H, T, 8, 0)
+        assert (blob[lay["word_off"]:] == 0xA5).all()
+        small.workspace_init(ws)
+    big.workspace_init(ws)
+    for T in (3000, 1400, 3000):
+        check(big, x[:T], ws, bits)
+    assert big.workspace_status(ws) == (0, 0)

@@ -2,7 +2,7 @@
 
 Some callers of the codec may not allocate device memory at the point where they encode (a serving
 loop that runs with a frozen memory pool, a plug-in inside a runtime that owns all device memory).
-For them the library keeps the encoder's look-back scratch in a fixed array of its own.  This test
+For them the library keeps the encoder's placement scratch in a fixed array of its own.  This test
 calls that entry point through the C ABI and requires the very same blob, byte for byte over every
 meaningful section, as the ordinary entry point gives with a caller-allocated workspace: twice in a
 row on different inputs, because the second call meets the first call's leftovers in the shared array.
@@ -49,6 +49,18 @@ def test_noalloc_matches_workspace_encode_twice(dtype):
         code = R.F16 if dtype == torch.float16 else R.BF16
         ref_blob = R.encode(synth.raw_u16(x.cpu()), code, 6.0, [2, 4, 8], 0.2)
         assert np.array_equal(synth.raw_u16(y.cpu()), R.decode(ref_blob))
+
+
+@pytest.mark.parametrize("variant", [B.VARIANT_MAGNITUDES, B.VARIANT_SIGNED_VALUES])
+def test_noalloc_calls_of_two_kernels(variant):
+    # the rows' sizes are summed in cells that every call has to find at 0: longer and shorter calls in turn, the longest the plan takes
+    plan = B.Plan(torch.float16, 256, 3000, 6.0, [2, 4, 8], 0.2, variant=variant)
+    for call, tokens in enumerate((3000, 1400, 3000, 40, 2999)):
+        x = _input(200 + call, tokens, 256, torch.float16)
+        blob = torch.zeros(plan.sizes(tokens)[0], dtype=torch.uint8, device="cuda")
+        plan.encode_noalloc(x.cuda(), blob)
+        torch.cuda.synchronize()
+        assert_blobs_equal(blob.cpu().numpy(), R.encode(synth.raw_u16(x), R.F16, 6.0, [2, 4, 8], 0.2, signed_values=variant == B.VARIANT_SIGNED_VALUES))
 
 
 def test_noalloc_refuses_plans_beyond_its_scratch():
