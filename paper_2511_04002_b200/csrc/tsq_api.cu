@@ -426,7 +426,7 @@ static int64_t direct_rows(const tsq_plan_t* plan) {
 // 8192 x 1024 22.5 / 24.0, 1000 x 8192 16.8 / 14.8.
 static bool few_rows(const tsq_plan_t* plan, int64_t tokens) {
   const int64_t segments = (plan->units + 31u) / 32u;
-  return segments <= 5 && (segments == 1 || tokens * segments <= 80 * static_cast<int64_t>(plan->sms));
+  return segments <= kFewSegments && (segments == 1 || tokens * segments <= 80 * static_cast<int64_t>(plan->sms));
 }
 
 // Instance of the one-kernel encoder: 128, 80 or 64 registers, so more CTAs per SM with each.  The one

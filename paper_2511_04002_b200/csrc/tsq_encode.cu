@@ -709,7 +709,7 @@ TwoPassShape two_pass_shape(const EncodeParams& p) {
                      static_cast<size_t>(pack_warps) * (2048u * static_cast<size_t>(groups) + sizeof(uint16_t) * kListCap)};
   };
   s.pack = pack_shape(segs <= 16 ? 2 : 4);
-  s.pack_few = segs <= 8 ? pack_shape(1) : s.pack;  // (few_rows in tsq_api.cu)
+  s.pack_few = segs <= kFewSegments ? pack_shape(1) : s.pack;  // (few_rows in tsq_api.cu)
   return s;
 }
 

@@ -157,6 +157,7 @@ struct TwoPassShape {
   bool sizes_full;
   PackShape pack, pack_few;  // pack_few: for calls that do not fill the device several times over
 };
+constexpr int kFewSegments = 5;  // rows of up to 5 x 1024 elements may take pack_few
 TwoPassShape two_pass_shape(const EncodeParams& p);
 cudaError_t two_pass_attrs(const EncodeParams& p, const TwoPassShape& s);
 cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s, bool few, cudaStream_t stream);
