@@ -493,8 +493,9 @@ static DecodeParams decode_params(const tsq_plan_t* plan, const void* blob_dev, 
 
 static tsq_status_t launch_decode_part(const tsq_plan_t* plan, DecodeParams& p, void* cuda_stream) {
   const int64_t tokens = p.tokens;
-  // A call of at most a row per SM lets the next grid in early (0.6 us per call at 64 rows).  A longer one does not: the next grid's CTAs
-  // wait where its own later ones should run (600 x 8192 5.3 us without, 7.2 us with; 16384 x 1024 16.5 and 20.4 us).
+  // A call of at most a row per SM lets the next grid in early (0.6 us per call at 64 rows).  A longer one does not, because it was slower
+  // (600 x 8192 5.3 us without, 7.2 us with; 16384 x 1024 16.5 and 20.4 us).  Why is not known: the next grid's CTAs are set up only once
+  // every CTA of this one has started, so they take the place of none.
   p.overlap_next = tokens <= static_cast<int64_t>(plan->sms) ? 1u : 0u;
   const cudaError_t e = launch_decode(p, plan->sms, plan->threads, plan->dec_smem, static_cast<cudaStream_t>(cuda_stream));
   g_launches.fetch_add(1);

@@ -13,10 +13,10 @@
 // x is read twice.  The forms that read it once (rows in shared memory or in registers, placement at once, by look-back, or put
 // off by a row's time) were all slower: in token order every row waits for the slowest of the rows before it, and a few rows in a
 // hundred take Algorithm 1 further than the first candidate (8192 x 8192 bf16 / 32768 x 4096 bf16 with 1 % outliers, us: persistent CTAs with a
-// ring of packed rows 87 / 190, one CTA per row 104 / 281, placement a row later 87 / 349, these kernels 65 / 126).
+// ring of packed rows 87 / 190, one CTA per row 104 / 281, placement a row later 87 / 349, these kernels at that time 65 / 126).
 //
-// What binds: DRAM and instruction issue about equally.  The two kernels move 332 MB at 8192 x 8192 bf16 (x twice, 8 % of the
-// second time from L2; 51 us at the copy rate) and issue every other to two cycles out of three.  So the passes work on two 16-bit elements
+// What binds: DRAM and instruction issue about equally.  The two kernels move about 320 MB at 8192 x 8192 bf16 (x twice; 50 us at
+// the copy rate) and issue in two cycles out of three.  So the passes work on two 16-bit elements
 // per 32-bit register and on two binary32 values per 64-bit register wherever they can, and what a row costs once is kept short.
 //
 // Arithmetic contract: the codes equal  clamp(rint(m / s) - zp, 0, Qmax)  with the IEEE binary32
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
       for (int i = 0; i < 4 * C; ++i) acc = add_differences<BF16>(x[i], hi2, t, acc);
       const int S = cta_sum(sh, sum_of(acc), 0u, nwarps);
       best.b = 8;
-      if (S <= p.s_max) {  // the 4-bit candidate may pass (3 to 7 % of the rows)
+      if (S <= p.s_max) {  // the 4-bit candidate may pass (0 to 6 % of a tensor's rows, and for nearly all of those it does)
         uint32_t turn_of_sum = 1u;
         best.b = descend<BF16>(
             p, x, range, S,

@@ -247,7 +247,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-// hi / Q, correctly rounded for every 16-bit hi (as in quick_level); *tie: Q divides hi's significand.
+// hi / Q, correctly rounded for every 16-bit hi (one Newton step on hi * fl(1 / Q)); *tie: Q divides hi's significand.
 template <int Q>
 __device__ __forceinline__ float divide_by(float hi, bool* tie) {
   constexpr float kInv = 1.0f / static_cast<float>(Q);

@@ -49,7 +49,7 @@ __device__ __forceinline__ bool given_up(const EncodeParams& p, uint32_t gen4, u
 // so the wait is one round trip past the last predecessor's store.  The sums are left by warp; the caller adds them up
 // behind its barrier.  (A walk back by one warp took 3600 of the 10100 cycles of a 64 x 4096 call: its first look found
 // nothing published, and every retry was another round trip.)  With many rows a thread's polls go out in batches, so that they
-// share a round trip: short rows have few threads to share them (2048 x 1024: 16.4 us, 19.3 in the pipelined kernel).
+// share a round trip: short rows have few threads to share them.
 constexpr uint32_t kPollBatch = 4u;
 template <bool BATCHES, int NW>
 __device__ __forceinline__ void direct_offsets(const EncodeParams& p, uint32_t gen4, uint32_t tile, RowShared<NW>& sh) {
@@ -110,8 +110,8 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
 // MAXT: the largest CTA the instance is launched with (rows of up to 8192 elements get the 256-thread instances).  MINB: 2, 3 or
 // 4 such CTAs' worth of registers, 128, 80 or 64 to a thread: a CTA spends most of its time waiting (its row, its barriers,
 // the rows before it), so a call of more rows than fit at once runs faster the more of them do.  SV: the signed-values variant.
-// DIRECT: calls of a few rows per SM (kByIndex, kByTicket): a row's offsets are read straight from the sizes of the rows before
-// it (direct_offsets) instead of walked back to.  With at most one row per SM (kByIndex) every CTA is resident, so row = CTA
+// DIRECT: where a row's number comes from (kByIndex, kByTicket); its offsets are read straight from the sizes of the rows before
+// it (direct_offsets).  With at most one row per SM (kByIndex) every CTA is resident, so row = CTA
 // index needs no ticket.
 // TOP84: the candidates end in 4 and 8 bits (magnitudes): the 4-bit candidate decided without forming codes (add_differences), so that a row's
 // sizes are published before its planes are formed, and the rows behind it find them when theirs are.

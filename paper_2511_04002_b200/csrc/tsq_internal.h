@@ -107,7 +107,7 @@ struct EncodeParams {
   unsigned long long* totals;                // where the part's end offsets go (host memory), or null
 };
 
-// The two widest candidates are 4 and 8 bits of a magnitude plan: the first decision can be taken on the 8-bit planes.
+// The two widest candidates are 4 and 8 bits of a magnitude plan: the first decision can be taken without forming codes (add_differences).
 inline bool ends_in_4_and_8(const EncodeParams& p) {
   return p.variant == 0u && p.n_bits >= 2 && p.bits[p.n_bits - 1] == 8 && p.bits[p.n_bits - 2] == 4;
 }

@@ -1,4 +1,4 @@
-"""The distortion sum that the two-kernel encoder forms without codes (add_differences, step_error in csrc/tsq_encode.cu), restated in numpy
+"""The distortion sum that the encoders form without codes (add_differences, step_error in csrc/tsq_encode_device.cuh), restated in numpy
 for every 16-bit magnitude of a row: with the corrections it is the sum over the true codes, without them it is never above it; and the
 one-FMA codes of the levels of 2, 3 and 4 bits.  The reciprocal instruction's last bits are not known here: everything has to hold
 for two units more and less in the factor (its error is below one, the product's half)."""

@@ -1,5 +1,5 @@
-"""Calls of a few rows per SM (offsets read directly, last row's CTA ends the call) at the edges of their range, several on one
-workspace, mixed with calls of the other kernels."""
+"""Calls of a few rows per SM (one kernel, offsets read directly, last row's CTA ends the call) at the edges of their range, several on one
+workspace, mixed with calls of two kernels."""
 import numpy as np
 import pytest
 import torch
@@ -11,6 +11,21 @@ from tests._parity import assert_blobs_equal, gpu_decode, gpu_encode
 from tests.test_gpu_parity import rand16
 
 pytestmark = pytest.mark.gpu
+
+
+def longest_call_of_one_kernel(plan, x, blob, ws):
+    """Rows of the longest call that takes one launch: asked of the library, which knows its kernels' occupancy."""
+    def launches(T):
+        before = B.kernel_launch_count()
+        plan.encode(x[:T], blob, ws)
+        return B.kernel_launch_count() - before
+
+    one, two = 1, x.shape[0]
+    assert launches(one) == 1 and launches(two) == 2
+    while two - one > 1:
+        T = (one + two) // 2
+        one, two = (T, two) if launches(T) == 1 else (one, T)
+    return one
 
 
 @pytest.mark.parametrize("hidden", [8, 1032, 4096, 16384])
@@ -57,16 +72,17 @@ def test_many_calls_back_to_back_on_one_stream():
 
 @pytest.mark.parametrize("bits", [[2, 4, 8], [2, 3, 6]])
 @pytest.mark.parametrize("dtype,hidden", [(torch.float16, 1032), (torch.bfloat16, 5120)])
-def test_every_instance_and_the_line_to_the_pipelined_kernel(dtype, hidden, bits):
+def test_every_instance_and_the_line_to_the_two_kernels(dtype, hidden, bits):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    sizes = [3 * sms + 5, 4 * sms + 9, 9 * sms, 10 * sms, 10 * sms + 1, 14 * sms, 14 * sms + 1]
-    plan = B.Plan(dtype, hidden, max(sizes), 6.0, bits, 0.2)
-    ws = plan.alloc(1)[1]
-    x = rand16((max(sizes), hidden), dtype, seed=hidden, scale=2.0, outlier_rate=0.01)
+    plan = B.Plan(dtype, hidden, 14 * sms + 1, 6.0, bits, 0.2)
+    blob, ws = plan.alloc(14 * sms + 1)
+    x = rand16((14 * sms + 1, hidden), dtype, seed=hidden, scale=2.0, outlier_rate=0.01)
     x[::3] = (x[::3].float().abs() * 0.2).to(dtype)              # rows without outliers
     x[1::5] = (x[1::5].float().abs() ** 3 * 0.05).to(dtype)      # rows that descend
     x[7::29] = (x[7::29].float().abs() * 0.1 + 3.0).to(dtype)    # rows that need the division instruction
-    for T in sizes:
+    line = longest_call_of_one_kernel(plan, x.cuda(), blob, ws)
+    # with rows of 5120 elements an SM holds 3, 4 and 6 CTAs of the three instances
+    for T in (3 * sms + 5, 4 * sms + 9, 5 * sms, line, line + 1, 9 * sms, 14 * sms + 1):
         blob = torch.zeros(plan.sizes(T)[0], dtype=torch.uint8, device="cuda")
         _, got, _ = gpu_encode(plan, x[:T], ws=ws, blob=blob)
         assert_blobs_equal(got, R.encode(synth.raw_u16(x[:T]), R.F16 if dtype == torch.float16 else R.BF16, 6.0, bits, 0.2))
@@ -74,7 +90,7 @@ def test_every_instance_and_the_line_to_the_pipelined_kernel(dtype, hidden, bits
 
 
 @pytest.mark.parametrize("hidden,signed", [(8200, False), (8200, True)])
-def test_long_rows_and_the_line_to_the_look_back(hidden, signed):
+def test_long_rows_and_the_line_to_the_two_kernels(hidden, signed):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     variant = B.VARIANT_SIGNED_VALUES if signed else B.VARIANT_MAGNITUDES
     plan = B.Plan(torch.bfloat16, hidden, 64 * sms + 1, 6.0, [2, 4, 8], 0.2, variant=variant)
@@ -82,25 +98,25 @@ def test_long_rows_and_the_line_to_the_look_back(hidden, signed):
     x = rand16((64 * sms + 1, hidden), torch.bfloat16, seed=7, scale=2.0, outlier_rate=0.01)
     x[::3] = (x[::3].float().abs() * 0.2).to(torch.bfloat16)
     x = x.cuda()
-    few = 7 * sms + 1
-    _, got, _ = gpu_encode(plan, x[:few].cpu(), ws=ws)
-    if not signed:
-        assert_blobs_equal(got, R.encode(synth.raw_u16(x[:few].cpu()), R.BF16, 6.0, [2, 4, 8], 0.2))
-    # both sides of the line decode to the same rows, in between to those of a short call
-    y = [torch.empty_like(x) for _ in range(2)]
-    for k, T in enumerate((64 * sms, 64 * sms + 1)):
+    line = longest_call_of_one_kernel(plan, x, blob, ws)
+    for T in (line, line + 1, 7 * sms + 1):
+        _, got, _ = gpu_encode(plan, x[:T].cpu(), ws=ws)
+        if T <= line + 1 or not signed:
+            assert_blobs_equal(got, R.encode(synth.raw_u16(x[:T].cpu()), R.BF16, 6.0, [2, 4, 8], 0.2, signed_values=signed))
+    # the rows of a call of one kernel decode as in calls of two
+    y = [torch.empty_like(x) for _ in range(3)]
+    sizes = (line, line + 1, 64 * sms + 1)
+    for k, T in enumerate(sizes):
         plan.encode(x[:T], blob, ws)
         plan.decode(blob, T, y[k][:T], ws)
-    plan.encode(x[:few], blob, ws)
-    short = torch.empty_like(x[:few])
-    plan.decode(blob, few, short, ws)
     assert plan.workspace_status(ws) == (0, 0)
-    assert torch.equal(y[0][:64 * sms].view(torch.int16), y[1][:64 * sms].view(torch.int16))
-    assert torch.equal(y[0][:few].view(torch.int16), short.view(torch.int16))
+    for k in (0, 1):
+        assert torch.equal(y[k][:sizes[k]].view(torch.int16), y[k + 1][:sizes[k]].view(torch.int16))
 
 
 def test_a_wait_that_runs_out_ends_a_call_of_many_turns():
-    # row 0 is never produced: one limit's worth of waiting for the whole call, not one for each turn of CTAs
+    # row 0 is never produced.  Two kernels, which wait for nothing: the call ends at once.  Parts of a host-buffer call, one kernel each and the
+    # longest calls of it, in several turns of CTAs: one limit's worth of waiting for the part, not one for each turn
     T, H = 30 * torch.cuda.get_device_properties(0).multi_processor_count, 8200
     plan = B.Plan(torch.bfloat16, H, T, 6.0, [2, 4, 8], 0.2)
     blob, ws = plan.alloc(T)
@@ -114,6 +130,17 @@ def test_a_wait_that_runs_out_ends_a_call_of_many_turns():
     torch.cuda.synchronize()
     assert plan.workspace_status(ws)[0] == 7 and plan.blob_info(blob).status == 7
     assert e0.elapsed_time(e1) < 40.0
+    plan.workspace_init(ws)
+    plan.workspace_set_wait_limit(ws, 3000)
+    ws.view(torch.int32)[1] = 1
+    x_host = x.cpu().pin_memory()
+    blob_host = torch.empty(blob.numel(), dtype=torch.uint8).pin_memory()
+    e0.record()
+    with pytest.raises(B.TsqError) as e:
+        plan.encode_host(x_host, blob_host, x, blob, ws)
+    e1.record()
+    torch.cuda.synchronize()
+    assert e.value.status == 7 and plan.workspace_status(ws)[0] == 7 and e0.elapsed_time(e1) < 40.0
     plan.workspace_init(ws)
     _, got, _ = gpu_encode(plan, x[:5].cpu(), ws=ws)
     assert_blobs_equal(got, R.encode(synth.raw_u16(x[:5].cpu()), R.BF16, 6.0, [2, 4, 8], 0.2))

@@ -48,9 +48,8 @@ def test_every_candidate_is_exercised(dtype, delta, bits):
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
 @pytest.mark.parametrize("shape", [(400, 10240), (330, 16384), (600, 8200), (700, 4104), (1000, 72), (450, 8192), (2000, 1024)])
-def test_many_rows_take_the_pipelined_or_the_row_kernel(dtype, shape):
-    # more rows than twice the SM count: rows of up to 8192 elements go through the pipelined kernel,
-    # longer ones through the row-at-a-time kernel
+def test_many_rows_take_one_or_two_kernels(dtype, shape):
+    # more rows than twice the SM count: calls of one kernel with several rows per SM, and of two
     x = rand16(shape, dtype, seed=shape[0] * 1000 + shape[1], scale=2.0, outlier_rate=0.02)
     x[::7] = (x[::7].float().abs() ** 3 * 0.05).to(dtype) * torch.sign(x[::7].float()).to(dtype)   # rows that descend
     full_parity(x, 6.0, [2, 3, 4, 8], 0.2, check_cross=False)
@@ -60,7 +59,7 @@ def test_many_rows_take_the_pipelined_or_the_row_kernel(dtype, shape):
 @pytest.mark.parametrize("shape", [(500, 4096), (420, 8192), (900, 264)])
 @pytest.mark.parametrize("delta", [0.2, 1e9])
 def test_many_rows_some_needing_the_division_instruction(dtype, shape, delta):
-    # the pipelined kernel's rolled path: rows whose zero-point is large (a narrow range far from zero) and,
+    # the ways apart from the packed steps: rows whose zero-point is large (a narrow range far from zero) and,
     # for bf16, rows whose scale is far outside the range of the FMA quotient, among ordinary rows
     T, H = shape
     x = rand16(shape, dtype, seed=T * 31 + H, scale=1.5, outlier_rate=0.0).float()
@@ -215,9 +214,8 @@ def test_c5_sweep(i_tok, i_rate, i_dtype):
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
 def test_long_rows_with_few_and_very_many_outliers_mixed(dtype):
-    # hidden 8192, more rows than a persistent CTA keeps in flight many times over, and rows with 0, 1, about 600
-    # and about 4000 outliers next to one another: the rows whose outliers do not fit a CTA's list are placed
-    # while ordinary rows queue behind them
+    # hidden 8192, many rows per SM, and rows with 0, 1, about 600 and about 4000 outliers next to one another: warps whose
+    # outliers fit their list beside warps whose do not
     T, H = 3100, 8192
     g = torch.Generator().manual_seed(77)
     v = torch.randn((T, H), generator=g)
@@ -239,7 +237,7 @@ def test_long_rows_with_few_and_very_many_outliers_mixed(dtype):
 
 @pytest.mark.parametrize("hidden,max_outliers", [(4096, 0), (5120, 0), (1000, 0), (4096, 300000)])
 def test_runs_of_rows_that_are_mostly_outliers(hidden, max_outliers):
-    # every persistent CTA meets several rows in a row whose outliers exceed its lists (a third to all of the row),
+    # several rows in a row whose outliers exceed the warps' lists (a third to all of the row),
     # between stretches of ordinary rows; the last case also runs out of CSR capacity in the middle of such a row
     T = 1500
     g = torch.Generator().manual_seed(hidden)

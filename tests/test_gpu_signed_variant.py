@@ -102,7 +102,7 @@ def test_c1_and_c3_workloads():
 
 
 def test_runs_of_rows_that_are_mostly_outliers():
-    # rows whose outliers exceed a persistent CTA's lists, several in a row, between stretches of ordinary rows
+    # rows whose outliers exceed the warps' lists, several in a row, between stretches of ordinary rows
     T, H = 1200, 4096
     g = torch.Generator().manual_seed(4096)
     v = torch.randn((T, H), generator=g)

@@ -1,9 +1,10 @@
 """A device-side wait that runs out ends in TSQ_ERR_TIMEOUT, quickly, and the buffers work again afterwards.
 
 The failure is made on the host: after the workspace is initialised, its ticket counter is set to 1, so that
-row 0 is never handed out and every other row's placement look-back waits for sizes that nobody publishes.  With
+row 0 is never handed out and every other row of a one-kernel call waits for sizes that nobody publishes.  With
 a wait limit of a few thousand polls every such wait gives up within milliseconds; nothing faults or spins
-without bound, and the kernel returns the status."""
+without bound, and the kernel returns the status.  (A call of two kernels waits for nothing: it finds the counter
+not 0, writes no row and returns the same status.)"""
 import time
 
 import numpy as np
@@ -20,7 +21,8 @@ TIMEOUT = 7
 
 
 @pytest.mark.parametrize("tokens,hidden", [(200, 512),     # one CTA per row, rows handed out by ticket (more rows than SMs)
-                                           (700, 1024)])   # the persistent kernel for many rows
+                                           (700, 1024),    # several rows per SM
+                                           (1500, 1024)])  # two kernels
 def test_wait_runs_out_into_timeout_status_and_workspace_recovers(tokens, hidden):
     g = torch.Generator().manual_seed(tokens)
     x_cpu = (torch.randn((tokens, hidden), generator=g) * 1.5).to(torch.float16).contiguous()

@@ -1,5 +1,6 @@
-"""The codes by one FMA, the quick 8-bit level and the certain differences on the bit-planes, checked on the CPU against the
-definitions: clamp(rint(fl(m / s))) with s = fl(hi / 127), and |(q >> 4) - low|."""
+"""The scale of the 8-bit level and its codes by one FMA (divide_by, middle_up, one_fma_factor in csrc/tsq_encode_device.cuh), checked on
+the CPU for every 16-bit maximum against the definition, clamp(rint(fl(m / s))) with s = fl(hi / 127); and what the sum of differences
+without codes rests on: |(q >> 4) - low| is 0 or 1, and which it is follows from the 8-bit code but next to a step."""
 import numpy as np
 import pytest
 
@@ -17,7 +18,7 @@ def fma(a, b, c):
 
 
 @pytest.mark.parametrize("fmt", ["f16", "bf16"])
-def test_quick_level_and_one_fma_codes_for_every_maximum(fmt):
+def test_scale_and_one_fma_codes_for_every_maximum(fmt):
     v = patterns(fmt)
     s = (v / f32(127)).astype(f32)
     ok = (s >= 2.0 ** -60) & (s <= 2.0 ** 60)
@@ -40,7 +41,7 @@ def test_quick_level_and_one_fma_codes_for_every_maximum(fmt):
             assert np.array_equal(np.rint((m / s[i]).astype(f32)), np.rint(m.astype(np.float64) * np.float64(factor[i]))), v[i]
 
 
-def test_certain_differences_match_the_definition():
+def test_differences_are_at_most_one_and_lie_between_the_steps():
     rng = np.random.default_rng(0)
     for hi in np.concatenate([rng.uniform(0.5, 60000, 300), [1.0, 127.0, 254.0]]).astype(np.float16).astype(f32):
         m = patterns("f16")
