@@ -52,10 +52,10 @@ KERNEL_SOURCES = {
     "decode": ("tsq_decode.cu", "tsq_device.cuh", "tsq_internal.h"),
 }
 NCU_TRAFFIC = {
-    "encode": {"sha256": "baf9476e9d4bda9eb41f4d4afa8f16dfb920496cff71841b49f831613a60de75",  # both kernels
-               "bytes_per_token": (123747328 + 3328 + 134421504 + 63116288) / 8192, "hidden": 8192, "dtype": "bf16"},
-    "decode": {"sha256": "07216779d4f0ba2db981a58b07c9a60216b6517b7a3d4fe69148b1ac166ae1f9",
-               "bytes_per_token": (68634112 + 119722750) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "encode": {"sha256": "5a49023ccf10a782890c3d493245c8ae20b796c407656da3e52aa0b62b8118ae",  # both kernels
+               "bytes_per_token": (134260000 + 6280000 + 122980000 + 62720000) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "decode": {"sha256": "d8ab6337f0ac1e5b270ed71b13b2abfb4f0f596dac117d2a668a47a0e4133a3f",
+               "bytes_per_token": (68620000 + 132850000) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
 KERNEL_NAMES = {"encode": "sizes_kernel + pack_kernel (encode_rows_kernel for few rows)", "decode": "decode_kernel"}
 

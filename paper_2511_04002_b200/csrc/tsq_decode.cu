@@ -3,7 +3,7 @@
 // outliers of T_above over their slots.  One CTA per token row; the row is assembled in shared
 // memory and leaves through one bulk asynchronous store.
 //
-// What bounds it: bytes, for calls of many rows (8192 x 8192 with every row at 8 bits: 34.6 to 35.6 us for 201 MB; a kernel that only widens as many bytes
+// What bounds it: bytes, for calls of many rows (8192 x 8192 with every row at 8 bits: 34.6 to 35.8 us for 201 MB; a kernel that only widens as many bytes
 // to 16 bits takes 33.4 us, 32768 x 4096 with 1 % outliers 69.5 against 63 us), two dependent round trips to memory and the launch for the others.
 // Threads in flight decide more than instructions: 32768 x 4096 took 77 us with 40 registers a thread and 302 instructions per warp and
 // group, 71.6 us with 32 and 379.  CTAs that stay and take several rows, and warps that send their 2 KB of a row by themselves, were
