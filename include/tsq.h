@@ -143,9 +143,9 @@ tsq_status_t tsq_workspace_init(const tsq_plan_t *plan, void *ws_dev, size_t ws_
 /*
  * Set how long the encoder's device-side waits may last before they give up with TSQ_ERR_TIMEOUT.  The
  * only such wait is for placement in calls of few rows: a row's offsets are the sums over every earlier row, and a
- * row polls the workspace until those rows have published their sizes.  (Calls of more rows go through two kernels that wait
- * for nothing; they end with TSQ_ERR_TIMEOUT when the workspace is not as a finished call leaves it, or was
- * initialised for fewer rows.)  `polls` counts polls of one
+ * row polls the workspace until those rows have published their sizes.  (Calls of more rows go through two kernels: the second
+ * starts while the first still runs and polls for rows that are being sized, with the built-in limit whatever is set here.  They end
+ * with TSQ_ERR_TIMEOUT when the workspace is not as a finished call leaves it, or was initialised for fewer rows.)  `polls` counts polls of one
  * row's size: one round trip apart for the first 32, then 1 us apart.  0 restores the built-in limit of 2^20 polls (about one
  * second), which is also what tsq_workspace_init sets.  With the built-in limit a wait can only run out
  * when the workspace was not initialised, is shared by calls that overlap on the GPU, or was
@@ -174,7 +174,7 @@ tsq_status_t tsq_encode(const tsq_plan_t *plan, const void *x_dev, int64_t token
  * all device memory, a thread that must never take the allocator's lock).  For them the placement
  * scratch lives in a fixed array inside the library image instead of in a caller-allocated workspace;
  * x_dev and blob_dev are still the caller's.
- *   - Limit: the plan's max_tokens must be <= 16384 (the array is 256 KiB + 256 B per device, held
+ *   - Limit: the plan's max_tokens must be <= 16384 (the array is 361 KB per device, held
  *     by every device that loads the library until the process exits); larger plans are refused with
  *     TSQ_ERR_UNSUPPORTED before anything is enqueued.
  *   - The call allocates and frees nothing.  The first call on a device looks up the array's device

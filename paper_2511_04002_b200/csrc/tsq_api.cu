@@ -51,7 +51,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // Scratch of tsq_encode_noalloc: a workspace that lives in the library image instead of in memory the
 // caller allocates.  Every device that loads the library holds its own copy until the process exits.
 constexpr unsigned long long kStaticMaxTokens = 16384;
-constexpr size_t kStaticWsBytes = (sizeof(WsControl) + 16ull * kStaticMaxTokens + 255ull) & ~255ull;
+constexpr size_t kStaticWsBytes = (sizeof(WsControl) + 8ull * desc_words(kStaticMaxTokens) + 255ull) & ~255ull;
 static __device__ __align__(256) unsigned char g_static_ws[kStaticWsBytes];
 
 // In host code `g_static_ws` is only a handle for the runtime, not an address a kernel may use: the
@@ -279,7 +279,7 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
   p->enc_threads = static_cast<int>(((p->units + p->enc_upt - 1) / p->enc_upt + 31u) / 32u * 32u);
   p->dec_smem = decode_smem_bytes(p->row_bytes, p->threads);
   const unsigned long long desc = T > 0 ? T : 1;
-  p->workspace_bytes = static_cast<size_t>(align16(sizeof(WsControl) + 16ull * desc));
+  p->workspace_bytes = static_cast<size_t>(align16(sizeof(WsControl) + 8ull * desc_words(desc)));
 
   int n_dev = 0;
   if (cudaGetDeviceCount(&n_dev) != cudaSuccess || device >= n_dev) {
@@ -420,7 +420,7 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 static int64_t direct_rows(const tsq_plan_t* plan) {
   if (plan->variant != 0u) return 8;
   const int64_t at_once = static_cast<int64_t>(plan->sms) * std::min(std::max(plan->rows_ctas[2], 1), 8);
-  return at_once + at_once / 16;  // (a sixteenth of a turn more does not count)
+  return std::min<int64_t>(at_once + at_once / 16, kOneKernelRows);  // (a sixteenth of a turn more does not count)
 }
 
 // Rows up to which the second of the two kernels takes 32 elements per thread instead of 64, for rows of up to 5120 elements: more warps share
@@ -541,8 +541,9 @@ tsq_status_t tsq_encode_noalloc(const tsq_plan_t* plan, const void* x_dev, int64
   // The array keeps whatever the last call left (including an unfinished call's tickets): start clean.
   // This also zeroes the generation counter and the recorded capacity: every call through this entry
   // point runs as generation 1, so the wrap-around path that reads the capacity is never taken here, and
-  // the rows that have been cleared are told with the call.
-  if (cudaMemsetAsync(ws, 0, plan->workspace_bytes, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
+  // the rows that have been cleared are told with the call.  (A call of one kernel uses the first words only.)
+  const size_t used = tokens > direct_rows(plan) ? plan->workspace_bytes : sizeof(WsControl) + 16u * static_cast<size_t>(tokens);
+  if (cudaMemsetAsync(ws, 0, used, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
     cudaGetLastError();
     return TSQ_ERR_CUDA;
   }

@@ -3,17 +3,23 @@
 //
 // Variable-length placement: where a token's planes and CSR entries start is an exclusive prefix sum over all earlier
 // tokens, and a token's sizes are known only after Algorithm 1 has run on it.  Calls of many rows therefore go through two
-// kernels that wait for nothing (here); calls of few rows through one that reads the sizes of the rows before it directly
+// kernels (here); calls of few rows through one that reads the sizes of the rows before it directly
 // (tsq_encode_rows.cu).
 //   sizes_kernel   one CTA per row: threshold, extremes, outlier count, Algorithm 1; leaves the row's bit-width, scale and
-//                  zero-point in the blob, its sizes and how its codes are formed in the workspace, and adds the sizes to cells for
-//                  the row's block of 32, 1024 and 32768 rows.
-//   pack_kernel    one CTA per row: its offsets from the cells (three loads per lane of one warp), codes -> bytes
-//                  (code | sign << 7) -> 8 x 32 bit transpose -> plane words, outlier entries.
+//                  zero-point in the blob, these, its sizes and how its codes are formed in its slot of the workspace, and adds the sizes to cells for
+//                  the row's block of 32, 1024 and 32768 rows.  It waits for nothing.
+//   pack_kernel    one CTA per row: its place from the slots and cells (four loads per lane of one warp), codes -> bytes
+//                  (code | sign << 7) -> 8 x 32 bit transpose -> plane words, outlier entries.  Its CTAs take the room that those of sizes_kernel leave, from
+//                  the first row on, while the last rows are still being sized; every row they may wait for is being sized by then.
+// The overlap fills the last, partly empty turn of the first kernel's CTAs and hides the second one's start (us, the second kernel behind the first / so:
+// 777 x 3000 bf16 10.9 / 8.6, 2048 x 5120 fp16 19.8 / 18.8, 4000 x 3000 25.1 / 20.5, 4096 x 4096 24.8 / 22.3, 10000 x 2048 32.4 / 27.6, 2000 x 16384 41.0 / 38.1, signed
+// 2048 x 5120 25.7 / 22.4, 8192 x 8192 62.4 / 61.6, 32768 x 4096 121.7 / 121.2).  What the place costs to read decides whether it pays: with every warp
+// reading its slot (relaxed loads go past L1) 8192 x 8192 took 66.7 us.
 // x is read twice.  The forms that read it once (rows in shared memory or in registers, placement at once, by look-back, or put
 // off by a row's time) were all slower: in token order every row waits for the slowest of the rows before it, and a few rows in a
 // hundred take Algorithm 1 further than the first candidate (8192 x 8192 bf16 / 32768 x 4096 bf16 with 1 % outliers, us: persistent CTAs with a
-// ring of packed rows 87 / 190, one CTA per row 104 / 281, placement a row later 87 / 349, these kernels at that time 65 / 126).
+// ring of packed rows 87 / 190, one CTA per row 104 / 281, placement a row later 87 / 349, these kernels at that time 65 / 126; CTAs that stay, with
+// the present arithmetic, a ring of two packed rows and cells instead of look-back 72 / 215).
 //
 // What binds: DRAM and instruction issue about equally.  The two kernels move 326 MB at 8192 x 8192 bf16 (x twice, 8 % of the
 // second time from L2; 50 us at the copy rate) and issue in two cycles out of three.  So the passes work on two 16-bit elements
@@ -47,9 +53,21 @@ constexpr int kKind84 = 0;      // magnitudes, candidates end in 4 and 8 bits: b
 constexpr int kKindExact = 1;   // any other candidates of the magnitudes: exact sums
 constexpr int kKindSigned = 2;  // signed values: exact sums
 
-// A row's size in its slot: outliers | bits << 17 | mode << 21 (the upper half stays 0: no tag of a direct call)
-__device__ __forceinline__ unsigned long long row_entry(uint32_t outliers, int b, uint32_t mode) {
-  return outliers | static_cast<uint32_t>(b) << 17 | mode << 21;
+// What the second kernel has to know of a row: outliers | bits << 17 | mode << 21
+__device__ __forceinline__ uint32_t row_entry(uint32_t outliers, int b, uint32_t mode) { return outliers | static_cast<uint32_t>(b) << 17 | mode << 21; }
+
+// A cell: outliers in the lower half, the sum of the rows' bits from bit 32, how many rows (or blocks of 1024 rows) have been added from kCellShift.
+constexpr uint32_t kCellShift = 51u;
+constexpr unsigned long long kCellRow = 1ull << kCellShift;
+constexpr uint32_t kCells32 = 64u, kCells1024 = 66u, kCells32768 = 68u, kCallWord = 70u;  // from block_at
+
+__device__ __forceinline__ unsigned long long* slot_of(const EncodeParams& p, uint32_t row) { return p.desc + block_at(row) + 2u * (row & 31u); }
+// A slot is one 128-bit word, so that what is read of it belongs together: the tag, the entry, the scale and the zero-point.
+__device__ __forceinline__ void store_slot(unsigned long long* slot, unsigned long long lo, unsigned long long hi) {
+  asm volatile("{.reg .b128 v; mov.b128 v, {%1, %2}; st.relaxed.gpu.global.b128 [%0], v;}" ::"l"(slot), "l"(lo), "l"(hi) : "memory");
+}
+__device__ __forceinline__ void load_slot(const unsigned long long* slot, unsigned long long& lo, unsigned long long& hi) {
+  asm volatile("{.reg .b128 v; ld.relaxed.gpu.global.b128 v, [%2]; mov.b128 {%0, %1}, v;}" : "=l"(lo), "=l"(hi) : "l"(slot) : "memory");
 }
 
 __device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long long v) {
@@ -181,7 +199,6 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
   using Shared = SizesShared<MAXT / 32>;
   __shared__ Shared sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  launch_dependents();
   if (tid >= nwarps && tid < static_cast<uint32_t>(Shared::kSlots)) {
     sh.warp_min[tid] = 0xffffu;
     sh.warp_max[tid] = KIND == kKind84 ? -32768 : 0;
@@ -190,6 +207,19 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
   }
   wait_for_prior_grids();
   const uint32_t tile = blockIdx.x;
+  uint32_t call = 0u;
+  if (tid == 0u) {
+    call = *reinterpret_cast<volatile const uint32_t*>(&p.ws->calls) + 1u;
+    if ((tile & 31u) == 0u) {
+      const uint32_t ticket = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket);
+      const uint32_t has_cells = *reinterpret_cast<volatile const uint32_t*>(&p.ws->desc_capacity);
+      st_relaxed_u64(p.desc + block_at(tile) + kCallWord, ticket == 0u && p.tokens <= max(has_cells, p.cleared_rows) ? call : 0u);
+      __threadfence();
+    }
+    // The second kernel's CTAs start once every CTA here has come this far: they find the call's number, and every row that they may have to wait for
+    // is being sized.  (By one thread: the first of a CTA's threads counts, and the number has to be there.)
+    launch_dependents();
+  }
   const uint4* xrow = reinterpret_cast<const uint4*>(p.x) + static_cast<size_t>(tile) * p.chunks;
   uint32_t x[4 * C];
   uint32_t nv = FULL ? C : 0u;
@@ -206,8 +236,6 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
     x[4 * j + 2] = c.z;
     x[4 * j + 3] = c.w;
   }
-  const uint32_t turn = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn) & 1u;
-  if (tile == 0u && tid == 0u) p.ws->sums_turn_next = turn ^ 1u;
   const uint32_t thr2 = p.thr16 * 0x10001u;
 
   uint32_t mn, cnt = 0u;
@@ -387,12 +415,18 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
   }
   if (best.b == 0) best = settle_exactly<BF16, C, SV>(p, xrow, pmin, pmax, sh);
   if (tid == 0) {
-    unsigned long long* cells = p.desc + 1;
-    const unsigned long long size = (static_cast<unsigned long long>(static_cast<uint32_t>(best.b) * p.lay.wpp) << 32) | row_cnt;
-    if ((tile | 31u) < p.tokens) red_add_u64(cells + 2u * ((tile & ~31u) + turn), size);
-    if ((tile | 1023u) < p.tokens) red_add_u64(cells + 2u * ((tile & ~1023u) + 2u + turn), size);
-    if ((tile | 32767u) < p.tokens) red_add_u64(cells + 2u * ((tile & ~32767u) + 4u + turn), size);
-    p.desc[2u * tile] = row_entry(row_cnt, best.b, best.mode);
+    unsigned long long* cells = p.desc + (call & 1u);
+    const unsigned long long size = kCellRow | static_cast<unsigned long long>(static_cast<uint32_t>(best.b)) << 32 | row_cnt;
+    store_slot(slot_of(p, tile), static_cast<unsigned long long>(call) << 32 | row_entry(row_cnt, best.b, best.mode),
+               static_cast<unsigned long long>(static_cast<uint32_t>(best.zp)) << 32 | __float_as_uint(best.s));
+    // (of blocks that have rows behind them)
+    if ((tile | 31u) + 1u < p.tokens) red_add_u64(cells + block_at(tile) + kCells32, size);
+    if ((tile | 32767u) + 1u < p.tokens) {  // the row that completes a block of 1024 adds it to the 32768's cell
+      const unsigned long long sum = atomicAdd(cells + block_at(tile & ~1023u) + kCells1024, size) + size;
+      if ((sum >> kCellShift) == 1024u) red_add_u64(cells + block_at(tile & ~32767u) + kCells32768, (sum & (kCellRow - 1u)) | kCellRow);
+    } else if ((tile | 1023u) + 1u < p.tokens) {
+      red_add_u64(cells + block_at(tile & ~1023u) + kCells1024, size);
+    }
     reinterpret_cast<uint8_t*>(p.blob + p.lay.off_bits)[tile] = static_cast<uint8_t>(best.b);
     reinterpret_cast<float*>(p.blob + p.lay.off_scale)[tile] = best.s;
     reinterpret_cast<int32_t*>(p.blob + p.lay.off_zp)[tile] = best.zp;
@@ -400,37 +434,71 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
 }
 
 constexpr uint32_t kListCap = 512u;  // entries of a warp's outlier list
+// Where a row goes and how its codes are formed
+struct Place {
+  uint32_t word_off, out_base, entry;
+  float s;
+  int zp;
+  uint32_t call;  // 0: the row is not to be written
+};
 template <int NW>
 struct PackShared {
   uint32_t cnt[NW];  // outliers by warp
-  uint32_t word_off, out_base;
-  uint32_t next_turn;  // of the cells, in the next call
-  uint32_t sound;      // the workspace is as a finished call leaves it and has cells for all of this call's rows
+  Place place;
 };
 
-// Words and outliers before row `tile`, by one warp (lane 0's result counts): the rows of its block of 32, the blocks of 32 before it in
-// its block of 1024, those of 1024 in its block of 32768, those of 32768 before it: three loads per lane, all in one round trip.
-__device__ __forceinline__ void sums_before(const EncodeParams& p, uint32_t next_turn, uint32_t tile, uint32_t lane, uint32_t* words, uint32_t* outliers) {
-  const unsigned long long* cells = p.desc + 1;
+__device__ __forceinline__ void load_cells(const unsigned long long* c, unsigned long long& a, unsigned long long& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(c) : "memory");
+}
+
+// Place of row `tile` by one warp: its own slot and those of the rows before it in its block of 32, the blocks of 32 before it in its block of 1024, those of
+// 1024 in its block of 32768, those of 32768 before it: four loads per lane, all in one round trip (both turns' cells: the call's number arrives with
+// them).  Returns the call's number, or ~0 while not all of these rows have been sized.
+__device__ __forceinline__ uint32_t place_row(const EncodeParams& p, uint32_t tile, Place& out) {
+  const uint32_t lane = threadIdx.x & 31u;
   const uint32_t row = (tile & ~31u) + lane, g = (tile & ~1023u) + 32u * lane, q = (tile & ~32767u) + 1024u * lane;
-  unsigned long long part = 0ull, g0 = 0ull, g1 = 0ull, q0 = 0ull, q1 = 0ull;
-  if (row < tile) {
-    const uint32_t e = static_cast<uint32_t>(p.desc[2u * row]);
-    part = (static_cast<unsigned long long>(((e >> 17) & 15u) * p.lay.wpp) << 32) | (e & 0x1ffffu);
+  constexpr unsigned long long kSums = kCellRow - 1u, k32 = 32ull << kCellShift, k1024 = 1024ull << kCellShift;
+  unsigned long long lo = 0ull, hi = 0ull, g0 = k32, g1 = k32, q0 = k1024, q1 = k1024;
+  const uint32_t call = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord));
+  if (row <= tile) load_slot(slot_of(p, row), lo, hi);
+  if (g + 31u < tile) load_cells(p.desc + block_at(g) + kCells32, g0, g1);
+  if (q + 1023u < tile) load_cells(p.desc + block_at(q) + kCells1024, q0, q1);
+  const uint32_t turn = call & 1u;
+  const unsigned long long of_g = turn ? g1 : g0, of_q = turn ? q1 : q0;
+  bool all = (row > tile || static_cast<uint32_t>(lo >> 32) == call) && (of_g >> kCellShift) == 32u && (of_q >> kCellShift) == 1024u;
+  const uint32_t entry = static_cast<uint32_t>(lo);
+  unsigned long long part = (of_g & kSums) + (of_q & kSums);
+  if (row < tile) part += static_cast<unsigned long long>((entry >> 17) & 15u) << 32 | (entry & 0x1ffffu);
+  for (unsigned long long c = 32768ull * lane; c + 32767ull < tile; c += 32ull * 32768ull) {
+    const unsigned long long v = ld_relaxed_u64(p.desc + block_at(static_cast<uint32_t>(c)) + kCells32768 + turn);
+    all = all && (v >> kCellShift) == 32u;
+    part += v & kSums;
   }
-  if (g + 31u < tile) {  // both turns' cells: which one counts arrives in the same round trip
-    g0 = cells[2u * g];
-    g1 = cells[2u * (g + 1u)];
+  const uint32_t words = __reduce_add_sync(kFull, static_cast<uint32_t>(part >> 32)) * p.lay.wpp;
+  const uint32_t outliers = __reduce_add_sync(kFull, static_cast<uint32_t>(part));
+  all = __all_sync(kFull, all) || call == 0u;
+  if (row == tile) out = Place{words, outliers, entry, __uint_as_float(static_cast<uint32_t>(hi)), static_cast<int>(hi >> 32), all ? call : 0u};
+  return all ? call : 0xffffffffu;
+}
+
+// The same, waited for.  The rows are being sized, so the wait ends; it has a limit for a workspace that two calls use at once, or that something else has
+// written to.  A row that gives up is not written, so the call must not end with TSQ_OK: call_state decides as direct_state does for calls of one
+// kernel (given_up there).
+__device__ __noinline__ void wait_for_place(const EncodeParams& p, uint32_t tile, Place& out) {
+  const uint32_t state4 = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord)) << 2;
+  for (uint32_t polls = 1u; place_row(p, tile, out) == 0xffffffffu; ++polls) {
+    uint32_t over = 0u;
+    if (polls > 32u && (threadIdx.x & 31u) == 0u) {
+      __nanosleep(1000u);
+      if (polls > kPollLimit) {
+        over = atomicMax(&p.ws->call_state, state4 | kWaitRanOut) != (state4 | kCallEnded) || polls > kPollLimit + 64u ? 1u : 0u;
+      } else {
+        over = *reinterpret_cast<volatile const uint32_t*>(&p.ws->call_state) == (state4 | kWaitRanOut) ? 1u : 0u;
+      }
+      if (over != 0u) atomicCAS(&p.ws->enc_status, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
+    }
+    if (__shfl_sync(kFull, over, 0) != 0u) return;  // (out.call is 0)
   }
-  if (q + 1023u < tile) {
-    q0 = cells[2u * (q + 2u)];
-    q1 = cells[2u * (q + 3u)];
-  }
-  const uint32_t turn = (next_turn & 1u) ^ 1u;
-  part += turn ? g1 + q1 : g0 + q0;
-  for (unsigned long long c = 32768ull * lane; c + 32767ull < tile; c += 32ull * 32768ull) part += cells[2u * (c + 4u + turn)];
-  *words = __reduce_add_sync(kFull, static_cast<uint32_t>(part >> 32));
-  *outliers = __reduce_add_sync(kFull, static_cast<uint32_t>(part));
 }
 
 template <bool BF16, int G, bool SV, bool FULL, int MAXT, int MINB>
@@ -439,9 +507,10 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   __shared__ PackShared<MAXT / 32> sh;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nt = blockDim.x, nwarps = nt >> 5;
+  // This grid starts while sizes_kernel still runs, whose CTAs have all seen the end of everything before it: the input can be read, and what that
+  // kernel leaves is polled for.  Row order: the rows sized first.
   launch_dependents();
-  wait_for_prior_grids();
-  const uint32_t tile = p.tokens - 1u - blockIdx.x;  // from the end: what sizes_kernel has read last is still in L2
+  const uint32_t tile = blockIdx.x;
   const uint4* xrow = reinterpret_cast<const uint4*>(p.x) + static_cast<size_t>(tile) * p.chunks;
   uint4* const park = reinterpret_cast<uint4*>(smem_dyn) + warp * (128u * G);
   uint16_t* const list = reinterpret_cast<uint16_t*>(smem_dyn + nwarps * (2048u * G)) + warp * kListCap;
@@ -454,28 +523,8 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (FULL || c0 + 32u * i < p.chunks) cp_async16(dst + 32u * i, xrow + c0 + 32u * i);
     }
   }
-  const uint32_t entry = static_cast<uint32_t>(p.desc[2u * tile]);
-  const float s = reinterpret_cast<const float*>(p.blob + p.lay.off_scale)[tile];
-  if (warp == nwarps - 1u) {
-    // The control block's words by one warp per CTA: every CTA of the call reads the same line, which takes one request after the other
-    // (us of a call with 2 words read by every warp / 3 by every warp / 3 by one warp: 2048 x 5120 22.0 / 24.5 / 18.6, 8192 x 8192 70.6 / 74.0 / 68.7,
-    // signed pair 2048 x 5120 40.8 / 44.6 / 38.3).
-    const uint32_t next = *reinterpret_cast<volatile const uint32_t*>(&p.ws->sums_turn_next);
-    const uint32_t ticket = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket);
-    const uint32_t has_cells = *reinterpret_cast<volatile const uint32_t*>(&p.ws->desc_capacity);
-    uint32_t w, o;
-    sums_before(p, next, tile, lane, &w, &o);
-    if (lane == 0) {
-      sh.word_off = w;
-      sh.out_base = o;
-      sh.next_turn = next;
-      sh.sound = ticket == 0u && p.tokens <= max(has_cells, p.cleared_rows) ? 1u : 0u;
-    }
-  }
+  if (warp == nwarps - 1u && place_row(p, tile, sh.place) == 0xffffffffu) wait_for_place(p, tile, sh.place);
   const uint32_t thr2 = p.thr16 * 0x10001u;
-  const int b = static_cast<int>((entry >> 17) & 15u);
-  const uint32_t mode = entry >> 21, row_cnt = entry & 0x1ffffu;
-  const uint32_t agg_w = static_cast<uint32_t>(b) * p.lay.wpp;
   uint32_t x[G][16], bitmap[G];
   cp_async_wait_all();
   __syncwarp();
@@ -495,22 +544,22 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   }
   // ---- outliers: bitmap of each group; where they are in the warp's part of the row, in order, into its list ----
   uint32_t all = 0u;
-#pragma unroll
-  for (int k = 0; k < G; ++k) bitmap[k] = 0u;
   const auto pattern_at = [&](int k, uint32_t e) {  // of element e of the lane's group in segment k, from the parked row
     return static_cast<uint32_t>(reinterpret_cast<const uint16_t*>(own + 128 * k)[8u * (((e >> 3) + rot) & 3u) + (e & 7u)]);
   };
-  if (row_cnt != 0u) {
+  uint32_t any = 0u;
 #pragma unroll
-    for (int k = 0; k < G; ++k) {
-      uint32_t nat = outliers_of(x[k], thr2);
-      if (!FULL) {
-        const uint32_t u = u0 + 32u * k;
-        const uint32_t chunks = 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
-        if (chunks < 4u) nat &= (1u << (8u * chunks)) - 1u;
-      }
-      bitmap[k] = nat;
+  for (int k = 0; k < G; ++k) {
+    uint32_t nat = outliers_of(x[k], thr2);
+    if (!FULL) {
+      const uint32_t u = u0 + 32u * k;
+      const uint32_t chunks = 4u * u < p.chunks ? min(p.chunks - 4u * u, 4u) : 0u;
+      if (chunks < 4u) nat &= (1u << (8u * chunks)) - 1u;
     }
+    bitmap[k] = nat;
+    any |= nat;
+  }
+  if (__any_sync(kFull, any != 0u)) {
     // how many come before the lane's in each segment, two segments to a register
     uint32_t at[G];
 #pragma unroll
@@ -539,11 +588,16 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       }
     }
     __syncwarp();
-    if (lane == 0u) sh.cnt[warp] = all;
   }
+  if (lane == 0u) sh.cnt[warp] = all;
   __syncthreads();
-  const uint32_t word_off = sh.word_off, out_base = sh.out_base, word_end = word_off + agg_w, out_end = out_base + row_cnt;
-  uint32_t status = sh.sound != 0u && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
+  const uint32_t entry = sh.place.entry, call = sh.place.call;
+  const float s = sh.place.s;
+  const int b = static_cast<int>((entry >> 17) & 15u);
+  const uint32_t mode = entry >> 21, row_cnt = entry & 0x1ffffu;
+  const uint32_t agg_w = static_cast<uint32_t>(b) * p.lay.wpp;
+  const uint32_t word_off = sh.place.word_off, out_base = sh.place.out_base, word_end = word_off + agg_w, out_end = out_base + row_cnt;
+  uint32_t status = call != 0u && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
   if (status == TSQ_OK) {
     uint32_t* wrow = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
     if (!SV && mode >= kOneUp) {
@@ -559,7 +613,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       Level best;
       best.s = s;
       best.r = __frcp_rn(s);
-      best.zp = reinterpret_cast<const int32_t*>(p.blob + p.lay.off_zp)[tile];
+      best.zp = sh.place.zp;
       best.qmax = SV ? (1 << b) - 1 : (1 << (b - 1)) - 1;
 #pragma unroll
       for (int k = 0; k < G; ++k) {
@@ -625,23 +679,38 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       o_out_ptr[tile + 1u] = out_end;
     }
     if (tile == p.tokens - 1u) {
+      // This CTA ends the call.  The grid after this one waits for this grid only: sizes_kernel must have ended by then.
+      wait_for_prior_grids();
+      if (call == 0u || atomicMax(&p.ws->call_state, call << 2 | kCallEnded) == (call << 2 | kWaitRanOut)) status = TSQ_ERR_TIMEOUT;
       if (status == TSQ_OK && out_end > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
       const bool ok = status != TSQ_ERR_TIMEOUT;
       end_part(p, status, ok ? word_end : 0u, ok ? out_end : 0u);
       if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
-      // (the slots of this call's rows carry no tag, and the other CTAs are still reading them)
-      next_generation(p, *reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u, p.tokens);
-      p.ws->sums_turn = sh.next_turn;
+      next_generation(p, *reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u);
+      if (call != 0u && call != kCallWrap) p.ws->calls = call;
     }
   }
   // ---- the cells that the next call adds to ----
   if (blockIdx.x < 32u) {
     const uint32_t blocks = max(p.ws->desc_capacity, p.tokens) >> 5;
     for (uint32_t i = blockIdx.x * nt + tid; i < blocks; i += min(gridDim.x, 32u) * nt) {
-      unsigned long long* c = p.desc + 64ull * i + 1u + 2u * (sh.next_turn & 1u);
-      c[0] = 0ull;
-      if ((i & 31u) == 0u) c[4] = 0ull;
-      if ((i & 1023u) == 0u) c[8] = 0ull;
+      unsigned long long* c = p.desc + block_at(32u * i) + ((call & 1u) ^ 1u);
+      c[kCells32] = 0ull;
+      if ((i & 31u) == 0u) c[kCells1024] = 0ull;
+      if ((i & 1023u) == 0u) c[kCells32768] = 0ull;
+    }
+  }
+  if (call == kCallWrap) {  // the numbers start over: once no CTA reads slots any more, no old one may be left
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(&p.ws->done, 1u) == gridDim.x - 1u) {
+        const uint32_t n = max(p.ws->desc_capacity, p.tokens);
+        for (uint32_t i = 0; i < n; ++i) store_slot(slot_of(p, i), 0ull, 0ull);
+        p.ws->call_state = 0u;
+        p.ws->calls = 0u;
+        p.ws->done = 0u;
+      }
     }
   }
 }

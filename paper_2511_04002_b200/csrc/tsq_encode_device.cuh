@@ -591,12 +591,11 @@ __device__ void end_part(const EncodeParams& p, uint32_t status, unsigned long l
   }
 }
 
-// The generation of the call that ends; after the last one they start over, and the slots from `first` on are wiped so that old tags
-// cannot alias.
-__device__ void next_generation(const EncodeParams& p, uint32_t g, uint32_t first) {
+// The generation of the call that ends; after the last one they start over, and the rows' words are wiped so that old tags cannot alias.
+__device__ void next_generation(const EncodeParams& p, uint32_t g) {
   if (g >= kGenWrap) {
-    const uint32_t n = max(p.ws->desc_capacity, p.tokens);
-    for (uint32_t i = first; i < n; ++i) p.desc[2ull * i] = 0ull;
+    const uint32_t n = min(max(p.ws->desc_capacity, p.tokens), kOneKernelRows);
+    for (uint32_t i = 0; i < n; ++i) p.desc[2ull * i] = 0ull;
     p.ws->direct_state = 0u;
     g = 0u;
   }
@@ -630,7 +629,7 @@ __device__ void finish_call(const EncodeParams& p, uint32_t gen4) {
   if (e != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, e);
   p.ws->ticket = 0u;
   p.ws->done = 0u;
-  next_generation(p, gen4 >> 2, 0u);
+  next_generation(p, gen4 >> 2);
 }
 
 // The per-token fields of the blob, written by one thread.

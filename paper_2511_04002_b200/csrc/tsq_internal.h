@@ -54,16 +54,22 @@ __host__ __device__ inline BlobLayout make_layout(uint32_t hidden, unsigned long
   return L;
 }
 
-// Workspace: a 64-byte control block and, per token t, two adjacent 64-bit words:
-//   desc[2 t]      the slot of row t.  Calls of one kernel: (tag << 32) | plane words << 17 | outliers, tag = generation * 4 + flag; stale
-//                  generations read as "not yet published", so nothing needs clearing between calls.  Calls of two kernels:
-//                  outliers | bits << 17 | mode << 21, upper half 0 (no tag: generations start at 1).
-//   desc[2 t + 1]  cells of calls of two kernels: plane words << 32 | outliers of a whole block of rows, two of each, used in turn.  Block of 32
-//                  rows that starts at row t: cells t and t + 1; of 1024 rows: t + 2, t + 3; of 32768 rows: t + 4, t + 5.  A call
-//                  adds to the cells of its turn, which the call before it has left at 0, and clears those of the other.
+// Workspace: a 64-byte control block and an array of 64-bit words (desc_words).
+//   Calls of one kernel, which have kOneKernelRows rows at most: word 2 r belongs to row r: (tag << 32) | plane words << 17 | outliers,
+//   tag = generation * 4 + kFlagAggregate; stale generations read as "not yet published", so nothing needs clearing between calls.
+//   Calls of two kernels: from word kBlocksAt on, five 128-byte lines per block of 32 rows (block_at).
+//     words 0 .. 63   slots, one 128-bit word per row: call << 32 | entry (row_entry) and zero-point << 32 | scale, where call is the call's number.
+//     words 64 .. 69  cells: how many rows of a whole block have been sized, the sum of their bits, their outliers (kCellRow); two of each, used in turn.
+//                     The block's 32 rows: 64, 65; 1024 rows that start here: 66, 67; 32768 rows: 68, 69 (these count blocks of 1024).  A call adds
+//                     to the cells of its turn, which the call before it has left at 0, and clears those of the other.
+//     word 70         the call's number, or 0 where the workspace is not fit for it, for the second kernel's CTAs of these rows.
+//   Slots and cells tell by themselves whether they are complete: the second kernel starts while the first still runs.
 // Where a word is does not depend on the number of tokens, so a workspace may serve plans of different sizes, as far as it has been
 // initialised: cells must be 0 when a call adds to them, and every call clears those of desc_capacity rows.  A call of two kernels with more
 // rows than that writes no row and ends with TSQ_ERR_TIMEOUT.  (Slots need no such bound: their tags tell.)
+// (The two kinds apart, because one-kernel calls are sensitive to where their words are: 128 x 4096 in 5.99 us with words at a stride of 16 bytes,
+// 6.10 with a gap every 32 rows, 6.12 at 8 or 32 bytes.  Cells in lines of their own: 10000 x 2048 27.6 us, 27.9 behind the slots in 72 words; 32 bytes
+// per row with the cells between the slots 30.0.)
 struct WsControl {
   uint32_t gen;          // generation of the last finished encode
   uint32_t ticket;       // next tile to hand out (self-resetting)
@@ -74,8 +80,8 @@ struct WsControl {
   uint32_t desc_capacity;  // rows whose slots and cells init has cleared
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
   uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut or kCallEnded, only ever grows
-  uint32_t sums_turn;      // calls of two kernels: whose turn the cells are, read by the first and written by the second kernel
-  uint32_t sums_turn_next; // the same for the next call, written by the first kernel and read by the second
+  uint32_t calls;          // number of the last call of two kernels that has ended: read by the first, written by the second kernel
+  uint32_t call_state;     // as direct_state, for calls of two kernels: number * 4 + kWaitRanOut or kCallEnded
   uint32_t pad[5];
 };
 static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
@@ -83,12 +89,18 @@ static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
 constexpr uint32_t kFlagAggregate = 1;
 constexpr uint32_t kWaitRanOut = 1, kCallEnded = 2;  // direct_state
 constexpr uint32_t kGenWrap = (1u << 30) - 2;
+constexpr uint32_t kCallWrap = (1u << 30) - 2;      // calls of two kernels are numbered 1 .. kCallWrap (even: the cells go on in turn)
+
+constexpr uint32_t kOneKernelRows = 2048;
+constexpr unsigned long long kBlocksAt = 2ull * kOneKernelRows + 8ull, kBlockWords = 80ull;
+__host__ __device__ constexpr unsigned long long desc_words(unsigned long long rows) { return kBlocksAt + kBlockWords * ((rows + 31ull) / 32ull); }
+__host__ __device__ inline unsigned long long block_at(uint32_t row) { return kBlocksAt + kBlockWords * (row >> 5); }
 
 struct EncodeParams {
   const uint16_t* x;
   unsigned char* blob;
   WsControl* ws;
-  unsigned long long* desc;                  // [2 * max_tokens] slots and cells
+  unsigned long long* desc;                  // [desc_words(max_tokens)], behind the control block
   BlobLayout lay;
   uint32_t tokens, hidden, units, chunks;   // units = ceil(H/32), chunks = H/8
   uint32_t thr16;                            // smallest non-negative 16-bit pattern with value >= tau
