@@ -160,7 +160,7 @@ tsq_status_t tsq_workspace_set_wait_limit(void *ws_dev, uint32_t polls, void *cu
 /*
  * Encode x (DEVICE, [tokens x hidden]) into blob (DEVICE, >= blob_bytes from tsq_plan_sizes,
  * 16-byte aligned): TS (Eq. "ts") + TAB-Q (Algorithm 1, token-wise) + bit-plane packing, one
- * kernel launch, or two for calls of more than a few rows per SM.  tokens == 0 writes an empty, valid blob.  Returns argument errors before
+ * kernel launch, or two for calls of more rows than the device has SMs.  tokens == 0 writes an empty, valid blob.  Returns argument errors before
  * anything is enqueued.
  */
 tsq_status_t tsq_encode(const tsq_plan_t *plan, const void *x_dev, int64_t tokens, void *blob_dev,

@@ -403,34 +403,26 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 }
 
 // Rows up to which a call goes through one kernel, whose rows read the sizes of the rows before them directly, instead of two.  The
-// second kernel costs a launch and a second read of the input; in the one kernel every row waits for the slowest row before it, which
-// is cheap while all rows are in flight at once (rows_ctas) and they are few enough to read each other's sizes (8 per SM).  us, one kernel /
-// two, each pair on the same tensors (n: normal values with 0.1 % outliers, n0: none, n1: 1 %, t3: Student-t nu = 3 with 0.1 %, t4: nu = 4 with 16
-// outlier channels):
-//   up to 2048 elements  1042 x 1976 fp16, 8 channels  9.3 / 10.9    1184 x 1024 bf16 t3   9.1 / 7.1     1500 x 1024 fp16 n   13.5 / 9.4
-//   up to 5120            300 x 4096 fp16 n            7.7 / 8.4      777 x 3000 bf16 n   10.2 / 10.9    1000 x 4096 fp16 n0  13.3 / 11.4
-//                        1500 x 4096 fp16 n1          17.3 / 11.4     700 x 4096 fp16 n    9.9 / 10.3
-//   up to 8192            300 x 8192 bf16 t3           9.2 / 9.8      600 x 8192 fp16 n   11.8 / 11.6    1000 x 8192 fp16 t4  20.0 / 13.7
-//   longer                300 x 12288 fp16 n          11.3 / 12.1     600 x 12288 fp16 n  17.6 / 12.8     600 x 16384 fp16 t4 23.1 / 16.3
-//   signed values          64 x 4096 fp16 n           12.4 / 7.9      300 x 4096 fp16 n   21.1 / 9.9      600 x 5120 fp16 t4  35.7 / 12.7
-// (Signed values: one row in ten has a code that needs the clamp, which the one kernel forms by the division instruction; 1 x 4096 4.1 / 5.9,
-// 8 x 4096 5.7 / 7.0, 16 x 4096 8.3 / 7.1.)  The line was drawn when two kernels took 1 to 3 us more than here, before one warp per CTA read the
-// control block (pack_kernel): by these figures rows of up to 5120 elements would have it at five to six rows per SM instead of six to eight
-// and a half.
+// second kernel costs a launch and a second read of the input, but starts while the first still runs; in the one kernel every row waits for the slowest
+// row before it, and with more than one row per SM the rows have to be numbered by ticket.  us, one kernel / two, each pair on the same tensors (bf16 or
+// fp16, normal values with 0.1 % outliers):
+//   up to a row per SM   64 x 4096  5.4 / 6.5    100 x 4096  5.7 / 6.4    148 x 4096  5.0 / 6.6    148 x 8192  5.2 / 7.1    148 x 10240 6.4 / 7.4    148 x 24576 8.4 / 10.5
+//     (rows of 8200 to 16384 elements lie on both sides: 32 x 16384 5.9 / 6.8, 64 x 16384 7.5 / 6.7, 100 x 12288 8.6 / 7.9)
+//   more                149 x 1024  6.3 / 6.1    149 x 4096  6.9 / 6.5    149 x 8192  7.3 / 7.2    149 x 16384 10.3 / 8.0   149 x 32768 16.0 / 14.6
+//                       600 x 1024  8.0 / 6.5    300 x 4096  7.0 / 6.9    777 x 3000 10.3 / 8.3    700 x 4096 10.1 / 8.5    600 x 8192 11.6 / 10.2
+// Signed values: one row in ten has a code that needs the clamp, which the one kernel forms by the division instruction (1 x 4096 4.1 / 5.9,
+// 8 x 4096 5.7 / 6.6, 16 x 4096 8.3 / 6.6).
 static int64_t direct_rows(const tsq_plan_t* plan) {
-  if (plan->variant != 0u) return 8;
-  const int64_t at_once = static_cast<int64_t>(plan->sms) * std::min(std::max(plan->rows_ctas[2], 1), 8);
-  return std::min<int64_t>(at_once + at_once / 16, kOneKernelRows);  // (a sixteenth of a turn more does not count)
+  return std::min<int64_t>(plan->variant != 0u ? 8 : plan->sms, kOneKernelRows);
 }
 
-// Rows up to which the second of the two kernels takes 32 elements per thread instead of 64, for rows of up to 5120 elements: more warps share
-// a row while they do not fill the device several times over, and rows of one segment of 1024 elements leave half of the wider threads
-// idle.  us, 32 / 64 elements: 300 x 4096 8.4 / 9.7, 2048 x 4096 13.4 / 15.1, 2048 x 5120 18.4 / 21.0, 4096 x 4096 24.2 / 24.9, 10000 x 2048 30.8 / 31.7,
-// 8192 x 4096 38.5 / 38.2, 8192 x 1024 23.4 / 23.9; 1000 x 8192 16.8 / 14.8.  (The line, 80 segments per SM, was drawn when warps were dearer, each of
-// them reading the control block: by these figures, the last pair apart, which is older, it would lie near 200.)
+// Whether the second of the two kernels takes 32 elements per thread instead of 64, for rows of up to 5120 elements.  An odd number of segments of
+// 1024 elements leaves half a warp's work idle with 64; otherwise more warps share a row while they do not fill the device several times over.  us,
+// 32 / 64 elements: 12000 x 3072 41.7 / 45.4, 10000 x 5120 55.4 / 55.6, 2048 x 5120 18.7 / 20.8; 3000 x 4096 17.1 / 17.6, 8192 x 2048 22.4 / 23.3, 4096 x 4096 21.3 / 22.1 (111
+// segments per SM), 4500 x 4096 22.9 / 22.6 (122), 10000 x 2048 27.7 / 27.5, 32768 x 4096 135 / 121.
 static bool few_rows(const tsq_plan_t* plan, int64_t tokens) {
   const int64_t segments = (plan->units + 31u) / 32u;
-  return segments <= kFewSegments && (segments == 1 || tokens * segments <= 80 * static_cast<int64_t>(plan->sms));
+  return segments <= kFewSegments && (segments % 2 == 1 || tokens * segments <= 120 * static_cast<int64_t>(plan->sms));
 }
 
 // Instance of the one-kernel encoder: 128, 80 or 64 registers, so more CTAs per SM with each.  The one

@@ -2,8 +2,8 @@
 // Eq. "Proposed") + bit-plane packing + CSR emission.
 //
 // Variable-length placement: where a token's planes and CSR entries start is an exclusive prefix sum over all earlier
-// tokens, and a token's sizes are known only after Algorithm 1 has run on it.  Calls of many rows therefore go through two
-// kernels (here); calls of few rows through one that reads the sizes of the rows before it directly
+// tokens, and a token's sizes are known only after Algorithm 1 has run on it.  Calls of more rows than the device has SMs therefore go through two
+// kernels (here), calls of fewer through one that reads the sizes of the rows before it directly
 // (tsq_encode_rows.cu).
 //   sizes_kernel   one CTA per row: threshold, extremes, outlier count, Algorithm 1; leaves the row's bit-width, scale and
 //                  zero-point in the blob, these, its sizes and how its codes are formed in its slot of the workspace, and adds the sizes to cells for
@@ -752,7 +752,8 @@ static EncodeKernel pack_of(const EncodeParams& p, const PackShape& s) {
     if (sv) return bf16 ? pack_kernel<true, 4, true, false, 512, 1> : pack_kernel<false, 4, true, false, 512, 1>;
     return bf16 ? pack_kernel<true, 4, false, false, 512, 1> : pack_kernel<false, 4, false, false, 512, 1>;
   }
-  if (s.groups == 1) return sv ? pack_instance<true, 1, 256, 4>(bf16, full) : pack_instance<false, 1, 256, 5>(bf16, full);
+  // (32 elements: rows of up to 5 warps, kFewSegments.  56 registers, 7 such CTAs per SM: 2048 x 5120 18.7 us, 19.0 with 48 registers, which spill)
+  if (s.groups == 1) return sv ? pack_instance<true, 1, 256, 4>(bf16, full) : pack_instance<false, 1, 160, 7>(bf16, full);
   if (sv) return pack_instance<true, 2, 256, 3>(bf16, full);
   return s.threads > 128 ? pack_instance<false, 2, 256, 3>(bf16, full) : pack_instance<false, 2, 128, 7>(bf16, full);
 }

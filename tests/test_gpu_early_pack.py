@@ -1,5 +1,6 @@
 """The second kernel of a two-kernel encode starts while the first still runs: rows that are sized late in front of rows that are packed early, calls one after
-another on one workspace with the numbers of calls starting over, blocks of 32, 1024 and 32768 rows that end with the call."""
+another on one workspace with the numbers of calls starting over, blocks of 32, 1024 and 32768 rows that end with the call, and the shapes of the second
+kernel on both sides of their line."""
 import pytest
 import torch
 
@@ -19,7 +20,7 @@ def reference(x, bits=(2, 4, 8), variant=0):
     return R.encode(synth.raw_u16(x), code, 6.0, list(bits), 0.2, signed_values=variant == 1)
 
 
-@pytest.mark.parametrize("tokens,hidden", [(1300, 1024), (2049, 64), (32769, 16)])
+@pytest.mark.parametrize("tokens,hidden", [(149, 1024), (151, 4096), (160, 8200), (2049, 64), (32769, 16)])
 def test_numbers_of_calls_start_over(tokens, hidden):
     plan = B.Plan(torch.float16, hidden, tokens, 6.0, [2, 4, 8], 0.2)
     ws = plan.alloc(1)[1]
@@ -51,6 +52,23 @@ def test_calls_one_after_another_with_other_inputs(variant):
     assert plan.workspace_status(ws) == (0, 0)
     for x, blob in zip(xs, blobs):
         assert_blobs_equal(blob.cpu().numpy(), reference(x, variant=variant))
+
+
+@pytest.mark.parametrize("hidden", [2048, 3072, 4096])
+def test_both_sides_of_the_line_between_the_pack_shapes(hidden):
+    segments = hidden // 1024
+    line = 120 * torch.cuda.get_device_properties(0).multi_processor_count // segments
+    plan = B.Plan(torch.bfloat16, hidden, line + 1, 6.0, [2, 4, 8], 0.2)
+    ws = plan.alloc(1)[1]
+    few = rows_of_every_kind(500, hidden, torch.bfloat16, hidden)
+    x = few.repeat((line + 500) // 500, 1)[: line + 1].contiguous()
+    ref = reference(x[: line + 1])
+    blob = torch.zeros(plan.sizes(line + 1)[0], dtype=torch.uint8, device="cuda")
+    plan.encode(x.cuda(), blob, ws)
+    assert_blobs_equal(blob.cpu().numpy(), ref)
+    blob = torch.zeros(plan.sizes(line)[0], dtype=torch.uint8, device="cuda")
+    plan.encode(x[:line].cuda(), blob, ws)
+    assert_blobs_equal(blob.cpu().numpy(), reference(x[:line]))
 
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
