@@ -52,10 +52,10 @@ KERNEL_SOURCES = {
     "decode": ("tsq_decode.cu", "tsq_device.cuh", "tsq_internal.h"),
 }
 NCU_TRAFFIC = {
-    "encode": {"sha256": "5a49023ccf10a782890c3d493245c8ae20b796c407656da3e52aa0b62b8118ae",  # both kernels
-               "bytes_per_token": (134260000 + 6280000 + 122980000 + 62720000) / 8192, "hidden": 8192, "dtype": "bf16"},
-    "decode": {"sha256": "d8ab6337f0ac1e5b270ed71b13b2abfb4f0f596dac117d2a668a47a0e4133a3f",
-               "bytes_per_token": (68620000 + 132850000) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "encode": {"sha256": "d989553c1d55d1a7ed3d5d4bf76418772445e85b293a0db041c70b43cd43ca87",  # both kernels
+               "bytes_per_token": (134260000 + 6780000 + 134280000 + 62880000) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "decode": {"sha256": "3d4351c9dbf7a28ed5fe0cdf1ce75e5421140b92b13577e16bf4708fe800f7f6",
+               "bytes_per_token": (68620000 + 132950000) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
 KERNEL_NAMES = {"encode": "sizes_kernel + pack_kernel (encode_rows_kernel for few rows)", "decode": "decode_kernel"}
 

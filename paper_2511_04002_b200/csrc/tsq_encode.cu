@@ -19,10 +19,10 @@
 // off by a row's time) were all slower: in token order every row waits for the slowest of the rows before it, and a few rows in a
 // hundred take Algorithm 1 further than the first candidate (8192 x 8192 bf16 / 32768 x 4096 bf16 with 1 % outliers, us: persistent CTAs with a
 // ring of packed rows 87 / 190, one CTA per row 104 / 281, placement a row later 87 / 349, these kernels at that time 65 / 126; CTAs that stay, with
-// the present arithmetic, a ring of two packed rows and cells instead of look-back 72 / 215).
+// the present arithmetic, a ring of two packed rows and cells instead of look-back 72 / 205).
 //
-// What binds: DRAM and instruction issue about equally.  The two kernels move 326 MB at 8192 x 8192 bf16 (x twice, 8 % of the
-// second time from L2; 50 us at the copy rate) and issue in two cycles out of three.  So the passes work on two 16-bit elements
+// What binds: instruction issue, and DRAM close behind it.  The two kernels issue in two cycles out of three, whether a turn of CTAs finds its input in
+// L2 or not, and move 338 MB at 8192 x 8192 bf16 (x twice; 52 us at the copy rate).  So the passes work on two 16-bit elements
 // per 32-bit register and on two binary32 values per 64-bit register wherever they can, and what a row costs once is kept short.
 //
 // Arithmetic contract: the codes equal  clamp(rint(m / s) - zp, 0, Qmax)  with the IEEE binary32
