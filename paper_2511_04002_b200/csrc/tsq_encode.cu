@@ -60,6 +60,7 @@ __device__ __forceinline__ uint32_t row_entry(uint32_t outliers, int b, uint32_t
 constexpr uint32_t kCellShift = 51u;
 constexpr unsigned long long kCellRow = 1ull << kCellShift;
 constexpr uint32_t kCells32 = 64u, kCells1024 = 66u, kCells32768 = 68u, kCallWord = 70u;  // from block_at
+constexpr uint32_t kUnfit = 1u << 31;  // beside the call's number: the workspace is not fit for the call, no row is to be written
 
 __device__ __forceinline__ unsigned long long* slot_of(const EncodeParams& p, uint32_t row) { return p.desc + block_at(row) + 2u * (row & 31u); }
 // A slot is one 128-bit word, so that what is read of it belongs together: the tag, the entry, the scale and the zero-point.
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
     if ((tile & 31u) == 0u) {
       const uint32_t ticket = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket);
       const uint32_t has_cells = *reinterpret_cast<volatile const uint32_t*>(&p.ws->desc_capacity);
-      st_relaxed_u64(p.desc + block_at(tile) + kCallWord, ticket == 0u && p.tokens <= max(has_cells, p.cleared_rows) ? call : 0u);
+      st_relaxed_u64(p.desc + block_at(tile) + kCallWord, ticket == 0u && p.tokens <= max(has_cells, p.cleared_rows) ? call : call | kUnfit);
       __threadfence();
     }
     // The second kernel's CTAs start once every CTA here has come this far: they find the call's number, and every row that they may have to wait for
@@ -439,7 +440,8 @@ struct Place {
   uint32_t word_off, out_base, entry;
   float s;
   int zp;
-  uint32_t call;  // 0: the row is not to be written
+  uint32_t call;
+  bool known;  // false: the row is not to be written
 };
 template <int NW>
 struct PackShared {
@@ -453,13 +455,13 @@ __device__ __forceinline__ void load_cells(const unsigned long long* c, unsigned
 
 // Place of row `tile` by one warp: its own slot and those of the rows before it in its block of 32, the blocks of 32 before it in its block of 1024, those of
 // 1024 in its block of 32768, those of 32768 before it: four loads per lane, all in one round trip (both turns' cells: the call's number arrives with
-// them).  Returns the call's number, or ~0 while not all of these rows have been sized.
-__device__ __forceinline__ uint32_t place_row(const EncodeParams& p, uint32_t tile, Place& out) {
+// them).  Returns false while not all of these rows have been sized.
+__device__ __forceinline__ bool place_row(const EncodeParams& p, uint32_t tile, Place& out) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t row = (tile & ~31u) + lane, g = (tile & ~1023u) + 32u * lane, q = (tile & ~32767u) + 1024u * lane;
   constexpr unsigned long long kSums = kCellRow - 1u, k32 = 32ull << kCellShift, k1024 = 1024ull << kCellShift;
   unsigned long long lo = 0ull, hi = 0ull, g0 = k32, g1 = k32, q0 = k1024, q1 = k1024;
-  const uint32_t call = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord));
+  const uint32_t word = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord)), call = word & ~kUnfit;
   if (row <= tile) load_slot(slot_of(p, row), lo, hi);
   if (g + 31u < tile) load_cells(p.desc + block_at(g) + kCells32, g0, g1);
   if (q + 1023u < tile) load_cells(p.desc + block_at(q) + kCells1024, q0, q1);
@@ -476,9 +478,9 @@ __device__ __forceinline__ uint32_t place_row(const EncodeParams& p, uint32_t ti
   }
   const uint32_t words = __reduce_add_sync(kFull, static_cast<uint32_t>(part >> 32)) * p.lay.wpp;
   const uint32_t outliers = __reduce_add_sync(kFull, static_cast<uint32_t>(part));
-  all = __all_sync(kFull, all) || call == 0u;
-  if (row == tile) out = Place{words, outliers, entry, __uint_as_float(static_cast<uint32_t>(hi)), static_cast<int>(hi >> 32), all ? call : 0u};
-  return all ? call : 0xffffffffu;
+  all = __all_sync(kFull, all);
+  if (row == tile) out = Place{words, outliers, entry, __uint_as_float(static_cast<uint32_t>(hi)), static_cast<int>(hi >> 32), call, all && word == call};
+  return all || word != call;
 }
 
 // The same, waited for.  The rows are being sized, so the wait ends; it has a limit for a workspace that two calls use at once, or that something else has
@@ -486,7 +488,7 @@ __device__ __forceinline__ uint32_t place_row(const EncodeParams& p, uint32_t ti
 // kernel (given_up there).
 __device__ __noinline__ void wait_for_place(const EncodeParams& p, uint32_t tile, Place& out) {
   const uint32_t state4 = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord)) << 2;
-  for (uint32_t polls = 1u; place_row(p, tile, out) == 0xffffffffu; ++polls) {
+  for (uint32_t polls = 1u; !place_row(p, tile, out); ++polls) {
     uint32_t over = 0u;
     if (polls > 32u && (threadIdx.x & 31u) == 0u) {
       __nanosleep(1000u);
@@ -497,7 +499,7 @@ __device__ __noinline__ void wait_for_place(const EncodeParams& p, uint32_t tile
       }
       if (over != 0u) atomicCAS(&p.ws->enc_status, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
     }
-    if (__shfl_sync(kFull, over, 0) != 0u) return;  // (out.call is 0)
+    if (__shfl_sync(kFull, over, 0) != 0u) return;  // (out.known is false)
   }
 }
 
@@ -523,7 +525,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (FULL || c0 + 32u * i < p.chunks) cp_async16(dst + 32u * i, xrow + c0 + 32u * i);
     }
   }
-  if (warp == nwarps - 1u && place_row(p, tile, sh.place) == 0xffffffffu) wait_for_place(p, tile, sh.place);
+  if (warp == nwarps - 1u && !place_row(p, tile, sh.place)) wait_for_place(p, tile, sh.place);
   const uint32_t thr2 = p.thr16 * 0x10001u;
   uint32_t x[G][16], bitmap[G];
   cp_async_wait_all();
@@ -597,7 +599,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   const uint32_t mode = entry >> 21, row_cnt = entry & 0x1ffffu;
   const uint32_t agg_w = static_cast<uint32_t>(b) * p.lay.wpp;
   const uint32_t word_off = sh.place.word_off, out_base = sh.place.out_base, word_end = word_off + agg_w, out_end = out_base + row_cnt;
-  uint32_t status = call != 0u && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
+  uint32_t status = sh.place.known && static_cast<unsigned long long>(word_off) + agg_w <= p.lay.words_capacity ? TSQ_OK : TSQ_ERR_TIMEOUT;
   if (status == TSQ_OK) {
     uint32_t* wrow = reinterpret_cast<uint32_t*>(p.blob + p.lay.off_words) + word_off;
     if (!SV && mode >= kOneUp) {
@@ -681,13 +683,13 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
     if (tile == p.tokens - 1u) {
       // This CTA ends the call.  The grid after this one waits for this grid only: sizes_kernel must have ended by then.
       wait_for_prior_grids();
-      if (call == 0u || atomicMax(&p.ws->call_state, call << 2 | kCallEnded) == (call << 2 | kWaitRanOut)) status = TSQ_ERR_TIMEOUT;
+      if (atomicMax(&p.ws->call_state, call << 2 | kCallEnded) == (call << 2 | kWaitRanOut)) status = TSQ_ERR_TIMEOUT;
       if (status == TSQ_OK && out_end > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
       const bool ok = status != TSQ_ERR_TIMEOUT;
       end_part(p, status, ok ? word_end : 0u, ok ? out_end : 0u);
       if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
       next_generation(p, *reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u);
-      if (call != 0u && call != kCallWrap) p.ws->calls = call;
+      if (call != kCallWrap) p.ws->calls = call;  // (after a call that has failed as well: its slots carry the number)
     }
   }
   // ---- the cells that the next call adds to ----

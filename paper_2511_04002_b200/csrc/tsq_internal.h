@@ -62,11 +62,12 @@ __host__ __device__ inline BlobLayout make_layout(uint32_t hidden, unsigned long
 //     words 64 .. 69  cells: how many rows of a whole block have been sized, the sum of their bits, their outliers (kCellRow); two of each, used in turn.
 //                     The block's 32 rows: 64, 65; 1024 rows that start here: 66, 67; 32768 rows: 68, 69 (these count blocks of 1024).  A call adds
 //                     to the cells of its turn, which the call before it has left at 0, and clears those of the other.
-//     word 70         the call's number, or 0 where the workspace is not fit for it, for the second kernel's CTAs of these rows.
+//     word 70         the call's number, with a mark (kUnfit) where the workspace is not fit for it, for the second kernel's CTAs of these rows.
 //   Slots and cells tell by themselves whether they are complete: the second kernel starts while the first still runs.
 // Where a word is does not depend on the number of tokens, so a workspace may serve plans of different sizes, as far as it has been
 // initialised: cells must be 0 when a call adds to them, and every call clears those of desc_capacity rows.  A call of two kernels with more
-// rows than that writes no row and ends with TSQ_ERR_TIMEOUT.  (Slots need no such bound: their tags tell.)
+// rows than that writes no row and ends with TSQ_ERR_TIMEOUT.  (Slots need no such bound: their tags tell.)  Every call has a number of its own, whatever
+// its status, and clears the other turn's cells: the call behind one that has failed finds nothing that it could take for its own.
 // (The two kinds apart, because one-kernel calls are sensitive to where their words are: 128 x 4096 in 5.99 us with words at a stride of 16 bytes,
 // 6.10 with a gap every 32 rows, 6.12 at 8 or 32 bytes.  Cells in lines of their own: 10000 x 2048 27.6 us, 27.9 behind the slots in 72 words; 32 bytes
 // per row with the cells between the slots 30.0.)
