@@ -144,8 +144,9 @@ tsq_status_t tsq_workspace_init(const tsq_plan_t *plan, void *ws_dev, size_t ws_
  * Set how long the encoder's device-side waits may last before they give up with TSQ_ERR_TIMEOUT.  The
  * only such wait is for placement in calls of few rows: a row's offsets are the sums over every earlier row, and a
  * row polls the workspace until those rows have published their sizes.  (Calls of more rows go through two kernels: the second
- * starts while the first still runs and polls for rows that are being sized, with the built-in limit whatever is set here.  They end
- * with TSQ_ERR_TIMEOUT when the workspace is not as a finished call leaves it, or was initialised for fewer rows.)  `polls` counts polls of one
+ * starts while the first still runs and polls for rows that are being sized, but no longer than the first takes, which waits for
+ * nothing: no limit is needed there, and a sound call never runs out, whatever is set here.  They end with TSQ_ERR_TIMEOUT when the
+ * workspace is not as a finished call leaves it, or was initialised for fewer rows.)  `polls` counts polls of one
  * row's size: one round trip apart for the first 32, then 1 us apart.  0 restores the built-in limit of 2^20 polls (about one
  * second), which is also what tsq_workspace_init sets.  With the built-in limit a wait can only run out
  * when the workspace was not initialised, is shared by calls that overlap on the GPU, or was

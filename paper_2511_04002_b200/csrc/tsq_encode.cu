@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(MAXT, MINB) sizes_kernel(const __grid_constant
   uint32_t call = 0u;
   if (tid == 0u) {
     call = *reinterpret_cast<volatile const uint32_t*>(&p.ws->calls) + 1u;
+    if (tile == 0u) reinterpret_cast<BlobHeader*>(p.blob)->status = TSQ_OK;  // (fail_call)
     if ((tile & 31u) == 0u) {
       const uint32_t ticket = *reinterpret_cast<volatile const uint32_t*>(&p.ws->ticket);
       const uint32_t has_cells = *reinterpret_cast<volatile const uint32_t*>(&p.ws->desc_capacity);
@@ -453,6 +454,12 @@ __device__ __forceinline__ void load_cells(const unsigned long long* c, unsigned
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(c) : "memory");
 }
 
+// What a call of two kernels has found wrong, for its blob and the workspace.  sizes_kernel has set the blob's status to 0.
+__device__ __forceinline__ void fail_call(const EncodeParams& p, uint32_t status) {
+  atomicMax(&reinterpret_cast<BlobHeader*>(p.blob)->status, status);
+  atomicCAS(&p.ws->enc_status, 0u, status);
+}
+
 // Place of row `tile` by one warp: its own slot and those of the rows before it in its block of 32, the blocks of 32 before it in its block of 1024, those of
 // 1024 in its block of 32768, those of 32768 before it: four loads per lane, all in one round trip (both turns' cells: the call's number arrives with
 // them).  Returns false while not all of these rows have been sized.
@@ -483,24 +490,18 @@ __device__ __forceinline__ bool place_row(const EncodeParams& p, uint32_t tile, 
   return all || word != call;
 }
 
-// The same, waited for.  The rows are being sized, so the wait ends; it has a limit for a workspace that two calls use at once, or that something else has
-// written to.  A row that gives up is not written, so the call must not end with TSQ_OK: call_state decides as direct_state does for calls of one
-// kernel (given_up there).
+// The same, waited for: the rows are being sized, so the wait ends, at the latest with the first kernel, whose end is waited for after some polls (a row's
+// time is a few microseconds).  Where the place is not known even then, something else has written to the workspace, or two calls use it at once: the row is
+// not written, and the blob's status says so (whichever of this and the CTA of the last row comes first: the largest status stays).
+constexpr uint32_t kPollsOfPlace = 64u;
 __device__ __noinline__ void wait_for_place(const EncodeParams& p, uint32_t tile, Place& out) {
-  const uint32_t state4 = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord)) << 2;
-  for (uint32_t polls = 1u; !place_row(p, tile, out); ++polls) {
-    uint32_t over = 0u;
-    if (polls > 32u && (threadIdx.x & 31u) == 0u) {
-      __nanosleep(1000u);
-      if (polls > kPollLimit) {
-        over = atomicMax(&p.ws->call_state, state4 | kWaitRanOut) != (state4 | kCallEnded) || polls > kPollLimit + 64u ? 1u : 0u;
-      } else {
-        over = *reinterpret_cast<volatile const uint32_t*>(&p.ws->call_state) == (state4 | kWaitRanOut) ? 1u : 0u;
-      }
-      if (over != 0u) atomicCAS(&p.ws->enc_status, 0u, static_cast<uint32_t>(TSQ_ERR_TIMEOUT));
-    }
-    if (__shfl_sync(kFull, over, 0) != 0u) return;  // (out.known is false)
+  for (uint32_t polls = 1u; polls <= kPollsOfPlace; ++polls) {
+    if (place_row(p, tile, out)) return;
+    if (polls > kPollsOfPlace / 2u) __nanosleep(1000u);
   }
+  wait_for_prior_grids();
+  if (place_row(p, tile, out)) return;
+  if ((threadIdx.x & 31u) == 0u) fail_call(p, TSQ_ERR_TIMEOUT);
 }
 
 template <bool BF16, int G, bool SV, bool FULL, int MAXT, int MINB>
@@ -683,11 +684,10 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
     if (tile == p.tokens - 1u) {
       // This CTA ends the call.  The grid after this one waits for this grid only: sizes_kernel must have ended by then.
       wait_for_prior_grids();
-      if (atomicMax(&p.ws->call_state, call << 2 | kCallEnded) == (call << 2 | kWaitRanOut)) status = TSQ_ERR_TIMEOUT;
       if (status == TSQ_OK && out_end > p.lay.outlier_capacity) status = TSQ_ERR_OUTLIER_OVERFLOW;
       const bool ok = status != TSQ_ERR_TIMEOUT;
-      end_part(p, status, ok ? word_end : 0u, ok ? out_end : 0u);
-      if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
+      write_header(p, ok ? word_end : 0u, ok ? out_end : 0u);
+      if (status != TSQ_OK) fail_call(p, status);
       next_generation(p, *reinterpret_cast<volatile const uint32_t*>(&p.ws->gen) + 1u);
       if (call != kCallWrap) p.ws->calls = call;  // (after a call that has failed as well: its slots carry the number)
     }
@@ -709,7 +709,6 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (atomicAdd(&p.ws->done, 1u) == gridDim.x - 1u) {
         const uint32_t n = max(p.ws->desc_capacity, p.tokens);
         for (uint32_t i = 0; i < n; ++i) store_slot(slot_of(p, i), 0ull, 0ull);
-        p.ws->call_state = 0u;
         p.ws->calls = 0u;
         p.ws->done = 0u;
       }

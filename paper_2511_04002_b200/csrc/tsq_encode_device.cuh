@@ -577,7 +577,7 @@ __device__ void write_header(const EncodeParams& p, unsigned long long total_wor
   h->outlier_capacity = static_cast<uint32_t>(p.lay.outlier_capacity);
 }
 
-// Ends a call, or a part of one: header, status, end offsets.
+// Ends a call of one kernel, or a part of one: header, status, end offsets.
 __device__ void end_part(const EncodeParams& p, uint32_t status, unsigned long long total_words, unsigned long long total_outliers) {
   if (p.totals) {
     p.totals[0] = total_words;

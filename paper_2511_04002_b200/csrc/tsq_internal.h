@@ -82,8 +82,7 @@ struct WsControl {
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
   uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut or kCallEnded, only ever grows
   uint32_t calls;          // number of the last call of two kernels that has ended: read by the first, written by the second kernel
-  uint32_t call_state;     // as direct_state, for calls of two kernels: number * 4 + kWaitRanOut or kCallEnded
-  uint32_t pad[5];
+  uint32_t pad[6];
 };
 static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
 
