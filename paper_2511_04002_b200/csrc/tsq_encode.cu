@@ -462,13 +462,17 @@ __device__ __forceinline__ void fail_call(const EncodeParams& p, uint32_t status
 
 // Place of row `tile` by one warp: its own slot and those of the rows before it in its block of 32, the blocks of 32 before it in its block of 1024, those of
 // 1024 in its block of 32768, those of 32768 before it: four loads per lane, all in one round trip (both turns' cells: the call's number arrives with
-// them).  Returns false while not all of these rows have been sized.
-__device__ __forceinline__ bool place_row(const EncodeParams& p, uint32_t tile, Place& out) {
+// them).  The number comes from a word that the first kernel has just written, and nothing but where these loads go (past L1) says that the word is not the last
+// call's yet, whose slots and cells may still be complete.  So it has to be one more than the number of the last call that has ended, a word that no kernel
+// writes while this is read, but for the CTA that ends this call: kUnsure then, and the first kernel's end is waited for.  `ended`: that has been done.
+constexpr int kPlaced = 0, kNotSized = 1, kUnsure = 2;
+__device__ __forceinline__ int place_row(const EncodeParams& p, uint32_t tile, bool ended, Place& out) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t row = (tile & ~31u) + lane, g = (tile & ~1023u) + 32u * lane, q = (tile & ~32767u) + 1024u * lane;
   constexpr unsigned long long kSums = kCellRow - 1u, k32 = 32ull << kCellShift, k1024 = 1024ull << kCellShift;
   unsigned long long lo = 0ull, hi = 0ull, g0 = k32, g1 = k32, q0 = k1024, q1 = k1024;
   const uint32_t word = static_cast<uint32_t>(ld_relaxed_u64(p.desc + block_at(tile) + kCallWord)), call = word & ~kUnfit;
+  const uint32_t last = *reinterpret_cast<volatile const uint32_t*>(&p.ws->calls);
   if (row <= tile) load_slot(slot_of(p, row), lo, hi);
   if (g + 31u < tile) load_cells(p.desc + block_at(g) + kCells32, g0, g1);
   if (q + 1023u < tile) load_cells(p.desc + block_at(q) + kCells1024, q0, q1);
@@ -487,7 +491,8 @@ __device__ __forceinline__ bool place_row(const EncodeParams& p, uint32_t tile, 
   const uint32_t outliers = __reduce_add_sync(kFull, static_cast<uint32_t>(part));
   all = __all_sync(kFull, all);
   if (row == tile) out = Place{words, outliers, entry, __uint_as_float(static_cast<uint32_t>(hi)), static_cast<int>(hi >> 32), call, all && word == call};
-  return all || word != call;
+  if (!ended && call != last + 1u) return kUnsure;
+  return all || word != call ? kPlaced : kNotSized;
 }
 
 // The same, waited for: the rows are being sized, so the wait ends, at the latest with the first kernel, whose end is waited for after some polls (a row's
@@ -495,12 +500,14 @@ __device__ __forceinline__ bool place_row(const EncodeParams& p, uint32_t tile, 
 // not written, and the blob's status says so (whichever of this and the CTA of the last row comes first: the largest status stays).
 constexpr uint32_t kPollsOfPlace = 64u;
 __device__ __noinline__ void wait_for_place(const EncodeParams& p, uint32_t tile, Place& out) {
-  for (uint32_t polls = 1u; polls <= kPollsOfPlace; ++polls) {
-    if (place_row(p, tile, out)) return;
+  int state = kNotSized;
+  for (uint32_t polls = 1u; state == kNotSized && polls <= kPollsOfPlace; ++polls) {
+    state = place_row(p, tile, false, out);
+    if (state == kPlaced) return;
     if (polls > kPollsOfPlace / 2u) __nanosleep(1000u);
   }
   wait_for_prior_grids();
-  if (place_row(p, tile, out)) return;
+  if (place_row(p, tile, true, out) == kPlaced) return;
   if ((threadIdx.x & 31u) == 0u) fail_call(p, TSQ_ERR_TIMEOUT);
 }
 
@@ -526,7 +533,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
       if (FULL || c0 + 32u * i < p.chunks) cp_async16(dst + 32u * i, xrow + c0 + 32u * i);
     }
   }
-  if (warp == nwarps - 1u && !place_row(p, tile, sh.place)) wait_for_place(p, tile, sh.place);
+  if (warp == nwarps - 1u && place_row(p, tile, false, sh.place) != kPlaced) wait_for_place(p, tile, sh.place);
   const uint32_t thr2 = p.thr16 * 0x10001u;
   uint32_t x[G][16], bitmap[G];
   cp_async_wait_all();
@@ -694,7 +701,7 @@ __global__ void __launch_bounds__(MAXT, MINB) pack_kernel(const __grid_constant_
   }
   // ---- the cells that the next call adds to ----
   if (blockIdx.x < 32u) {
-    const uint32_t blocks = max(p.ws->desc_capacity, p.tokens) >> 5;
+    const uint32_t blocks = max(*reinterpret_cast<volatile const uint32_t*>(&p.ws->desc_capacity), p.tokens) >> 5;
     for (uint32_t i = blockIdx.x * nt + tid; i < blocks; i += min(gridDim.x, 32u) * nt) {
       unsigned long long* c = p.desc + block_at(32u * i) + ((call & 1u) ^ 1u);
       c[kCells32] = 0ull;

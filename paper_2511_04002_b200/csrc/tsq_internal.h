@@ -138,8 +138,9 @@ struct DecodeParams {
 };
 
 // Launch with programmatic stream serialisation: the grid's CTAs may be set up while the stream's previous grid still runs
-// (where that is one of this library's kernels, which allow it from their start), and each begins with
-// wait_for_prior_grids().  Only the launch overlaps: a kernel reads and writes nothing before that wait.
+// (where that is one of this library's kernels, which allow it from their start).  All but pack_kernel begin with wait_for_prior_grids() and
+// read and write nothing before it: only the launch overlaps.  pack_kernel follows sizes_kernel, whose CTAs have all been through that wait
+// when it starts, and reads the input and what sizes_kernel publishes without it.
 template <typename... Args>
 cudaError_t launch_overlapped(void (*kernel)(Args...), int grid, int threads, size_t smem, cudaStream_t stream, const Args&... args) {
   cudaLaunchConfig_t config = {};
