@@ -103,7 +103,7 @@ __device__ __forceinline__ void finish_direct(const EncodeParams& p, uint32_t ge
   const bool ok = status != TSQ_ERR_TIMEOUT;
   end_part(p, status, ok ? total_w : 0ull, ok ? total_o : 0ull);
   if (status != TSQ_OK) atomicCAS(&p.ws->enc_status, 0u, status);
-  p.ws->ticket = 0u;  // every CTA has taken its own
+  if (p.direct_tiles == kByIndex) p.ws->ticket = 0u;  // (rows by ticket: the CTA that has taken the last one)
   p.ws->gen = gen4 >> 2;
 }
 
@@ -134,7 +134,14 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_rows_kernel(const __grid_co
 
   uint32_t tile = blockIdx.x;
   if (DIRECT != kByIndex) {
-    if (tid == 0) sh.tile = atomicAdd(&p.ws->ticket, 1u);
+    if (tid == 0) {
+      // the number in the lower half, how many CTAs have taken theirs in the upper: the last to take one re-arms the counter.  (The CTA that ends the call must
+      // not: where a call starts with a counter that is not 0, so that rows are missing, CTAs that have not taken theirs yet would be given the first rows,
+      // as of the next call, and the next part of a host-buffer call would wait for a limit of its own.)
+      const uint32_t t = atomicAdd(&p.ws->ticket, 0x10001u);
+      if ((t >> 16) == gridDim.x - 1u) p.ws->ticket = 0u;
+      sh.tile = t & 0xffffu;
+    }
     __syncthreads();
     tile = sh.tile;
   }

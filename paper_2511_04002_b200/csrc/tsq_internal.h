@@ -73,7 +73,7 @@ __host__ __device__ inline BlobLayout make_layout(uint32_t hidden, unsigned long
 // per row with the cells between the slots 30.0.)
 struct WsControl {
   uint32_t gen;          // generation of the last finished encode
-  uint32_t ticket;       // next tile to hand out (self-resetting)
+  uint32_t ticket;       // next row to hand out, and from bit 16 how many CTAs have taken one (0 between calls)
   uint32_t done;         // CTAs that have finished (self-resetting)
   uint32_t err;          // first error of the running encode
   uint32_t enc_status;   // first encode error since init (sticky)
