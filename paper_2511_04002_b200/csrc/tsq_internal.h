@@ -80,14 +80,14 @@ struct WsControl {
   uint32_t dec_status;   // first decode error since init (sticky)
   uint32_t desc_capacity;  // rows whose slots and cells init has cleared
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
-  uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut or kCallEnded, only ever grows
+  uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut, kCallEnded or kEndedRanOut, only ever grows
   uint32_t calls;          // number of the last call of two kernels that has ended: read by the first, written by the second kernel
   uint32_t pad[6];
 };
 static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
 
 constexpr uint32_t kFlagAggregate = 1;
-constexpr uint32_t kWaitRanOut = 1, kCallEnded = 2;  // direct_state
+constexpr uint32_t kWaitRanOut = 1, kCallEnded = 2, kEndedRanOut = 3;  // direct_state
 constexpr uint32_t kGenWrap = (1u << 30) - 2;
 constexpr uint32_t kCallWrap = (1u << 30) - 2;      // calls of two kernels are numbered 1 .. kCallWrap (even: the cells go on in turn)
 

@@ -1,4 +1,6 @@
 """Parts of host-buffer calls with more rows than SMs: the one-kernel encoder with rows by ticket, which no other call takes."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -9,6 +11,10 @@ from paper_2511_04002_b200 import binding as B
 pytestmark = pytest.mark.gpu
 TIMEOUT = 7
 TICKET = 1                                                     # 32-bit word of the workspace's control block
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
 
 
 class Call:
@@ -55,3 +61,22 @@ def test_a_part_without_its_first_row_leaves_the_next_ones_theirs(hidden, part):
         assert np.array_equal(call.blob[at + part:at + T].cpu().numpy(), want)
     call.plan.workspace_init(call.ws)
     assert call() == 0
+
+
+def test_one_limit_for_a_part_of_two_turns():
+    # the last row's CTA ends the call while other CTAs of the second turn have just started to poll: they must find that a wait has run out, not that the call
+    # has ended, after which they would wait for a limit of their own
+    part, hidden = 6 * sms(), 8200
+    x = torch.randn((3 * part, hidden), generator=torch.Generator().manual_seed(1)).to(torch.bfloat16)
+    call = Call(B.Plan(torch.bfloat16, hidden, 3 * part, 6.0, [2, 4, 8], 0.2), x)
+    assert call() == 0
+    ms = []
+    for _ in range(24):
+        call.plan.workspace_init(call.ws)
+        call.plan.workspace_set_wait_limit(call.ws, 20000)
+        call.word(TICKET, 1)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        assert call() == TIMEOUT
+        ms.append(1e3 * (time.perf_counter() - t0))
+    assert max(ms) < 1.5 * min(ms), ms                         # one limit, not two
