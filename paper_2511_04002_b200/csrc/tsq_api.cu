@@ -227,6 +227,7 @@ const char* tsq_status_string(tsq_status_t status) {
 uint64_t tsq_kernel_launch_count(void) { return g_launches.load(); }
 
 static int64_t direct_rows(const tsq_plan_t* plan);
+static int64_t longest_part(const tsq_plan_t* plan);
 tsq_status_t tsq_plan(tsq_plan_t** out, int device, tsq_dtype_t dtype, int32_t hidden, int64_t max_tokens, float tau,
                       const int32_t* bits, int32_t n_bits, float delta, int64_t max_outliers) {
   return tsq_plan_variant(out, device, dtype, hidden, max_tokens, tau, bits, n_bits, delta, max_outliers, TSQ_VARIANT_MAGNITUDES);
@@ -302,9 +303,9 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
     kernel_of.n_bits = n_bits;
     for (int i = 0; i < 8; ++i) kernel_of.bits[i] = p->bits[i];
     p->ends_in_4_and_8 = ends_in_4_and_8(kernel_of);
-    // only what calls of max_tokens can take: the occupancy queries are most of what a plan costs
+    // only what calls of max_tokens, or parts of them, can take: the occupancy queries are most of what a plan costs
     p->sms = sms;
-    const int64_t rows = static_cast<int64_t>(T);
+    const int64_t rows = std::min<int64_t>(static_cast<int64_t>(T), longest_part(p));
     for (int i = 0; i < 3; ++i) {
       p->rows_ctas[i] = i > 0 ? p->rows_ctas[i - 1] : 0;
       if (i == 0 || rows > static_cast<int64_t>(sms) * p->rows_ctas[i]) {
@@ -312,7 +313,7 @@ tsq_status_t tsq_plan_variant(tsq_plan_t** out, int device, tsq_dtype_t dtype, i
       }
     }
     p->two_pass = two_pass_shape(kernel_of);
-    if (rows > direct_rows(p)) ok = ok && two_pass_attrs(kernel_of, p->two_pass) == cudaSuccess;
+    if (static_cast<int64_t>(T) > direct_rows(p)) ok = ok && two_pass_attrs(kernel_of, p->two_pass) == cudaSuccess;
   }
   cudaSetDevice(prev_dev);
   if (!ok || sms < 1) {
@@ -425,9 +426,12 @@ static bool few_rows(const tsq_plan_t* plan, int64_t tokens) {
   return segments <= kFewSegments && (segments % 2 == 1 || tokens * segments <= 120 * static_cast<int64_t>(plan->sms));
 }
 
+// Rows of the longest part of a host-buffer call (part_rows): a part is a call of one kernel.
+static int64_t longest_part(const tsq_plan_t* plan) { return std::min<int64_t>(6 * static_cast<int64_t>(plan->sms), kOneKernelRows); }
+
 // Instance of the one-kernel encoder: 128, 80 or 64 registers, so more CTAs per SM with each.  The one
 // that takes the rows in the fewest turns (a sixteenth of a turn more does not count), of those the one with the most registers:
-// 2048 x 5120 37.1, 33.2 and 30.5 us, 1500 x 4096 19.7, 17.6 and 19.6 us, 600 x 4096 10.2, 12.3 and 12.3 us.
+// 600 x 4096 10.2, 12.3 and 12.3 us.  (Only parts of host-buffer calls, longest_part, have more than a row per SM.)
 static int rows_instance(const tsq_plan_t* plan, int64_t tokens) {
   int best = 0;
   int64_t fewest = INT64_MAX;
@@ -455,7 +459,7 @@ static tsq_status_t enqueue_encode(const tsq_plan_t* plan, const void* x_dev, in
   // few rows: one CTA per row (a call without rows still launches one CTA, which writes the header).  Up to one CTA per SM is
   // resident whatever the CTA's size: such a call needs no tickets.
   const int grid = tokens > 0 ? static_cast<int>(tokens) : 1;
-  p.direct_tiles = tokens <= plan->sms ? 1u : 2u;
+  p.direct_tiles = 1u;
   const cudaError_t e = launch_encode_rows(p, grid, plan->enc_threads, plan->enc_upt, rows_instance(plan, tokens), static_cast<cudaStream_t>(cuda_stream));
   g_launches.fetch_add(1);
   return e == cudaSuccess ? TSQ_OK : TSQ_ERR_CUDA;
@@ -587,7 +591,7 @@ static int64_t part_rows(const tsq_plan_t* plan, int64_t tokens) {
   if (cudaGetDevice(&device) != cudaSuccess || device != plan->device) return tokens;  // the copy streams belong to the plan's device
   const int64_t row = static_cast<int64_t>(plan->row_bytes), parts = std::min<int64_t>(3, tokens * row / (4 << 20));
   if (parts < 2) return tokens;
-  const int64_t rows = std::min((tokens + parts - 1) / parts, 6 * static_cast<int64_t>(plan->sms));
+  const int64_t rows = std::min((tokens + parts - 1) / parts, longest_part(plan));
   return rows * row < (1 << 20) ? tokens : rows;
 }
 

@@ -81,7 +81,7 @@ struct WsControl {
   uint32_t desc_capacity;  // rows whose slots and cells init has cleared
   uint32_t poll_limit;     // polls before a device-side wait gives up; 0 = the built-in limit
   uint32_t direct_state;   // calls with direct offsets: generation * 4 + kWaitRanOut, kCallEnded or kEndedRanOut, only ever grows
-  uint32_t calls;          // number of the last call of two kernels that has ended: read by the first, written by the second kernel
+  uint32_t calls;          // number of the last call of two kernels that has ended: read by both kernels, written by the second as the call ends
   uint32_t pad[6];
 };
 static_assert(sizeof(WsControl) == 64, "control block is 64 bytes");
