@@ -131,8 +131,8 @@ tsq_status_t tsq_plan_sizes(const tsq_plan_t *plan, int64_t tokens, tsq_sizes_t 
 
 /*
  * Zero a workspace (DEVICE, workspace_bytes, 16-byte aligned) on `cuda_stream`.  Required once
- * before the buffer's first use and after any TSQ_ERR_TIMEOUT; encode and decode leave it ready
- * for the next call.  One workspace serves one call at a time: calls that may overlap on the GPU
+ * before the buffer's first use and after any TSQ_ERR_TIMEOUT or TSQ_ERR_CUDA; encode and decode leave it ready
+ * for the next call otherwise.  One workspace serves one call at a time: calls that may overlap on the GPU
  * need separate workspaces.  A workspace that plans of different max_tokens share is to be initialised
  * through the plan with the most: it is cleared as far as that plan needs it, and a call of two kernels
  * (tsq_encode) with more rows writes no row and ends with TSQ_ERR_TIMEOUT.  (Variable-length placement, the prefix sums behind word_off and
@@ -161,7 +161,7 @@ tsq_status_t tsq_workspace_set_wait_limit(void *ws_dev, uint32_t polls, void *cu
 /*
  * Encode x (DEVICE, [tokens x hidden]) into blob (DEVICE, >= blob_bytes from tsq_plan_sizes,
  * 16-byte aligned): TS (Eq. "ts") + TAB-Q (Algorithm 1, token-wise) + bit-plane packing, one
- * kernel launch, or two for calls of more rows than the device has SMs.  tokens == 0 writes an empty, valid blob.  Returns argument errors before
+ * kernel launch, or two for calls of more rows than the device has SMs (signed values: more than 8).  tokens == 0 writes an empty, valid blob.  Returns argument errors before
  * anything is enqueued.
  */
 tsq_status_t tsq_encode(const tsq_plan_t *plan, const void *x_dev, int64_t tokens, void *blob_dev,

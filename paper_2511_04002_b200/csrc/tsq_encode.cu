@@ -801,7 +801,12 @@ cudaError_t launch_encode_two_pass(const EncodeParams& p, const TwoPassShape& s,
   const int grid = static_cast<int>(p.tokens);
   const PackShape& pack = few ? s.pack_few : s.pack;
   const cudaError_t e = launch_overlapped(sizes_of(p, s), grid, s.sizes_threads, 0, stream, p);
-  return e != cudaSuccess ? e : launch_overlapped(pack_of(p, pack), grid, pack.threads, pack.smem, stream, p);
+  if (e != cudaSuccess) return e;
+  const cudaError_t e2 = launch_overlapped(pack_of(p, pack), grid, pack.threads, pack.smem, stream, p);
+  // Without the second kernel nobody advances the number that the first has left slots and cells under, and the next call would take them for its own:
+  // the workspace counts as not initialised from here on.
+  if (e2 != cudaSuccess) cudaMemsetAsync(&p.ws->desc_capacity, 0, sizeof p.ws->desc_capacity, stream);
+  return e2;
 }
 
 }  // namespace tsq
