@@ -52,10 +52,10 @@ KERNEL_SOURCES = {
     "decode": ("tsq_decode.cu", "tsq_device.cuh", "tsq_internal.h"),
 }
 NCU_TRAFFIC = {
-    "encode": {"sha256": "d989553c1d55d1a7ed3d5d4bf76418772445e85b293a0db041c70b43cd43ca87",  # both kernels
-               "bytes_per_token": (134260000 + 6780000 + 134280000 + 62880000) / 8192, "hidden": 8192, "dtype": "bf16"},
-    "decode": {"sha256": "3d4351c9dbf7a28ed5fe0cdf1ce75e5421140b92b13577e16bf4708fe800f7f6",
-               "bytes_per_token": (68620000 + 132950000) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "encode": {"sha256": "3ad56d2c10611ffcb48192ebd50e7325bfa0fb8cea32b4f6828eb59f12b94fc7",  # both kernels
+               "bytes_per_token": (134270000 + 6840000 + 134280000 + 62600000) / 8192, "hidden": 8192, "dtype": "bf16"},
+    "decode": {"sha256": "abb607620f1b51a17588ccd966fcd0cff2b5e4be6bbf6552234c61fe0f9d55fc",
+               "bytes_per_token": (68620000 + 133010000) / 8192, "hidden": 8192, "dtype": "bf16"},
 }
 KERNEL_NAMES = {"encode": "sizes_kernel + pack_kernel (encode_rows_kernel for few rows)", "decode": "decode_kernel"}
 

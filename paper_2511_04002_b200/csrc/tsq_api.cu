@@ -408,7 +408,8 @@ static EncodeParams encode_params(const tsq_plan_t* plan, const void* x_dev, int
 // row before it, and with more than one row per SM the rows have to be numbered by ticket.  us, one kernel / two, each pair on the same tensors (bf16 or
 // fp16, normal values with 0.1 % outliers):
 //   up to a row per SM   64 x 4096  5.4 / 6.5    100 x 4096  5.7 / 6.4    148 x 4096  5.0 / 6.6    148 x 8192  5.2 / 7.1    148 x 10240 6.4 / 7.4    148 x 24576 8.4 / 10.5
-//     (rows of 8200 to 16384 elements lie on both sides: 32 x 16384 5.9 / 6.8, 64 x 16384 7.5 / 6.7, 100 x 12288 8.6 / 7.9)
+//     (not all: 32 x 16384 5.9 / 6.8, but 64 x 16384 7.5 / 6.7 and 100 x 12288 8.6 / 7.9.  The line is the same for all lengths, and calls of 64 to 148 rows of
+//     8200 to 16384 elements are on the slower side of it.)
 //   more                149 x 1024  6.3 / 6.1    149 x 4096  6.9 / 6.5    149 x 8192  7.3 / 7.2    149 x 16384 10.3 / 8.0   149 x 32768 16.0 / 14.6
 //                       600 x 1024  8.0 / 6.5    300 x 4096  7.0 / 6.9    777 x 3000 10.3 / 8.3    700 x 4096 10.1 / 8.5    600 x 8192 11.6 / 10.2
 // Signed values: one row in ten has a code that needs the clamp, which the one kernel forms by the division instruction (1 x 4096 4.1 / 5.9,

@@ -13,7 +13,7 @@
 //                  the first row on, while the last rows are still being sized; every row they may wait for is being sized by then.
 // The overlap fills the last, partly empty turn of the first kernel's CTAs and hides the second one's start (us, the second kernel behind the first / so:
 // 777 x 3000 bf16 10.9 / 8.6, 2048 x 5120 fp16 19.8 / 18.8, 4000 x 3000 25.1 / 20.5, 4096 x 4096 24.8 / 22.3, 10000 x 2048 32.4 / 27.6, 2000 x 16384 41.0 / 38.1, signed
-// 2048 x 5120 25.7 / 22.4, 8192 x 8192 62.4 / 61.6, 32768 x 4096 121.7 / 121.2).  What the place costs to read decides whether it pays: with every warp
+// 2048 x 5120 25.7 / 22.4; 8192 x 8192 62.4 / 61.6 and 32768 x 4096 121.7 / 121.2 differ by no more than calls timed in turn do).  What the place costs to read decides whether it pays: with every warp
 // reading its slot (relaxed loads go past L1) 8192 x 8192 took 66.7 us.
 // x is read twice.  The forms that read it once (rows in shared memory or in registers, placement at once, by look-back, or put
 // off by a row's time) were all slower: in token order every row waits for the slowest of the rows before it, and a few rows in a

@@ -86,7 +86,8 @@ __device__ __forceinline__ Level2 make_level2(const Level& c) {
 }
 // The signed values of the two elements of a 16-bit pair as packed binary32, each by a mixed addition of -0 (exact, for subnormal values too).  That takes
 // one cycle of the FMA pipe per element, where the conversion of a binary16 value takes two and a bfloat16 pair took a multiply-add and a logic
-// instruction, which are half rate both: encode 8192 x 8192 62.2 -> 60.9 us fp16 and 63.2 -> 62.6 bf16, signed 2048 x 5120 fp16 29.6 -> 25.7.
+// instruction, which are half rate both: encode 8192 x 8192 62.2 -> 60.9 us fp16, signed 2048 x 5120 fp16 29.6 -> 25.7 (8192 x 8192 bf16 63.2 -> 62.6 is
+// within what two runs differ by).
 template <bool BF16>
 __device__ __forceinline__ uint64_t values2(uint32_t x) {
   float lo, hi;
